@@ -116,13 +116,14 @@ typedef struct {
 
 /* Statistics of the last cf_count / cf_batch_count call on a context. */
 typedef struct {
-    int64_t evaluated_pairs;   /* separations computed by the pair kernel (i x j per work item) */
+    int64_t evaluated_pairs;   /* pairs the pair kernel resolves: i x j per work item (those it rules out
+                                  by a bounding box, without forming the separation, among them) */
     int64_t rechecked_pairs;   /* pairs within the FP32 error band of an edge, redone in FP64 */
     int64_t work_items;        /* (i tile, j range) items of the pair kernel */
     int64_t cells;             /* cells per catalogue */
     int grid[3];               /* cells per axis */
     int refine[3];             /* refinement used */
-    int variant;               /* pair kernel variant used */
+    int variant;               /* pair kernel form used (always 1: one form is built) */
     int ncat;                  /* catalogues in the call */
     float ms_build;            /* cell build + work list (CUDA events) */
     float ms_pair;             /* pair kernel (CUDA events on the context stream) */
@@ -142,8 +143,8 @@ cf_status cf_destroy(void *ctx);
 const char *cf_last_error(const void *ctx);
 
 /* Options (0 = default).  CF_OPT_MEM_CAP caps the context's device scratch in bytes so that
- * a request above it fails with CF_ERR_OOM instead of allocating; CF_OPT_VARIANT pins the
- * pair-kernel variant; CF_OPT_TILE pins the i-tile size (32..128); CF_OPT_JCHUNK pins the
+ * a request above it fails with CF_ERR_OOM instead of allocating; CF_OPT_VARIANT is
+ * accepted without effect (the pair kernel has one form); CF_OPT_TILE pins the i-tile size (32..128); CF_OPT_JCHUNK pins the
  * j range length per work item; CF_OPT_QUEUE sets the FP64 recheck queue capacity;
  * CF_OPT_CTAS_PER_SM sets the persistent grid; CF_OPT_AUDIT = 1 sends every pair the pair
  * kernel evaluates to the FP64 recheck instead of binning it in FP32, so the call returns the FP64
@@ -161,8 +162,8 @@ typedef enum {
     CF_OPT_CTAS_PER_SM = 6,
     CF_OPT_AUDIT = 7,
     CF_OPT_ITER_LIMIT = 8,
-    CF_OPT_WARPS = 9,        /* warps per CTA of the pair kernel: up to 16 for the direct form with
-                                weights or ravg, up to 8 otherwise (0 = as many as fit) */
+    CF_OPT_WARPS = 9,        /* warps per CTA of the pair kernel: up to 16 with weights or ravg, up to 8
+                                otherwise (0 = as many as fit) */
     CF_OPT_REFINE = 10,      /* refinement factor used when params.refine is 0 */
     CF_OPT_CELL_PRUNE = 11,  /* 0 (default): skip cell pairs whose points' bounding boxes lie farther
                                 apart than the largest edge (and pimax along z for rp-pi / wp);
@@ -215,10 +216,11 @@ cf_status cf_get_stats(const void *ctx, cf_stats *out);
  * (npibins+1 values, rp-pi / wp / mocks) receive the FP32 error band of each squared edge / pi
  * edge (mocks: of each squared pi edge):
  * an FP32 value within a band of an edge is re-evaluated in FP64.  With nv > 0, `values` are
- * classified through the same lookup table the pair kernel uses (which = 0: squared r / rp /
+ * classified through the full lookup table (which decides every pair near an edge in the pair kernel;
+ * the kernel's smaller table and its pi multiplication agree with it elsewhere) (which = 0: squared r / rp /
  * chord; which = 1: |dz|, or pi^2 for mocks): classes[i] = bin index, 0xFE outside every bin, 0xFF within a band.
- * which = 2 / 3 classify the same way as the direct pair kernel does (an FP32 cut at the table's
- * tail, then the lookup without its upper clamp); 0xFD there would mean an index past the table.
+ * which = 2 / 3 classify with an FP32 cut at the table's tail in place of the lookup's upper clamp;
+ * 0xFD there would mean an index past the table.
  * Adding 4 to `which` plans DD(theta) on the angular grid (CF_OPT_THETA_GRID = 1): grid[] then
  * reports the bands, the most RA cells of a band, and 1. 
  * Grid and refinement: Sec. 4.1-4.2; bins in squared space: Sec. 4.7. */

@@ -205,15 +205,7 @@ static int check_points(CfCtx *C, const cf_params *p, const cf_points *d)
     } while (0)
 #define CF_CU(x, what) CF_TRY(C->cuda((x), what))
 
-// the work list and the order the pair kernel takes it in (one index per item, then the ordering
-// pass's per-block class sizes)
-static int ensure_items(CfCtx *C, size_t cap)
-{
-    cap = std::max<size_t>(1, cap);
-    CF_TRY(C->ensure(B_ITEMS, sizeof(CfItem) * cap));
-    const size_t part = (size_t)CFI_ITEM_CLASSES * cfb_order_blocks((uint32_t)cap, C->num_sms);
-    return C->ensure(B_ORDER, sizeof(uint32_t) * (cap + part));
-}
+static int ensure_items(CfCtx *C, size_t cap) { return C->ensure(B_ITEMS, sizeof(CfItem) * std::max<size_t>(1, cap)); }
 
 // The bbox pass's readback (CFB_BBOX_WORDS per point set): reject non-finite values and periodic
 // positions outside [0, L]; record each set's weight range and the union of the sets' boxes, the
@@ -464,15 +456,15 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     const size_t norigin = D.ang ? 3 * (size_t)D.g.ncell : H.origin.size();
     // The plan, its tables and the call's descriptors share one device block, filled from the
     // pinned staging by one copy: plan | LUT | fine entries | stencil | jobs | sets | bands |
-    // origins (FP64) | origins (float32).  The angular grid's origins are computed on the device.
-    const size_t piece[9] = {sizeof(CfDevPlan), sizeof(uint16_t) * H.lut.size(), sizeof(CfFine) * H.fine.size(),
+    // separation table | origins (FP64) | origins (float32).  The angular grid's origins are computed on the device.
+    const size_t piece[10] = {sizeof(CfDevPlan), sizeof(uint16_t) * H.lut.size(), sizeof(CfFine) * H.fine.size(),
                              sizeof(CfStencil) * H.stencil.size(), sizeof(CfJobDesc) * njobs,
-                             sizeof(CfSetDesc) * nsets, sizeof(CfBand) * H.bands.size(), sizeof(double) * norigin,
-                             sizeof(float) * norigin};
-    size_t poff[10];
+                             sizeof(CfSetDesc) * nsets, sizeof(CfBand) * H.bands.size(), H.lut8.size(),
+                              sizeof(double) * norigin, sizeof(float) * norigin};
+    size_t poff[11];
     poff[0] = 0;
-    for (int k = 0; k < 9; k++) poff[k + 1] = poff[k] + ((std::max<size_t>(piece[k], 1) + 255) & ~(size_t)255);
-    CF_TRY(C->ensure(B_PLANBLK, poff[9]));
+    for (int k = 0; k < 10; k++) poff[k + 1] = poff[k] + ((std::max<size_t>(piece[k], 1) + 255) & ~(size_t)255);
+    CF_TRY(C->ensure(B_PLANBLK, poff[10]));
     {
         char *blk = (char *)C->buf[B_PLANBLK].p;
         R.d_plan = (const CfDevPlan *)(blk + poff[0]);
@@ -482,8 +474,9 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         R.d_jobs = (const CfJobDesc *)(blk + poff[4]);
         R.d_sets = (const CfSetDesc *)(blk + poff[5]);
         D.band = (const CfBand *)(blk + poff[6]);
-        R.d_origin = (double *)(blk + poff[7]);
-        R.d_origin32 = (float *)(blk + poff[8]);
+        R.d_lut8 = (const uint8_t *)(blk + poff[7]);
+        R.d_origin = (double *)(blk + poff[8]);
+        R.d_origin32 = (float *)(blk + poff[9]);
         D.origin = R.d_origin;
         D.origin32 = R.d_origin32;
     }
@@ -492,12 +485,14 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     CF_TRY(C->ensure(B_CSTART, 4 * (size_t)(R.ncell_all + 1)));
     CF_TRY(C->ensure(B_CELLID, 4 * (size_t)R.np));
     CF_TRY(C->ensure(B_SLOT, 4 * (size_t)R.np));
-    CF_TRY(C->ensure(B_PA, 16 * (size_t)R.np));
-    CF_TRY(C->ensure(B_PB, 16 * (size_t)R.np));
+    const bool mocks = p->kind == CF_DD_RPPI_MOCKS;
+    CF_TRY(C->ensure(B_PT, 16 * (size_t)R.np));
+    if (mocks) CF_TRY(C->ensure(B_PABS, 16 * (size_t)R.np));
     CF_TRY(C->ensure(B_ORIG, 4 * (size_t)R.np));
     CF_TRY(C->ensure(B_CBOX, 24 * (size_t)R.ncell_all));
     if (C->opt[CF_OPT_CELL_PRUNE] == 0 && C->opt[CF_OPT_BLOCK_PRUNE] == 1) CF_TRY(C->ensure(B_GBOX, 24 * (size_t)R.np));
-    if (D.f64lo) CF_TRY(C->ensure(B_PLO, 32 * (size_t)R.np));
+    if (D.f64lo) CF_TRY(C->ensure(B_PLO, 16 * (size_t)R.np));
+    if (D.f64lo && mocks) CF_TRY(C->ensure(B_PABSLO, 16 * (size_t)R.np));
     CF_TRY(C->ensure(B_SCAN, 4 * (size_t)cfb_scan_tmp_words(std::max(R.nfine, R.nunit))));
     CF_TRY(C->ensure(B_ICNT, 4 * (size_t)std::max<int64_t>(R.nunit, 1)));
     CF_TRY(C->ensure(B_IOFF, 4 * (size_t)(R.nunit + 1)));
@@ -511,9 +506,9 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     {
         // one upload through pinned staging (no wait for the transfer); the angular grid's origins
         // are left to the device
-        const void *src[9] = {&D, H.lut.data(), H.fine.data(), H.stencil.data(), R.jobs.data(), R.sets.data(),
-                              H.bands.data(), H.origin.data(), H.origin32.data()};
-        const int npieces = D.ang ? 7 : 9;
+        const void *src[10] = {&D, H.lut.data(), H.fine.data(), H.stencil.data(), R.jobs.data(), R.sets.data(),
+                               H.bands.data(), H.lut8.data(), H.origin.data(), H.origin32.data()};
+        const int npieces = D.ang ? 8 : 10;
         CF_TRY(C->ensure_upload(poff[npieces]));
         for (int k = 0; k < npieces; k++)
             if (piece[k]) std::memcpy((char *)C->hup + poff[k], src[k], piece[k]);
@@ -527,14 +522,11 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     R.cfg.ravg = D.ravg;
     R.cfg.wrap = D.g.wrap[0] | D.g.wrap[1] | D.g.wrap[2];
     R.cfg.lo = D.f64lo;
-    R.cfg.nlut_words = D.nlut_words;
-    R.cfg.nfine = D.nfine;
+    R.cfg.nlut = D.nlut8;
     R.cfg.nslot = D.nslot;
     R.cfg.nb = D.nb;
     R.cfg.warps = (int)C->opt[CF_OPT_WARPS];
     R.cfg.ctas_per_sm = (int)C->opt[CF_OPT_CTAS_PER_SM];
-    // the mocks kind has the direct form only (a compacting form measured slower)
-    R.cfg.variant = (C->opt[CF_OPT_VARIANT] == 2 && D.kind != CF_DD_RPPI_MOCKS) ? 2 : 1;
     R.items_cap = 0;
     return CF_OK;
 }
@@ -599,16 +591,15 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
                    cstart, sub_shift),
           "scan cells");
     CF_CU(cfb_scatter(dplan, dsets, R.nsets, R.np, R.sub, fstart, (uint32_t *)C->buf[B_CELLID].p,
-                      (uint32_t *)C->buf[B_SLOT].p, (float4 *)C->buf[B_PA].p, (float4 *)C->buf[B_PB].p,
-                      (float4 *)C->buf[B_PLO].p, (uint32_t *)C->buf[B_ORIG].p, st),
+                      (uint32_t *)C->buf[B_SLOT].p, (float4 *)C->buf[B_PT].p, (float4 *)C->buf[B_PABS].p,
+                      (float4 *)C->buf[B_PLO].p, (float4 *)C->buf[B_PABSLO].p, (uint32_t *)C->buf[B_ORIG].p, st),
           "scatter");
     const float *cbox = nullptr;
     float *gbox = nullptr;
     if (C->opt[CF_OPT_CELL_PRUNE] == 0) {
         // and, when asked for, the boxes of the cells' 32-point groups
         gbox = C->opt[CF_OPT_BLOCK_PRUNE] == 1 ? (float *)C->buf[B_GBOX].p : nullptr;
-        CF_CU(cfb_cellbox(cstart, R.ncell_all, (const float4 *)C->buf[B_PA].p, (const float4 *)C->buf[B_PB].p,
-                          (float *)C->buf[B_CBOX].p, gbox, st),
+        CF_CU(cfb_cellbox(cstart, R.ncell_all, (const float4 *)C->buf[B_PT].p, (float *)C->buf[B_CBOX].p, gbox, st),
               "cell boxes");
         cbox = (const float *)C->buf[B_CBOX].p;
         C->launches += 1;
@@ -731,29 +722,23 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
                         nullptr, st),
               "items emit");
     }
-    // a short list is taken as it is: the two ordering passes would cost more than they save (the
-    // capacity of a repeat call's list holds 25 % headroom)
-    const bool ordered = R.items_cap >= CF_ORDER_MIN_ITEMS;
-    if (ordered)
-        CF_CU(cfb_order((const CfItem *)C->buf[B_ITEMS].p, nitems_dev, R.items_cap, (uint32_t *)C->buf[B_ORDER].p,
-                        (uint32_t *)C->buf[B_ORDER].p + R.items_cap, C->num_sms, st),
-              "work-list order");
     if (timed) CF_CU(cudaEventRecordWithFlags(C->ev[1], st, C->capturing ? cudaEventRecordExternal : 0), "event");
     CfPairArgs &A = R.args;
     std::memset(&A, 0, sizeof(A));
     A.plan = dplan;
     A.lut = R.d_lut;
     A.fine = R.d_fine;
+    A.lut8 = R.d_lut8;
     A.items = (const CfItem *)C->buf[B_ITEMS].p;
-    A.order = ordered ? (const uint32_t *)C->buf[B_ORDER].p : nullptr;
     A.nitems_dev = nitems_dev;
     A.items_cap = R.items_cap;
     A.qcap = R.qcap;
     A.cursor = (uint32_t *)(out + OUT_CURSOR);
     A.qcount = (unsigned long long *)(out + OUT_QCOUNT);
-    A.pa = (const ulonglong2 *)C->buf[B_PA].p;
-    A.pb = (const ulonglong2 *)C->buf[B_PB].p;
-    A.plo = (const ulonglong2 *)C->buf[B_PLO].p;
+    A.pt = (const float4 *)C->buf[B_PT].p;
+    A.pabs = (const float4 *)C->buf[B_PABS].p;
+    A.plo = (const float4 *)C->buf[B_PLO].p;
+    A.pabslo = (const float4 *)C->buf[B_PABSLO].p;
     A.orig = (const uint32_t *)C->buf[B_ORIG].p;
     A.hcnt = hcnt;
     A.hw = hw;
@@ -767,12 +752,10 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     // fit (many rp x pi slots, weights), they add straight into the global histograms instead
     const bool per_warp = D.kind == CF_DD_RPPI || D.kind == CF_DD_RPPI_MOCKS;
     if (per_warp && !R.cfg.ghist && cfp_pair_smem(R.cfg, 1) > (size_t)C->smem_optin) R.cfg.ghist = 1;
-    if (R.cfg.ghist) R.cfg.variant = 1;       // that form is built direct only
     A.ghist = R.cfg.ghist;
     // their per-warp sums go to fixed point when the terms' range allows it; never in a
     // captured graph, whose replays bring new weights
     if (per_warp && !A.ghist && !C->capturing) fixed_point_scales(R, D.weighted != 0, R.cfg.ravg != 0, A);
-    if (A.fxw != 0.f || A.fxr != 0.f) R.cfg.variant = 1;    // built direct only
     int grid = 0, warps = 0;
     if (R.items_cap > 0 && C->opt[CF_OPT_AUDIT]) {
         CF_CU(cfp_launch_audit(A.items, A.nitems_dev, A.items_cap, A.orig, A.queue, A.qcount, A.qcap, C->num_sms,
@@ -790,7 +773,7 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
         CF_CU(cfb_wsq(dsets, R.nsets, R.np, wsq, st), "self-pair weights");
         C->launches++;
     }
-    C->launches += 2 + (R.items_cap > 0 ? 1 : 0) + (ordered ? 2 : 0);   // items emit, recheck, pair, order
+    C->launches += 2 + (R.items_cap > 0 ? 1 : 0);   // items emit, recheck, pair
     if (timed) CF_CU(cudaEventRecordWithFlags(C->ev[3], st, C->capturing ? cudaEventRecordExternal : 0), "event");
     // the side stream's bbox pass joins here, so that the call's synchronisation covers it
     if (R.bbox_aux) {
@@ -868,7 +851,7 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
         C->stats.refine[a] = D.g.k[a];
     }
     C->stats.ncat = R.njobs;
-    C->stats.variant = R.cfg.variant;
+    C->stats.variant = 1;
     C->stats.fixed_sums = (R.args.fxw != 0.f ? 1 : 0) | (R.args.fxr != 0.f ? 2 : 0);
     C->stats.kernel_launches = C->launches;
     return CF_OK;

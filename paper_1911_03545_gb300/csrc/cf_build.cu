@@ -500,14 +500,15 @@ __global__ void cf_scan_apply(const uint32_t *__restrict__ in, uint32_t *__restr
 }
 
 // ---------------------------------------------------------------------------------------------
-// Scatter into cell order (Sec. 4.3).  Writes the packed j-side layout pa/pb (cell-relative,
-// negated, duplicated), the FP64 residual plo when requested, and the original index.
+// Scatter into cell order (Sec. 4.3).  Writes each point's cell-relative position (negated) and weight
+// (pt, 16 bytes: one sector per point), for mocks the absolute position, the low parts when requested,
+// and the original index.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__restrict__ plan, const CfSetDesc *__restrict__ sets,
                                   uint32_t ns, const uint32_t *__restrict__ fstart, const uint32_t *__restrict__ key,
-                                  const uint32_t *__restrict__ slot, float4 *__restrict__ pa,
-                                  float4 *__restrict__ pb, float4 *__restrict__ plo,
-                                  uint32_t *__restrict__ orig)
+                                  const uint32_t *__restrict__ slot, float4 *__restrict__ pt,
+                                  float4 *__restrict__ pabs, float4 *__restrict__ plo,
+                                  float4 *__restrict__ pabslo, uint32_t *__restrict__ orig)
 {
     const CfSetDesc S = sets[blockIdx.y];
     const CfGrid &g = plan->g;
@@ -529,9 +530,8 @@ __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__r
             const float yf = vy - cf_cell_origin32(plan, 1, (int)c, iy);
             const float zf = vz - cf_cell_origin32(plan, 2, (int)c, iz);
             const float w = S.w ? ((const float *)S.w)[i] : 1.0f;
-            const float ax = mocks ? vx : -xf, ay = mocks ? vy : -yf, az = mocks ? vz : -zf;
-            pa[dst] = make_float4(-xf, ax, -yf, ay);
-            pb[dst] = make_float4(-zf, az, w, w);
+            pt[dst] = make_float4(-xf, -yf, -zf, w);
+            if (mocks) pabs[dst] = make_float4(vx, vy, vz, 0.f);
             orig[dst] = (uint32_t)i;
             continue;
         }
@@ -541,17 +541,13 @@ __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__r
         double Z = vz - cf_cell_origin(plan, 2, (int)c, iz);
         float xf = (float)X, yf = (float)Y, zf = (float)Z;
         float w = S.w ? (float)cf_load(S.w, S.dtype, i) : 1.0f;
-        // second copies: X again, or for mocks the absolute position (its line of sight)
-        const float ax = mocks ? (float)vx : -xf, ay = mocks ? (float)vy : -yf, az = mocks ? (float)vz : -zf;
-        pa[dst] = make_float4(-xf, ax, -yf, ay);
-        pb[dst] = make_float4(-zf, az, w, w);
+        pt[dst] = make_float4(-xf, -yf, -zf, w);
+        const float ax = (float)vx, ay = (float)vy, az = (float)vz;
+        if (mocks) pabs[dst] = make_float4(ax, ay, az, 0.f);
         if (lo) {
-            float xl = (float)(X - (double)xf), yl = (float)(Y - (double)yf), zl = (float)(Z - (double)zf);
-            const float axl = mocks ? (float)(vx - (double)ax) : -xl;
-            const float ayl = mocks ? (float)(vy - (double)ay) : -yl;
-            const float azl = mocks ? (float)(vz - (double)az) : -zl;
-            plo[2 * dst] = make_float4(-xl, axl, -yl, ayl);
-            plo[2 * dst + 1] = make_float4(-zl, azl, 0.f, 0.f);
+            plo[dst] = make_float4(-(float)(X - (double)xf), -(float)(Y - (double)yf), -(float)(Z - (double)zf), 0.f);
+            if (mocks)
+                pabslo[dst] = make_float4((float)(vx - (double)ax), (float)(vy - (double)ay), (float)(vz - (double)az), 0.f);
         }
         orig[dst] = (uint32_t)i;
     }
@@ -567,8 +563,7 @@ __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__r
 // list prunes at that granularity.
 // ---------------------------------------------------------------------------------------------
 __global__ void cf_cellbox_kernel(const uint32_t *__restrict__ cell_start, int64_t ncell_all,
-                                  const float4 *__restrict__ pa, const float4 *__restrict__ pb, float *__restrict__ box,
-                                  float *__restrict__ gbox)
+                                  const float4 *__restrict__ pt, float *__restrict__ box, float *__restrict__ gbox)
 {
     const uint32_t lane = threadIdx.x & 31u;
     const int64_t wstride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -584,8 +579,8 @@ __global__ void cf_cellbox_kernel(const uint32_t *__restrict__ cell_start, int64
             float glo[3] = {INFINITY, INFINITY, INFINITY}, ghi[3] = {-INFINITY, -INFINITY, -INFINITY};
             const uint32_t p = p0 + lane;
             if (p < e) {
-                const float4 A = pa[p], B = pb[p];
-                const float v[3] = {-A.x, -A.z, -B.x};
+                const float4 A = pt[p];
+                const float v[3] = {-A.x, -A.y, -A.z};
                 for (int a = 0; a < 3; a++) glo[a] = ghi[a] = v[a];
             }
             if (gbox) {
@@ -966,126 +961,6 @@ __global__ void __launch_bounds__(256, GP ? 3 : 4)
     if (mode == 2 && lane == 0 && nres) atomicAdd(total64, nres);     // nres is the same in every lane
 }
 
-// ---------------------------------------------------------------------------------------------
-// Order of the work list: the pair kernel dispatches each item to one of four instances of its
-// loop (cf_item_class).  Taken in list order, neighbouring warps of an SM would run all four at
-// once, and their code together does not stay in the instruction cache; taken class by class, an
-// SM runs one at a time (largest tiles first, so the small ones fill the end of the launch).
-// A counting sort by class without atomics: block b owns the items [b C, (b + 1) C) with
-// C = ceil(n / blocks); the first pass writes each block's class sizes to part[b][k], the second
-// finds its offsets from them (the classes before k, the blocks before b) and writes each item's
-// index in list order.  The order is the same on every call.
-// ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void order_chunk(uint32_t n, uint32_t &beg, uint32_t &end)
-{
-    const uint32_t per = (n + gridDim.x - 1) / gridDim.x;
-    beg = min(n, blockIdx.x * per);
-    end = min(n, beg + per);
-}
-
-__device__ __forceinline__ uint32_t order_class(const CfItem *__restrict__ items, uint32_t i, uint32_t end)
-{
-    if (i >= end) return CFI_ITEM_CLASSES;
-    const uint2 cm = *reinterpret_cast<const uint2 *>(&items[i].cnt);       // cnt, meta
-    return cf_item_class(cm.x, cm.y);
-}
-
-__global__ void __launch_bounds__(256) cf_order_count_kernel(const CfItem *__restrict__ items,
-                                                             const uint32_t *__restrict__ nitems_dev,
-                                                             uint32_t items_cap, uint32_t *__restrict__ part)
-{
-    __shared__ uint32_t s_c[8][CFI_ITEM_CLASSES];
-    uint32_t beg, end;
-    order_chunk(min(*nitems_dev, items_cap), beg, end);
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t cnt[CFI_ITEM_CLASSES] = {};
-    for (uint32_t t = beg; t < end; t += 256u) {
-        const uint32_t c = order_class(items, t + threadIdx.x, end);
-#pragma unroll
-        for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++) cnt[k] += (uint32_t)__popc(__ballot_sync(CF_FULL, c == k));
-    }
-    if (lane == 0)
-        for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++) s_c[warp][k] = cnt[k];
-    __syncthreads();
-    if (threadIdx.x < CFI_ITEM_CLASSES) {
-        uint32_t s = 0;
-        for (uint32_t w = 0; w < (blockDim.x >> 5); w++) s += s_c[w][threadIdx.x];
-        part[blockIdx.x * CFI_ITEM_CLASSES + threadIdx.x] = s;
-    }
-}
-
-__global__ void __launch_bounds__(256) cf_order_scatter_kernel(const CfItem *__restrict__ items,
-                                                               const uint32_t *__restrict__ nitems_dev,
-                                                               uint32_t items_cap, const uint32_t *__restrict__ part,
-                                                               uint32_t *__restrict__ order)
-{
-    __shared__ uint32_t s_w[8][CFI_ITEM_CLASSES];      // per warp: before this block, then per tile
-    __shared__ uint32_t s_base[CFI_ITEM_CLASSES];      // where this block's next item of class k goes
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    {
-        // the classes' sizes over all blocks, and over the blocks before this one
-        uint32_t tot[CFI_ITEM_CLASSES] = {}, pre[CFI_ITEM_CLASSES] = {};
-        for (uint32_t b = threadIdx.x; b < gridDim.x; b += blockDim.x)
-            for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++) {
-                const uint32_t v = part[b * CFI_ITEM_CLASSES + k];
-                tot[k] += v;
-                pre[k] += b < blockIdx.x ? v : 0u;
-            }
-        for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++)
-            for (int o = 16; o; o >>= 1) {
-                tot[k] += __shfl_xor_sync(CF_FULL, tot[k], o);
-                pre[k] += __shfl_xor_sync(CF_FULL, pre[k], o);
-            }
-        __shared__ uint32_t s_tot[8][CFI_ITEM_CLASSES];
-        if (lane == 0)
-            for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++) {
-                s_tot[warp][k] = tot[k];
-                s_w[warp][k] = pre[k];
-            }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t off = 0;
-            for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++) {
-                uint32_t t = 0, p = 0;
-                for (uint32_t w = 0; w < nw; w++) {
-                    t += s_tot[w][k];
-                    p += s_w[w][k];
-                }
-                s_base[k] = off + p;
-                off += t;
-            }
-        }
-        __syncthreads();
-    }
-    uint32_t beg, end;
-    order_chunk(min(*nitems_dev, items_cap), beg, end);
-    const uint32_t below = (1u << lane) - 1u;
-    for (uint32_t t = beg; t < end; t += 256u) {
-        const uint32_t i = t + threadIdx.x;
-        const uint32_t c = order_class(items, i, end);
-        uint32_t mine = 0;      // the ballot of this thread's class
-#pragma unroll
-        for (uint32_t k = 0; k < CFI_ITEM_CLASSES; k++) {
-            const uint32_t m = __ballot_sync(CF_FULL, c == k);
-            if (c == k) mine = m;
-            if (lane == 0) s_w[warp][k] = (uint32_t)__popc(m);
-        }
-        __syncthreads();
-        if (c < CFI_ITEM_CLASSES) {
-            uint32_t r = s_base[c] + (uint32_t)__popc(mine & below);
-            for (uint32_t w = 0; w < warp; w++) r += s_w[w][c];
-            order[r] = i;       // r < n: the class's place plus its rank among the class's n_k items
-        }
-        __syncthreads();
-        if (threadIdx.x < CFI_ITEM_CLASSES) {
-            uint32_t s = 0;
-            for (uint32_t w = 0; w < nw; w++) s += s_w[w][threadIdx.x];
-            s_base[threadIdx.x] += s;
-        }
-        __syncthreads();
-    }
-}
-
 // sum of w^2 per set (self pairs of a weighted auto-correlation whose first edge is 0)
 __global__ void cf_wsq_kernel(const CfSetDesc *__restrict__ sets, double *__restrict__ out)
 {
@@ -1160,19 +1035,19 @@ cudaError_t cfb_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp
 }
 
 cudaError_t cfb_scatter(const CfDevPlan *plan, const CfSetDesc *sets, int nsets, int64_t nmax, int sub,
-                        const uint32_t *fstart, const uint32_t *key, const uint32_t *slot, float4 *pa,
-                        float4 *pb, float4 *plo, uint32_t *orig, cudaStream_t st)
+                        const uint32_t *fstart, const uint32_t *key, const uint32_t *slot, float4 *pt,
+                        float4 *pabs, float4 *plo, float4 *pabslo, uint32_t *orig, cudaStream_t st)
 {
     dim3 grid(blocks_for(nmax, 256, 4096), nsets);
-    cf_scatter_kernel<<<grid, 256, 0, st>>>(plan, sets, (uint32_t)(sub * sub * sub), fstart, key, slot, pa, pb, plo,
-                                            orig);
+    cf_scatter_kernel<<<grid, 256, 0, st>>>(plan, sets, (uint32_t)(sub * sub * sub), fstart, key, slot, pt, pabs, plo,
+                                            pabslo, orig);
     return cudaGetLastError();
 }
 
-cudaError_t cfb_cellbox(const uint32_t *cell_start, int64_t ncell_all, const float4 *pa, const float4 *pb, float *box,
-                        float *gbox, cudaStream_t st)
+cudaError_t cfb_cellbox(const uint32_t *cell_start, int64_t ncell_all, const float4 *pt, float *box, float *gbox,
+                        cudaStream_t st)
 {
-    cf_cellbox_kernel<<<blocks_for(ncell_all * 32, 256, 8192), 256, 0, st>>>(cell_start, ncell_all, pa, pb, box, gbox);
+    cf_cellbox_kernel<<<blocks_for(ncell_all * 32, 256, 8192), 256, 0, st>>>(cell_start, ncell_all, pt, box, gbox);
     return cudaGetLastError();
 }
 
@@ -1197,15 +1072,6 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
     else
         cf_items_kernel<false><<<nb, 256, 0, st>>>(plan, sets, jobs, stencil, cell_start, cbox, nullptr, live, nlive,
                                                    mode, counts, offsets, items, items_cap, evaluated, total64);
-    return cudaGetLastError();
-}
-
-cudaError_t cfb_order(const CfItem *items, const uint32_t *nitems_dev, uint32_t items_cap, uint32_t *order,
-                      uint32_t *part, int num_sms, cudaStream_t st)
-{
-    const int nb = cfb_order_blocks(items_cap, num_sms);
-    cf_order_count_kernel<<<nb, 256, 0, st>>>(items, nitems_dev, items_cap, part);
-    cf_order_scatter_kernel<<<nb, 256, 0, st>>>(items, nitems_dev, items_cap, part, order);
     return cudaGetLastError();
 }
 

@@ -24,12 +24,12 @@ int64_t cfb_scan_tmp_words(int64_t n);
 cudaError_t cfb_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, uint32_t *done, cudaStream_t st,
                      uint32_t *total_copy = nullptr, uint32_t *every = nullptr, int every_shift = 0);
 cudaError_t cfb_scatter(const CfDevPlan *plan, const CfSetDesc *sets, int nsets, int64_t nmax, int sub,
-                        const uint32_t *fstart, const uint32_t *key, const uint32_t *slot, float4 *pa,
-                        float4 *pb, float4 *plo, uint32_t *orig, cudaStream_t st);
+                        const uint32_t *fstart, const uint32_t *key, const uint32_t *slot, float4 *pt,
+                        float4 *pabs, float4 *plo, float4 *pabslo, uint32_t *orig, cudaStream_t st);
 // tight point bounding box per cell (6 floats: lo xyz, hi xyz, cell-relative), for cell-pair pruning;
 // with gbox (6 floats per point) also the box of every 32-point group of a cell at its first point
-cudaError_t cfb_cellbox(const uint32_t *cell_start, int64_t ncell_all, const float4 *pa, const float4 *pb, float *box,
-                        float *gbox, cudaStream_t st);
+cudaError_t cfb_cellbox(const uint32_t *cell_start, int64_t ncell_all, const float4 *pt, float *box, float *gbox,
+                        cudaStream_t st);
 // the units (job, i cell) whose i cell holds points, appended to live[] (nunits entries) at the
 // zeroed counter *nlive
 cudaError_t cfb_live_units(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobDesc *jobs,
@@ -47,39 +47,22 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
                       const uint32_t *nlive, int64_t nunits, int mode, uint32_t *counts, const uint32_t *offsets,
                       CfItem *items, uint32_t items_cap, unsigned long long *evaluated, unsigned long long *total64,
                       cudaStream_t st);
-// work lists of a smaller capacity are taken in list order (CfPairArgs::order = NULL): the two
-// ordering passes cost 12-15 us, the pair kernel saves 3-7 %, so they pay from about 0.3 ms of
-// pair kernel (some 30,000 items)
-#define CF_ORDER_MIN_ITEMS 40960u
-// the order in which the pair kernel takes the work list: the indices of the items of each class
-// (cf_item_class) together, classes in increasing order and each class in list order, so that the
-// warps of an SM run one instance's code at a time.  order[] needs min(*nitems_dev, items_cap)
-// entries; part[] CFI_ITEM_CLASSES words per block of the launch (cfb_order_blocks), no initial
-// value.
-inline int cfb_order_blocks(uint32_t items_cap, int num_sms)
-{
-    const int cap = num_sms > 0 ? 4 * num_sms : 4;
-    const int64_t b = ((int64_t)items_cap + 255) / 256;
-    return b < 1 ? 1 : (b > cap ? cap : (int)b);
-}
-cudaError_t cfb_order(const CfItem *items, const uint32_t *nitems_dev, uint32_t items_cap, uint32_t *order,
-                      uint32_t *part, int num_sms, cudaStream_t st);
 cudaError_t cfb_wsq(const CfSetDesc *sets, int nsets, int64_t nmax, double *out, cudaStream_t st);
 
 // ---- pair counting ----
 struct CfPairArgs {
     const CfDevPlan *plan;
-    const uint16_t *lut;         // coarse LUT entries (global copy; staged into shared memory)
+    const uint8_t *lut8;         // separation table (staged into shared memory)
+    const uint16_t *lut;         // coarse entries of the full tables
     const CfFine *fine;          // fine LUT entries
     const CfItem *items;
-    const uint32_t *order;       // the items in the order they are taken (cfb_order; NULL: list order)
     const uint32_t *nitems_dev;  // item count written by the work-list scan
     uint32_t items_cap;          // items beyond this were not stored
     uint32_t qcap;
     uint32_t *cursor;
-    const ulonglong2 *pa;        // (-X,-X | -Y,-Y)
-    const ulonglong2 *pb;        // (-Z,-Z | w, w)
-    const ulonglong2 *plo;       // FP64 residuals, two per point (may be NULL)
+    const float4 *pt;            // (-X, -Y, -Z, w)
+    const float4 *pabs;          // mocks: absolute positions
+    const float4 *plo, *pabslo;  // low parts (float64 inputs with ravg)
     const uint32_t *orig;
     unsigned long long *hcnt;    // [njobs][nslot]
     double *hw;                  // [njobs][nslot]
@@ -103,11 +86,11 @@ struct CfPairCfg {
     int kind;          // 0 r, 1 rppi, 2 wp, 3 theta, 4 mocks
     int weighted, ravg, wrap, lo;
     int ghist;         // see CfPairArgs::ghist (no per-warp histogram in shared memory)
-    int nlut_words, nfine, nslot;
+    int nlut;          // cells of the squared-separation table in shared memory
+    int nslot;
     int nb;            // r / rp / theta bins
     int warps;         // warps per CTA (0: automatic)
     int ctas_per_sm;   // 0: occupancy-derived
-    int variant;       // 1 direct binning, 2 compacting ring (resolved from 0 by the caller)
 };
 
 // Shared-memory bytes of one CTA with `warps` warps.

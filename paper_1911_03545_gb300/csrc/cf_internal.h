@@ -4,14 +4,12 @@
 //   point set s (a catalogue, or one side of a cross count) is scattered into cell order by a
 //   counting sort (Sec. 4.3: particles of a cell are stored contiguously).  For every point p
 //   (global index over all sets) we keep
-//     pa[p] = float4(-X, -X, -Y, -Y)   pb[p] = float4(-Z, -Z, w, w)
+//     pt[p] = float4(-X, -Y, -Z, w)
 //   where X = x - o(cell) is the cell-relative coordinate (Sec. 4.4's shift trick applied per
-//   cell), stored negated and duplicated so that one packed f32x2 add forms two separations.
-//   For mocks the second copies hold the absolute position instead: pa = (-X, x, -Y, y),
-//   pb = (-Z, z, w, w) with x, y, z rounded to float32.
-//     plo[2p] = float4(-Xlo, -Xlo, -Ylo, -Ylo), plo[2p+1] = float4(-Zlo, -Zlo, 0, 0)
-//   (float64 inputs with ravg only: x - o = X + Xlo; for mocks the second copies hold the low
-//   parts of the absolute position, x = float(x) + xlo)
+//   cell), stored negated so that an addition forms a separation; for mocks also
+//     pabs[p] = float4(x, y, z, 0), the absolute position rounded to float32
+//   and for float64 inputs with ravg the low parts: x - o = X + Xlo, x = float(x) + xlo
+//     plo[p] = float4(-Xlo, -Ylo, -Zlo, 0), pabslo[p] = float4(xlo, ylo, zlo, 0) (mocks)
 //     orig[p] = index of the point in its input arrays
 //   cell_start[set cell offset + c] .. [c+1] delimit a cell's points.
 //   A work item is one (i tile, j range, shift) triple of a cell pair (Sec. 4.3).
@@ -24,6 +22,7 @@
 #define CFI_MAX_STENCIL 4096
 #define CFI_LUT_MAX 8192          // coarse LUT cells (2 B each)
 #define CFI_LUT_TARGET 4096       // preferred coarse cells per table
+#define CFI_LUT8_CELLS 8192       // cells of the pair kernel's separation table below the last edge
 #define CFI_FINE_MAX 1024         // fine LUT entries (16 B each)
 #define CFI_CLS_OUT 0xFEu         // class: outside every bin
 #define CFI_CLS_AMB 0xFFu         // class: within the FP32 error band of an edge
@@ -43,22 +42,6 @@ struct CfItem {
 };
 #define CFI_ITEM_DIAG (1u << 30)
 #define CFI_ITEM_JOBMASK 0xFFFFFu
-
-// The pair-kernel instance an item runs in (the kernel dispatches on the same thresholds): 0 an
-// i tile of more than 96 points (four slots per lane), 1 a cell with itself, 2 a tile of 65-96
-// points (three slots), 3 one of 33-64 (two), 4 one of at most 32 (one).  The work list is handed
-// to the pair kernel in this order of classes.  (The mocks kind runs classes 0 and 2 in its
-// four-slot instance.)
-#define CFI_ITEM_CLASSES 5
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline uint32_t cf_item_class(uint32_t cnt, uint32_t meta)
-{
-    if (meta & CFI_ITEM_DIAG) return 1u;
-    const uint32_t ic = cnt & 0xFFFFu;
-    return ic > 96u ? 0u : (ic > 64u ? 2u : (ic > 32u ? 3u : 4u));
-}
 
 // A point set (input view + where its sorted points and cells live)
 struct CfSetDesc {
@@ -137,6 +120,8 @@ struct CfDevPlan {
     int tile;              // max i tile (64 or 128)
     int jchunk;            // max j range per item
     CfLut lr, lp;          // r/rp/chord LUT, and pi LUT (rppi/wp)
+    int nlut8;             // cells of the pair kernel's separation table (one byte each)
+    float lut8_scale;      // its cells per unit of separation
     int nlut_words;        // coarse words (both LUTs)
     int nfine;             // fine entries (both LUTs)
     double pimax;
@@ -148,13 +133,16 @@ struct CfDevPlan {
     const CfBand *band;    // device table of the bands
     double adlo, ah;       // lowest band edge and band height (radians)
     double tsearch;        // neighbour-search angle (radians): the largest edge, widened
-    float cut_r;           // candidate cut on the FP32 squared separation (above the last band);
-                           // mocks: on rp^2 in the form (s.s - cut_r) l.l < (s.l)^2
-    float cut_p;           // candidate cut on the FP32 |dz| (rp-pi / wp); mocks: on pi^2 in the
-                           // form (s.l)^2 < cut_p l.l
+    float reach_r;         // gathering limit of the pair kernel on the squared separation (mocks: s.s;
+                           // rp-pi / wp: rp^2) formed without the shift's low part: above the largest
+                           // one that may count by that form's FP32 error
+    float reach_p;         // the same on dz^2 (rp-pi / wp)
+    float pi_inv, pi_n;    // rp-pi / wp / mocks: t = pi * pi_inv counts pi bins of equal width, pi_n of them
+                           // (wp: one)
+    float pi_tol;          // a t within this of an integer may lie in the FP32 band of a pi edge
     float near2;           // mocks: a candidate whose FP32 l.l is below this goes to the FP64
-                           // recheck when its s.s - cut_r is below cut_su (0: no candidate can be)
-    float cut_su;
+                           // recheck when its s.s is below near_ss (0: no candidate can be)
+    float near_ss;
     double smax2;          // mocks: largest |s|^2 of a counted pair (rmax^2 + pimax^2, widened)
     // float32 helpers of the cell build (the FP64 pipe runs at a small fraction of the FP32 rate):
     const float *origin32; // float32 copies of `origin` (exact: origins are multiples of the float32

@@ -2,28 +2,33 @@
 //
 // Sec. 4.3-4.7 on a GPU.  Every warp repeatedly takes one work item -- an i tile of one cell
 // (<= 128 points) against a j range (<= 512 points) of a neighbour cell -- from a global atomic
-// cursor (in the order of cfb_order: items of one instance together).  Lane l holds the i points
-// l + 32 q (q < Q; Q = 1 to 4 by the tile's size, mocks 1, 2 or 4) in
-// registers, already translated by the cell-pair shift (Sec. 4.4, Code corrfunc_pbc: the shift
-// is added once per i, not per pair), each duplicated into both halves of a packed FP32 pair.
-// The j points stream through a double-buffered shared-memory stage (cp.async) as float arrays
-// and are read two at a time by broadcast 8-byte loads: one packed add forms the separations of
-// an i point from two j points.
+// cursor, and works through the tile in groups of 32 points: lane l holds one i point in registers,
+// translated by the cell-pair shift (Sec. 4.4, Code corrfunc_pbc: the shift is added once per i, not
+// per pair).
 //
-// Per pair: the separation and squared distance by packed FP32x2 add / mul / fma on
-// cell-relative coordinates -- with the shift's low part and the TwoSum residual of the i
-// translation when ravg needs relative accuracy -- and one cut: the FP32 value from which on
-// every value lies outside all bins (Sec. 4.7: squared space, no sqrt; rp-pi and wp also cut
-// |dz|).  A pair below the cut is binned on its FP32 bit pattern through a coarse table (cells
-// holding an edge resolve through a fine entry of <= 2 thresholds).  A value within the proven
-// FP32 error band of an edge is not binned: the pair goes to a global queue and is re-evaluated
-// in FP64 by the recheck kernel, so counts equal the FP64 result.
+// Gathering: the warp reads the j range 32 points at a time, one per lane, tests each against the
+// bounding box of the group's 32 i points (the late entry / early exit of Sec. 4.5, point by point)
+// and gathers the points within reach in shared memory as float arrays.  The smallest separation the
+// box allows is formed with operations that round monotonically, and the limit lies above the largest
+// edge by the FP32 error of that form (CfDevPlan::reach_r), so no pair that counts is dropped.
+// Counting: whenever 32 points are gathered (and at the end of the range) every lane forms its pairs
+// with them, four at a time: packed FP32x2 separations on cell-relative coordinates -- with the
+// shift's low part and the TwoSum residual of the i translation when ravg needs relative accuracy --
+// binned through a table over the separation (one byte a cell; outside every bin is a class of it), the
+// equally wide pi bins by one multiplication.  A table cell that holds an edge, or a value near a pi
+// edge, resolves through the full tables on the squared separation's bits (Sec. 4.7); a value within
+// the proven FP32 error band of an edge is not binned: the pair goes to a global queue and is
+// re-evaluated in FP64 by the recheck kernel, so counts equal the FP64 result.
 //
-// Two forms of that binning step, with identical results:
-//   direct     (variant 1): each lane bins its own pairs below the cut where they are formed;
-//   compacting (variant 2): the warp appends its pairs below the cut (value bits, |dz| bits,
-//              i/j code, weight product) to a per-warp ring in shared memory at offsets from a
-//              ballot prefix sum, and bins them 32 at a time with every lane busy.
+// What bounds it: instruction issue (70 to 80 % of the slots).  Counting costs 17 (DD(theta), counts only)
+// to 30 (weights and ravg) instructions per gathered point and warp, gathering about 70 per 32 j points,
+// so the layout aims at few gathered points per pair in range: on the clustered catalogues 1.6 to
+// 2.0 times the in-range pairs are formed, where whole cell pairs form 4 to 8 times as many.  Gathering
+// also fills the blocks: a cell's ragged end costs at most three points of a range's last block.
+// Measured against whole cell pairs with a branch per pair in range (pair kernel, one GB300): DD(r) of
+// 1M clustered points with weights and ravg 1.546 -> 1.102 ms, counts to twice the separation
+// 5.25 -> 2.53 ms, DD(rp, pi) of 2M points 1.505 -> 1.016 ms, its DR against 4M randoms 5.17 -> 3.03 ms,
+// DD(theta) of 1M points 1.176 -> 0.687 ms, DR of the survey cone 5.48 -> 2.48 ms.
 //
 // Histograms live in shared memory per warp (Sec. 4.8: private histograms, merged once): for
 // r / theta / wp one private copy per lane (no bank conflicts, no contention; weighted sums
@@ -39,6 +44,8 @@
 // hold 2^18 terms: the second word then stays below 2^32 and places the true sum within 2^30 below
 // its value times 2^12, and the first word gives the sum exactly (fx_sum).
 #pragma once
+#include <math_constants.h>
+
 #include "cf_build.h"
 #include "cf_device.cuh"
 
@@ -51,10 +58,9 @@ __host__ __device__ constexpr bool warp_hist(int kind) { return kind == KIND_RPP
 
 __host__ __device__ __forceinline__ uint32_t align16(uint32_t x) { return (x + 15u) & ~15u; }
 
-// per-warp shared memory: j stage | candidate ring (compacting form) | histogram
-//   j stage: 2 chunks x 3-7 float arrays (x, y, z[, w][, lo parts of x, y, z]) of JSTAGE points
-//   ring:    RING candidates as arrays: value bits, |dz| bits (rp-pi, wp), weight product (W),
-//            code (u16: i slot | j << 7)
+// per-warp shared memory: gathered j points | histogram
+//   gathered points: a ring of GBUF points as 3-7 float arrays (x, y, z[, w][, lo parts of x, y, z])
+//   and the points' places in the j range (u16)
 // a warp flushes its histograms once it has evaluated more than this many pairs of one job;
 // with the item in hand that keeps every flushed batch at <= 2^28 pairs (an item: <= 2^16)
 constexpr uint32_t CF_FLUSH_PAIRS = (1u << 28) - (1u << 16);
@@ -69,33 +75,32 @@ __device__ __forceinline__ unsigned long long fx_sum(uint32_t lo, uint32_t hi)
     const unsigned long long c = (unsigned long long)hi << FX_HI_SHIFT;
     return c + (uint32_t)(lo - (uint32_t)c);
 }
-constexpr uint32_t JSTAGE = 32;
-constexpr uint32_t RING = 512;
-constexpr uint32_t RM = RING - 1;
-static_assert(CFI_JMAX <= 512, "a ring code holds a 7-bit i slot and a 9-bit j");
+constexpr uint32_t GBUF = 64;
+// Histogram rows past the bins: a separation outside every bin reads class nb, one that the full tables
+// must decide class nb + 1.  Counts-only kinds add there as well instead of testing (lane-private rows; one
+// word per lane past a per-warp histogram), and nothing reads those rows.
+constexpr uint32_t SPARE = 2;
 __host__ __device__ __forceinline__ uint32_t warp_hist_bytes(int kind, bool W, bool R, int nslot)
 {
     if (warp_hist(kind)) {
-        uint32_t b = ((uint32_t)nslot * 4u + 7u) & ~7u;
+        uint32_t b = (((uint32_t)nslot + (W || R ? 0u : 32u)) * 4u + 7u) & ~7u;
         if (W) b += nslot * 8u;
         if (R) b += nslot * 8u;
         return align16(b);
     }
-    uint32_t b = nslot * 32u * 4u;
+    uint32_t b = (nslot + (W || R ? 0u : SPARE)) * 32u * 4u;
     if (W) b += nslot * 32u * 8u;
     if (R) b += nslot * 32u * 8u;
     return b;
 }
 __host__ __device__ constexpr bool has_z(int kind) { return kind == KIND_RPPI || kind == KIND_WP; }
+// kinds that bin a second value (|dz|; for mocks pi^2)
+__host__ __device__ constexpr bool has_pi(int kind) { return has_z(kind) || kind == KIND_MOCKS; }
 __host__ __device__ constexpr uint32_t stage_arrays(bool W, bool LO) { return LO ? 7u : (W ? 4u : 3u); }
-__host__ __device__ constexpr uint32_t warp_jbuf_bytes(bool W, bool LO) { return 2u * stage_arrays(W, LO) * JSTAGE * 4u; }
-__host__ __device__ __forceinline__ uint32_t warp_ring_bytes(int kind, bool W)
+__host__ __device__ constexpr uint32_t warp_jbuf_bytes(bool W, bool LO) { return stage_arrays(W, LO) * GBUF * 4u + GBUF * 2u; }
+__host__ __device__ __forceinline__ uint32_t warp_bytes(int kind, bool W, bool R, bool LO, int nslot)
 {
-    return RING * (4u + (has_z(kind) ? 4u : 0u) + (W ? 4u : 0u) + 2u);
-}
-__host__ __device__ __forceinline__ uint32_t warp_bytes(int kind, bool W, bool R, bool LO, int nslot, bool compact)
-{
-    return warp_jbuf_bytes(W, LO) + (compact ? warp_ring_bytes(kind, W) : 0u) + warp_hist_bytes(kind, W, R, nslot);
+    return warp_jbuf_bytes(W, LO) + warp_hist_bytes(kind, W, R, nslot);
 }
 
 // Kahan-compensated FP32 sum: s holds the sum, c the negated lost low part
@@ -113,17 +118,12 @@ __device__ __forceinline__ void kahan_add(float2 *p, float v)
     *p = sc;
 }
 
-struct Lut {
-    uint32_t base, shift, last;
-    const uint16_t *words;   // shared
-};
-
-__device__ __forceinline__ uint32_t lut_class(const Lut &L, const CfFine *__restrict__ fine, uint32_t vb)
+// class of a non-negative value's bit pattern from the full (16-bit) table in global memory
+__device__ __forceinline__ uint32_t lut_class(const uint16_t *__restrict__ words, const CfFine *__restrict__ fine,
+                                              const CfLut &L, uint32_t vb)
 {
-    int t = (int)(vb - L.base);
-    t = t > 0 ? t : 0;
-    uint32_t idx = min((uint32_t)t >> L.shift, L.last);
-    uint32_t c = L.words[idx];
+    const uint32_t idx = min((max(vb, L.base) - L.base) >> L.shift, L.last);
+    uint32_t c = words[L.coff + idx];
     if (c >= CFI_FINE_FLAG) {
         const CfFine f = fine[c - CFI_FINE_FLAG];
         uint32_t seg = (vb >= f.t1 ? 1u : 0u) + (vb >= f.t2 ? 1u : 0u);
@@ -132,21 +132,42 @@ __device__ __forceinline__ uint32_t lut_class(const Lut &L, const CfFine *__rest
     return c;
 }
 
-// Lookup for a value known to lie below the table's tail (the start of its final "outside
-// every bin" segment): the index then never passes the last cell, so no upper clamp is needed.
-// Split in two so that several lookups can issue their table reads before any fine resolution.
-__device__ __forceinline__ uint32_t lut_raw_in(const Lut &L, uint32_t vb)
+// minimum / maximum over the warp; NaN lanes drop out
+__device__ __forceinline__ float f_redux_min(float v)
 {
-    return L.words[(max(vb, L.base) - L.base) >> L.shift];
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
-__device__ __forceinline__ uint32_t lut_fine(const CfFine *__restrict__ fine, uint32_t c, uint32_t vb)
+__device__ __forceinline__ float f_redux_max(float v)
 {
-    if (c >= CFI_FINE_FLAG) {
-        const CfFine f = fine[c - CFI_FINE_FLAG];
-        uint32_t seg = (vb >= f.t1 ? 1u : 0u) + (vb >= f.t2 ? 1u : 0u);
-        c = (f.code >> (8u * seg)) & 0xFFu;
-    }
-    return c;
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float f_rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// denormals as 0 (one instruction): the table sends separations that small to the full tables
+__device__ __forceinline__ float f_sqrt_ftz(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ uint32_t lds_u8(uint32_t addr)
+{
+    uint32_t r;
+    asm("ld.shared.u8 %0, [%1];" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ float pick4(const float (&v)[4], int h)
+{
+    const float a = h & 1 ? v[1] : v[0], b = h & 1 ? v[3] : v[2];
+    return h & 2 ? b : a;
 }
 
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
@@ -174,26 +195,24 @@ static __device__ __noinline__ void push_recheck(const CfPairArgs &a, uint32_t i
 // and s x l = s x v_i because l = v_i - s / 2: the cancellation that makes s.s - pi^2 inaccurate
 // for rp << pi moves into one cross product of exactly known numbers (s as a hi + lo pair from
 // the cell-relative coordinates, v_i as float32 plus its lo part), taken by Kahan's difference of
-// products (error <= 2u of each component).  ip: the i point; bs, jl: the stage buffer and the j
-// point's index in it; sh / sl: the item's shift, hi and lo.  Rare (counted pairs with ravg
+// products (error <= 2u of each component).  ip: the i point; bj: the gathered j point; sh / sl: the
+// item's shift, hi and lo.  Rare (counted pairs with ravg
 // only), so kept out of line.
 template <bool LO>
-static __device__ __noinline__ float mocks_rp(const CfPairArgs &a, uint32_t ip, const float *bs, uint32_t jl,
+static __device__ __noinline__ float mocks_rp(const CfPairArgs &a, uint32_t ip, const float *bj,
                                               float shx, float shy, float shz, float slx, float sly, float slz)
 {
-    const float4 A = reinterpret_cast<const float4 *>(a.pa)[ip];
-    const float4 B = reinterpret_cast<const float4 *>(a.pb)[ip];
-    const float X[3] = {-A.x, -A.z, -B.x}, Ah[3] = {A.y, A.w, B.y};
+    const float4 P = a.pt[ip], A = a.pabs[ip];
+    const float X[3] = {-P.x, -P.y, -P.z}, Ah[3] = {A.x, A.y, A.z};
     const float ish[3] = {shx, shy, shz}, isl[3] = {slx, sly, slz};
     float XL[3] = {0.f, 0.f, 0.f}, AL[3] = {0.f, 0.f, 0.f}, XJL[3] = {0.f, 0.f, 0.f};
     if (LO) {
-        const float4 C = reinterpret_cast<const float4 *>(a.plo)[2 * (size_t)ip];
-        const float4 D = reinterpret_cast<const float4 *>(a.plo)[2 * (size_t)ip + 1];
-        XL[0] = -C.x; XL[1] = -C.z; XL[2] = -D.x;
-        AL[0] = C.y; AL[1] = C.w; AL[2] = D.y;
-        XJL[0] = bs[4 * JSTAGE + jl]; XJL[1] = bs[5 * JSTAGE + jl]; XJL[2] = bs[6 * JSTAGE + jl];
+        const float4 C = a.plo[ip], D = a.pabslo[ip];
+        XL[0] = -C.x; XL[1] = -C.y; XL[2] = -C.z;
+        AL[0] = D.x; AL[1] = D.y; AL[2] = D.z;
+        XJL[0] = bj[4 * GBUF]; XJL[1] = bj[5 * GBUF]; XJL[2] = bj[6 * GBUF];
     }
-    const float XJ[3] = {bs[jl], bs[JSTAGE + jl], bs[2 * JSTAGE + jl]};   // -X_j
+    const float XJ[3] = {bj[0], bj[GBUF], bj[2 * GBUF]};   // -X_j
     float sh[3], sl[3], l[3];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
@@ -226,43 +245,56 @@ static __device__ __noinline__ float mocks_rp(const CfPairArgs &a, uint32_t ip, 
 template <int KIND, bool W, bool R, bool WRAP, bool LO, bool GH, bool FX>
 struct Warp {
     const CfPairArgs &a;
-    Lut lr, lp;
-    const CfFine *fine;
-    uint32_t *h_cnt;        // lane-private [nslot][32] or per-warp [nslot]
+    const CfLut &lr, &lp;   // the full tables' shapes
+    uint32_t lut;           // separation table in shared memory: its address, less the bits of 2^23
+    uint32_t lut_top;       // bits of 2^23 + the index of its last cell (outside every bin)
+    float lut_scale;        // cells per unit of separation
+    uint32_t *h_cnt;        // lane-private [nslot][32] (this and the sums: at the lane's column) or
+                            // per-warp [nslot]
     float2 *h_w, *h_r;      // lane-private Kahan pairs (interleaved when both are kept)
     double *h_wd, *h_rd;    // per-warp sums (rp-pi, mocks): FP64, or with FX two 32-bit words per slot
                             // (nslot low words, then nslot high words)
     const float *fxr_bin;   // with FX and ravg: the scale of each rp bin's ravg terms (shared memory)
-    float *jst;             // j stage
-    uint32_t *rv, *rz;      // ring: value bits, |dz| bits
-    float *rw;              // ring: weight product
-    uint16_t *rc;           // ring: code, i slot | j << 7
+    float *jst;             // gathered j points
+    uint16_t *gj;           // their places in the j range
     int lane, nb, npi, nslot;
-    uint32_t icnt, ibeg, jbeg, job, head, tail, ltmask;
-    float cut_r, cut_p;
+    uint32_t jbeg, job;
+    float reach_r, reach_p; // the gathering limits (see CfDevPlan)
+    float pi_inv, pi_n, pi_tol;     // 1 / pi bin width, pi bins, distance from an edge below which the table decides
     float Lx, Ly, Lz, iLx, iLy, iLz;
-    float near2, cut_su;    // mocks: the near-observer test (near2 = 0: off)
-    float ish[3], isl[3];   // mocks with ravg: the item's shift, hi and lo
+    float near2, near_ss;   // mocks: the near-observer test (near2 = 0: off)
 
-    __device__ Warp(const CfPairArgs &args) : a(args) {}
+    __device__ Warp(const CfPairArgs &args) : a(args), lr(args.plan->lr), lp(args.plan->lp) {}
+
+    // index of a gathered point among the sorted points
+    __device__ __forceinline__ uint32_t gidx(const float *bs, uint32_t k) const { return jbeg + gj[(bs - jst) + k]; }
+
+    // Table classes of two separations (bin; nb: outside every bin; nb + 1: for the full tables to decide).
+    // The cell is the separation times lut_scale, rounded to an integer by adding 2^23; values past the
+    // table and NaN clamp to its last cell.
+    __device__ __forceinline__ void lut2(float r0, float r1, uint32_t &c0, uint32_t &c1) const
+    {
+        const u64 n = f2_fma(f2_pack(r0, r1), f2_pack(lut_scale, lut_scale), f2_pack(8388608.0f, 8388608.0f));
+        c0 = lds_u8(lut + min(f2_lo_bits(n), lut_top));
+        c1 = lds_u8(lut + min(f2_hi_bits(n), lut_top));
+    }
 
     __device__ __forceinline__ void push(uint32_t ip, uint32_t jp) { push_recheck(a, ip, jp, job); }
 
-    __device__ __forceinline__ void acc_lp(uint32_t c, float d2, float wp)
+    __device__ __forceinline__ void acc_lp(uint32_t c, float r, float wp)
     {
-        uint32_t idx = c * 32u + lane;
+        const uint32_t idx = c * 32u;       // the histogram pointers carry the lane
         atomicAdd(h_cnt + idx, 1u);
-        float r = 0.f;
-        if (R) {
-            r = f_sqrt_approx(d2);
-            if (KIND == KIND_THETA) r = 2.0f * asinf(0.5f * r) * 57.29577951308232f;
-        }
+        if (R && KIND == KIND_THETA) r = 2.0f * asinf(0.5f * r) * 57.29577951308232f;
         if (W && R) {
-            // both sums of a lane's bin sit in one float4: one 16-byte load and store
-            float4 *p = reinterpret_cast<float4 *>(h_w) + idx;
-            float4 v = *p;
-            kahan_step(v.x, v.y, wp);
-            kahan_step(v.z, v.w, wp * r);
+            // both sums of a lane's bin sit in one 16-byte word (sums, then their compensations): one load,
+            // one packed compensated step, one store
+            ulonglong2 *p = reinterpret_cast<ulonglong2 *>(h_w) + idx;
+            ulonglong2 v = *p;
+            const u64 y = f2_sub(f2_pack(wp, __fmul_rn(wp, r)), v.y);
+            const u64 t = f2_add(v.x, y);
+            v.y = f2_sub(f2_sub(t, v.x), y);
+            v.x = t;
             *p = v;
         } else {
             if (W) kahan_add(h_w + idx, wp);
@@ -270,25 +302,19 @@ struct Warp {
         }
     }
 
-    __device__ __forceinline__ void acc_sh(uint32_t slot, uint32_t rbin, float rp2, float wp)
+    __device__ __forceinline__ void acc_sh(uint32_t slot, uint32_t rbin, float r, float wp)
     {
         if (GH) {
             // no per-warp histogram: straight into the job's global one
             const size_t g = (size_t)job * (uint32_t)nslot + slot;
             atomicAdd(a.hcnt + g, 1ull);
             if (W) atomicAdd(a.hw + g, (double)wp);
-            if (R) {
-                const float r = f_sqrt_approx(rp2);
-                atomicAdd(a.hr + g, (double)(W ? wp * r : r));
-            }
+            if (R) atomicAdd(a.hr + g, (double)(W ? wp * r : r));
             return;
         }
         atomicAdd(h_cnt + slot, 1u);
         if (W) add_sum(h_wd, slot, wp, a.fxw);
-        if (R) {
-            float r = f_sqrt_approx(rp2);
-            add_sum(h_rd, slot, W ? wp * r : r, FX ? fxr_bin[rbin] : 0.f);
-        }
+        if (R) add_sum(h_rd, slot, W ? wp * r : r, FX ? fxr_bin[rbin] : 0.f);
     }
 
     // One term of a per-warp sum: with FX m = round(t * scale) into the slot's two 32-bit words (m
@@ -305,511 +331,299 @@ struct Warp {
         }
     }
 
-    // Histogram slot of N pairs that passed the FP32 cut (squared separation below cut_r and,
-    // for rp-pi and wp, |dz| below cut_p), or K_AMB (re-evaluate in FP64) or K_OUT (outside
-    // every bin).  The table reads of all N are issued before any fine resolution.
-    static constexpr uint32_t K_AMB = 0xFFFFFFFFu, K_OUT = 0xFFFFFFFEu;
-    template <int N>
-    __device__ __forceinline__ void classify(const uint32_t (&vb)[N], const uint32_t (&zb)[N], uint32_t (&k)[N],
-                                             uint32_t (&kr)[N]) const
+    // The i point of a lane, translated by the item's shift.  A lane past the tile holds NaN: every
+    // separation it forms is NaN, which the table puts outside every bin.
+    struct IPoint {
+        u64 s[3], e[3];         // x_i + shift, and with ravg its low part (in both halves)
+        u64 a[3];               // mocks: the absolute position
+        float w;
+        uint32_t p;             // its index among the sorted points
+    };
+
+    __device__ __forceinline__ void load_i(const CfItem &it, uint32_t ip, bool live, IPoint &I) const
     {
-        uint32_t cr[N], cz[N];
+        I.p = ip;
+        I.w = 0.f;
 #pragma unroll
-        for (int n = 0; n < N; n++) {
-            cr[n] = lut_raw_in(lr, vb[n]);
-            cz[n] = has_z(KIND) ? lut_raw_in(lp, zb[n]) : 0u;
+        for (int d = 0; d < 3; d++) {
+            I.s[d] = f2_pack(CUDART_NAN_F, CUDART_NAN_F);
+            I.e[d] = I.a[d] = 0ull;
+        }
+        if (!live) return;
+        const float4 P = a.pt[ip];
+        const float X[3] = {-P.x, -P.y, -P.z};
+        float XL[3] = {0.f, 0.f, 0.f};
+        if (LO) {
+            const float4 l = a.plo[ip];
+            XL[0] = -l.x;
+            XL[1] = -l.y;
+            XL[2] = -l.z;
+        }
+        if (KIND == KIND_MOCKS) {
+            const float4 q = a.pabs[ip];
+            I.a[0] = f2_pack(q.x, q.x);
+            I.a[1] = f2_pack(q.y, q.y);
+            I.a[2] = f2_pack(q.z, q.z);
         }
 #pragma unroll
-        for (int n = 0; n < N; n++) {
-            cr[n] = lut_fine(fine, cr[n], vb[n]);
-            if (has_z(KIND)) cz[n] = lut_fine(fine, cz[n], zb[n]);
-            if (KIND == KIND_R || KIND == KIND_THETA) {
-                k[n] = cr[n] < (uint32_t)nb ? cr[n] : (cr[n] == CFI_CLS_AMB ? K_AMB : K_OUT);
+        for (int d = 0; d < 3; d++) {
+            if (R) {
+                float s, e;
+                two_sum(X[d], it.s[d], s, e);
+                I.s[d] = f2_pack(s, s);
+                const float l = (e + it.slo[d]) + XL[d];
+                I.e[d] = f2_pack(l, l);
             } else {
-                // the pi table starts at 0 with bin 0, so below cut_p it yields a bin or AMB
-                if (max(cr[n], cz[n]) < CFI_CLS_OUT) k[n] = KIND == KIND_RPPI ? cr[n] * npi + cz[n] : cr[n];
-                else k[n] = cr[n] != CFI_CLS_OUT ? K_AMB : K_OUT;
+                const float s = X[d] + it.s[d];
+                I.s[d] = f2_pack(s, s);
             }
-            kr[n] = cr[n];
         }
+        I.w = P.w;
     }
 
-    __device__ __forceinline__ void finish(uint32_t k, uint32_t kr, uint32_t vb, float wp, uint32_t il, uint32_t j)
+    // Add the pair with the gathered point bj (weight wj) to the histogram: rp (or r) bin cr, pi bin cz,
+    // FP32 separation r
+    __device__ __forceinline__ void add_pair(const CfItem &it, const IPoint &I, uint32_t cr, uint32_t cz, float r,
+                                             float wj, const float *bj)
     {
-        if (k < K_OUT) {
-            if (warp_hist(KIND)) acc_sh(k, kr, __uint_as_float(vb), wp);
-            else acc_lp(k, __uint_as_float(vb), wp);
-        } else if (k == K_AMB) {
-            push(ibeg + il, jbeg + j);
-        }
-    }
-
-    __device__ __forceinline__ void bin_in(uint32_t vb, uint32_t zb, float wp, uint32_t il, uint32_t j)
-    {
-        const uint32_t v[1] = {vb}, z[1] = {zb};
-        uint32_t k[1], kr[1];
-        classify<1>(v, z, k, kr);
-        finish(k[0], kr[0], vb, wp, il, j);
-    }
-
-    // bin the ring's candidates with every lane busy: two per lane while 64 are queued, then
-    // 32 at a time; with all = true also the last, partial pass
-    __device__ __forceinline__ void drain(bool all)
-    {
-        __syncwarp();
-        while (tail - head >= 64u) {
-            const uint32_t e0 = (head + lane) & RM, e1 = (head + 32u + lane) & RM;
-            const uint32_t v[2] = {rv[e0], rv[e1]};
-            const uint32_t z[2] = {has_z(KIND) ? rz[e0] : 0u, has_z(KIND) ? rz[e1] : 0u};
-            const uint32_t c0 = rc[e0], c1 = rc[e1];
-            const float w0 = W ? rw[e0] : 0.f, w1 = W ? rw[e1] : 0.f;
-            uint32_t k[2], kr[2];
-            classify<2>(v, z, k, kr);
-            finish(k[0], kr[0], v[0], w0, c0 & 0x7Fu, c0 >> 7);
-            finish(k[1], kr[1], v[1], w1, c1 & 0x7Fu, c1 >> 7);
-            head += 64u;
-        }
-        for (;;) {
-            const uint32_t left = tail - head;
-            if (left == 0u || (!all && left < 32u)) break;
-            const uint32_t n = min(left, 32u);
-            if ((uint32_t)lane < n) {
-                const uint32_t e = (head + lane) & RM;
-                const uint32_t c = rc[e];
-                bin_in(rv[e], has_z(KIND) ? rz[e] : 0u, W ? rw[e] : 0.f, c & 0x7Fu, c >> 7);
-            }
-            head += n;
-        }
-        __syncwarp();
-    }
-
-    // Stage chunk c of the j range into its buffer: arrays 0 x, 1 y, 2 z, 3 w, 4-6 lo parts of
-    // x, y, z (all negated as stored); a j past the end of the range reads the far-away sentinel
-    __device__ __forceinline__ void stage(uint32_t c, uint32_t jcnt)
-    {
-        constexpr uint32_t NA = stage_arrays(W, LO);
-        float *bs = jst + (c & 1u) * NA * JSTAGE;
-        const uint32_t j = c * JSTAGE + lane;
-        if (j < jcnt) {
-            const float *fa = reinterpret_cast<const float *>(a.pa + jbeg + j);
-            const float *fb = reinterpret_cast<const float *>(a.pb + jbeg + j);
-            cp_async4(bs + lane, fa);
-            cp_async4(bs + JSTAGE + lane, fa + 2);
-            cp_async4(bs + 2 * JSTAGE + lane, fb);
-            if (W) cp_async4(bs + 3 * JSTAGE + lane, fb + 2);
-            if (LO) {
-                const float *fl = reinterpret_cast<const float *>(a.plo + 2 * (size_t)(jbeg + j));
-                cp_async4(bs + 4 * JSTAGE + lane, fl);
-                cp_async4(bs + 5 * JSTAGE + lane, fl + 2);
-                cp_async4(bs + 6 * JSTAGE + lane, fl + 4);
-            }
+        const float wp = W ? __fmul_rn(I.w, wj) : 0.f;
+        if (KIND == KIND_MOCKS) {
+            if (R) r = mocks_rp<LO>(a, I.p, bj, it.s[0], it.s[1], it.s[2], it.slo[0], it.slo[1], it.slo[2]);
+            acc_sh(cr * (uint32_t)npi + cz, cr, r, wp);
+        } else if (KIND == KIND_RPPI) {
+            acc_sh(cr * (uint32_t)npi + cz, cr, r, wp);
         } else {
-            bs[lane] = 1e18f;
-            bs[JSTAGE + lane] = 1e18f;
-            bs[2 * JSTAGE + lane] = 1e18f;
-            if (W) bs[3 * JSTAGE + lane] = 0.f;
-            if (LO) bs[4 * JSTAGE + lane] = bs[5 * JSTAGE + lane] = bs[6 * JSTAGE + lane] = 0.f;
+            acc_lp(cr, r, wp);
         }
     }
 
-    // One work item.  Q = i slots per lane; DIAG: the i tile and the j range are the same cell
-    // (only j > i counts; one instance with Q = 4 serves every tile size, the slots past the
-    // tile skipped at run time); COMPACT selects the binning form.
-    template <int Q, bool DIAG, bool COMPACT>
+    // Bin the pairs of this lane's i point with the gathered j points j4 .. j4 + 3 (of the block at bs).
+    // All four are formed and classified at once (independent chains, packed arithmetic); there is no
+    // test for "in range" before the table: a value past the last edge reads the class outside every
+    // bin.  dg: a cell paired with itself; gathered points before position skip do not count for this
+    // lane.
+    __device__ __forceinline__ void bin4(const CfItem &it, const IPoint &I, const float *bs, uint32_t j4, bool dg,
+                                         uint32_t skip)
+    {
+        const float *b = bs + j4;
+        const ulonglong2 xj = *reinterpret_cast<const ulonglong2 *>(b);
+        const ulonglong2 yj = *reinterpret_cast<const ulonglong2 *>(b + GBUF);
+        const ulonglong2 zj = *reinterpret_cast<const ulonglong2 *>(b + 2 * GBUF);
+        u64 q[2], z[2] = {0ull, 0ull};
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            u64 dx = f2_add(I.s[0], h ? xj.y : xj.x), dy = f2_add(I.s[1], h ? yj.y : yj.x),
+                dz = f2_add(I.s[2], h ? zj.y : zj.x);
+            if (R) {
+                u64 ex = I.e[0], ey = I.e[1], ez = I.e[2];
+                if (LO) {
+                    ex = f2_add(ex, *reinterpret_cast<const u64 *>(b + 4 * GBUF + 2 * h));
+                    ey = f2_add(ey, *reinterpret_cast<const u64 *>(b + 5 * GBUF + 2 * h));
+                    ez = f2_add(ez, *reinterpret_cast<const u64 *>(b + 6 * GBUF + 2 * h));
+                }
+                dx = f2_add(dx, ex);
+                dy = f2_add(dy, ey);
+                dz = f2_add(dz, ez);
+            }
+            if (WRAP) {
+                if (Lx > 0.f) dx = wrap2(dx, Lx, iLx);
+                if (Ly > 0.f) dy = wrap2(dy, Ly, iLy);
+                if (Lz > 0.f) dz = wrap2(dz, Lz, iLz);
+            }
+            if (KIND == KIND_MOCKS) {
+                // DD(rp, pi) of observed positions (Appendix A.2.1): pi^2 = (s.l)^2 / l.l and rp^2 =
+                // |s x A_i|^2 / l.l (s x A_i = s x l, because l = A_i - s / 2), whose error scales with
+                // rp where s.s - pi^2 would lose everything below the rounding of s.s when rp << pi
+                const u64 ax = I.a[0], ay = I.a[1], az = I.a[2];
+                const u64 NH = f2_pack(-0.5f, -0.5f);
+                const u64 lx = f2_fma(dx, NH, ax), ly = f2_fma(dy, NH, ay), lz = f2_fma(dz, NH, az);
+                const u64 sl = f2_fma(dz, lz, f2_fma(dy, ly, f2_mul(dx, lx)));
+                const u64 ll = f2_fma(lz, lz, f2_fma(ly, ly, f2_mul(lx, lx)));
+                const u64 cx = f2_sub(f2_mul(dy, az), f2_mul(dz, ay));
+                const u64 cy = f2_sub(f2_mul(dz, ax), f2_mul(dx, az));
+                const u64 cz = f2_sub(f2_mul(dx, ay), f2_mul(dy, ax));
+                const u64 c2 = f2_fma(cz, cz, f2_fma(cy, cy, f2_mul(cx, cx)));
+                const u64 r = f2_pack(f_rcp_approx(f2_lo(ll)), f_rcp_approx(f2_hi(ll)));
+                q[h] = f2_mul(c2, r);
+                z[h] = f2_mul(f2_mul(sl, sl), r);
+                if (near2 > 0.f) {
+                    // a midpoint near the observer, where the error bounds do not hold: FP64 when its
+                    // s.s may count
+                    const u64 ss = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+                    const bool n0 = f2_lo(ll) < near2, n1 = f2_hi(ll) < near2;
+                    if (n0 && f2_lo(ss) < near_ss && (!dg || j4 + 2 * h >= skip)) push(I.p, gidx(bs, j4 + 2 * h));
+                    if (n1 && f2_hi(ss) < near_ss && (!dg || j4 + 2 * h + 1 >= skip)) push(I.p, gidx(bs, j4 + 2 * h + 1));
+                    const float nan = CUDART_NAN_F;
+                    q[h] = f2_pack(n0 ? nan : f2_lo(q[h]), n1 ? nan : f2_hi(q[h]));
+                }
+            } else {
+                q[h] = f2_fma(dy, dy, f2_mul(dx, dx));
+                if (!has_pi(KIND)) q[h] = f2_fma(dz, dz, q[h]);
+                else z[h] = dz & 0x7FFFFFFF7FFFFFFFull;
+            }
+        }
+        float v2[4] = {f2_lo(q[0]), f2_hi(q[0]), f2_lo(q[1]), f2_hi(q[1])};
+        if (dg) {
+#pragma unroll
+            for (int h = 0; h < 4; h++) v2[h] = j4 + h < skip ? CUDART_NAN_F : v2[h];
+        }
+        uint32_t c[4], cz[4] = {0u, 0u, 0u, 0u};
+        float r4[4], T[4] = {0.f, 0.f, 0.f, 0.f}, F[4] = {1.f, 1.f, 1.f, 1.f};
+#pragma unroll
+        for (int h = 0; h < 4; h++) r4[h] = f_sqrt_ftz(v2[h]);
+        lut2(r4[0], r4[1], c[0], c[1]);
+        lut2(r4[2], r4[3], c[2], c[3]);
+        if (has_pi(KIND)) {
+            // the pi bins are equally wide: t = pi / width, its nearest integer by the 2^23 trick, and the
+            // distance from it, which also says whether a pi edge is near
+            const u64 MAGIC = f2_pack(8388608.0f, 8388608.0f);
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                u64 p = z[h];
+                if (KIND == KIND_MOCKS) p = f2_pack(f_sqrt_ftz(f2_lo(p)), f_sqrt_ftz(f2_hi(p)));
+                const u64 t = f2_mul(p, f2_pack(pi_inv, pi_inv));
+                const u64 n = f2_add(t, MAGIC);
+                const u64 f = f2_sub(t, f2_sub(n, MAGIC));
+                T[2 * h] = f2_lo(t);
+                T[2 * h + 1] = f2_hi(t);
+                F[2 * h] = f2_lo(f);
+                F[2 * h + 1] = f2_hi(f);
+                cz[2 * h] = (f2_lo_bits(n) - 0x4B000000u) + (uint32_t)((int)f2_lo_bits(f) >> 31);
+                cz[2 * h + 1] = (f2_hi_bits(n) - 0x4B000000u) + (uint32_t)((int)f2_hi_bits(f) >> 31);
+            }
+        }
+        bool odd = max(max(c[0], c[1]), max(c[2], c[3])) > (uint32_t)nb;
+        if (has_pi(KIND)) odd = odd || fminf(fminf(fabsf(F[0]), fabsf(F[1])), fminf(fabsf(F[2]), fabsf(F[3]))) < pi_tol;
+        if (odd) {
+            // a table cell with an edge in it or a value near a pi edge (one pair in a thousand): the full
+            // tables decide, and what they call ambiguous goes to the FP64 recheck
+            uint32_t todo = 0;
+#pragma unroll
+            for (int h = 0; h < 4; h++) {
+                const bool d = c[h] > (uint32_t)nb || (has_pi(KIND) && c[h] < (uint32_t)nb && fabsf(F[h]) < pi_tol);
+                todo |= (d ? 1u : 0u) << h;
+                c[h] = d ? (uint32_t)nb : c[h];
+            }
+            const float z4[4] = {f2_lo(z[0]), f2_hi(z[0]), f2_lo(z[1]), f2_hi(z[1])};
+            for (; todo; todo &= todo - 1u) {
+                const int h = __ffs(todo) - 1;
+                const uint32_t kr = lut_class(a.lut, a.fine, lr, __float_as_uint(pick4(v2, h)));
+                const uint32_t kz = has_pi(KIND) ? lut_class(a.lut, a.fine, lp, __float_as_uint(pick4(z4, h))) : 0u;
+                if (kr == CFI_CLS_OUT || kz == CFI_CLS_OUT) continue;
+                if (max(kr, kz) == CFI_CLS_AMB) push(I.p, gidx(bs, j4 + h));
+                else add_pair(it, I, kr, kz, R ? f_sqrt_approx(pick4(v2, h)) : 0.f, W ? b[3 * GBUF + h] : 0.f, b + h);
+            }
+        }
+        float wj[4] = {0.f, 0.f, 0.f, 0.f};
+        if (W) {
+            const float4 t = *reinterpret_cast<const float4 *>(b + 3 * GBUF);
+            wj[0] = t.x; wj[1] = t.y; wj[2] = t.z; wj[3] = t.w;
+        }
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            bool in = c[h] < (uint32_t)nb;
+            if (has_pi(KIND)) in = in && T[h] < pi_n;
+            if (W || R || GH) {
+                if (in) add_pair(it, I, c[h], cz[h], r4[h], wj[h], b + h);
+            } else if (KIND == KIND_RPPI || KIND == KIND_MOCKS) {
+                atomicAdd(h_cnt + (in ? c[h] * (uint32_t)npi + cz[h] : (uint32_t)(nslot + lane)), 1u);
+            } else if (KIND == KIND_WP) {
+                atomicAdd(h_cnt + (in ? c[h] : (uint32_t)nb) * 32u, 1u);
+            } else {
+                atomicAdd(h_cnt + c[h] * 32u, 1u);
+            }
+        }
+    }
+
+    // One work item: its i tile in groups of 32 points; for each the j points within reach of the
+    // group's bounding box are gathered in shared memory and counted 32 at a time.
     __device__ __forceinline__ void run(const CfItem &it)
     {
-        // direct form: r and theta issue the distances of all slots before binning any (more
-        // independent chains); rp-pi and wp, whose binning is larger, bin each slot right away
-        constexpr bool SPLIT = !has_z(KIND);
-        icnt = it.cnt & 0xFFFFu;
-        const uint32_t jcnt = it.cnt >> 16;
-        ibeg = it.ibeg;
-        jbeg = it.jbeg;
+        const uint32_t icnt = it.cnt & 0xFFFFu, jcnt = it.cnt >> 16;
+        const bool diag = (it.meta & CFI_ITEM_DIAG) != 0;
         job = it.meta & CFI_ITEM_JOBMASK;
-        u64 sx[Q], sy[Q], sz[Q], ex[Q], ey[Q], ez[Q], wi[Q];
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            const uint32_t il = lane + 32u * q;
-            float vs[3], ve[3], vw = 0.f;
-#pragma unroll
-            for (int d = 0; d < 3; d++) { vs[d] = 1e18f; ve[d] = 0.f; }
-            // empty slots sit far outside every bin (1e18^2 < FLT_MAX); in wrap mode the
-            // minimum image would fold them back, so there they are also masked by icnt
-            if (il < icnt) {
-                const ulonglong2 A = a.pa[ibeg + il], B = a.pb[ibeg + il];
-                const float X[3] = {-f2_lo(A.x), -f2_lo(A.y), -f2_lo(B.x)};
-                float XL[3] = {0.f, 0.f, 0.f};
-                if (LO) {
-                    const ulonglong2 C = a.plo[2 * (size_t)(ibeg + il)], D = a.plo[2 * (size_t)(ibeg + il) + 1];
-                    XL[0] = -f2_lo(C.x);
-                    XL[1] = -f2_lo(C.y);
-                    XL[2] = -f2_lo(D.x);
-                }
-#pragma unroll
-                for (int d = 0; d < 3; d++) {
-                    if (R) {
-                        float s, e;
-                        two_sum(X[d], it.s[d], s, e);
-                        vs[d] = s;
-                        ve[d] = (e + it.slo[d]) + XL[d];
-                    } else {
-                        vs[d] = X[d] + it.s[d];
-                    }
-                }
-                vw = f2_lo(B.y);
-            }
-            sx[q] = f2_pack(vs[0], vs[0]);
-            sy[q] = f2_pack(vs[1], vs[1]);
-            sz[q] = f2_pack(vs[2], vs[2]);
-            ex[q] = f2_pack(ve[0], ve[0]);
-            ey[q] = f2_pack(ve[1], ve[1]);
-            ez[q] = f2_pack(ve[2], ve[2]);
-            wi[q] = f2_pack(vw, vw);
-        }
-        constexpr uint32_t NA = stage_arrays(W, LO);
-        const uint32_t nchunk = (jcnt + JSTAGE - 1) / JSTAGE;
-        stage(0, jcnt);
-        cp_async_commit();
-        for (uint32_t c = 0; c < nchunk; c++) {
-            if (c + 1 < nchunk) stage(c + 1, jcnt);
-            cp_async_commit();
-            cp_async_wait<1>();
-            __syncwarp();
-            const float *bs = jst + (c & 1u) * NA * JSTAGE;
-            const uint32_t j0 = c * JSTAGE;
-            const uint32_t n = min(JSTAGE, jcnt - j0);
-            // within a cell paired with itself, slot q (i >= 32 q) has a live pair in this
-            // chunk (j <= 32 c + 31) only if q <= c, and none past the tile
-            const int nq = DIAG ? min((int)((icnt + 31u) >> 5), (int)c + 1) : Q;
-#pragma unroll 1
-            for (uint32_t jj = 0; jj < n; jj += 2) {
-                const uint32_t j = j0 + jj;
-                const u64 xj = *reinterpret_cast<const u64 *>(bs + jj);
-                const u64 yj = *reinterpret_cast<const u64 *>(bs + JSTAGE + jj);
-                const u64 zj = *reinterpret_cast<const u64 *>(bs + 2 * JSTAGE + jj);
-                // the j weights, read once for all slots (rp-pi / wp bin where formed)
-                const u64 wjd = (W && !SPLIT && !COMPACT) ? *reinterpret_cast<const u64 *>(bs + 3 * JSTAGE + jj) : 0ull;
-                u64 lx = 0, ly = 0, lz = 0;
-                if (LO) {
-                    lx = *reinterpret_cast<const u64 *>(bs + 4 * JSTAGE + jj);
-                    ly = *reinterpret_cast<const u64 *>(bs + 5 * JSTAGE + jj);
-                    lz = *reinterpret_cast<const u64 *>(bs + 6 * JSTAGE + jj);
-                }
-                // the distances and cuts of every slot first (independent chains), then the
-                // binning; in the compacting form bits 2q and 2q + 1 of m: slot q's pair with j
-                // and with j + 1 is below the cut
-                u64 v2[Q], az[Q];
-                bool p0[Q], p1[Q];
-                uint32_t m = 0;
-#pragma unroll
-                for (int q = 0; q < Q; q++) {
-                    v2[q] = az[q] = 0ull;
-                    p0[q] = p1[q] = false;
-                    if (DIAG && q >= nq) continue;
-                    u64 dx = f2_add(sx[q], xj), dy = f2_add(sy[q], yj), dz = f2_add(sz[q], zj);
-                    if (R) {
-                        dx = f2_add(dx, LO ? f2_add(ex[q], lx) : ex[q]);
-                        dy = f2_add(dy, LO ? f2_add(ey[q], ly) : ey[q]);
-                        dz = f2_add(dz, LO ? f2_add(ez[q], lz) : ez[q]);
-                    }
-                    if (WRAP) {
-                        if (Lx > 0.f) dx = wrap2(dx, Lx, iLx);
-                        if (Ly > 0.f) dy = wrap2(dy, Ly, iLy);
-                        if (Lz > 0.f) dz = wrap2(dz, Lz, iLz);
-                    }
-                    const uint32_t il = lane + 32u * q;
-                    bool in0, in1;
-                    v2[q] = f2_mul(dx, dx);
-                    v2[q] = f2_fma(dy, dy, v2[q]);
-                    if (KIND == KIND_R || KIND == KIND_THETA) {
-                        v2[q] = f2_fma(dz, dz, v2[q]);
-                        in0 = f2_lo(v2[q]) < cut_r;
-                        in1 = f2_hi(v2[q]) < cut_r;
-                    } else {
-                        az[q] = dz & 0x7FFFFFFF7FFFFFFFull;
-                        in0 = f2_lo(v2[q]) < cut_r && f2_lo(az[q]) < cut_p;
-                        in1 = f2_hi(v2[q]) < cut_r && f2_hi(az[q]) < cut_p;
-                    }
-                    // within a cell paired with itself only j > i counts; in wrap mode the
-                    // minimum image folds the far-away sentinels back, so mask them here
-                    if (DIAG) {
-                        in0 = in0 && j > il;
-                        in1 = in1 && j + 1 > il;
-                    }
-                    if (WRAP) {
-                        const bool li = il < icnt;
-                        in0 = in0 && li;
-                        in1 = in1 && li && j + 1 < jcnt;
-                    }
-                    p0[q] = in0;
-                    p1[q] = in1;
-                    if (COMPACT) {
-                        m |= (in0 ? 1u : 0u) << (2 * q);
-                        m |= (in1 ? 2u : 0u) << (2 * q);
-                    } else if (!SPLIT && (in0 || in1)) {
-                        // direct form, rp-pi / wp: bin where formed
-                        const u64 wp = W ? f2_mul(wi[q], wjd) : 0ull;
-                        if (in0) bin_in(f2_lo_bits(v2[q]), f2_lo_bits(az[q]), f2_lo(wp), il, j);
-                        if (in1) bin_in(f2_hi_bits(v2[q]), f2_hi_bits(az[q]), f2_hi(wp), il, j + 1);
-                    }
-                }
-                if (!COMPACT && SPLIT) {
-                    // direct form, r / theta: bin after every slot's distances are issued (the j
-                    // weights read once for all slots)
-                    const u64 wj = W ? *reinterpret_cast<const u64 *>(bs + 3 * JSTAGE + jj) : 0ull;
-#pragma unroll
-                    for (int q = 0; q < Q; q++) {
-                        if (p0[q] || p1[q]) {
-                            const uint32_t il = lane + 32u * q;
-                            const u64 wp = W ? f2_mul(wi[q], wj) : 0ull;
-                            if (p0[q]) bin_in(f2_lo_bits(v2[q]), f2_lo_bits(az[q]), f2_lo(wp), il, j);
-                            if (p1[q]) bin_in(f2_hi_bits(v2[q]), f2_hi_bits(az[q]), f2_hi(wp), il, j + 1);
-                        }
-                    }
-                }
-                if (COMPACT && __any_sync(CF_FULL, m != 0u)) {
-                    // offsets of this lane's candidates: a prefix sum of the per-lane counts
-                    // (<= 2Q) from one ballot per bit of the count
-                    const u64 wj = W ? *reinterpret_cast<const u64 *>(bs + 3 * JSTAGE + jj) : 0ull;
-                    const uint32_t cnt = __popc(m);
-                    constexpr int CB = Q == 1 ? 2 : (Q == 2 ? 3 : 4);
-                    uint32_t pre = 0, tot = 0;
-#pragma unroll
-                    for (int b = 0; b < CB; b++) {
-                        const uint32_t bal = __ballot_sync(CF_FULL, (cnt >> b) & 1u);
-                        pre += (uint32_t)__popc(bal & ltmask) << b;
-                        tot += (uint32_t)__popc(bal) << b;
-                    }
-                    uint32_t pos = tail + pre;
-#pragma unroll
-                    for (int q = 0; q < Q; q++) {
-                        const uint32_t mq = (m >> (2 * q)) & 3u;
-                        if (!mq) continue;
-                        const u64 wp = W ? f2_mul(wi[q], wj) : 0ull;
-                        const uint32_t code = (lane + 32u * q) | (j << 7);
-                        if (mq & 1u) {
-                            const uint32_t e = pos & RM;
-                            rv[e] = f2_lo_bits(v2[q]);
-                            if (has_z(KIND)) rz[e] = f2_lo_bits(az[q]);
-                            rc[e] = (uint16_t)code;
-                            if (W) rw[e] = f2_lo(wp);
-                            pos++;
-                        }
-                        if (mq & 2u) {
-                            const uint32_t e = pos & RM;
-                            rv[e] = f2_hi_bits(v2[q]);
-                            if (has_z(KIND)) rz[e] = f2_hi_bits(az[q]);
-                            rc[e] = (uint16_t)(code + 128u);    // j + 1
-                            if (W) rw[e] = f2_hi(wp);
-                            pos++;
-                        }
-                    }
-                    // the ring held < 32 candidates and took <= 64 Q: at most 287 of RING
-                    tail += tot;
-                    if (tail - head >= 32u) drain(false);
-                }
-            }
-            __syncwarp();       // the chunk buffer is refilled two chunks later
-        }
-        cp_async_wait<0>();
-        __syncwarp();
-        if (COMPACT) drain(true);
-    }
-
-    // ---- DD(rp, pi) of observed positions (Appendix A.2.1) ----
-    // Bin one mocks candidate from its FP32 |s x A_i|^2, (s.l)^2 and l.l: pi^2 = (s.l)^2 / l.l and
-    // rp^2 = |s x A_i|^2 / l.l (s x A_i = s x l), whose error scales with rp where s.s - pi^2 would
-    // lose everything below the rounding of s.s when rp << pi.  il, j: the pair within the item
-    // (j's chunk is the one staged now).
-    __device__ __forceinline__ void bin_mocks(float c2, float sl2, float ll, float wp, uint32_t il, uint32_t j)
-    {
-        if (near2 > 0.f && ll < near2) {
-            push(ibeg + il, jbeg + j);        // midpoint near the observer: FP64
-            return;
-        }
-        const float r = __fdividef(1.0f, ll);
-        const float pi2 = sl2 * r;
-        const float rp2 = c2 * r;
-        const uint32_t cr = lut_class(lr, fine, __float_as_uint(rp2));
-        const uint32_t cz = lut_class(lp, fine, __float_as_uint(pi2));
-        if (cr == CFI_CLS_OUT || cz == CFI_CLS_OUT) return;
-        if (max(cr, cz) == CFI_CLS_AMB) {
-            push(ibeg + il, jbeg + j);
-            return;
-        }
-        const uint32_t slot = cr * (uint32_t)npi + cz;
-        if (GH) {
-            const size_t g = (size_t)job * (uint32_t)nslot + slot;
-            atomicAdd(a.hcnt + g, 1ull);
-            if (W) atomicAdd(a.hw + g, (double)wp);
-            if (R) {
-                constexpr uint32_t NA = stage_arrays(W, LO);
-                const float *bs = jst + ((j / JSTAGE) & 1u) * NA * JSTAGE;
-                const float rr = mocks_rp<LO>(a, ibeg + il, bs, j % JSTAGE, ish[0], ish[1], ish[2], isl[0], isl[1],
-                                              isl[2]);
-                atomicAdd(a.hr + g, (double)(W ? wp * rr : rr));
-            }
-            return;
-        }
-        atomicAdd(h_cnt + slot, 1u);
-        if (W) add_sum(h_wd, slot, wp, a.fxw);
-        if (R) {
-            // the j point is in the stage buffer of its chunk
-            constexpr uint32_t NA = stage_arrays(W, LO);
-            const float *bs = jst + ((j / JSTAGE) & 1u) * NA * JSTAGE;
-            const float rr = mocks_rp<LO>(a, ibeg + il, bs, j % JSTAGE, ish[0], ish[1], ish[2], isl[0], isl[1],
-                                          isl[2]);
-            add_sum(h_rd, slot, W ? wp * rr : rr, FX ? fxr_bin[cr] : 0.f);
-        }
-    }
-
-    // One work item of the mocks kind (the direct form; Q and DIAG as in run).  Per pair, packed
-    // FP32x2: s = v_i - v_j (cell-relative), l = A_i - s / 2, u = s.s - cut_r, s.l, l.l; the
-    // candidate cut needs no division: rp^2 = s.s - pi^2 < cut_r and pi^2 < cut_p become
-    // u l.l < (s.l)^2 < cut_p l.l (cut_r lies above the last edge by twice this form's error).
-    // When either pair of a slot passes, |s x A_i|^2 of both is formed packed and each passing
-    // pair is binned by bin_mocks where it was formed.  (A compacting form -- candidates to a
-    // per-warp ring by ballot prefix, binned 32 at a time -- was measured slower: 4.69 against
-    // 4.32 ms on the 200k x 2M survey cone, more warp instructions and full-width shared
-    // atomics on few slots.)
-    template <int Q, bool DIAG>
-    __device__ __forceinline__ void run_mocks(const CfItem &it)
-    {
-        icnt = it.cnt & 0xFFFFu;
-        const uint32_t jcnt = it.cnt >> 16;
-        ibeg = it.ibeg;
         jbeg = it.jbeg;
-        job = it.meta & CFI_ITEM_JOBMASK;
-        if (R) {
-#pragma unroll
-            for (int d = 0; d < 3; d++) { ish[d] = it.s[d]; isl[d] = it.slo[d]; }
-        }
-        u64 sx[Q], sy[Q], sz[Q], ex[Q], ey[Q], ez[Q], ax[Q], ay[Q], az[Q], wi[Q];
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            const uint32_t il = lane + 32u * q;
-            float vs[3], ve[3], va[3], vw = 0.f;
-#pragma unroll
-            for (int d = 0; d < 3; d++) { vs[d] = 1e18f; ve[d] = 0.f; va[d] = 0.f; }
-            if (il < icnt) {
-                const ulonglong2 A = a.pa[ibeg + il], B = a.pb[ibeg + il];
-                const float X[3] = {-f2_lo(A.x), -f2_lo(A.y), -f2_lo(B.x)};
-                va[0] = f2_hi(A.x);
-                va[1] = f2_hi(A.y);
-                va[2] = f2_hi(B.x);
-                float XL[3] = {0.f, 0.f, 0.f};
-                if (LO) {
-                    const ulonglong2 C = a.plo[2 * (size_t)(ibeg + il)], D = a.plo[2 * (size_t)(ibeg + il) + 1];
-                    XL[0] = -f2_lo(C.x);
-                    XL[1] = -f2_lo(C.y);
-                    XL[2] = -f2_lo(D.x);
-                }
-#pragma unroll
-                for (int d = 0; d < 3; d++) {
-                    if (R) {
-                        float t, e;
-                        two_sum(X[d], it.s[d], t, e);
-                        vs[d] = t;
-                        ve[d] = (e + it.slo[d]) + XL[d];
-                    } else {
-                        vs[d] = X[d] + it.s[d];
-                    }
-                }
-                vw = f2_lo(B.y);
-            }
-            sx[q] = f2_pack(vs[0], vs[0]);
-            sy[q] = f2_pack(vs[1], vs[1]);
-            sz[q] = f2_pack(vs[2], vs[2]);
-            ex[q] = f2_pack(ve[0], ve[0]);
-            ey[q] = f2_pack(ve[1], ve[1]);
-            ez[q] = f2_pack(ve[2], ve[2]);
-            ax[q] = f2_pack(va[0], va[0]);
-            ay[q] = f2_pack(va[1], va[1]);
-            az[q] = f2_pack(va[2], va[2]);
-            wi[q] = f2_pack(vw, vw);
-        }
-        const u64 NH = f2_pack(-0.5f, -0.5f), NCR = f2_pack(-cut_r, -cut_r), CP = f2_pack(cut_p, cut_p);
-        constexpr uint32_t NA = stage_arrays(W, LO);
-        const uint32_t nchunk = (jcnt + JSTAGE - 1) / JSTAGE;
-        stage(0, jcnt);
-        cp_async_commit();
-        for (uint32_t c = 0; c < nchunk; c++) {
-            if (c + 1 < nchunk) stage(c + 1, jcnt);
-            cp_async_commit();
-            cp_async_wait<1>();
-            __syncwarp();
-            const float *bs = jst + (c & 1u) * NA * JSTAGE;
-            const uint32_t j0 = c * JSTAGE;
-            const uint32_t n = min(JSTAGE, jcnt - j0);
-            const int nq = DIAG ? min((int)((icnt + 31u) >> 5), (int)c + 1) : Q;
+        const uint32_t upto = 0xFFFFFFFFu >> (31 - lane);       // the lanes up to this one
 #pragma unroll 1
-            for (uint32_t jj = 0; jj < n; jj += 2) {
-                const uint32_t j = j0 + jj;
-                const u64 xj = *reinterpret_cast<const u64 *>(bs + jj);
-                const u64 yj = *reinterpret_cast<const u64 *>(bs + JSTAGE + jj);
-                const u64 zj = *reinterpret_cast<const u64 *>(bs + 2 * JSTAGE + jj);
-                u64 lxj = 0, lyj = 0, lzj = 0;
-                if (LO) {
-                    lxj = *reinterpret_cast<const u64 *>(bs + 4 * JSTAGE + jj);
-                    lyj = *reinterpret_cast<const u64 *>(bs + 5 * JSTAGE + jj);
-                    lzj = *reinterpret_cast<const u64 *>(bs + 6 * JSTAGE + jj);
-                }
-#pragma unroll
-                for (int q = 0; q < Q; q++) {
-                    if (DIAG && q >= nq) continue;
-                    u64 dx = f2_add(sx[q], xj), dy = f2_add(sy[q], yj), dz = f2_add(sz[q], zj);
-                    if (R) {
-                        dx = f2_add(dx, LO ? f2_add(ex[q], lxj) : ex[q]);
-                        dy = f2_add(dy, LO ? f2_add(ey[q], lyj) : ey[q]);
-                        dz = f2_add(dz, LO ? f2_add(ez[q], lzj) : ez[q]);
-                    }
-                    const u64 lx = f2_fma(dx, NH, ax[q]), ly = f2_fma(dy, NH, ay[q]), lz = f2_fma(dz, NH, az[q]);
-                    u64 uu = f2_fma(dx, dx, NCR);
-                    uu = f2_fma(dy, dy, uu);
-                    uu = f2_fma(dz, dz, uu);
-                    u64 sl = f2_mul(dx, lx);
-                    sl = f2_fma(dy, ly, sl);
-                    sl = f2_fma(dz, lz, sl);
-                    u64 ll = f2_mul(lx, lx);
-                    ll = f2_fma(ly, ly, ll);
-                    ll = f2_fma(lz, lz, ll);
-                    const u64 sl2 = f2_mul(sl, sl);
-                    const u64 m = f2_mul(uu, ll);
-                    const u64 cpl = f2_mul(CP, ll);
-                    bool in0 = f2_lo(m) < f2_lo(sl2) && f2_lo(sl2) < f2_lo(cpl);
-                    bool in1 = f2_hi(m) < f2_hi(sl2) && f2_hi(sl2) < f2_hi(cpl);
-                    if (near2 > 0.f) {
-                        // a midpoint near the observer makes the multiplied cut meaningless:
-                        // there only s.s decides, and the pair goes to FP64
-                        if (f2_lo(ll) < near2) in0 = f2_lo(uu) < cut_su;
-                        if (f2_hi(ll) < near2) in1 = f2_hi(uu) < cut_su;
-                    }
-                    const uint32_t il = lane + 32u * q;
-                    // empty slots and j past the range hold far-away sentinels whose products
-                    // overflow; mask them by index rather than rely on those comparisons
-                    in0 = in0 && il < icnt;
-                    in1 = in1 && il < icnt && j + 1 < jcnt;
-                    if (DIAG) {
-                        in0 = in0 && j > il;
-                        in1 = in1 && j + 1 > il;
-                    }
-                    if (in0 || in1) {
-                        // |s x A_i|^2 of both pairs at once
-                        const u64 cx = f2_sub(f2_mul(dy, az[q]), f2_mul(dz, ay[q]));
-                        const u64 cy = f2_sub(f2_mul(dz, ax[q]), f2_mul(dx, az[q]));
-                        const u64 cz = f2_sub(f2_mul(dx, ay[q]), f2_mul(dy, ax[q]));
-                        const u64 c2 = f2_fma(cz, cz, f2_fma(cy, cy, f2_mul(cx, cx)));
-                        const u64 wj = W ? *reinterpret_cast<const u64 *>(bs + 3 * JSTAGE + jj) : 0ull;
-                        const u64 wp = W ? f2_mul(wi[q], wj) : 0ull;
-                        if (in0) bin_mocks(f2_lo(c2), f2_lo(sl2), f2_lo(ll), f2_lo(wp), il, j);
-                        if (in1) bin_mocks(f2_hi(c2), f2_hi(sl2), f2_hi(ll), f2_hi(wp), il, j + 1);
-                    }
-                }
+        for (uint32_t i0 = 0; i0 < icnt; i0 += 32u) {
+            // a cell paired with itself: only j > i counts, so the points from this group on
+            uint32_t j0 = diag ? i0 : 0u;
+            const float4 *pj = a.pt + (jbeg + j0 + lane), *lj = LO ? a.plo + (jbeg + j0 + lane) : nullptr;
+            float4 P = make_float4(0.f, 0.f, 0.f, 0.f), Q = P;
+            if (j0 + lane < jcnt) {
+                P = *pj;
+                if (LO) Q = *lj;
             }
-            __syncwarp();       // the chunk buffer is refilled two chunks later
+            IPoint I;
+            load_i(it, it.ibeg + i0 + lane, i0 + lane < icnt, I);
+            float lo[3], hi[3];     // the group's box; the NaN of an empty lane drops out
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                lo[d] = f_redux_min(f2_lo(I.s[d]));
+                hi[d] = f_redux_max(f2_lo(I.s[d]));
+            }
+            // head: where the block to count next starts in the ring (0 or 32); fill: points gathered there
+            uint32_t head = 0, fill = 0, skip = 0;
+            bool dg = diag;
+            for (;;) {
+#pragma unroll 1
+                while (fill < 32u && j0 < jcnt) {
+                    const float4 C = P, E = Q;
+                    const bool live = j0 + lane < jcnt;
+                    j0 += 32u;
+                    pj += 32;
+                    if (LO) lj += 32;
+                    if (j0 + lane < jcnt) {
+                        P = *pj;
+                        if (LO) Q = *lj;
+                    }
+                    bool keep = live;
+                    if (!WRAP) {
+                        // the smallest separation a point of the group can have from this j point:
+                        // each operation rounds monotonically, so a point is only dropped when all 32
+                        // pairs lie past the limit
+                        const float gx = fmaxf(fmaxf(lo[0] + C.x, -hi[0] - C.x), 0.f);
+                        const float gy = fmaxf(fmaxf(lo[1] + C.y, -hi[1] - C.y), 0.f);
+                        const float gz = fmaxf(fmaxf(lo[2] + C.z, -hi[2] - C.z), 0.f);
+                        float t = fmaf(gy, gy, fmaf(gx, gx, -reach_r));
+                        if (has_z(KIND)) keep = keep && fmaf(gz, gz, -reach_p) < 0.f;
+                        else t = fmaf(gz, gz, t);
+                        keep = keep && t < 0.f;
+                    }
+                    const uint32_t m = __ballot_sync(CF_FULL, keep);
+                    const uint32_t rank = __popc(m & upto);
+                    if (keep) {
+                        const uint32_t k = (head + fill + rank - 1u) & (GBUF - 1u);
+                        float *q = jst + k;
+                        q[0] = C.x;
+                        q[GBUF] = C.y;
+                        q[2 * GBUF] = C.z;
+                        if (W) q[3 * GBUF] = C.w;
+                        if (LO) {
+                            q[4 * GBUF] = E.x;
+                            q[5 * GBUF] = E.y;
+                            q[6 * GBUF] = E.z;
+                        }
+                        gj[k] = (uint16_t)(j0 - 32u + lane);
+                    }
+                    // in a cell paired with itself the group's own points come first: those up to lane i
+                    // (i itself among them) do not count for it
+                    if (dg && fill == 0u) skip = rank;
+                    fill += __popc(m);
+                }
+                if (fill == 0u) break;
+                if (fill < 32u && lane < 3) jst[(head + fill + lane) & (GBUF - 1u)] = CUDART_NAN_F;    // up to a multiple of four
+                __syncwarp();
+                const float *bs = jst + head;
+                const uint32_t n = min(fill, 32u);
+#pragma unroll 1
+                for (uint32_t j4 = 0; j4 < n; j4 += 4u) bin4(it, I, bs, j4, dg, skip);
+                __syncwarp();       // the block's place is filled again
+                head ^= 32u;
+                fill -= n;
+                dg = false;
+            }
         }
-        cp_async_wait<0>();
-        __syncwarp();
     }
 
     __device__ void flush(uint32_t jb)
@@ -844,20 +658,21 @@ struct Warp {
                     }
                 }
             } else {
-                constexpr int ST = (W && R) ? 2 : 1;     // float2 stride of the Kahan sums
                 for (int l = 0; l < 32; l++) {
-                    int idx = sl * 32 + ((l + lane) & 31);
+                    const int idx = sl * 32 + ((l + lane) & 31) - lane;
                     c += h_cnt[idx];
                     h_cnt[idx] = 0;
-                    if (W) {
-                        float2 v = h_w[ST * idx];
-                        ws += (double)v.x - (double)v.y;
-                        h_w[ST * idx] = make_float2(0.f, 0.f);
-                    }
-                    if (R) {
-                        float2 v = h_r[ST * idx];
-                        rs += (double)v.x - (double)v.y;
-                        h_r[ST * idx] = make_float2(0.f, 0.f);
+                    if (W && R) {
+                        float4 *q = reinterpret_cast<float4 *>(h_w) + idx;
+                        const float4 v = *q;
+                        ws += (double)v.x - (double)v.z;
+                        rs += (double)v.y - (double)v.w;
+                        *q = make_float4(0.f, 0.f, 0.f, 0.f);
+                    } else if (W || R) {
+                        float2 *q = (W ? h_w : h_r) + idx;
+                        const float2 v = *q;
+                        (W ? ws : rs) += (double)v.x - (double)v.y;
+                        *q = make_float2(0.f, 0.f);
                     }
                 }
             }
@@ -874,26 +689,23 @@ struct Warp {
 // launcher takes as many as fit); count-only CTAs are small, and a budget for 4 of 256 threads per
 // SM (64 registers, no spills in the rp-pi instances) keeps more of them resident than one for 3.
 __host__ __device__ constexpr int pair_max_threads(bool W, bool R) { return (W || R) ? 512 : 256; }
-__host__ __device__ constexpr int pair_min_blocks(bool W, bool R) { return (!W && !R) ? 4 : 1; }
+__host__ __device__ constexpr int pair_min_blocks(bool W, bool R) { return (!W && !R) ? 3 : 1; }
 
-template <int KIND, bool W, bool R, bool WRAP, bool LO, bool COMPACT, bool GH, bool FX>
+template <int KIND, bool W, bool R, bool WRAP, bool LO, bool GH, bool FX>
 __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
     pair_kernel(const CfPairArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const CfDevPlan *__restrict__ P = a.plan;
-    const int nlw = P->nlut_words, nf = P->nfine;
-    uint16_t *s_lut = (uint16_t *)smem;
-    CfFine *s_fine = (CfFine *)(smem + align16(2u * nlw));
-    float *s_fxr = (float *)(s_fine + nf);      // rp-pi / mocks: per rp bin scale of the ravg terms
+    const uint32_t nl4 = align16((uint32_t)P->nlut8) / 4u;
+    float *s_fxr = (float *)(smem + 4u * nl4);          // rp-pi / mocks: per rp bin scale of the ravg terms
     unsigned char *wbase = (unsigned char *)s_fxr + (warp_hist(KIND) ? align16(4u * (uint32_t)a.nb) : 0u);
-    for (int i = threadIdx.x; i < nlw; i += blockDim.x) s_lut[i] = a.lut[i];
-    for (int i = threadIdx.x; i < nf; i += blockDim.x) s_fine[i] = a.fine[i];
+    for (uint32_t i = threadIdx.x; i < nl4; i += blockDim.x) ((uint32_t *)smem)[i] = ((const uint32_t *)a.lut8)[i];
     if (FX && R)
         for (int i = threadIdx.x; i < a.nb; i += blockDim.x) s_fxr[i] = a.fxr_bin[i];
     const int hslots = GH ? 0 : a.nslot;        // slots of the per-warp histogram
-    const uint32_t wb = warp_bytes(KIND, W, R, LO, hslots, COMPACT);
-    const uint32_t hoff = warp_jbuf_bytes(W, LO) + (COMPACT ? warp_ring_bytes(KIND, W) : 0u);
+    const uint32_t wb = warp_bytes(KIND, W, R, LO, hslots);
+    const uint32_t hoff = warp_jbuf_bytes(W, LO);
     unsigned char *my = wbase + (size_t)(threadIdx.x >> 5) * wb;
     {
         // zero this warp's histogram (the buffers need no initial value)
@@ -908,42 +720,35 @@ __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
     w.nb = a.nb;
     w.npi = a.npi;
     w.nslot = a.nslot;
-    w.fine = s_fine;
     w.fxr_bin = s_fxr;
-    w.lr = {P->lr.base, P->lr.shift, P->lr.last, s_lut + P->lr.coff};
-    w.lp = {P->lp.base, P->lp.shift, P->lp.last, s_lut + P->lp.coff};
-    w.cut_r = P->cut_r;
-    w.cut_p = P->cut_p;
+    w.lut = (uint32_t)__cvta_generic_to_shared(smem) - 0x4B000000u;
+    w.lut_top = 0x4B000000u + (uint32_t)P->nlut8 - 1u;
+    w.lut_scale = P->lut8_scale;
+    w.reach_r = P->reach_r;
+    w.reach_p = P->reach_p;
+    w.pi_inv = P->pi_inv;
+    w.pi_n = P->pi_n;
+    w.pi_tol = P->pi_tol;
     w.near2 = P->near2;
-    w.cut_su = P->cut_su;
+    w.near_ss = P->near_ss;
     w.Lx = a.L[0]; w.Ly = a.L[1]; w.Lz = a.L[2];
     w.iLx = a.L[0] > 0.f ? 1.0f / a.L[0] : 0.f;
     w.iLy = a.L[1] > 0.f ? 1.0f / a.L[1] : 0.f;
     w.iLz = a.L[2] > 0.f ? 1.0f / a.L[2] : 0.f;
-    w.ltmask = (1u << w.lane) - 1u;
-    w.head = w.tail = 0u;
     w.jst = (float *)my;
-    {
-        unsigned char *q = my + warp_jbuf_bytes(W, LO);
-        w.rv = (uint32_t *)q;
-        q += RING * 4u;
-        w.rz = has_z(KIND) ? (uint32_t *)q : nullptr;
-        q += has_z(KIND) ? RING * 4u : 0u;
-        w.rw = W ? (float *)q : nullptr;
-        q += W ? RING * 4u : 0u;
-        w.rc = (uint16_t *)q;
-    }
+    w.gj = (uint16_t *)(my + stage_arrays(W, LO) * GBUF * 4u);
     w.h_cnt = (uint32_t *)(my + hoff);
     if (warp_hist(KIND)) {
-        uint32_t o = ((uint32_t)hslots * 4u + 7u) & ~7u;
+        uint32_t o = (((uint32_t)hslots + (W || R ? 0u : 32u)) * 4u + 7u) & ~7u;
         w.h_wd = (double *)(my + hoff + o);
         w.h_rd = (double *)(my + hoff + o + (W ? hslots * 8u : 0u));
         w.h_w = w.h_r = nullptr;
     } else {
         uint32_t o = a.nslot * 32u * 4u;
-        // with both sums they interleave (float4 per lane and bin: w, w-comp, r, r-comp)
-        w.h_w = (float2 *)(my + hoff + o);
-        w.h_r = (W && R) ? w.h_w + 1 : (float2 *)(my + hoff + o + (W ? a.nslot * 32u * 8u : 0u));
+        // with both sums they interleave (float4 per lane and bin: w, r, their compensations)
+        w.h_w = (float2 *)(my + hoff + o) + (W && R ? 2 : 1) * w.lane;
+        w.h_r = w.h_w;      // only one of them is kept on its own
+        w.h_cnt += w.lane;
         w.h_wd = w.h_rd = nullptr;
     }
 
@@ -957,49 +762,33 @@ __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
     if (w.lane == 0) t = atomicAdd(a.cursor, 1u);
     t = __shfl_sync(CF_FULL, t, 0);
     CfItem it;
-    if (t < nitems) it = a.items[a.order ? a.order[t] : t];
+    if (t < nitems) it = a.items[t];
     for (;;) {
         if (t >= nitems) break;
         uint32_t tn = 0;
         if (w.lane == 0) tn = atomicAdd(a.cursor, 1u);
         tn = __shfl_sync(CF_FULL, tn, 0);
         CfItem nx;
-        if (tn < nitems) nx = a.items[a.order ? a.order[tn] : tn];
+        if (tn < nitems) nx = a.items[tn];
         const int job = (int)(it.meta & CFI_ITEM_JOBMASK);
         if (job != cur || pend > (FX ? FX_FLUSH_PAIRS : CF_FLUSH_PAIRS)) {
             if (cur >= 0) w.flush((uint32_t)cur);
             cur = job;
             pend = 0;
         }
-        const bool diag = (it.meta & CFI_ITEM_DIAG) != 0;
-        const uint32_t ic = it.cnt & 0xFFFFu;
-        pend += ic * (it.cnt >> 16);
-        // the instances below are the classes of cf_item_class; the work list comes ordered by
-        // class, so the warps of an SM mostly run one instance (its code stays in the
-        // instruction cache)
-        if (KIND == KIND_MOCKS) {
-            if (diag) w.template run_mocks<4, true>(it);
-            else if (ic <= 32u) w.template run_mocks<1, false>(it);
-            else if (ic <= 64u) w.template run_mocks<2, false>(it);
-            else w.template run_mocks<4, false>(it);
-        } else {
-            if (diag) w.template run<4, true, COMPACT>(it);
-            else if (ic <= 32u) w.template run<1, false, COMPACT>(it);
-            else if (ic <= 64u) w.template run<2, false, COMPACT>(it);
-            else if (ic <= 96u) w.template run<3, false, COMPACT>(it);
-            else w.template run<4, false, COMPACT>(it);
-        }
+        pend += (it.cnt & 0xFFFFu) * (it.cnt >> 16);
+        w.run(it);
         t = tn;
         it = nx;
     }
     if (cur >= 0) w.flush((uint32_t)cur);
 }
 
-template <int KIND, bool W, bool R, bool WRAP, bool LO, bool COMPACT, bool GH = false, bool FX = false>
+template <int KIND, bool W, bool R, bool WRAP, bool LO, bool GH = false, bool FX = false>
 cudaError_t launch_variant(const CfPairCfg &c, const CfPairArgs &a, int num_sms, cudaStream_t st, int *grid_out,
                            int *warps_out)
 {
-    auto k = pair_kernel<KIND, W, R, WRAP, LO, COMPACT, GH, FX>;
+    auto k = pair_kernel<KIND, W, R, WRAP, LO, GH, FX>;
     int dev;
     cudaGetDevice(&dev);
     int maxsm = 0;
@@ -1027,20 +816,18 @@ cudaError_t launch_variant(const CfPairCfg &c, const CfPairArgs &a, int num_sms,
     return cudaGetLastError();
 }
 
-// variant 1 = direct, 2 = compacting (0 picks one per kind: see cfp_default_variant)
+// global histograms (rp-pi and mocks tables too large for shared memory), fixed-point per-warp sums, or
+// the plain form
 template <int KIND, bool W, bool R, bool WRAP, bool LO>
 cudaError_t launch_one(const CfPairCfg &c, const CfPairArgs &a, int num_sms, cudaStream_t st, int *grid_out,
                        int *warps_out)
 {
-    // global histograms (rp-pi tables too large for shared memory): the direct form only
     if constexpr (warp_hist(KIND))
-        if (c.ghist) return launch_variant<KIND, W, R, WRAP, LO, false, true>(c, a, num_sms, st, grid_out, warps_out);
-    // fixed-point per-warp sums: the direct form only
+        if (c.ghist) return launch_variant<KIND, W, R, WRAP, LO, true>(c, a, num_sms, st, grid_out, warps_out);
     if constexpr (warp_hist(KIND) && (W || R))
         if (a.fxw != 0.f || a.fxr != 0.f)
-            return launch_variant<KIND, W, R, WRAP, LO, false, false, true>(c, a, num_sms, st, grid_out, warps_out);
-    if (c.variant == 2) return launch_variant<KIND, W, R, WRAP, LO, true>(c, a, num_sms, st, grid_out, warps_out);
-    return launch_variant<KIND, W, R, WRAP, LO, false>(c, a, num_sms, st, grid_out, warps_out);
+            return launch_variant<KIND, W, R, WRAP, LO, false, true>(c, a, num_sms, st, grid_out, warps_out);
+    return launch_variant<KIND, W, R, WRAP, LO>(c, a, num_sms, st, grid_out, warps_out);
 }
 
 }  // namespace cfpair

@@ -229,6 +229,34 @@ bool build_lut(const std::vector<Seg> &segs, CfLut &L, std::vector<uint16_t> &wo
     return false;
 }
 
+// The pair kernel's table: equally wide cells of the separation itself, s = sqrt(v).  Cell i holds
+// the values whose product with `scale` rounds to i: s in [(i - 1/2) / scale, (i + 1/2) / scale], here
+// widened by 2^-20 of itself for the kernel's approximate square root (2^-22) and rounded product.  A
+// cell within one segment gets its bin, or nb outside every bin; a cell that any band or edge
+// touches gets nb + 1 (the kernel then asks the full tables).  Pairs of a catalogue crowd at the large
+// separations, where these cells are narrow against the bins: one in a thousand pairs falls into a
+// cell with an edge, against one in 250 with cells equally wide in the bit pattern of v.  The last cell
+// lies past the last edge; the kernel clamps there.  Cell 0 always goes to the full tables (the
+// kernel's square root takes denormals as 0).
+void build_lut8(const std::vector<Seg> &segs, int nb, std::vector<uint8_t> &lut, float &scale)
+{
+    auto root = [](uint32_t bits) {
+        float v;
+        std::memcpy(&v, &bits, 4);
+        return std::sqrt(std::min((double)v, 3.4028234663852886e38));
+    };
+    const double w = 1.0 / 1048576.0;
+    scale = (float)(CFI_LUT8_CELLS / root(segs.back().start));
+    const int last = (int)std::ceil(root(segs.back().start) * scale * (1 + w) + 0.5);
+    lut.assign(last + 1, (uint8_t)(nb + 1));
+    for (size_t k = 0; k < segs.size(); k++) {
+        if (segs[k].cls == CFI_CLS_AMB) continue;
+        const int lo = std::max(1, (int)std::ceil(root(segs[k].start) * scale * (1 + w) + 0.5));
+        const int hi = k + 1 == segs.size() ? last : (int)std::floor(root(segs[k + 1].start) * scale * (1 - w) - 0.5);
+        for (int i = lo; i <= hi && i <= last; i++) lut[i] = (uint8_t)(segs[k].cls == CFI_CLS_OUT ? nb : (int)segs[k].cls);
+    }
+}
+
 }  // namespace
 
 namespace {
@@ -484,18 +512,22 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
     // float64 inputs round to float32 (epsX), or keep a lo part when ravg is requested.
     const double u = U32;
     const bool precise = D.ravg;
+    double delta1[3];
     for (int a = 0; a < 3; a++) {
         double amax = D.ang ? 1.01 : std::max(std::fabs(G.lo[a]), std::fabs(G.lo[a] + extent[a]));
         double Q = ulp32_of_magnitude(std::max(amax, 1e-300));
         double M = D.ang ? Mang[a] : (G.wrap[a] ? (extent[a] + 2 * G.width[a]) : ((G.k[a] + 1) * G.width[a]));
         M = M * 1.001 + 4 * Q;
         double epsX = 0;
+        const double epsX1 = f64 ? u * (G.width[a] + 2 * Q) + 2 * U64 * amax : 0.0;
         if (f64) epsX = D.f64lo ? (2 * U64 * 2 * amax + u * u * (G.width[a] + 2 * Q)) : (u * (G.width[a] + 2 * Q) + 2 * U64 * amax);
         double wrapterm = G.wrap[a] ? u * G.L[a] : 0.0;
         double truth = 2 * U64 * (M + G.L[a] + amax);
         double delta;
+        // gathering forms separations without the low parts
+        delta1[a] = u * M + u * M + 2 * epsX1 + wrapterm + truth;
         if (precise) delta = 4 * u * u * M + 2 * epsX + wrapterm + truth;
-        else delta = u * M + u * M + 2 * epsX + wrapterm + truth;
+        else delta = delta1[a];
         H.delta[a] = delta;
         H.M[a] = M;
     }
@@ -516,9 +548,26 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
         for (int m = 0; m <= p->npibins; m++)
             H.band_p[m] = SAFETY * (H.theta_rel * D.pe[m] + H.delta[2] + 4 * U64 * D.pe[m]);
     }
+    // Gathering limits.  The kernel's t = s^2 - limit starts the chain at -limit, so each of its (at most
+    // three) roundings is up to u limit: a pair below the last edge e has t < 0 when
+    // limit >= e^2 + |error of s^2| + 3u limit; |dz| below pimax likewise.  The band of the largest
+    // edge for the plain separation (which carries the factor-4 margin) covers the first two terms.
+    auto ceil32 = [](double v) {
+        const uint32_t b = cfp_float_ceil_bits(v);
+        float f;
+        std::memcpy(&f, &b, 4);
+        return f;
+    };
+    const double reach2 = mocks ? D.smax2 : D.e2[D.nb];
+    D.reach_r = ceil32((reach2 + band_sq(reach2, naxes, u, delta1)) * (1.0 + 16 * u));
+    D.reach_p = 0.0f;
+    if (rppi_like) {
+        const double z = p->pimax + SAFETY * (u * p->pimax + delta1[2] + 4 * U64 * p->pimax);
+        D.reach_p = ceil32(z * z * (1.0 + 16 * u));
+    }
     H.eta = 0.0;
     D.near2 = 0.0f;
-    D.cut_su = 0.0f;
+    D.near_ss = 0.0f;
     if (mocks) {
         // Error model of the mocks kernel (Appendix A.2.1 evaluated in FP32).  Per pair: s from
         // the cell-relative coordinates (per-axis error <= delta, Dl2 its 2-norm), l = A_i - s/2
@@ -527,9 +576,8 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
         // near2 = S^2 goes to the FP64 recheck, so every other one has |l| >= 0.999 S and
         // |A_i| <= 1.51 |l|.  Both values divide
         // by l.l through one reciprocal (<= 2 ulp) and a product.
-        double Dl = 0.0, Dl2 = 0.0;
+        double Dl2 = 0.0;
         for (int a = 0; a < 3; a++) {
-            Dl += H.delta[a];
             Dl2 += H.delta[a] * H.delta[a];
         }
         Dl2 = std::sqrt(Dl2);
@@ -570,22 +618,13 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
             const double Sm = std::sqrt(rpm * rpm + D.pe[m]) * 1.001;
             H.band_p[m] = SAFETY * epi(std::sqrt(D.pe[m]) * 1.0001 + 1e-300, Sm, rpm) + truth * Sm * Sm;
         }
-        // Candidate cuts in the multiplied form (s.s - cut_r) l.l < (s.l)^2 < cut_p l.l, loose by
-        // twice the error of that form: s.s (input error, the chain from -cut_r), pi^2 as above
-        // with the full |s| in place of rp, and the form's own roundings.
-        const double Cbound = 1.1 * S2;
+        // |s.s - its FP32 value| for |s| <= Sx
+        double Dl = 0.0;
+        for (int a = 0; a < 3; a++) Dl += H.delta[a];
         auto ess = [&](double Sx) {
             const double a = Sx + Dl;
-            return 2 * Sx * Dl + Dl * Dl + 3 * u * (Cbound + a * a) + u * a * a;
+            return 2 * Sx * Dl + Dl * Dl + 3 * u * a * a;
         };
-        const double Smax = S * 1.001;
-        const double ecut = ess(Smax) + epi(p->pimax * 1.001, Smax, Smax) + u * (D.e2[D.nb] + S2);
-        const double Cr = D.e2[D.nb] + 2 * SAFETY * ecut + 8 * u * S2;
-        const double Cp = pm2 + 2 * H.band_p[p->npibins] + 8 * u * pm2;
-        D.cut_r = (float)Cr;
-        if ((double)D.cut_r < Cr) D.cut_r = std::nextafter(D.cut_r, INFINITY);
-        D.cut_p = (float)Cp;
-        if ((double)D.cut_p < Cp) D.cut_p = std::nextafter(D.cut_p, INFINITY);
         // Near the observer: a candidate with |s| up to the stencil's reach may have a midpoint
         // within S of the origin unless every point is at least that far plus half the reach.
         double reach = 0.0;
@@ -601,11 +640,32 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
         }
         if (!(vmin - 0.5 * reach >= 1.01 * S)) {
             D.near2 = (float)S2;
-            // s.s - cut_r of a near candidate that may count: s.s <= S^2 (1 + 1e-4) + 2 ess(S)
-            const double su = S2 * (1 + 1e-4) + 2 * ess(S) - (double)D.cut_r;
-            D.cut_su = (float)su;
-            if ((double)D.cut_su < su) D.cut_su = std::nextafter(D.cut_su, INFINITY);
+            // s.s of a near candidate that may count
+            D.near_ss = ceil32(S2 * (1 + 1e-4) + 2 * ess(S));
         }
+    }
+    // ---- pi bins by multiplication ----
+    // t = fl(pi32 * pi_inv) is off the exact pi / width by the FP32 error of pi (the band of a pi edge
+    // over the width; mocks: the band of the squared edge over 2 pi, and sqrt's error) and by the
+    // roundings of pi_inv and of the product.  A t farther than pi_tol from every integer therefore lies
+    // in no band and in the bin floor(t); the others go through the table.
+    D.pi_inv = D.pi_n = D.pi_tol = 0.0f;
+    if (rppi_like || mocks) {
+        const int n = p->kind == CF_WP ? 1 : p->npibins;
+        const double w = p->pimax / n;
+        double off = 0.0;
+        for (int m = 1; m <= p->npibins; m++) {
+            double b = H.band_p[m];
+            if (mocks) {
+                // |sqrt(v) - p| for |v - p^2| <= b
+                const double q = std::sqrt(D.pe[m]);
+                b = b < D.pe[m] ? q - std::sqrt(D.pe[m] - b) : q;
+            }
+            off = std::max(off, b);
+        }
+        D.pi_n = (float)n;
+        D.pi_inv = (float)(n / p->pimax);
+        D.pi_tol = ceil32(1.01 * off / w + 16 * u * n);
     }
     // ---- lookup tables ----
     {
@@ -614,6 +674,9 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
             err = "bin edges too close together for the FP32 lookup table";
             return CF_ERR_ARG;
         }
+        build_lut8(segs, D.nb, H.lut8, D.lut8_scale);
+        D.nlut8 = (int)H.lut8.size();
+        H.lut8.resize((H.lut8.size() + 15) & ~(size_t)15, (uint8_t)D.nb);
     }
     if (rppi_like || mocks) {
         std::vector<double> pe(D.pe, D.pe + p->npibins + 1);
@@ -626,16 +689,6 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
             return CF_ERR_ARG;
         }
     }
-    // candidate cuts of the pair kernel's first phase: the FP32 value at which the final
-    // "outside every bin" segment of each table starts
-    if (!mocks) {
-        float f;
-        std::memcpy(&f, &D.lr.tail, 4);
-        D.cut_r = f;
-        if (rppi_like) std::memcpy(&f, &D.lp.tail, 4);
-        else f = INFINITY;
-        D.cut_p = f;
-    }
     D.nlut_words = (int)H.lut.size();
     D.nfine = (int)H.fine.size();
     return CF_OK;
@@ -646,8 +699,8 @@ uint32_t cfp_lut_class(const CfHostPlan &H, int which, uint32_t vb)
 {
     const CfLut &L = (which & 1) ? H.d.lp : H.d.lr;
     if (which & 2) {
-        // the direct pair kernel: an FP32 cut at the tail, then the lookup without upper clamp
-        // (lut_class_in in cf_pair.cuh); 0xFD flags an index past the table
+        // an FP32 cut at the tail, then the lookup without upper clamp; 0xFD flags an index past the
+        // table
         if (vb >= L.tail) return CFI_CLS_OUT;
         const uint32_t idx = (std::max(vb, L.base) - L.base) >> L.shift;
         if (idx > L.last) return 0xFDu;

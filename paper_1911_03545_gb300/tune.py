@@ -1,8 +1,7 @@
 """Autotuner for the pair-counting launch configuration.
 
 Knobs (all results are identical across them; only speed changes):
-  variant pair-kernel form: 1 bins every pair where it is formed, 2 compacts the candidates
-          of each lane into a per-warp ring first
+  variant accepted for stored configurations; the pair kernel has one form
   refine  sub-cells per Rmax cell (Sec. 4.2): 1, 2, 3
   warps   warps per CTA of the persistent pair kernel (CTA shape; occupancy follows from the
           shared-memory histograms): 0 (as many as fit), 12, 8, 6, 4
@@ -44,7 +43,7 @@ MARGIN = 0.01
 
 def knobs_for(p, block: bool = False) -> dict:
     """The knobs that can change anything for this kind: the angular grid exists for DD(theta)
-    only, and the mocks kind has the direct form only."""
+    only, and the mocks kind has no form to choose."""
     k = dict(KNOBS)
     if p.kind != CF_DD_THETA:
         k.pop("thetagrid")

@@ -1,0 +1,58 @@
+"""The pair kernel's gathering step at the sizes where it can go wrong: group and block edges (32), the
+padding to a multiple of four, ranges of which nothing or everything is within reach, cells paired with
+themselves, every kind, counts only and with sums (counts bit-exact, sums to 1e-6 as everywhere)."""
+import numpy as np
+import pytest
+
+import gen
+from tests.gpu_util import assert_match, gpu_count, oracle_count
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    c = cf.cf_create(0, torch.cuda.current_stream())
+    yield c
+    cf.cf_destroy(c)
+
+
+def _groups(n, seed, centre, dtype):
+    """n points in each of three tight groups: two within reach of each other, one in the next cell but
+    mostly out of reach, interleaved so that kept and dropped points alternate along a cell."""
+    r = np.random.Generator(np.random.PCG64(seed))
+    c = np.array(centre)[:, None] + np.array([[0.0, 3.0, 7.5], [0.0, 1.0, 6.0], [0.0, -2.0, 5.0]])
+    p = c[:, None, :] + r.normal(0.0, 0.6, size=(3, n, 3))
+    p = p.reshape(3, -1).astype(dtype)
+    w = r.uniform(0.5, 1.5, p.shape[1]).astype(dtype)
+    return gen.Catalogue(p[0].copy(), p[1].copy(), p[2].copy(), w)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 31, 32, 33, 63, 65, 100, 171])
+@pytest.mark.parametrize("kind", ["r", "rppi", "wp", "theta", "mocks"])
+def test_gathered_blocks(ctx, kind, n):
+    for sums, dtype in ((False, np.float32), (True, np.float32), (True, np.float64)):
+        edges = gen.log_edges(0.05, 8.0, 9)
+        kw = dict(periodic=False, weighted=sums, ravg=sums)
+        centre = (20.0, 20.0, 20.0)
+        if kind == "theta":
+            edges = gen.log_edges(0.2, 14.0, 9)
+        if kind == "mocks":
+            centre = (70.0, 60.0, 80.0)
+        if kind in ("rppi", "wp"):
+            kw.update(periodic=True, box=40.0)
+        if kind in ("rppi", "wp", "mocks"):
+            kw.update(pimax=6.0, npibins=7)
+        d1, d2 = _groups(n, 100 + n, centre, dtype), _groups(2 * n + 1, 200 + n, centre, dtype)
+        if kind == "theta":
+            for d in (d1, d2):
+                r = np.sqrt(d.x.astype(np.float64) ** 2 + d.y.astype(np.float64) ** 2 + d.z.astype(np.float64) ** 2)
+                d.x, d.y, d.z = ((v / r).astype(dtype) for v in (d.x, d.y, d.z))
+        for auto in (True, False):
+            got = gpu_count(ctx, kind, edges, d1, None if auto else d2, autocorr=auto, **kw)
+            exp = oracle_count(kind, edges, d1, None if auto else d2, autocorr=auto, mode="brute", **kw)
+            assert_match(got, exp, sums, sums)
