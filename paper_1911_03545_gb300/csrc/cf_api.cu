@@ -748,6 +748,23 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     A.nb = D.nb;
     A.npi = D.npi;
     A.nslot = D.nslot;
+    auto twice = [](float v) {
+        uint32_t b;
+        std::memcpy(&b, &v, 4);
+        return (uint64_t)b << 32 | b;
+    };
+    A.lut_scale2 = twice(D.lut8_scale);
+    A.pi_inv2 = twice(D.pi_inv);
+    A.nlut8 = (uint32_t)D.nlut8;
+    A.lut_top = 0x4B000000u + A.nlut8 - 1u;
+    A.reach_r = D.reach_r;
+    A.reach_p = D.reach_p;
+    A.pi_half = 0.5f - D.pi_tol;
+    A.pi_top = 0x4B000000u + (uint32_t)D.pi_n;
+    A.near2 = D.near2;
+    A.near_ss = D.near_ss;
+    A.lr = D.lr;
+    A.lp = D.lp;
     // rp-pi / mocks keep one histogram per warp in shared memory; when even one warp's does not
     // fit (many rp x pi slots, weights), they add straight into the global histograms instead
     const bool per_warp = D.kind == CF_DD_RPPI || D.kind == CF_DD_RPPI_MOCKS;

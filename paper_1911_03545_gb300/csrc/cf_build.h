@@ -71,6 +71,14 @@ struct CfPairArgs {
     unsigned long long *qcount;  // queued pairs, 64-bit so that it cannot wrap (entries >= qcap are dropped)
     float L[3];                  // periodic sides (wrap axes)
     int nb, npi, nslot;
+    // the plan's constants (CfDevPlan) as kernel parameters: constant operands instead of registers
+    uint64_t lut_scale2;         // lut8_scale, pi_inv in both halves of a packed pair
+    uint64_t pi_inv2;
+    uint32_t nlut8, lut_top;     // cells of lut8, and the bits of 2^23 + the last one's index
+    float reach_r, reach_p, near2, near_ss;
+    float pi_half;               // 1/2 - pi_tol: a fraction of pi / width farther from 1/2 may lie near a pi edge
+    uint32_t pi_top;             // bits of 2^23 + the number of pi bins
+    CfLut lr, lp;
     int ghist;                   // 1: rp-pi / mocks add straight into hcnt/hw/hr (global atomics):
                                  // their per-warp histogram does not fit in shared memory
     float fxw;                   // rp-pi / mocks per-warp weight sums in fixed point (two 32-bit words

@@ -16,6 +16,12 @@ __device__ __forceinline__ u64 f2_add(u64 a, u64 b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+__device__ __forceinline__ u64 f2_add_rm(u64 a, u64 b)      // rounded down
+{
+    u64 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 __device__ __forceinline__ u64 f2_sub(u64 a, u64 b)
 {
     u64 r;
@@ -44,6 +50,29 @@ __device__ __forceinline__ float f2_lo(u64 v) { return __uint_as_float((uint32_t
 __device__ __forceinline__ float f2_hi(u64 v) { return __uint_as_float((uint32_t)(v >> 32)); }
 __device__ __forceinline__ uint32_t f2_lo_bits(u64 v) { return (uint32_t)v; }
 __device__ __forceinline__ uint32_t f2_hi_bits(u64 v) { return (uint32_t)(v >> 32); }
+
+// ---- asynchronous global -> shared copy of 16 bytes, grouped and awaited ----
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// minimum / maximum over the warp; NaN lanes drop out
+__device__ __forceinline__ float cf_redux_min(float v)
+{
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float cf_redux_max(float v)
+{
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
 
 // sqrt.approx.f32: relative error within a few ulp; used only for ravg sums (1e-6 tolerance)
 __device__ __forceinline__ float f_sqrt_approx(float x)

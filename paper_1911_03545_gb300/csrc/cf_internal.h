@@ -22,7 +22,8 @@
 #define CFI_MAX_STENCIL 4096
 #define CFI_LUT_MAX 8192          // coarse LUT cells (2 B each)
 #define CFI_LUT_TARGET 4096       // preferred coarse cells per table
-#define CFI_LUT8_CELLS 8192       // cells of the pair kernel's separation table below the last edge
+#define CFI_LUT8_CELLS 16384      // cells of the pair kernel's separation table below the last edge
+#define CFI_LUT8_CELLS_SUMS 8192  // the same with weights or ravg, whose histograms fill shared memory
 #define CFI_FINE_MAX 1024         // fine LUT entries (16 B each)
 #define CFI_CLS_OUT 0xFEu         // class: outside every bin
 #define CFI_CLS_AMB 0xFFu         // class: within the FP32 error band of an edge
@@ -137,9 +138,9 @@ struct CfDevPlan {
                            // rp-pi / wp: rp^2) formed without the shift's low part: above the largest
                            // one that may count by that form's FP32 error
     float reach_p;         // the same on dz^2 (rp-pi / wp)
-    float pi_inv, pi_n;    // rp-pi / wp / mocks: t = pi * pi_inv counts pi bins of equal width, pi_n of them
-                           // (wp: one)
-    float pi_tol;          // a t within this of an integer may lie in the FP32 band of a pi edge
+    int pi_n;              // rp-pi / wp / mocks: pi bins, all of one width (wp: one bin)
+    float pi_inv;          // 1 / that width: bin floor(pi * pi_inv)
+    float pi_tol;          // a pi * pi_inv within this of an integer may lie in the FP32 band of a pi edge
     float near2;           // mocks: a candidate whose FP32 l.l is below this goes to the FP64
                            // recheck when its s.s is below near_ss (0: no candidate can be)
     float near_ss;

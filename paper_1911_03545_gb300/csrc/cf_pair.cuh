@@ -58,7 +58,8 @@ __host__ __device__ constexpr bool warp_hist(int kind) { return kind == KIND_RPP
 
 __host__ __device__ __forceinline__ uint32_t align16(uint32_t x) { return (x + 15u) & ~15u; }
 
-// per-warp shared memory: gathered j points | histogram
+// per-warp shared memory: (counts only) two work items, the current and the next | gathered j points |
+// histogram
 //   gathered points: a ring of GBUF points as 3-7 float arrays (x, y, z[, w][, lo parts of x, y, z])
 //   and the points' places in the j range (u16)
 // a warp flushes its histograms once it has evaluated more than this many pairs of one job;
@@ -76,6 +77,13 @@ __device__ __forceinline__ unsigned long long fx_sum(uint32_t lo, uint32_t hi)
     return c + (uint32_t)(lo - (uint32_t)c);
 }
 constexpr uint32_t GBUF = 64;
+// bits of 2^23: a value below 2^22 added to it has its integer part in the low bits of the sum
+constexpr uint32_t MAGIC_BITS = 0x4B000000u;
+// Counts-only instances run 32 warps per SM on 64 registers: they keep the work item and the next one in
+// shared memory (24 registers otherwise).  The others have the registers and need the shared memory.
+__host__ __device__ constexpr bool smem_items(bool W, bool R) { return !W && !R; }
+__host__ __device__ constexpr uint32_t item_bytes(bool W, bool R) { return smem_items(W, R) ? 2u * sizeof(CfItem) : 0u; }
+static_assert(sizeof(CfItem) % 16 == 0, "items are copied 16 bytes at a time");
 // Histogram rows past the bins: a separation outside every bin reads class nb, one that the full tables
 // must decide class nb + 1.  Counts-only kinds add there as well instead of testing (lane-private rows; one
 // word per lane past a per-warp histogram), and nothing reads those rows.
@@ -97,10 +105,21 @@ __host__ __device__ constexpr bool has_z(int kind) { return kind == KIND_RPPI ||
 // kinds that bin a second value (|dz|; for mocks pi^2)
 __host__ __device__ constexpr bool has_pi(int kind) { return has_z(kind) || kind == KIND_MOCKS; }
 __host__ __device__ constexpr uint32_t stage_arrays(bool W, bool LO) { return LO ? 7u : (W ? 4u : 3u); }
-__host__ __device__ constexpr uint32_t warp_jbuf_bytes(bool W, bool LO) { return stage_arrays(W, LO) * GBUF * 4u + GBUF * 2u; }
+__host__ __device__ constexpr uint32_t warp_jbuf_bytes(bool W, bool R, bool LO)
+{
+    return item_bytes(W, R) + stage_arrays(W, LO) * GBUF * 4u + GBUF * 2u;
+}
 __host__ __device__ __forceinline__ uint32_t warp_bytes(int kind, bool W, bool R, bool LO, int nslot)
 {
-    return warp_jbuf_bytes(W, LO) + warp_hist_bytes(kind, W, R, nslot);
+    return warp_jbuf_bytes(W, R, LO) + warp_hist_bytes(kind, W, R, nslot);
+}
+
+// per-CTA shared memory past the separation table: the ravg scales per rp bin (rp-pi, mocks), or the
+// spare row of the sums of the other kinds (a count, and two Kahan pairs at most, per lane)
+__host__ __device__ __forceinline__ uint32_t cta_extra_bytes(int kind, bool W, bool R, int nb)
+{
+    if (warp_hist(kind)) return align16(4u * (uint32_t)nb);
+    return W || R ? 32u * 20u : 0u;
 }
 
 // Kahan-compensated FP32 sum: s holds the sum, c the negated lost low part
@@ -132,19 +151,6 @@ __device__ __forceinline__ uint32_t lut_class(const uint16_t *__restrict__ words
     return c;
 }
 
-// minimum / maximum over the warp; NaN lanes drop out
-__device__ __forceinline__ float f_redux_min(float v)
-{
-    float r;
-    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ float f_redux_max(float v)
-{
-    float r;
-    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
 __device__ __forceinline__ float f_rcp_approx(float x)
 {
     float r;
@@ -245,68 +251,68 @@ static __device__ __noinline__ float mocks_rp(const CfPairArgs &a, uint32_t ip, 
 template <int KIND, bool W, bool R, bool WRAP, bool LO, bool GH, bool FX>
 struct Warp {
     const CfPairArgs &a;
-    const CfLut &lr, &lp;   // the full tables' shapes
-    uint32_t lut;           // separation table in shared memory: its address, less the bits of 2^23
-    uint32_t lut_top;       // bits of 2^23 + the index of its last cell (outside every bin)
-    float lut_scale;        // cells per unit of separation
+    uint32_t lut;           // separation table in shared memory: its address, less MAGIC_BITS
     uint32_t *h_cnt;        // lane-private [nslot][32] (this and the sums: at the lane's column) or
                             // per-warp [nslot]
-    float2 *h_w, *h_r;      // lane-private Kahan pairs (interleaved when both are kept)
+    float2 *h_w;            // lane-private Kahan pairs of the sum kept (interleaved when both are)
+    uint32_t *d_cnt;        // the CTA's spare row: count and sums nobody reads
+    float2 *d_w;
     double *h_wd, *h_rd;    // per-warp sums (rp-pi, mocks): FP64, or with FX two 32-bit words per slot
                             // (nslot low words, then nslot high words)
     const float *fxr_bin;   // with FX and ravg: the scale of each rp bin's ravg terms (shared memory)
     float *jst;             // gathered j points
     uint16_t *gj;           // their places in the j range
-    int lane, nb, npi, nslot;
-    uint32_t jbeg, job;
-    float reach_r, reach_p; // the gathering limits (see CfDevPlan)
-    float pi_inv, pi_n, pi_tol;     // 1 / pi bin width, pi bins, distance from an edge below which the table decides
+    int lane;
     float Lx, Ly, Lz, iLx, iLy, iLz;
-    float near2, near_ss;   // mocks: the near-observer test (near2 = 0: off)
 
-    __device__ Warp(const CfPairArgs &args) : a(args), lr(args.plan->lr), lp(args.plan->lp) {}
+    __device__ Warp(const CfPairArgs &args) : a(args) {}
 
     // index of a gathered point among the sorted points
-    __device__ __forceinline__ uint32_t gidx(const float *bs, uint32_t k) const { return jbeg + gj[(bs - jst) + k]; }
+    __device__ __forceinline__ uint32_t gidx(const CfItem &it, const float *bs, uint32_t k) const
+    {
+        return it.jbeg + gj[(bs - jst) + k];
+    }
+    static __device__ __forceinline__ uint32_t job(const CfItem &it) { return it.meta & CFI_ITEM_JOBMASK; }
 
     // Table classes of two separations (bin; nb: outside every bin; nb + 1: for the full tables to decide).
     // The cell is the separation times lut_scale, rounded to an integer by adding 2^23; values past the
     // table and NaN clamp to its last cell.
     __device__ __forceinline__ void lut2(float r0, float r1, uint32_t &c0, uint32_t &c1) const
     {
-        const u64 n = f2_fma(f2_pack(r0, r1), f2_pack(lut_scale, lut_scale), f2_pack(8388608.0f, 8388608.0f));
-        c0 = lds_u8(lut + min(f2_lo_bits(n), lut_top));
-        c1 = lds_u8(lut + min(f2_hi_bits(n), lut_top));
+        const u64 n = f2_fma(f2_pack(r0, r1), a.lut_scale2, f2_pack(8388608.0f, 8388608.0f));
+        c0 = lds_u8(lut + min(f2_lo_bits(n), a.lut_top));
+        c1 = lds_u8(lut + min(f2_hi_bits(n), a.lut_top));
     }
 
-    __device__ __forceinline__ void push(uint32_t ip, uint32_t jp) { push_recheck(a, ip, jp, job); }
+    __device__ __forceinline__ void push(const CfItem &it, uint32_t ip, uint32_t jp) { push_recheck(a, ip, jp, job(it)); }
 
-    __device__ __forceinline__ void acc_lp(uint32_t c, float r, float wp)
+    // Add to a lane's histogram of r, theta or wp, in bin c where `in` holds and in the CTA's spare row
+    // otherwise (no branch: the four pairs' chains overlap)
+    __device__ __forceinline__ void add_lane(bool in, uint32_t c, float r, float wp)
     {
         const uint32_t idx = c * 32u;       // the histogram pointers carry the lane
-        atomicAdd(h_cnt + idx, 1u);
+        atomicAdd(in ? h_cnt + idx : d_cnt, 1u);
         if (R && KIND == KIND_THETA) r = 2.0f * asinf(0.5f * r) * 57.29577951308232f;
         if (W && R) {
             // both sums of a lane's bin sit in one 16-byte word (sums, then their compensations): one load,
             // one packed compensated step, one store
-            ulonglong2 *p = reinterpret_cast<ulonglong2 *>(h_w) + idx;
+            ulonglong2 *p = reinterpret_cast<ulonglong2 *>(in ? h_w + 2u * idx : d_w);
             ulonglong2 v = *p;
             const u64 y = f2_sub(f2_pack(wp, __fmul_rn(wp, r)), v.y);
             const u64 t = f2_add(v.x, y);
             v.y = f2_sub(f2_sub(t, v.x), y);
             v.x = t;
             *p = v;
-        } else {
-            if (W) kahan_add(h_w + idx, wp);
-            if (R) kahan_add(h_r + idx, r);
+        } else if (W || R) {
+            kahan_add(in ? h_w + idx : d_w, W ? wp : r);
         }
     }
 
-    __device__ __forceinline__ void acc_sh(uint32_t slot, uint32_t rbin, float r, float wp)
+    __device__ __forceinline__ void acc_sh(const CfItem &it, uint32_t slot, uint32_t rbin, float r, float wp)
     {
         if (GH) {
             // no per-warp histogram: straight into the job's global one
-            const size_t g = (size_t)job * (uint32_t)nslot + slot;
+            const size_t g = (size_t)job(it) * (uint32_t)a.nslot + slot;
             atomicAdd(a.hcnt + g, 1ull);
             if (W) atomicAdd(a.hw + g, (double)wp);
             if (R) atomicAdd(a.hr + g, (double)(W ? wp * r : r));
@@ -325,7 +331,7 @@ struct Warp {
             uint32_t *w = reinterpret_cast<uint32_t *>(h);
             const uint32_t m = __float2uint_rn(t * scale);
             atomicAdd(w + slot, m);
-            atomicAdd(w + nslot + slot, m >> FX_HI_SHIFT);
+            atomicAdd(w + a.nslot + slot, m >> FX_HI_SHIFT);
         } else {
             atomicAdd(h + slot, (double)t);
         }
@@ -388,12 +394,13 @@ struct Warp {
     {
         const float wp = W ? __fmul_rn(I.w, wj) : 0.f;
         if (KIND == KIND_MOCKS) {
-            if (R) r = mocks_rp<LO>(a, I.p, bj, it.s[0], it.s[1], it.s[2], it.slo[0], it.slo[1], it.slo[2]);
-            acc_sh(cr * (uint32_t)npi + cz, cr, r, wp);
+            if (R) r = mocks_rp<LO>(a, I.p, bj, it.s[0], it.s[1], it.s[2], it.slo[0], it.slo[1],
+                                     it.slo[2]);
+            acc_sh(it, cr * (uint32_t)a.npi + cz, cr, r, wp);
         } else if (KIND == KIND_RPPI) {
-            acc_sh(cr * (uint32_t)npi + cz, cr, r, wp);
+            acc_sh(it, cr * (uint32_t)a.npi + cz, cr, r, wp);
         } else {
-            acc_lp(cr, r, wp);
+            add_lane(true, cr, r, wp);
         }
     }
 
@@ -446,13 +453,13 @@ struct Warp {
                 const u64 r = f2_pack(f_rcp_approx(f2_lo(ll)), f_rcp_approx(f2_hi(ll)));
                 q[h] = f2_mul(c2, r);
                 z[h] = f2_mul(f2_mul(sl, sl), r);
-                if (near2 > 0.f) {
+                if (a.near2 > 0.f) {
                     // a midpoint near the observer, where the error bounds do not hold: FP64 when its
                     // s.s may count
                     const u64 ss = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
-                    const bool n0 = f2_lo(ll) < near2, n1 = f2_hi(ll) < near2;
-                    if (n0 && f2_lo(ss) < near_ss && (!dg || j4 + 2 * h >= skip)) push(I.p, gidx(bs, j4 + 2 * h));
-                    if (n1 && f2_hi(ss) < near_ss && (!dg || j4 + 2 * h + 1 >= skip)) push(I.p, gidx(bs, j4 + 2 * h + 1));
+                    const bool n0 = f2_lo(ll) < a.near2, n1 = f2_hi(ll) < a.near2;
+                    if (n0 && f2_lo(ss) < a.near_ss && (!dg || j4 + 2 * h >= skip)) push(it, I.p, gidx(it, bs, j4 + 2 * h));
+                    if (n1 && f2_hi(ss) < a.near_ss && (!dg || j4 + 2 * h + 1 >= skip)) push(it, I.p, gidx(it, bs, j4 + 2 * h + 1));
                     const float nan = CUDART_NAN_F;
                     q[h] = f2_pack(n0 ? nan : f2_lo(q[h]), n1 ? nan : f2_hi(q[h]));
                 }
@@ -468,49 +475,48 @@ struct Warp {
             for (int h = 0; h < 4; h++) v2[h] = j4 + h < skip ? CUDART_NAN_F : v2[h];
         }
         uint32_t c[4], cz[4] = {0u, 0u, 0u, 0u};
-        float r4[4], T[4] = {0.f, 0.f, 0.f, 0.f}, F[4] = {1.f, 1.f, 1.f, 1.f};
+        float r4[4];
 #pragma unroll
         for (int h = 0; h < 4; h++) r4[h] = f_sqrt_ftz(v2[h]);
         lut2(r4[0], r4[1], c[0], c[1]);
         lut2(r4[2], r4[3], c[2], c[3]);
+        float F[4] = {0.f, 0.f, 0.f, 0.f};
         if (has_pi(KIND)) {
-            // the pi bins are equally wide: t = pi / width, its nearest integer by the 2^23 trick, and the
-            // distance from it, which also says whether a pi edge is near
-            const u64 MAGIC = f2_pack(8388608.0f, 8388608.0f);
+            // the pi bins are equally wide: with t = pi / width, t + 2^23 rounded down holds the bin in its
+            // low bits, and the fraction's distance from 1/2 says whether a pi edge is near
+            const u64 MAGIC = f2_pack(8388608.0f, 8388608.0f), HALF = f2_pack(-0.5f, -0.5f);
 #pragma unroll
             for (int h = 0; h < 2; h++) {
                 u64 p = z[h];
                 if (KIND == KIND_MOCKS) p = f2_pack(f_sqrt_ftz(f2_lo(p)), f_sqrt_ftz(f2_hi(p)));
-                const u64 t = f2_mul(p, f2_pack(pi_inv, pi_inv));
-                const u64 n = f2_add(t, MAGIC);
-                const u64 f = f2_sub(t, f2_sub(n, MAGIC));
-                T[2 * h] = f2_lo(t);
-                T[2 * h + 1] = f2_hi(t);
+                const u64 t = f2_mul(p, a.pi_inv2);
+                const u64 n = f2_add_rm(t, MAGIC);
+                const u64 f = f2_add(f2_sub(t, f2_sub(n, MAGIC)), HALF);
                 F[2 * h] = f2_lo(f);
                 F[2 * h + 1] = f2_hi(f);
-                cz[2 * h] = (f2_lo_bits(n) - 0x4B000000u) + (uint32_t)((int)f2_lo_bits(f) >> 31);
-                cz[2 * h + 1] = (f2_hi_bits(n) - 0x4B000000u) + (uint32_t)((int)f2_hi_bits(f) >> 31);
+                cz[2 * h] = f2_lo_bits(n);
+                cz[2 * h + 1] = f2_hi_bits(n);
             }
         }
-        bool odd = max(max(c[0], c[1]), max(c[2], c[3])) > (uint32_t)nb;
-        if (has_pi(KIND)) odd = odd || fminf(fminf(fabsf(F[0]), fabsf(F[1])), fminf(fabsf(F[2]), fabsf(F[3]))) < pi_tol;
+        bool odd = max(max(c[0], c[1]), max(c[2], c[3])) > (uint32_t)a.nb;
+        if (has_pi(KIND)) odd = odd || fmaxf(fmaxf(fabsf(F[0]), fabsf(F[1])), fmaxf(fabsf(F[2]), fabsf(F[3]))) > a.pi_half;
         if (odd) {
             // a table cell with an edge in it or a value near a pi edge (one pair in a thousand): the full
             // tables decide, and what they call ambiguous goes to the FP64 recheck
             uint32_t todo = 0;
 #pragma unroll
             for (int h = 0; h < 4; h++) {
-                const bool d = c[h] > (uint32_t)nb || (has_pi(KIND) && c[h] < (uint32_t)nb && fabsf(F[h]) < pi_tol);
+                const bool d = c[h] > (uint32_t)a.nb || (has_pi(KIND) && c[h] < (uint32_t)a.nb && fabsf(F[h]) > a.pi_half);
                 todo |= (d ? 1u : 0u) << h;
-                c[h] = d ? (uint32_t)nb : c[h];
+                c[h] = d ? (uint32_t)a.nb : c[h];
             }
             const float z4[4] = {f2_lo(z[0]), f2_hi(z[0]), f2_lo(z[1]), f2_hi(z[1])};
             for (; todo; todo &= todo - 1u) {
                 const int h = __ffs(todo) - 1;
-                const uint32_t kr = lut_class(a.lut, a.fine, lr, __float_as_uint(pick4(v2, h)));
-                const uint32_t kz = has_pi(KIND) ? lut_class(a.lut, a.fine, lp, __float_as_uint(pick4(z4, h))) : 0u;
+                const uint32_t kr = lut_class(a.lut, a.fine, a.lr, __float_as_uint(pick4(v2, h)));
+                const uint32_t kz = has_pi(KIND) ? lut_class(a.lut, a.fine, a.lp, __float_as_uint(pick4(z4, h))) : 0u;
                 if (kr == CFI_CLS_OUT || kz == CFI_CLS_OUT) continue;
-                if (max(kr, kz) == CFI_CLS_AMB) push(I.p, gidx(bs, j4 + h));
+                if (max(kr, kz) == CFI_CLS_AMB) push(it, I.p, gidx(it, bs, j4 + h));
                 else add_pair(it, I, kr, kz, R ? f_sqrt_approx(pick4(v2, h)) : 0.f, W ? b[3 * GBUF + h] : 0.f, b + h);
             }
         }
@@ -521,28 +527,42 @@ struct Warp {
         }
 #pragma unroll
         for (int h = 0; h < 4; h++) {
-            bool in = c[h] < (uint32_t)nb;
-            if (has_pi(KIND)) in = in && T[h] < pi_n;
-            if (W || R || GH) {
-                if (in) add_pair(it, I, c[h], cz[h], r4[h], wj[h], b + h);
+            bool in = c[h] < (uint32_t)a.nb;
+            if (has_pi(KIND)) in = in && cz[h] < a.pi_top;
+            const uint32_t kz = cz[h] - MAGIC_BITS;
+            if ((W || R) && !warp_hist(KIND)) {
+                add_lane(in, c[h], r4[h], W ? __fmul_rn(I.w, wj[h]) : 0.f);
+            } else if (W || R || GH) {
+                if (in) add_pair(it, I, c[h], kz, r4[h], wj[h], b + h);
             } else if (KIND == KIND_RPPI || KIND == KIND_MOCKS) {
-                atomicAdd(h_cnt + (in ? c[h] * (uint32_t)npi + cz[h] : (uint32_t)(nslot + lane)), 1u);
+                atomicAdd(h_cnt + (in ? c[h] * (uint32_t)a.npi + kz : (uint32_t)(a.nslot + lane)), 1u);
             } else if (KIND == KIND_WP) {
-                atomicAdd(h_cnt + (in ? c[h] : (uint32_t)nb) * 32u, 1u);
+                atomicAdd(h_cnt + (in ? c[h] : (uint32_t)a.nb) * 32u, 1u);
             } else {
                 atomicAdd(h_cnt + c[h] * 32u, 1u);
             }
         }
     }
 
+    // Whether a separation of at least (gx, gy, gz) per axis (negative: 0) may count.  Every operation from
+    // the boxes on rounds monotonically, so what fails here holds no pair below the limit.
+    __device__ __forceinline__ bool within(float gx, float gy, float gz) const
+    {
+        gx = fmaxf(gx, 0.f);
+        gy = fmaxf(gy, 0.f);
+        gz = fmaxf(gz, 0.f);
+        float t = fmaf(gy, gy, fmaf(gx, gx, -a.reach_r));
+        if (has_z(KIND)) return t < 0.f && fmaf(gz, gz, -a.reach_p) < 0.f;
+        t = fmaf(gz, gz, t);
+        return t < 0.f;
+    }
+
     // One work item: its i tile in groups of 32 points; for each the j points within reach of the
     // group's bounding box are gathered in shared memory and counted 32 at a time.
     __device__ __forceinline__ void run(const CfItem &it)
     {
-        const uint32_t icnt = it.cnt & 0xFFFFu, jcnt = it.cnt >> 16;
+        const uint32_t icnt = it.cnt & 0xFFFFu, jcnt = it.cnt >> 16, jbeg = it.jbeg;
         const bool diag = (it.meta & CFI_ITEM_DIAG) != 0;
-        job = it.meta & CFI_ITEM_JOBMASK;
-        jbeg = it.jbeg;
         const uint32_t upto = 0xFFFFFFFFu >> (31 - lane);       // the lanes up to this one
 #pragma unroll 1
         for (uint32_t i0 = 0; i0 < icnt; i0 += 32u) {
@@ -559,8 +579,8 @@ struct Warp {
             float lo[3], hi[3];     // the group's box; the NaN of an empty lane drops out
 #pragma unroll
             for (int d = 0; d < 3; d++) {
-                lo[d] = f_redux_min(f2_lo(I.s[d]));
-                hi[d] = f_redux_max(f2_lo(I.s[d]));
+                lo[d] = cf_redux_min(f2_lo(I.s[d]));
+                hi[d] = cf_redux_max(f2_lo(I.s[d]));
             }
             // head: where the block to count next starts in the ring (0 or 32); fill: points gathered there
             uint32_t head = 0, fill = 0, skip = 0;
@@ -569,7 +589,7 @@ struct Warp {
 #pragma unroll 1
                 while (fill < 32u && j0 < jcnt) {
                     const float4 C = P, E = Q;
-                    const bool live = j0 + lane < jcnt;
+                    const uint32_t j = j0 + lane;
                     j0 += 32u;
                     pj += 32;
                     if (LO) lj += 32;
@@ -577,19 +597,10 @@ struct Warp {
                         P = *pj;
                         if (LO) Q = *lj;
                     }
-                    bool keep = live;
-                    if (!WRAP) {
-                        // the smallest separation a point of the group can have from this j point:
-                        // each operation rounds monotonically, so a point is only dropped when all 32
-                        // pairs lie past the limit
-                        const float gx = fmaxf(fmaxf(lo[0] + C.x, -hi[0] - C.x), 0.f);
-                        const float gy = fmaxf(fmaxf(lo[1] + C.y, -hi[1] - C.y), 0.f);
-                        const float gz = fmaxf(fmaxf(lo[2] + C.z, -hi[2] - C.z), 0.f);
-                        float t = fmaf(gy, gy, fmaf(gx, gx, -reach_r));
-                        if (has_z(KIND)) keep = keep && fmaf(gz, gz, -reach_p) < 0.f;
-                        else t = fmaf(gz, gz, t);
-                        keep = keep && t < 0.f;
-                    }
+                    bool keep = j < jcnt;
+                    if (!WRAP)
+                        keep = keep && within(fmaxf(lo[0] + C.x, -hi[0] - C.x), fmaxf(lo[1] + C.y, -hi[1] - C.y),
+                                              fmaxf(lo[2] + C.z, -hi[2] - C.z));
                     const uint32_t m = __ballot_sync(CF_FULL, keep);
                     const uint32_t rank = __popc(m & upto);
                     if (keep) {
@@ -604,7 +615,7 @@ struct Warp {
                             q[5 * GBUF] = E.y;
                             q[6 * GBUF] = E.z;
                         }
-                        gj[k] = (uint16_t)(j0 - 32u + lane);
+                        gj[k] = (uint16_t)j;
                     }
                     // in a cell paired with itself the group's own points come first: those up to lane i
                     // (i itself among them) do not count for it
@@ -630,8 +641,8 @@ struct Warp {
     {
         if (GH) return;         // nothing held per warp
         __syncwarp();
-        const size_t g0 = (size_t)jb * nslot;
-        for (int sl = lane; sl < nslot; sl += 32) {
+        const size_t g0 = (size_t)jb * a.nslot;
+        for (int sl = lane; sl < a.nslot; sl += 32) {
             unsigned long long c = 0;
             double ws = 0.0, rs = 0.0;
             if (warp_hist(KIND)) {
@@ -640,8 +651,8 @@ struct Warp {
                 if (W) {
                     if (FX) {
                         uint32_t *w = reinterpret_cast<uint32_t *>(h_wd);
-                        ws = (double)fx_sum(w[sl], w[nslot + sl]) * a.ifxw;
-                        w[sl] = w[nslot + sl] = 0u;
+                        ws = (double)fx_sum(w[sl], w[a.nslot + sl]) * a.ifxw;
+                        w[sl] = w[a.nslot + sl] = 0u;
                     } else {
                         ws = h_wd[sl];
                         h_wd[sl] = 0.0;
@@ -650,8 +661,8 @@ struct Warp {
                 if (R) {
                     if (FX) {
                         uint32_t *w = reinterpret_cast<uint32_t *>(h_rd);
-                        rs = (double)fx_sum(w[sl], w[nslot + sl]) / (double)fxr_bin[sl / npi];
-                        w[sl] = w[nslot + sl] = 0u;
+                        rs = (double)fx_sum(w[sl], w[a.nslot + sl]) / (double)fxr_bin[sl / a.npi];
+                        w[sl] = w[a.nslot + sl] = 0u;
                     } else {
                         rs = h_rd[sl];
                         h_rd[sl] = 0.0;
@@ -669,7 +680,7 @@ struct Warp {
                         rs += (double)v.y - (double)v.w;
                         *q = make_float4(0.f, 0.f, 0.f, 0.f);
                     } else if (W || R) {
-                        float2 *q = (W ? h_w : h_r) + idx;
+                        float2 *q = h_w + idx;
                         const float2 v = *q;
                         (W ? ws : rs) += (double)v.x - (double)v.y;
                         *q = make_float2(0.f, 0.f);
@@ -689,7 +700,7 @@ struct Warp {
 // launcher takes as many as fit); count-only CTAs are small, and a budget for 4 of 256 threads per
 // SM (64 registers, no spills in the rp-pi instances) keeps more of them resident than one for 3.
 __host__ __device__ constexpr int pair_max_threads(bool W, bool R) { return (W || R) ? 512 : 256; }
-__host__ __device__ constexpr int pair_min_blocks(bool W, bool R) { return (!W && !R) ? 3 : 1; }
+__host__ __device__ constexpr int pair_min_blocks(bool W, bool R) { return (!W && !R) ? 4 : 1; }
 
 template <int KIND, bool W, bool R, bool WRAP, bool LO, bool GH, bool FX>
 __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
@@ -697,15 +708,16 @@ __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const CfDevPlan *__restrict__ P = a.plan;
-    const uint32_t nl4 = align16((uint32_t)P->nlut8) / 4u;
-    float *s_fxr = (float *)(smem + 4u * nl4);          // rp-pi / mocks: per rp bin scale of the ravg terms
-    unsigned char *wbase = (unsigned char *)s_fxr + (warp_hist(KIND) ? align16(4u * (uint32_t)a.nb) : 0u);
+    const uint32_t nl4 = align16(a.nlut8) / 4u;
+    // rp-pi / mocks: per rp bin scale of the ravg terms; else with sums the spare row
+    float *s_fxr = (float *)(smem + 4u * nl4);
+    unsigned char *wbase = (unsigned char *)s_fxr + cta_extra_bytes(KIND, W, R, a.nb);
     for (uint32_t i = threadIdx.x; i < nl4; i += blockDim.x) ((uint32_t *)smem)[i] = ((const uint32_t *)a.lut8)[i];
     if (FX && R)
         for (int i = threadIdx.x; i < a.nb; i += blockDim.x) s_fxr[i] = a.fxr_bin[i];
     const int hslots = GH ? 0 : a.nslot;        // slots of the per-warp histogram
     const uint32_t wb = warp_bytes(KIND, W, R, LO, hslots);
-    const uint32_t hoff = warp_jbuf_bytes(W, LO);
+    const uint32_t hoff = warp_jbuf_bytes(W, R, LO);
     unsigned char *my = wbase + (size_t)(threadIdx.x >> 5) * wb;
     {
         // zero this warp's histogram (the buffers need no initial value)
@@ -717,37 +729,27 @@ __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
 
     Warp<KIND, W, R, WRAP, LO, GH, FX> w(a);
     w.lane = threadIdx.x & 31;
-    w.nb = a.nb;
-    w.npi = a.npi;
-    w.nslot = a.nslot;
     w.fxr_bin = s_fxr;
-    w.lut = (uint32_t)__cvta_generic_to_shared(smem) - 0x4B000000u;
-    w.lut_top = 0x4B000000u + (uint32_t)P->nlut8 - 1u;
-    w.lut_scale = P->lut8_scale;
-    w.reach_r = P->reach_r;
-    w.reach_p = P->reach_p;
-    w.pi_inv = P->pi_inv;
-    w.pi_n = P->pi_n;
-    w.pi_tol = P->pi_tol;
-    w.near2 = P->near2;
-    w.near_ss = P->near_ss;
+    w.lut = (uint32_t)__cvta_generic_to_shared(smem) - MAGIC_BITS;
     w.Lx = a.L[0]; w.Ly = a.L[1]; w.Lz = a.L[2];
     w.iLx = a.L[0] > 0.f ? 1.0f / a.L[0] : 0.f;
     w.iLy = a.L[1] > 0.f ? 1.0f / a.L[1] : 0.f;
     w.iLz = a.L[2] > 0.f ? 1.0f / a.L[2] : 0.f;
-    w.jst = (float *)my;
-    w.gj = (uint16_t *)(my + stage_arrays(W, LO) * GBUF * 4u);
+    w.jst = (float *)(my + item_bytes(W, R));
+    w.gj = (uint16_t *)(my + item_bytes(W, R) + stage_arrays(W, LO) * GBUF * 4u);
     w.h_cnt = (uint32_t *)(my + hoff);
     if (warp_hist(KIND)) {
         uint32_t o = (((uint32_t)hslots + (W || R ? 0u : 32u)) * 4u + 7u) & ~7u;
         w.h_wd = (double *)(my + hoff + o);
         w.h_rd = (double *)(my + hoff + o + (W ? hslots * 8u : 0u));
-        w.h_w = w.h_r = nullptr;
+        w.h_w = nullptr;
     } else {
         uint32_t o = a.nslot * 32u * 4u;
         // with both sums they interleave (float4 per lane and bin: w, r, their compensations)
         w.h_w = (float2 *)(my + hoff + o) + (W && R ? 2 : 1) * w.lane;
-        w.h_r = w.h_w;      // only one of them is kept on its own
+        // (counts only: there is neither a sum nor a spare row)
+        w.d_cnt = W || R ? (uint32_t *)s_fxr + w.lane : nullptr;
+        w.d_w = W || R ? (float2 *)(s_fxr + 32) + (W && R ? 2 : 1) * w.lane : nullptr;
         w.h_cnt += w.lane;
         w.h_wd = w.h_rd = nullptr;
     }
@@ -757,30 +759,51 @@ __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
     // pairs evaluated since the last flush: a warp flushes at the latest every 2^28 (an item holds
     // at most 128 x 512 = 2^16), so no 32-bit count and no fixed-point sum it holds can overflow
     uint32_t pend = 0;
-    // the next item's index and descriptor are fetched before the current item is processed
-    uint32_t t = 0;
+    // the next item is fetched while the current one is processed
+    uint32_t t = 0, at = 0;
     if (w.lane == 0) t = atomicAdd(a.cursor, 1u);
     t = __shfl_sync(CF_FULL, t, 0);
-    CfItem it;
-    if (t < nitems) it = a.items[t];
-    for (;;) {
-        if (t >= nitems) break;
+    CfItem *ring = (CfItem *)my;
+    CfItem nx;
+    auto fetch = [&](uint32_t k) {
+        if (smem_items(W, R)) {
+            if (k < nitems && w.lane < (int)(sizeof(CfItem) / 16))
+                cp_async16((uint4 *)(ring + at) + w.lane, (const uint4 *)(a.items + k) + w.lane);
+            cp_async_commit();
+        } else if (k < nitems) {
+            nx = a.items[k];
+        }
+    };
+    fetch(t);
+    while (t < nitems) {
         uint32_t tn = 0;
         if (w.lane == 0) tn = atomicAdd(a.cursor, 1u);
         tn = __shfl_sync(CF_FULL, tn, 0);
-        CfItem nx;
-        if (tn < nitems) nx = a.items[tn];
-        const int job = (int)(it.meta & CFI_ITEM_JOBMASK);
-        if (job != cur || pend > (FX ? FX_FLUSH_PAIRS : CF_FLUSH_PAIRS)) {
-            if (cur >= 0) w.flush((uint32_t)cur);
-            cur = job;
-            pend = 0;
+        auto count = [&](const CfItem &it) {
+            const int job = (int)w.job(it);
+            if (job != cur || pend > (FX ? FX_FLUSH_PAIRS : CF_FLUSH_PAIRS)) {
+                if (cur >= 0) w.flush((uint32_t)cur);
+                cur = job;
+                pend = 0;
+            }
+            pend += (it.cnt & 0xFFFFu) * (it.cnt >> 16);
+            w.run(it);
+        };
+        if (smem_items(W, R)) {
+            cp_async_wait_all();
+            __syncwarp();           // the current item is there, and nobody reads the other place any more
+            const CfItem *it = ring + at;
+            at ^= 1u;
+            fetch(tn);
+            count(*it);
+        } else {
+            const CfItem it = nx;
+            fetch(tn);
+            count(it);
         }
-        pend += (it.cnt & 0xFFFFu) * (it.cnt >> 16);
-        w.run(it);
         t = tn;
-        it = nx;
     }
+    if (smem_items(W, R)) cp_async_wait_all();
     if (cur >= 0) w.flush((uint32_t)cur);
 }
 

@@ -238,7 +238,7 @@ bool build_lut(const std::vector<Seg> &segs, CfLut &L, std::vector<uint16_t> &wo
 // cell with an edge, against one in 250 with cells equally wide in the bit pattern of v.  The last cell
 // lies past the last edge; the kernel clamps there.  Cell 0 always goes to the full tables (the
 // kernel's square root takes denormals as 0).
-void build_lut8(const std::vector<Seg> &segs, int nb, std::vector<uint8_t> &lut, float &scale)
+void build_lut8(const std::vector<Seg> &segs, int cells, int nb, std::vector<uint8_t> &lut, float &scale)
 {
     auto root = [](uint32_t bits) {
         float v;
@@ -246,7 +246,7 @@ void build_lut8(const std::vector<Seg> &segs, int nb, std::vector<uint8_t> &lut,
         return std::sqrt(std::min((double)v, 3.4028234663852886e38));
     };
     const double w = 1.0 / 1048576.0;
-    scale = (float)(CFI_LUT8_CELLS / root(segs.back().start));
+    scale = (float)(cells / root(segs.back().start));
     const int last = (int)std::ceil(root(segs.back().start) * scale * (1 + w) + 0.5);
     lut.assign(last + 1, (uint8_t)(nb + 1));
     for (size_t k = 0; k < segs.size(); k++) {
@@ -649,7 +649,8 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
     // over the width; mocks: the band of the squared edge over 2 pi, and sqrt's error) and by the
     // roundings of pi_inv and of the product.  A t farther than pi_tol from every integer therefore lies
     // in no band and in the bin floor(t); the others go through the table.
-    D.pi_inv = D.pi_n = D.pi_tol = 0.0f;
+    D.pi_n = 0;
+    D.pi_inv = D.pi_tol = 0.0f;
     if (rppi_like || mocks) {
         const int n = p->kind == CF_WP ? 1 : p->npibins;
         const double w = p->pimax / n;
@@ -663,9 +664,9 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
             }
             off = std::max(off, b);
         }
-        D.pi_n = (float)n;
+        D.pi_n = n;
         D.pi_inv = (float)(n / p->pimax);
-        D.pi_tol = ceil32(1.01 * off / w + 16 * u * n);
+        D.pi_tol = ceil32(1.01 * off / w + 16 * u * n + 4 * u);
     }
     // ---- lookup tables ----
     {
@@ -674,7 +675,7 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
             err = "bin edges too close together for the FP32 lookup table";
             return CF_ERR_ARG;
         }
-        build_lut8(segs, D.nb, H.lut8, D.lut8_scale);
+        build_lut8(segs, D.weighted || D.ravg ? CFI_LUT8_CELLS_SUMS : CFI_LUT8_CELLS, D.nb, H.lut8, D.lut8_scale);
         D.nlut8 = (int)H.lut8.size();
         H.lut8.resize((H.lut8.size() + 15) & ~(size_t)15, (uint8_t)D.nb);
     }
