@@ -248,6 +248,27 @@ static int cf_check_bbox(CfCtx *C, CfRun &R, const unsigned long long *bb, doubl
     return CF_OK;
 }
 
+// Shape of the work items where the options leave it open: i tiles of 64 points against j ranges of 256.
+// Smaller items balance better over the warps and cost more items (and build time).  Measured, whole call
+// against 128 x 512: DD(r) of 10k points 174 -> 135 us with 64 x 128 (1,222 items are too few for 4,864 warps),
+// wp of 100k 222 -> 183 us, DD(r) of 200k with sums 568 -> 528 us with 64 x 128; DD(r) of 1M with sums
+// 1.213 -> 1.177 ms, DD(rp, pi) of 2M 1.191 -> 1.168 ms with 64 x 256 (64 x 128: 1.207 and 1.171).  Dense cells
+// make long lists of items whatever their shape: at 1000 points per cell 64 x 256 took 2.735 ms against 2.587 with
+// 128 x 512, at 56 x 558 (survey cone, data x randoms) 64 x 512 2.70 ms, 64 x 256 2.72 and 128 x 512 2.82.
+static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
+{
+    double da = 0.0, db = 0.0;      // mean points per cell, i and j side
+    for (const CfJobDesc &J : R.jobs) {
+        da = std::max(da, (double)R.sets[J.a].n / D.g.ncell);
+        db = std::max(db, (double)R.sets[J.b].n / D.g.ncell);
+    }
+    D.tile = tile ? tile : (da >= 400.0 || R.coarse ? 128 : 64);
+    D.jchunk = jchunk ? jchunk : (db >= 400.0 || R.coarse ? CFI_JMAX : (R.npts <= 400000 ? 128 : 256));
+}
+
+// work lists longer than this (3 GB) are made again with the largest items when their shape was left open
+static const uint32_t CF_FINE_ITEMS = 1u << 26;
+
 int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &pts,
                const std::vector<CfJobDesc> &jobs, CfRun &R)
 {
@@ -396,8 +417,8 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     int refine[3];
     for (int a = 0; a < 3; a++)
         refine[a] = p->refine[a] > 0 ? p->refine[a] : (C->opt[CF_OPT_REFINE] > 0 ? (int)C->opt[CF_OPT_REFINE] : 1);
-    int tile = C->opt[CF_OPT_TILE] > 0 ? (int)std::min<int64_t>(128, std::max<int64_t>(32, C->opt[CF_OPT_TILE])) : 128;
-    int jchunk = C->opt[CF_OPT_JCHUNK] > 0 ? (int)std::min<int64_t>(CFI_JMAX, C->opt[CF_OPT_JCHUNK]) : CFI_JMAX;
+    const int tile = C->opt[CF_OPT_TILE] > 0 ? (int)std::min<int64_t>(128, std::max<int64_t>(32, C->opt[CF_OPT_TILE])) : 0;
+    const int jchunk = C->opt[CF_OPT_JCHUNK] > 0 ? (int)std::min<int64_t>(CFI_JMAX, C->opt[CF_OPT_JCHUNK]) : 0;
     // |v| of the point nearest the observer (its square was summed in float32 for float32 inputs:
     // a few roundings high or low)
     const double vmin = std::isfinite(vmin2) ? std::sqrt(vmin2) * (1.0 - 1e-6) : 0.0;
@@ -417,8 +438,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         put(&vmin, sizeof(vmin));
         if (key != C->plan_key) {
             C->plan_key.clear();
-            rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, tile, jchunk, &H, err, angular ? 1 : 0,
-                               vmin);
+            rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0, vmin);
             if (rc) return C->fail(rc, err);
             C->plan_key = key;
         }
@@ -426,6 +446,8 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     CfDevPlan &D = H.d;
     D.nsets = nsets;
     D.njobs = njobs;
+    R.coarse = !C->coarse_key.empty() && C->coarse_key == C->plan_key;
+    item_shape(R, tile, jchunk, D);
     R.ncell = D.g.ncell;
     for (int s = 0; s < nsets; s++) R.sets[s].cbeg = (int64_t)s * R.ncell;
     R.ncell_all = R.ncell * nsets;
@@ -894,7 +916,8 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     // the work list depends on the plan and on the pruning and order options
     const std::string ikey = C->plan_key + std::to_string(C->opt[CF_OPT_CELL_PRUNE]) + "/" +
                              std::to_string(C->opt[CF_OPT_CELL_ORDER]) + "/" +
-                             std::to_string(C->opt[CF_OPT_BLOCK_PRUNE]);
+                             std::to_string(C->opt[CF_OPT_BLOCK_PRUNE]) + "/" + std::to_string(R.plan.d.tile) + "x" +
+                             std::to_string(R.plan.d.jchunk);
     // a call on the same plan sized the work list before: take that size with headroom, count and
     // write the list in one pass, and let cf_finish run the count again in the rare case that the
     // list outgrew it
@@ -909,6 +932,15 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
               "items total");
         CF_CU(cudaStreamSynchronize(st), "items sync");
         R.items_cap = *(const uint32_t *)C->hpin;
+    }
+    // concentrated points make far more items than their mean density says: take the largest ones then
+    auto too_fine = [&] {
+        return R.items_cap > CF_FINE_ITEMS && !R.coarse && R.plan.d.tile * R.plan.d.jchunk < 128 * CFI_JMAX &&
+               C->opt[CF_OPT_TILE] == 0 && C->opt[CF_OPT_JCHUNK] == 0;
+    };
+    if (!R.fused_items && too_fine()) {
+        C->coarse_key = C->plan_key;
+        return cf_run(C, p, pts, jobs, res);
     }
     CF_TRY(ensure_items(C, R.items_cap));
     for (int attempt = 0; attempt < 4; attempt++) {
@@ -931,6 +963,11 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
             return CF_OK;
         }
         if (retry == 1) CF_TRY(C->ensure(B_QUEUE, 16 * (size_t)R.qcap));
+        if (retry == 2 && too_fine()) {
+            C->coarse_key = C->plan_key;
+            C->items_hint = 0;
+            return cf_run(C, p, pts, jobs, res);
+        }
         if (retry == 2) CF_TRY(ensure_items(C, R.items_cap));
     }
     return C->fail(CF_ERR_INTERNAL, "recheck queue kept overflowing");

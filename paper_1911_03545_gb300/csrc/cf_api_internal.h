@@ -74,6 +74,7 @@ struct CfRun {
     bool self_pairs = false;
     double bbox[6] = {0, 0, 0, 0, 0, 0};   // union of the sets' boxes the plan was made for
     double vmin2 = 0.0;            // smallest |v|^2 over the points (mocks: the plan's near-observer test)
+    bool coarse = false;           // largest work items: finer ones made too long a list
     bool angular = false;          // DD(theta) on the angular grid (needs unit vectors)
     bool bbox_deferred = false;    // periodic call planned from L: its bbox is checked after the final sync
     bool fused_items = false;      // the work list is counted and written in one pass (size known)
@@ -108,6 +109,7 @@ struct CfCtx {
     int num_sms = 1;
     int smem_optin = 0;            // largest dynamic shared memory of one CTA (opt-in)
     std::string plan_key;          // inputs of the plan held in run.plan (empty: none)
+    std::string coarse_key;        // plan whose work list is made of the largest items (see CF_FINE_ITEMS)
     std::string err;
     size_t mem_cap = 0, mem_used = 0;
     Buf buf[B_COUNT_];
