@@ -419,6 +419,11 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         refine[a] = p->refine[a] > 0 ? p->refine[a] : (C->opt[CF_OPT_REFINE] > 0 ? (int)C->opt[CF_OPT_REFINE] : 1);
     const int tile = C->opt[CF_OPT_TILE] > 0 ? (int)std::min<int64_t>(128, std::max<int64_t>(32, C->opt[CF_OPT_TILE])) : 0;
     const int jchunk = C->opt[CF_OPT_JCHUNK] > 0 ? (int)std::min<int64_t>(CFI_JMAX, C->opt[CF_OPT_JCHUNK]) : 0;
+    // a call that leaves the refinement and the order inside the cells open leaves the cells' width open too
+    // (the audit has a limit on the pairs of the work list, which wider cells make longer)
+    bool open_grid = !angular && C->opt[CF_OPT_REFINE] == 0 && C->opt[CF_OPT_CELL_ORDER] == 0 && !C->opt[CF_OPT_AUDIT];
+    for (int a = 0; a < 3; a++) open_grid = open_grid && p->refine[a] == 0;
+    const double fill = open_grid ? CFI_MIN_FILL : 0.0;
     // |v| of the point nearest the observer (its square was summed in float32 for float32 inputs:
     // a few roundings high or low)
     const double vmin = std::isfinite(vmin2) ? std::sqrt(vmin2) * (1.0 - 1e-6) : 0.0;
@@ -433,12 +438,17 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         put(bbox, sizeof(bbox));
         put(&R.npts, sizeof(R.npts));
         const int ints[6] = {any_f64 ? 1 : 0, refine[0] * 16 + refine[1] * 4 + refine[2], tile, jchunk, angular ? 1 : 0,
-                             0};
+                             open_grid ? 1 : 0};
         put(ints, sizeof(ints));
         put(&vmin, sizeof(vmin));
         if (key != C->plan_key) {
             C->plan_key.clear();
-            rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0, vmin);
+            rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0, vmin,
+                               fill * nsets);
+            // wider cells have wider error bands: what fails with them may pass without
+            if (rc && fill > 0.0)
+                rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0,
+                                   vmin);
             if (rc) return C->fail(rc, err);
             C->plan_key = key;
         }

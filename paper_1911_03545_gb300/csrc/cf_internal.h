@@ -28,6 +28,8 @@
 #define CFI_CLS_OUT 0xFEu         // class: outside every bin
 #define CFI_CLS_AMB 0xFFu         // class: within the FP32 error band of an edge
 #define CFI_FINE_FLAG 0x100u      // coarse entry >= this: index of a fine entry + flag
+#define CFI_MIN_FILL 40.0         // points per cell and set below which the cells are widened (widen_cells)
+#define CFI_WIDEN_MIN 32768       // points of a call below which they are not
 #define CFI_JMAX 512              // longest j range of a work item (9-bit j in a candidate)
 
 // Pair-kernel item (48 bytes, three 16-byte loads)
