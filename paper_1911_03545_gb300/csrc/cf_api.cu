@@ -266,6 +266,26 @@ static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
     D.jchunk = jchunk ? jchunk : (db >= 400.0 || R.coarse ? CFI_JMAX : (R.npts <= 400000 ? 128 : 256));
 }
 
+// points of a call up to which one launch builds it
+static const int64_t CF_ONE_MAX = 262144;
+
+// work-list capacity (48 bytes an item) up to which a call on a new plan takes an estimate instead of
+// counting the items first
+static const uint64_t CF_GUESS_MAX = 1u << 21;
+
+static uint64_t items_guess(const CfRun &R)
+{
+    const CfDevPlan &D = R.plan.d;
+    double n = 4096.0;
+    for (const CfJobDesc &J : R.jobs) {
+        const double na = (double)R.sets[J.a].n, nb = (double)R.sets[J.b].n, nc = (double)D.g.ncell;
+        const double cells = std::min(nc, na);      // i cells that may hold points
+        const double pairs = D.ang ? 25.0 : (J.autoc ? 0.5 * (R.nst + 1) : (double)R.nst);
+        n += cells * std::min(pairs, nb) * (na / cells / D.tile + 1.0) * (nb / std::min(nc, std::max(1.0, nb)) / D.jchunk + 1.0);
+    }
+    return n < 4e18 ? (uint64_t)n : (uint64_t)4e18;
+}
+
 // work lists longer than this (3 GB) are made again with the largest items when their shape was left open
 static const uint32_t CF_FINE_ITEMS = 1u << 26;
 
@@ -479,6 +499,13 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     // a grid with more cells than points (most of them empty): list the units with points first,
     // so that the work-list pass does not spend a warp iteration on each empty cell
     R.live_units = R.nunit >= 65536 && R.nunit > R.npts;
+    R.one_build = !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
+    if (R.one_build && C->one_blocks < 0) {
+        CF_TRY(C->ensure(B_BAR, 64));
+        CF_CU(cudaMemsetAsync(C->buf[B_BAR].p, 0, 64, st), "memset barrier");
+        C->one_blocks = cfb_one_init(C->num_sms);
+    }
+    R.one_build = R.one_build && C->one_blocks > 0;
     R.nslot = (size_t)D.nslot;
     R.hsz = R.nslot * njobs;
     R.self_pairs = p->edges[0] == 0.0;
@@ -525,7 +552,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     if (C->opt[CF_OPT_CELL_PRUNE] == 0 && C->opt[CF_OPT_BLOCK_PRUNE] == 1) CF_TRY(C->ensure(B_GBOX, 24 * (size_t)R.np));
     if (D.f64lo) CF_TRY(C->ensure(B_PLO, 16 * (size_t)R.np));
     if (D.f64lo && mocks) CF_TRY(C->ensure(B_PABSLO, 16 * (size_t)R.np));
-    CF_TRY(C->ensure(B_SCAN, 4 * (size_t)cfb_scan_tmp_words(std::max(R.nfine, R.nunit))));
+    CF_TRY(C->ensure(B_SCAN, 4 * (size_t)std::max<int64_t>(C->num_sms, cfb_scan_tmp_words(std::max(R.nfine, R.nunit)))));
     CF_TRY(C->ensure(B_ICNT, 4 * (size_t)std::max<int64_t>(R.nunit, 1)));
     CF_TRY(C->ensure(B_IOFF, 4 * (size_t)(R.nunit + 1)));
     if (R.live_units) CF_TRY(C->ensure(B_LIVE, 4 * (size_t)R.nunit));
@@ -608,6 +635,45 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
     uint32_t *cnt = (uint32_t *)C->buf[B_CNT].p, *cstart = (uint32_t *)C->buf[B_CSTART].p;
     char *out = (char *)C->buf[B_OUT].p;
     uint32_t *fstart = (uint32_t *)C->buf[B_FSTART].p;
+    if (R.one_build && R.fused_items) {
+        CfOneBuild S;
+        std::memset(&S, 0, sizeof(S));
+        S.plan = dplan;
+        S.sets = dsets;
+        S.jobs = djobs;
+        S.stencil = R.d_stencil;
+        S.nsets = R.nsets;
+        S.sub = R.sub;
+        S.npts = (uint32_t)R.npts;
+        S.nfine = (uint32_t)R.nfine;
+        S.zero = (uint32_t *)out;
+        S.zero_words = (uint32_t)(readback_bytes(R) / 4);
+        S.bar = (uint32_t *)C->buf[B_BAR].p;
+        S.late = S.bar + 2;
+        S.part = (uint32_t *)C->buf[B_SCAN].p;
+        S.count = cnt;
+        S.key = (uint32_t *)C->buf[B_CELLID].p;
+        S.slot = (uint32_t *)C->buf[B_SLOT].p;
+        S.fstart = fstart;
+        S.cell_start = cstart;
+        S.orig = (uint32_t *)C->buf[B_ORIG].p;
+        S.pt = (float4 *)C->buf[B_PT].p;
+        S.pabs = (float4 *)C->buf[B_PABS].p;
+        S.plo = (float4 *)C->buf[B_PLO].p;
+        S.pabslo = (float4 *)C->buf[B_PABSLO].p;
+        S.cbox = C->opt[CF_OPT_CELL_PRUNE] == 0 ? (float *)C->buf[B_CBOX].p : nullptr;
+        S.items = (CfItem *)C->buf[B_ITEMS].p;
+        S.items_cap = R.items_cap;
+        S.nitems = (uint32_t *)(out + OUT_NITEMS);
+        S.evaluated = (unsigned long long *)(out + OUT_EVAL);
+        S.total64 = (unsigned long long *)(out + OUT_ITEMS64);
+        CF_CU(cfb_one_build(S, C->one_blocks, st), "build");
+        R.cbox = S.cbox;
+        R.gbox = nullptr;
+        R.listed = true;
+        C->launches += 1;
+        return CF_OK;
+    }
     if (R.plan.d.ang) {
         CF_CU(cfb_ang_origins(dplan, R.plan.d.g.ncell, R.d_origin, R.d_origin32, st), "cell origins");
         C->launches += 1;
@@ -731,13 +797,17 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     // evaluated pairs, the work cursor, the queue length, the histograms and w^2 sums (and for the
     // one-pass work list its two length counters): one memset
     const size_t zero_from = R.fused_items ? 0 : OUT_EVAL;
-    CF_CU(cudaMemsetAsync(out + zero_from, 0, readback_bytes(R) - zero_from, st), "memset");
+    const bool listed = R.listed;       // the build has zeroed them and written the list
+    R.listed = false;
+    if (!listed) CF_CU(cudaMemsetAsync(out + zero_from, 0, readback_bytes(R) - zero_from, st), "memset");
     uint32_t *nitems_dev = ioff + R.nunit;
     const uint32_t *cstart = (const uint32_t *)C->buf[B_CSTART].p;
     const uint32_t *live = R.live_units ? (const uint32_t *)C->buf[B_LIVE].p : nullptr;
     const uint32_t *nlive = R.live_units ? (const uint32_t *)(out + OUT_NLIVE) : nullptr;
-    if (R.fused_items) {
-        nitems_dev = (uint32_t *)(out + OUT_NITEMS);
+    if (R.fused_items) nitems_dev = (uint32_t *)(out + OUT_NITEMS);
+    if (listed) {
+        // nothing left to do
+    } else if (R.fused_items) {
         if (R.live_units) {
             // the memset above cleared the list's count: list the units with points again
             CF_CU(cfb_live_units(dplan, dsets, djobs, cstart, R.nunit, (uint32_t *)live, (uint32_t *)nlive, st),
@@ -817,12 +887,15 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     C->last_grid = grid;
     C->last_warps = warps;
     if (timed) CF_CU(cudaEventRecordWithFlags(C->ev[2], st, C->capturing ? cudaEventRecordExternal : 0), "event");
-    CF_CU(cfp_launch_recheck(dplan, dsets, djobs, A.queue, A.qcount, R.qcap, A.hcnt, A.hw, A.hr, C->num_sms, st), "recheck");
+    CF_CU(cfp_launch_recheck(dplan, dsets, djobs, A.queue, A.qcount, R.qcap, A.hcnt, A.hw, A.hr,
+                             listed ? (const uint32_t *)C->buf[B_BAR].p + 2 : nullptr, (uint32_t *)(out + OUT_LATE),
+                             C->num_sms, st),
+          "recheck");
     if (R.self_pairs && D.weighted) {
         CF_CU(cfb_wsq(dsets, R.nsets, R.np, wsq, st), "self-pair weights");
         C->launches++;
     }
-    C->launches += 2 + (R.items_cap > 0 ? 1 : 0);   // items emit, recheck, pair
+    C->launches += (listed ? 1 : 2) + (R.items_cap > 0 ? 1 : 0);   // items emit, recheck, pair
     if (timed) CF_CU(cudaEventRecordWithFlags(C->ev[3], st, C->capturing ? cudaEventRecordExternal : 0), "event");
     // the side stream's bbox pass joins here, so that the call's synchronisation covers it
     if (R.bbox_aux) {
@@ -841,6 +914,10 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
     const unsigned long long qn = *(const unsigned long long *)(h + OUT_QCOUNT);
     const uint32_t nitems = *(const uint32_t *)(h + OUT_NITEMS);
     *retry = 0;
+    if (*(const uint32_t *)(h + OUT_LATE)) {
+        C->one_blocks = -1;         // start the barrier afresh
+        return C->fail(CF_ERR_TIMEOUT, "the build gave up waiting at a barrier");
+    }
     // work items and queue entries are indexed in 32 bits, with headroom for the grid-stride
     // loops and the work cursor's overshoot
     if (*(const unsigned long long *)(h + OUT_ITEMS64) > CF_MAX_ENTRIES)
@@ -931,12 +1008,25 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     // a call on the same plan sized the work list before: take that size with headroom, count and
     // write the list in one pass, and let cf_finish run the count again in the rare case that the
     // list outgrew it
+    R.listed = false;
     R.fused_items = C->items_hint && C->items_key == ikey;
+    uint32_t cap = C->items_hint;
+    if (!R.fused_items && !C->opt[CF_OPT_AUDIT] && !C->mem_cap) {
+        // a new plan: the size that evenly spread points would need, while that is modest; a longer list
+        // only costs a second attempt, whose pair kernel the first one leaves out
+        const uint64_t guess = items_guess(R);
+        if (guess <= CF_GUESS_MAX && ensure_items(C, guess) == CF_OK) {
+            R.fused_items = true;
+            cap = (uint32_t)guess;
+        }
+    }
+    if (R.fused_items) {
+        R.items_cap = cap;
+        CF_TRY(ensure_items(C, cap));
+    }
     CF_CU(cudaEventRecord(C->ev[0], st), "event");
     CF_TRY(cf_enqueue_build(C, R));
-    if (R.fused_items) {
-        R.items_cap = C->items_hint;
-    } else {
+    if (!R.fused_items) {
         // size the work list from the device count (one small readback)
         CF_CU(cudaMemcpyAsync(C->hpin, (uint32_t *)C->buf[B_IOFF].p + R.nunit, 4, cudaMemcpyDeviceToHost, st),
               "items total");

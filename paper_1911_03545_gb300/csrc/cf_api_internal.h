@@ -12,7 +12,7 @@
 enum CfBuf {
     B_IN, B_SETS, B_BBOX, B_PLAN, B_LUT, B_FINE, B_STENCIL, B_JOBS, B_CNT, B_CSTART, B_CELLID, B_SLOT,
     B_PT, B_PABS, B_PLO, B_PABSLO, B_ORIG, B_SCAN, B_ICNT, B_IOFF, B_ITEMS, B_HCNT, B_HW, B_HR, B_QUEUE, B_WSQ, B_MISC, B_ORIGIN,
-    B_CBOX, B_FSTART, B_BANDS, B_ORIGIN32, B_OUT, B_PLANBLK, B_GBOX, B_LIVE, B_COUNT_
+    B_CBOX, B_FSTART, B_BANDS, B_ORIGIN32, B_OUT, B_PLANBLK, B_GBOX, B_LIVE, B_BAR, B_COUNT_
 };
 
 // B_OUT: the counters and histograms one call reads back, laid out as the host copy of them (one
@@ -20,7 +20,7 @@ enum CfBuf {
 // of units with points in their i cell (u32, when the work list visits only those), the same length in 64 bits,
 // evaluated pairs, the pair kernel's work cursor (u32), recheck-queue length, then from OUT_HIST
 // hcnt[hsz] (u64), hw[hsz], hr[hsz] (f64) and the sum of w^2 per point set (f64); at OUT_SCAN the
-// tickets of the build's two scans.  The build zeroes the first OUT_HIST bytes, the count phase
+// tickets of the build's two scans, at OUT_LATE a flag that the one-launch build gave up at a barrier.  The build zeroes the first OUT_HIST bytes, the count phase
 // everything from OUT_EVAL on (from 0 for the one-pass work list), each with one memset.
 #define OUT_NITEMS 0
 #define OUT_NLIVE 4
@@ -29,6 +29,7 @@ enum CfBuf {
 #define OUT_CURSOR 24
 #define OUT_QCOUNT 32
 #define OUT_SCAN 40
+#define OUT_LATE 48
 #define OUT_HIST 64
 
 struct DeviceGuard {
@@ -78,6 +79,8 @@ struct CfRun {
     bool angular = false;          // DD(theta) on the angular grid (needs unit vectors)
     bool bbox_deferred = false;    // periodic call planned from L: its bbox is checked after the final sync
     bool fused_items = false;      // the work list is counted and written in one pass (size known)
+    bool listed = false;           // the build has written the work list and zeroed the call's counters
+    bool one_build = false;        // the build is one launch (cfb_one_build)
     bool live_units = false;       // the work list visits only the units whose i cell holds points
     bool bbox_aux = false;         // the bbox pass runs on the side stream: join before the readback
     // the call's plan, tables and descriptors inside the B_PLANBLK device block
@@ -127,6 +130,7 @@ struct CfCtx {
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     CfRun run;
     int last_grid = 0, last_warps = 0;
+    int one_blocks = -1;           // blocks of the one-launch build (0: not taken, -1: not asked yet)
     int launches = 0;              // kernels launched by the current call
     uint64_t gen = 0;              // bumped whenever device or pinned scratch is reallocated
     cudaGraph_t graph = nullptr;

@@ -226,79 +226,84 @@ __device__ __forceinline__ uint32_t cf_morton3(uint32_t x, uint32_t y, uint32_t 
            ((y & 1u) << 1) | (z & 1u);
 }
 
+// The counting-sort key of point i of a set
+__device__ __forceinline__ uint32_t cf_point_key(const CfDevPlan *__restrict__ plan, const CfSetDesc &S, int64_t i, int sub)
+{
+    const CfGrid &g = plan->g;
+    const bool f32 = S.dtype == CF_F32;
+    // float32 inputs stay float32 here (the FP64 pipe runs at a small fraction of the FP32 rate)
+    float xf[3];
+    double xd[3] = {0.0, 0.0, 0.0};
+    if (f32) {
+        xf[0] = ((const float *)S.x)[i];
+        xf[1] = ((const float *)S.y)[i];
+        xf[2] = ((const float *)S.z)[i];
+    } else {
+        xd[0] = ((const double *)S.x)[i];
+        xd[1] = ((const double *)S.y)[i];
+        xd[2] = ((const double *)S.z)[i];
+        for (int a = 0; a < 3; a++) xf[a] = (float)xd[a];
+    }
+    uint32_t sa[3] = {0u, 0u, 0u};
+    uint32_t c;
+    if (plan->ang) {
+        // angular grid: declination band of the vector's direction (atan2 of z over the projected
+        // length: independent of |v| and well conditioned at the poles), then right-ascension
+        // cell in [0, 2 pi).  Float32 is enough: any cell choice is correct as long as the point
+        // lies in the cell's box, whose margin (2e-6) is far above these ~1e-7 errors.
+        const double dec = (double)atan2f(xf[2], sqrtf(xf[0] * xf[0] + xf[1] * xf[1]));
+        double ra = (double)atan2f(xf[1], xf[0]);
+        if (ra < 0.0) ra += 2.0 * M_PI;
+        int b = (int)floor((dec - plan->adlo) / plan->ah);
+        b = b < 0 ? 0 : (b > plan->nband - 1 ? plan->nband - 1 : b);
+        const CfBand &B = plan->band[b];
+        const double tr = ra * B.inv_w;
+        int r = (int)floor(tr);
+        r = r < 0 ? 0 : (r > B.nra - 1 ? B.nra - 1 : r);
+        c = (uint32_t)(B.base + r);
+        const double fr[2] = {(dec - B.dlo) / (B.dhi - B.dlo), tr - (double)r};
+        for (int a = 0; a < 2; a++) {
+            const int s = (int)(fr[a] * sub);
+            sa[a] = (uint32_t)(s < 0 ? 0 : (s > sub - 1 ? sub - 1 : s));
+        }
+    } else {
+        int ia[3];
+        for (int a = 0; a < 3; a++) {
+            // the cell coordinate in float32 decides the cell as the FP64 one would, unless it
+            // lies within the plan's guard of a cell boundary: then (and for float64 inputs) FP64
+            float fr;
+            int cc;
+            const float t32 = (xf[a] - plan->lo32[a]) * plan->inv32[a];
+            const float f32c = floorf(t32), r32 = t32 - f32c;
+            if (f32 && r32 >= plan->cguard[a] && r32 <= 1.0f - plan->cguard[a]) {
+                cc = (int)f32c;
+                fr = r32;
+            } else {
+                const double x = f32 ? (double)xf[a] : xd[a];
+                const double t = (x - g.lo[a]) * g.inv[a];
+                const double ft = floor(t);
+                cc = (int)ft;
+                fr = (float)(t - ft);
+            }
+            cc = cc < 0 ? 0 : (cc > g.n[a] - 1 ? g.n[a] - 1 : cc);
+            ia[a] = cc;
+            // the sub-cell orders points inside the cell; it does not change any result
+            const int s = (int)(fr * (float)sub);
+            sa[a] = (uint32_t)(s < 0 ? 0 : (s > sub - 1 ? sub - 1 : s));
+        }
+        c = (uint32_t)((ia[0] * g.n[1] + ia[1]) * g.n[2] + ia[2]);
+    }
+    return ((uint32_t)S.cbeg + c) * (uint32_t)(sub * sub * sub) + (sub > 1 ? cf_morton3(sa[0], sa[1], sa[2], sub) : 0u);
+}
+
 __global__ void __launch_bounds__(256, 6) cf_assign_kernel(const CfDevPlan *__restrict__ plan, const CfSetDesc *__restrict__ sets, int sub,
                                  uint32_t *__restrict__ count, uint32_t *__restrict__ key,
                                  uint32_t *__restrict__ slot)
 {
     const CfSetDesc S = sets[blockIdx.y];
-    const CfGrid &g = plan->g;
-    const uint32_t ns = (uint32_t)(sub * sub * sub);
-    const bool f32 = S.dtype == CF_F32;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < S.n; i += (int64_t)gridDim.x * blockDim.x) {
-        // float32 inputs stay float32 here (the FP64 pipe runs at a small fraction of the FP32 rate)
-        float xf[3];
-        double xd[3] = {0.0, 0.0, 0.0};
-        if (f32) {
-            xf[0] = ((const float *)S.x)[i];
-            xf[1] = ((const float *)S.y)[i];
-            xf[2] = ((const float *)S.z)[i];
-        } else {
-            xd[0] = ((const double *)S.x)[i];
-            xd[1] = ((const double *)S.y)[i];
-            xd[2] = ((const double *)S.z)[i];
-            for (int a = 0; a < 3; a++) xf[a] = (float)xd[a];
-        }
-        uint32_t sa[3] = {0u, 0u, 0u};
-        uint32_t c;
-        if (plan->ang) {
-            // angular grid: declination band of the vector's direction (atan2 of z over the projected
-            // length: independent of |v| and well conditioned at the poles), then right-ascension
-            // cell in [0, 2 pi).  Float32 is enough: any cell choice is correct as long as the point
-            // lies in the cell's box, whose margin (2e-6) is far above these ~1e-7 errors.
-            const double dec = (double)atan2f(xf[2], sqrtf(xf[0] * xf[0] + xf[1] * xf[1]));
-            double ra = (double)atan2f(xf[1], xf[0]);
-            if (ra < 0.0) ra += 2.0 * M_PI;
-            int b = (int)floor((dec - plan->adlo) / plan->ah);
-            b = b < 0 ? 0 : (b > plan->nband - 1 ? plan->nband - 1 : b);
-            const CfBand &B = plan->band[b];
-            const double tr = ra * B.inv_w;
-            int r = (int)floor(tr);
-            r = r < 0 ? 0 : (r > B.nra - 1 ? B.nra - 1 : r);
-            c = (uint32_t)(B.base + r);
-            const double fr[2] = {(dec - B.dlo) / (B.dhi - B.dlo), tr - (double)r};
-            for (int a = 0; a < 2; a++) {
-                const int s = (int)(fr[a] * sub);
-                sa[a] = (uint32_t)(s < 0 ? 0 : (s > sub - 1 ? sub - 1 : s));
-            }
-        } else {
-            int ia[3];
-            for (int a = 0; a < 3; a++) {
-                // the cell coordinate in float32 decides the cell as the FP64 one would, unless it
-                // lies within the plan's guard of a cell boundary: then (and for float64 inputs) FP64
-                float fr;
-                int cc;
-                const float t32 = (xf[a] - plan->lo32[a]) * plan->inv32[a];
-                const float f32c = floorf(t32), r32 = t32 - f32c;
-                if (f32 && r32 >= plan->cguard[a] && r32 <= 1.0f - plan->cguard[a]) {
-                    cc = (int)f32c;
-                    fr = r32;
-                } else {
-                    const double x = f32 ? (double)xf[a] : xd[a];
-                    const double t = (x - g.lo[a]) * g.inv[a];
-                    const double ft = floor(t);
-                    cc = (int)ft;
-                    fr = (float)(t - ft);
-                }
-                cc = cc < 0 ? 0 : (cc > g.n[a] - 1 ? g.n[a] - 1 : cc);
-                ia[a] = cc;
-                // the sub-cell orders points inside the cell; it does not change any result
-                const int s = (int)(fr * (float)sub);
-                sa[a] = (uint32_t)(s < 0 ? 0 : (s > sub - 1 ? sub - 1 : s));
-            }
-            c = (uint32_t)((ia[0] * g.n[1] + ia[1]) * g.n[2] + ia[2]);
-        }
-        const uint32_t k = ((uint32_t)S.cbeg + c) * ns + (sub > 1 ? cf_morton3(sa[0], sa[1], sa[2], sub) : 0u);
-        int64_t p = S.pbeg + i;
+        const uint32_t k = cf_point_key(plan, S, i, sub);
+        const int64_t p = S.pbeg + i;
         key[p] = k;
         slot[p] = atomicAdd(count + k, 1u);
     }
@@ -504,6 +509,48 @@ __global__ void cf_scan_apply(const uint32_t *__restrict__ in, uint32_t *__restr
 // (pt, 16 bytes: one sector per point), for mocks the absolute position, the low parts when requested,
 // and the original index.
 // ---------------------------------------------------------------------------------------------
+// Point i of a set, whose key is k, into its place dst
+__device__ __forceinline__ void cf_scatter_point(const CfDevPlan *__restrict__ plan, const CfSetDesc &S, int64_t i,
+                                                 uint32_t k, uint32_t ns, int64_t dst, float4 *pt, float4 *pabs,
+                                                 float4 *plo, float4 *pabslo, uint32_t *orig)
+{
+    const CfGrid &g = plan->g;
+    const int lo = plan->f64lo;
+    const uint32_t c = k / ns - (uint32_t)S.cbeg;
+    const int iz = c % g.n[2];
+    const int iy = (c / g.n[2]) % g.n[1];
+    const int ix = c / (g.n[2] * g.n[1]);
+    const bool mocks = plan->kind == CF_DD_RPPI_MOCKS;
+    if (S.dtype == CF_F32 && !lo) {
+        // float32 inputs: x - o is exact in float32 (o is a multiple of the float32 spacing at
+        // the cell's magnitude and lies between 0 and x), the same value the FP64 form rounds to
+        const float vx = ((const float *)S.x)[i], vy = ((const float *)S.y)[i], vz = ((const float *)S.z)[i];
+        const float xf = vx - cf_cell_origin32(plan, 0, (int)c, ix);
+        const float yf = vy - cf_cell_origin32(plan, 1, (int)c, iy);
+        const float zf = vz - cf_cell_origin32(plan, 2, (int)c, iz);
+        const float w = S.w ? ((const float *)S.w)[i] : 1.0f;
+        pt[dst] = make_float4(-xf, -yf, -zf, w);
+        if (mocks) pabs[dst] = make_float4(vx, vy, vz, 0.f);
+        orig[dst] = (uint32_t)i;
+        return;
+    }
+    const double vx = cf_load(S.x, S.dtype, i), vy = cf_load(S.y, S.dtype, i), vz = cf_load(S.z, S.dtype, i);
+    double X = vx - cf_cell_origin(plan, 0, (int)c, ix);
+    double Y = vy - cf_cell_origin(plan, 1, (int)c, iy);
+    double Z = vz - cf_cell_origin(plan, 2, (int)c, iz);
+    float xf = (float)X, yf = (float)Y, zf = (float)Z;
+    float w = S.w ? (float)cf_load(S.w, S.dtype, i) : 1.0f;
+    pt[dst] = make_float4(-xf, -yf, -zf, w);
+    const float ax = (float)vx, ay = (float)vy, az = (float)vz;
+    if (mocks) pabs[dst] = make_float4(ax, ay, az, 0.f);
+    if (lo) {
+        plo[dst] = make_float4(-(float)(X - (double)xf), -(float)(Y - (double)yf), -(float)(Z - (double)zf), 0.f);
+        if (mocks)
+            pabslo[dst] = make_float4((float)(vx - (double)ax), (float)(vy - (double)ay), (float)(vz - (double)az), 0.f);
+    }
+    orig[dst] = (uint32_t)i;
+}
+
 __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__restrict__ plan, const CfSetDesc *__restrict__ sets,
                                   uint32_t ns, const uint32_t *__restrict__ fstart, const uint32_t *__restrict__ key,
                                   const uint32_t *__restrict__ slot, float4 *__restrict__ pt,
@@ -511,45 +558,10 @@ __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__r
                                   float4 *__restrict__ pabslo, uint32_t *__restrict__ orig)
 {
     const CfSetDesc S = sets[blockIdx.y];
-    const CfGrid &g = plan->g;
-    const int lo = plan->f64lo;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < S.n; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t p = S.pbeg + i;
+        const int64_t p = S.pbeg + i;
         const uint32_t k = key[p];
-        const uint32_t c = k / ns - (uint32_t)S.cbeg;
-        int iz = c % g.n[2];
-        int iy = (c / g.n[2]) % g.n[1];
-        int ix = c / (g.n[2] * g.n[1]);
-        int64_t dst = fstart[k] + slot[p];
-        const bool mocks = plan->kind == CF_DD_RPPI_MOCKS;
-        if (S.dtype == CF_F32 && !lo) {
-            // float32 inputs: x - o is exact in float32 (o is a multiple of the float32 spacing at
-            // the cell's magnitude and lies between 0 and x), the same value the FP64 form rounds to
-            const float vx = ((const float *)S.x)[i], vy = ((const float *)S.y)[i], vz = ((const float *)S.z)[i];
-            const float xf = vx - cf_cell_origin32(plan, 0, (int)c, ix);
-            const float yf = vy - cf_cell_origin32(plan, 1, (int)c, iy);
-            const float zf = vz - cf_cell_origin32(plan, 2, (int)c, iz);
-            const float w = S.w ? ((const float *)S.w)[i] : 1.0f;
-            pt[dst] = make_float4(-xf, -yf, -zf, w);
-            if (mocks) pabs[dst] = make_float4(vx, vy, vz, 0.f);
-            orig[dst] = (uint32_t)i;
-            continue;
-        }
-        const double vx = cf_load(S.x, S.dtype, i), vy = cf_load(S.y, S.dtype, i), vz = cf_load(S.z, S.dtype, i);
-        double X = vx - cf_cell_origin(plan, 0, (int)c, ix);
-        double Y = vy - cf_cell_origin(plan, 1, (int)c, iy);
-        double Z = vz - cf_cell_origin(plan, 2, (int)c, iz);
-        float xf = (float)X, yf = (float)Y, zf = (float)Z;
-        float w = S.w ? (float)cf_load(S.w, S.dtype, i) : 1.0f;
-        pt[dst] = make_float4(-xf, -yf, -zf, w);
-        const float ax = (float)vx, ay = (float)vy, az = (float)vz;
-        if (mocks) pabs[dst] = make_float4(ax, ay, az, 0.f);
-        if (lo) {
-            plo[dst] = make_float4(-(float)(X - (double)xf), -(float)(Y - (double)yf), -(float)(Z - (double)zf), 0.f);
-            if (mocks)
-                pabslo[dst] = make_float4((float)(vx - (double)ax), (float)(vy - (double)ay), (float)(vz - (double)az), 0.f);
-        }
-        orig[dst] = (uint32_t)i;
+        cf_scatter_point(plan, S, i, k, ns, (int64_t)fstart[k] + slot[p], pt, pabs, plo, pabslo, orig);
     }
 }
 
@@ -562,47 +574,52 @@ __global__ void __launch_bounds__(256, 6) cf_scatter_kernel(const CfDevPlan *__r
 // cell (counted from the cell's first point), at gbox[6 p] for the group's first point p; the work
 // list prunes at that granularity.
 // ---------------------------------------------------------------------------------------------
+// one warp: the box of cell c
+__device__ __forceinline__ void cf_cell_box(const uint32_t *cell_start, int64_t c, const float4 *pt, float *box, float *gbox)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t b = cell_start[c], e = cell_start[c + 1];
+    if (b == e) {
+        // most cells of a fine grid are empty: no reduction for them (b, e are warp-uniform)
+        if (lane < 6u) box[6 * c + lane] = lane < 3u ? INFINITY : -INFINITY;
+        return;
+    }
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    for (uint32_t p0 = b; p0 < e; p0 += 32u) {
+        float glo[3] = {INFINITY, INFINITY, INFINITY}, ghi[3] = {-INFINITY, -INFINITY, -INFINITY};
+        const uint32_t p = p0 + lane;
+        if (p < e) {
+            const float4 A = pt[p];
+            const float v[3] = {-A.x, -A.y, -A.z};
+            for (int a = 0; a < 3; a++) glo[a] = ghi[a] = v[a];
+        }
+        if (gbox) {
+            for (int o = 16; o; o >>= 1)
+                for (int a = 0; a < 3; a++) {
+                    glo[a] = fminf(glo[a], __shfl_xor_sync(CF_FULL, glo[a], o));
+                    ghi[a] = fmaxf(ghi[a], __shfl_xor_sync(CF_FULL, ghi[a], o));
+                }
+            if (lane < 6u) gbox[6 * (size_t)p0 + lane] = lane < 3u ? glo[lane] : ghi[lane - 3u];
+        }
+        for (int a = 0; a < 3; a++) {
+            lo[a] = fminf(lo[a], glo[a]);
+            hi[a] = fmaxf(hi[a], ghi[a]);
+        }
+    }
+    for (int o = 16; o; o >>= 1)
+        for (int a = 0; a < 3; a++) {
+            lo[a] = fminf(lo[a], __shfl_xor_sync(CF_FULL, lo[a], o));
+            hi[a] = fmaxf(hi[a], __shfl_xor_sync(CF_FULL, hi[a], o));
+        }
+    if (lane < 6u) box[6 * c + lane] = lane < 3u ? lo[lane] : hi[lane - 3u];
+}
+
 __global__ void cf_cellbox_kernel(const uint32_t *__restrict__ cell_start, int64_t ncell_all,
                                   const float4 *__restrict__ pt, float *__restrict__ box, float *__restrict__ gbox)
 {
-    const uint32_t lane = threadIdx.x & 31u;
     const int64_t wstride = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < ncell_all; c += wstride) {
-        const uint32_t b = cell_start[c], e = cell_start[c + 1];
-        if (b == e) {
-            // most cells of a fine grid are empty: no reduction for them (b, e are warp-uniform)
-            if (lane < 6u) box[6 * c + lane] = lane < 3u ? INFINITY : -INFINITY;
-            continue;
-        }
-        float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-        for (uint32_t p0 = b; p0 < e; p0 += 32u) {
-            float glo[3] = {INFINITY, INFINITY, INFINITY}, ghi[3] = {-INFINITY, -INFINITY, -INFINITY};
-            const uint32_t p = p0 + lane;
-            if (p < e) {
-                const float4 A = pt[p];
-                const float v[3] = {-A.x, -A.y, -A.z};
-                for (int a = 0; a < 3; a++) glo[a] = ghi[a] = v[a];
-            }
-            if (gbox) {
-                for (int o = 16; o; o >>= 1)
-                    for (int a = 0; a < 3; a++) {
-                        glo[a] = fminf(glo[a], __shfl_xor_sync(CF_FULL, glo[a], o));
-                        ghi[a] = fmaxf(ghi[a], __shfl_xor_sync(CF_FULL, ghi[a], o));
-                    }
-                if (lane < 6u) gbox[6 * (size_t)p0 + lane] = lane < 3u ? glo[lane] : ghi[lane - 3u];
-            }
-            for (int a = 0; a < 3; a++) {
-                lo[a] = fminf(lo[a], glo[a]);
-                hi[a] = fmaxf(hi[a], ghi[a]);
-            }
-        }
-        for (int o = 16; o; o >>= 1)
-            for (int a = 0; a < 3; a++) {
-                lo[a] = fminf(lo[a], __shfl_xor_sync(CF_FULL, lo[a], o));
-                hi[a] = fmaxf(hi[a], __shfl_xor_sync(CF_FULL, hi[a], o));
-            }
-        if (lane < 6u) box[6 * c + lane] = lane < 3u ? lo[lane] : hi[lane - 3u];
-    }
+    for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c < ncell_all; c += wstride)
+        cf_cell_box(cell_start, c, pt, box, gbox);
 }
 
 // The units (job, i cell) whose i cell holds points, in any order, and their number in *nlive
@@ -650,15 +667,14 @@ __global__ void cf_live_units_kernel(const CfDevPlan *__restrict__ plan, const C
 // instead of (job, cell).
 // GP: the instance with group pruning (its group code holds registers the other need not pay for)
 template <bool GP>
-__global__ void __launch_bounds__(256, GP ? 3 : 4)
-    cf_items_kernel(const CfDevPlan *__restrict__ plan, const CfSetDesc *__restrict__ sets,
+__device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan, const CfSetDesc *__restrict__ sets,
                                 const CfJobDesc *__restrict__ jobs, const CfStencil *__restrict__ stencil,
-                                const uint32_t *__restrict__ cell_start, const float *__restrict__ cbox,
-                                const float *__restrict__ gbox, const uint32_t *__restrict__ live,
-                                const uint32_t *__restrict__ nlive, int mode,
-                                uint32_t *__restrict__ counts, const uint32_t *__restrict__ offsets,
-                                CfItem *__restrict__ items, uint32_t items_cap,
-                                unsigned long long *__restrict__ evaluated, unsigned long long *__restrict__ total64)
+                                const uint32_t *cell_start, const float *cbox,
+                                const float *gbox, const uint32_t *live,
+                                const uint32_t *nlive, int mode,
+                                uint32_t *counts, const uint32_t *offsets,
+                                CfItem *items, uint32_t items_cap,
+                                unsigned long long *evaluated, unsigned long long *total64, uint32_t bid, uint32_t nblk)
 {
     const CfGrid &g = plan->g;
     const int nst = g.nstencil;
@@ -678,7 +694,7 @@ __global__ void __launch_bounds__(256, GP ? 3 : 4)
     const int64_t wpb = blockDim.x >> 5, warp = threadIdx.x >> 5;
     // with a list of the units whose i cell holds points, only those (the same count in every thread)
     const int64_t nloop = live ? (int64_t)min(*nlive, (uint32_t)nunit) : nunit;
-    for (int64_t ub = blockIdx.x * wpb; ub < nloop; ub += (int64_t)gridDim.x * wpb) {
+    for (int64_t ub = bid * wpb; ub < nloop; ub += (int64_t)nblk * wpb) {
         if (mode == 2) {
             if (threadIdx.x == 0) s_n = 0;
             __syncthreads();
@@ -961,6 +977,168 @@ __global__ void __launch_bounds__(256, GP ? 3 : 4)
     if (mode == 2 && lane == 0 && nres) atomicAdd(total64, nres);     // nres is the same in every lane
 }
 
+template <bool GP>
+__global__ void __launch_bounds__(256, GP ? 3 : 4)
+    cf_items_kernel(const CfDevPlan *__restrict__ plan, const CfSetDesc *__restrict__ sets,
+                                const CfJobDesc *__restrict__ jobs, const CfStencil *__restrict__ stencil,
+                                const uint32_t *__restrict__ cell_start, const float *__restrict__ cbox,
+                                const float *__restrict__ gbox, const uint32_t *__restrict__ live,
+                                const uint32_t *__restrict__ nlive, int mode,
+                                uint32_t *__restrict__ counts, const uint32_t *__restrict__ offsets,
+                                CfItem *__restrict__ items, uint32_t items_cap,
+                                unsigned long long *__restrict__ evaluated, unsigned long long *__restrict__ total64)
+{
+    cf_items_body<GP>(plan, sets, jobs, stencil, cell_start, cbox, gbox, live, nlive, mode, counts, offsets, items,
+                      items_cap, evaluated, total64, blockIdx.x, gridDim.x);
+}
+
+// ---------------------------------------------------------------------------------------------
+// The whole build in one cooperative launch: one block per SM and a barrier over the grid between the
+// steps (zero the counters, assign, scan, scatter, cell boxes, work list).  Eight separate launches and
+// memsets cost 3 to 5 us each, most of it launch latency, ramp and tail.  The points of all sets are one
+// index range.  Only plain (coherent) loads read what the kernel wrote.
+// ---------------------------------------------------------------------------------------------
+
+// Barrier over the grid (all blocks are resident: cooperative launch).  bar[0] counts arrivals and is back at 0
+// after each barrier, bar[1] counts barriers; both start at 0 once and keep across launches.  A wait is
+// bounded: past the limit the block reports it and goes on to its end (ok = false), and the host
+// fails the call.
+__device__ __forceinline__ bool cf_grid_barrier(uint32_t *bar, uint32_t *late)
+{
+    __shared__ bool s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_ok = true;
+        const uint32_t gen = *(volatile uint32_t *)(bar + 1);
+        __threadfence();
+        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+            *(volatile uint32_t *)bar = 0u;
+            __threadfence();
+            atomicAdd(bar + 1, 1u);
+        } else {
+            uint32_t n = 0;
+            while (*(volatile uint32_t *)(bar + 1) == gen) {
+                if (++n > (1u << 22)) {
+                    atomicExch(late, 1u);
+                    s_ok = false;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+    return s_ok;
+}
+
+__global__ void __launch_bounds__(CFB_ONE_THREADS, 1) cf_one_build_kernel(const CfOneBuild A)
+{
+    const uint32_t rank = blockIdx.x, nct = gridDim.x;
+    const uint32_t tid = rank * blockDim.x + threadIdx.x, nth = nct * blockDim.x;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t ns = (uint32_t)(A.sub * A.sub * A.sub);
+    __shared__ uint32_t s_warp[CFB_ONE_THREADS / 32];
+    // ---- counters ----
+    for (uint32_t i = tid; i < A.nfine; i += nth) A.count[i] = 0u;
+    for (uint32_t i = tid; i < A.zero_words; i += nth) A.zero[i] = 0u;
+    if (!cf_grid_barrier(A.bar, A.late)) return;
+    // the set of point p: the last one that starts at or before it
+    auto set_of = [&](uint32_t p) {
+        int lo = 0, hi = A.nsets - 1;
+        while (lo < hi) {
+            const int m = (lo + hi + 1) >> 1;
+            if (A.sets[m].pbeg <= (int64_t)p) lo = m;
+            else hi = m - 1;
+        }
+        return lo;
+    };
+    // ---- assign ----
+    for (uint32_t p = tid; p < A.npts; p += nth) {
+        const CfSetDesc &S = A.sets[set_of(p)];
+        const uint32_t k = cf_point_key(A.plan, S, (int64_t)p - S.pbeg, A.sub);
+        A.key[p] = k;
+        A.slot[p] = atomicAdd(A.count + k, 1u);
+    }
+    if (!cf_grid_barrier(A.bar, A.late)) return;
+    // ---- scan: each block a contiguous share of the keys; the blocks' totals through global memory ----
+    const uint32_t per = ((A.nfine + nct - 1) / nct + 3u) & ~3u;
+    const uint32_t k0 = min(rank * per, A.nfine), k1 = min(k0 + per, A.nfine);
+    auto block_sum = [&](uint32_t v) {          // the sum over the block, in every thread
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(CF_FULL, v, o);
+        __syncthreads();
+        if (lane == 0) s_warp[warp] = v;
+        __syncthreads();
+        uint32_t t = lane < blockDim.x / 32 ? s_warp[lane] : 0u;
+        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(CF_FULL, t, o);
+        return t;
+    };
+    {
+        uint32_t v = 0;
+        for (uint32_t i = k0 + threadIdx.x; i < k1; i += blockDim.x) v += A.count[i];
+        v = block_sum(v);
+        if (threadIdx.x == 0) A.part[rank] = v;
+    }
+    if (!cf_grid_barrier(A.bar, A.late)) return;
+    uint32_t carry = 0;
+    for (uint32_t r = threadIdx.x; r < rank; r += blockDim.x) carry += A.part[r];
+    carry = block_sum(carry);
+    const uint32_t cmask = ns - 1u;
+    const int cshift = 31 - __clz(ns);
+    for (uint32_t b0 = k0; b0 < k1; b0 += 4u * blockDim.x) {
+        // four consecutive keys per thread
+        const uint32_t i = b0 + 4u * threadIdx.x;
+        uint32_t v[4], sum = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            v[q] = i + q < k1 ? A.count[i + q] : 0u;
+            sum += v[q];
+        }
+        uint32_t x = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(CF_FULL, x, o);
+            if ((int)lane >= o) x += t;
+        }
+        __syncthreads();
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        uint32_t w = lane < blockDim.x / 32 ? s_warp[lane] : 0u, wi = w;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(CF_FULL, wi, o);
+            if ((int)lane >= o) wi += t;
+        }
+        uint32_t pre = carry + __shfl_sync(CF_FULL, wi - w, warp) + x - sum;
+        carry += __shfl_sync(CF_FULL, wi, 31);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (i + q >= k1) break;
+            A.fstart[i + q] = pre;
+            if (((i + q) & cmask) == 0u) A.cell_start[(i + q) >> cshift] = pre;
+            pre += v[q];
+        }
+    }
+    if (tid == 0) {
+        A.fstart[A.nfine] = A.npts;
+        A.cell_start[A.nfine >> cshift] = A.npts;
+    }
+    if (!cf_grid_barrier(A.bar, A.late)) return;
+    // ---- scatter ----
+    for (uint32_t p = tid; p < A.npts; p += nth) {
+        const CfSetDesc &S = A.sets[set_of(p)];
+        const uint32_t k = A.key[p];
+        cf_scatter_point(A.plan, S, (int64_t)p - S.pbeg, k, ns, (int64_t)A.fstart[k] + A.slot[p], A.pt, A.pabs, A.plo,
+                         A.pabslo, A.orig);
+    }
+    if (!cf_grid_barrier(A.bar, A.late)) return;
+    // ---- cell boxes ----
+    if (A.cbox) {
+        for (uint32_t c = tid >> 5; c < (A.nfine >> cshift); c += nth >> 5) cf_cell_box(A.cell_start, c, A.pt, A.cbox, nullptr);
+        if (!cf_grid_barrier(A.bar, A.late)) return;
+    }
+    // ---- work list ----
+    cf_items_body<false>(A.plan, A.sets, A.jobs, A.stencil, A.cell_start, A.cbox, nullptr, nullptr, nullptr, 2, A.nitems,
+                         nullptr, A.items, A.items_cap, A.evaluated, A.total64, rank, nct);
+}
+
 // sum of w^2 per set (self pairs of a weighted auto-correlation whose first edge is 0)
 __global__ void cf_wsq_kernel(const CfSetDesc *__restrict__ sets, double *__restrict__ out)
 {
@@ -1073,6 +1251,24 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
         cf_items_kernel<false><<<nb, 256, 0, st>>>(plan, sets, jobs, stencil, cell_start, cbox, nullptr, live, nlive,
                                                    mode, counts, offsets, items, items_cap, evaluated, total64);
     return cudaGetLastError();
+}
+
+int cfb_one_init(int num_sms)
+{
+    int per_sm = 0, coop = 0, dev = 0;
+    cudaGetDevice(&dev);
+    const bool ok = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cf_one_build_kernel, CFB_ONE_THREADS, 0) ==
+                        cudaSuccess && per_sm >= 1;
+    cudaGetLastError();
+    return ok ? num_sms : 0;
+}
+
+cudaError_t cfb_one_build(const CfOneBuild &A, int blocks, cudaStream_t st)
+{
+    CfOneBuild arg = A;
+    void *args[1] = {&arg};
+    return cudaLaunchCooperativeKernel((const void *)cf_one_build_kernel, dim3(blocks), dim3(CFB_ONE_THREADS), args, 0, st);
 }
 
 cudaError_t cfb_wsq(const CfSetDesc *sets, int nsets, int64_t nmax, double *out, cudaStream_t st)

@@ -47,6 +47,32 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
                       const uint32_t *nlive, int64_t nunits, int mode, uint32_t *counts, const uint32_t *offsets,
                       CfItem *items, uint32_t items_cap, unsigned long long *evaluated, unsigned long long *total64,
                       cudaStream_t st);
+// The whole build, from zeroing the call's counters to the work list, in one cooperative launch of one block
+// per SM: see cf_one_build_kernel.  3-D grids without group pruning only.
+#define CFB_ONE_THREADS 512
+struct CfOneBuild {
+    const CfDevPlan *plan;
+    const CfSetDesc *sets;
+    const CfJobDesc *jobs;
+    const CfStencil *stencil;
+    int nsets, sub;
+    uint32_t npts, nfine;
+    uint32_t *zero;              // counters and histograms of the call
+    uint32_t zero_words;
+    uint32_t *bar;               // the grid barrier's two words (0 before the first launch)
+    uint32_t *late;              // set when a barrier was given up
+    uint32_t *part;              // one word per block
+    uint32_t *count, *key, *slot, *fstart, *cell_start, *orig;
+    float4 *pt, *pabs, *plo, *pabslo;
+    float *cbox;                 // NULL: no boxes, every stencil neighbour is visited
+    CfItem *items;
+    uint32_t items_cap;
+    uint32_t *nitems;
+    unsigned long long *evaluated, *total64;
+};
+// once per context, on its device: blocks of the launch (0: the device does not take it)
+int cfb_one_init(int num_sms);
+cudaError_t cfb_one_build(const CfOneBuild &A, int blocks, cudaStream_t st);
 cudaError_t cfb_wsq(const CfSetDesc *sets, int nsets, int64_t nmax, double *out, cudaStream_t st);
 
 // ---- pair counting ----
@@ -115,4 +141,5 @@ cudaError_t cfp_launch_audit(const CfItem *items, const uint32_t *nitems_dev, ui
                              cudaStream_t st);
 cudaError_t cfp_launch_recheck(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobDesc *jobs,
                                const uint4 *queue, const unsigned long long *qcount, uint32_t qcap,
-                               unsigned long long *hcnt, double *hw, double *hr, int num_sms, cudaStream_t st);
+                               unsigned long long *hcnt, double *hw, double *hr, const uint32_t *late, uint32_t *flag,
+                               int num_sms, cudaStream_t st);

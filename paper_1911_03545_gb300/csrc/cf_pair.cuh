@@ -754,7 +754,8 @@ __global__ void __launch_bounds__(pair_max_threads(W, R), pair_min_blocks(W, R))
         w.h_wd = w.h_rd = nullptr;
     }
 
-    const uint32_t nitems = min(*a.nitems_dev, a.items_cap);
+    // a list that was cut off is made again: nothing to count then
+    const uint32_t nitems = *a.nitems_dev <= a.items_cap ? *a.nitems_dev : 0u;
     int cur = -1;
     // pairs evaluated since the last flush: a warp flushes at the latest every 2^28 (an item holds
     // at most 128 x 512 = 2^16), so no 32-bit count and no fixed-point sum it holds can overflow

@@ -32,8 +32,10 @@ __global__ void cf_recheck_kernel(const CfDevPlan *__restrict__ P, const CfSetDe
                                   const CfJobDesc *__restrict__ jobs, const uint4 *__restrict__ queue,
                                   const unsigned long long *__restrict__ qcount, uint32_t qcap,
                                   unsigned long long *__restrict__ hcnt, double *__restrict__ hw,
-                                  double *__restrict__ hr)
+                                  double *__restrict__ hr, const uint32_t *__restrict__ late, uint32_t *flag)
 {
+    // a build that gave up at a barrier: into the words the host reads back
+    if (late && blockIdx.x == 0 && threadIdx.x == 0 && *late) *flag = 1u;
     const uint32_t n = (uint32_t)min(*qcount, (unsigned long long)qcap);
     const int kind = P->kind, nb = P->nb, npi = P->npi, nslot = P->nslot;
     const double L0 = P->g.periodic ? P->g.L[0] : 0.0;
@@ -132,9 +134,10 @@ cudaError_t cfp_launch_audit(const CfItem *items, const uint32_t *nitems_dev, ui
 
 cudaError_t cfp_launch_recheck(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobDesc *jobs,
                                const uint4 *queue, const unsigned long long *qcount, uint32_t qcap,
-                               unsigned long long *hcnt, double *hw, double *hr, int num_sms, cudaStream_t st)
+                               unsigned long long *hcnt, double *hw, double *hr, const uint32_t *late, uint32_t *flag,
+                               int num_sms, cudaStream_t st)
 {
-    cf_recheck_kernel<<<num_sms * 2, 256, 0, st>>>(plan, sets, jobs, queue, qcount, qcap, hcnt, hw, hr);
+    cf_recheck_kernel<<<num_sms * 2, 256, 0, st>>>(plan, sets, jobs, queue, qcount, qcap, hcnt, hw, hr, late, flag);
     return cudaGetLastError();
 }
 
