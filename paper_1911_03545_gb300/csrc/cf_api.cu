@@ -483,16 +483,6 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     R.ncell_all = R.ncell * nsets;
     if (R.ncell_all >= ((int64_t)1 << 31)) return C->fail(CF_ERR_ARG, "too many cells");
     R.nst = D.g.nstencil;
-    // points sort by (cell, Morton sub-cell): the finest order whose key array stays within about
-    // twice the points (and 1M keys)
-    {
-        const int64_t want = C->opt[CF_OPT_CELL_ORDER];
-        const int64_t lim = std::max<int64_t>(2 * R.npts, (int64_t)1 << 20);
-        if (want == 1 || want == 2 || want == 4) R.sub = (int)want;
-        else R.sub = R.ncell_all * 64 <= lim ? 4 : (R.ncell_all * 8 <= lim ? 2 : 1);
-        R.nfine = R.ncell_all * R.sub * R.sub * R.sub;
-        if (R.nfine >= ((int64_t)1 << 31)) return C->fail(CF_ERR_ARG, "too many cells");
-    }
     R.nunit = (int64_t)njobs * R.ncell;      // work-list units: one per (job, i cell)
     if (R.nunit >= ((int64_t)1 << 31)) return C->fail(CF_ERR_ARG, "work list too large");
     R.np = std::max<int64_t>(R.npts, 1);
@@ -500,6 +490,21 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     // so that the work-list pass does not spend a warp iteration on each empty cell
     R.live_units = R.nunit >= 65536 && R.nunit > R.npts;
     R.one_build = !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
+    // points sort by (cell, Morton sub-cell): the finest order whose key array stays within about
+    // twice the points (and 1M keys).  The one-launch build scans the keys in shared memory, so it takes fewer:
+    // sub-cells of 1/8 or a whole cell in place of 1/64 there cost the pair kernel 1 % at 200k points and
+    // nothing measurable below.
+    {
+        const int64_t want = C->opt[CF_OPT_CELL_ORDER];
+        const int64_t lim = R.one_build && R.ncell_all <= CFB_ONE_KEYS
+                                ? std::min<int64_t>(std::max<int64_t>(2 * R.npts, 16384), CFB_ONE_KEYS)
+                                : std::max<int64_t>(2 * R.npts, (int64_t)1 << 20);
+        if (want == 1 || want == 2 || want == 4) R.sub = (int)want;
+        else R.sub = R.ncell_all * 64 <= lim ? 4 : (R.ncell_all * 8 <= lim ? 2 : 1);
+        R.nfine = R.ncell_all * R.sub * R.sub * R.sub;
+        if (R.nfine >= ((int64_t)1 << 31)) return C->fail(CF_ERR_ARG, "too many cells");
+    }
+    R.one_build = R.one_build && R.nfine <= CFB_ONE_KEYS;
     if (R.one_build && C->one_blocks < 0) {
         CF_TRY(C->ensure(B_BAR, 64));
         CF_CU(cudaMemsetAsync(C->buf[B_BAR].p, 0, 64, st), "memset barrier");
@@ -540,6 +545,12 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         D.origin32 = R.d_origin32;
     }
     CF_TRY(C->ensure(B_CNT, 4 * (size_t)(R.nfine + 1)));
+    if (R.one_build) {
+        // the one-launch build's own key counts: zero before and after each of its launches
+        const uint64_t g = C->gen;
+        CF_TRY(C->ensure(B_ONECNT, 4 * (((size_t)R.nfine + 3) & ~(size_t)3)));
+        if (C->gen != g) C->one_clean = false;
+    }
     CF_TRY(C->ensure(B_FSTART, 4 * (size_t)(R.nfine + 1)));
     CF_TRY(C->ensure(B_CSTART, 4 * (size_t)(R.ncell_all + 1)));
     CF_TRY(C->ensure(B_CELLID, 4 * (size_t)R.np));
@@ -650,11 +661,9 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
         S.zero_words = (uint32_t)(readback_bytes(R) / 4);
         S.bar = (uint32_t *)C->buf[B_BAR].p;
         S.late = S.bar + 2;
-        S.part = (uint32_t *)C->buf[B_SCAN].p;
-        S.count = cnt;
+        S.count = (uint32_t *)C->buf[B_ONECNT].p;
         S.key = (uint32_t *)C->buf[B_CELLID].p;
         S.slot = (uint32_t *)C->buf[B_SLOT].p;
-        S.fstart = fstart;
         S.cell_start = cstart;
         S.orig = (uint32_t *)C->buf[B_ORIG].p;
         S.pt = (float4 *)C->buf[B_PT].p;
@@ -667,6 +676,9 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
         S.nitems = (uint32_t *)(out + OUT_NITEMS);
         S.evaluated = (unsigned long long *)(out + OUT_EVAL);
         S.total64 = (unsigned long long *)(out + OUT_ITEMS64);
+        // a new buffer, or one that a launch may have left half done
+        if (!C->one_clean) CF_CU(cudaMemsetAsync(S.count, 0, C->buf[B_ONECNT].cap, st), "memset counts");
+        if (!C->capturing) C->one_clean = true;
         CF_CU(cfb_one_build(S, C->one_blocks, st), "build");
         R.cbox = S.cbox;
         R.gbox = nullptr;
@@ -915,7 +927,8 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
     const uint32_t nitems = *(const uint32_t *)(h + OUT_NITEMS);
     *retry = 0;
     if (*(const uint32_t *)(h + OUT_LATE)) {
-        C->one_blocks = -1;         // start the barrier afresh
+        C->one_blocks = -1;         // start the barrier and the key counts afresh
+        C->one_clean = false;
         return C->fail(CF_ERR_TIMEOUT, "the build gave up waiting at a barrier");
     }
     // work items and queue entries are indexed in 32 bits, with headroom for the grid-stride

@@ -12,7 +12,7 @@
 enum CfBuf {
     B_IN, B_SETS, B_BBOX, B_PLAN, B_LUT, B_FINE, B_STENCIL, B_JOBS, B_CNT, B_CSTART, B_CELLID, B_SLOT,
     B_PT, B_PABS, B_PLO, B_PABSLO, B_ORIG, B_SCAN, B_ICNT, B_IOFF, B_ITEMS, B_HCNT, B_HW, B_HR, B_QUEUE, B_WSQ, B_MISC, B_ORIGIN,
-    B_CBOX, B_FSTART, B_BANDS, B_ORIGIN32, B_OUT, B_PLANBLK, B_GBOX, B_LIVE, B_BAR, B_COUNT_
+    B_CBOX, B_FSTART, B_BANDS, B_ORIGIN32, B_OUT, B_PLANBLK, B_GBOX, B_LIVE, B_BAR, B_ONECNT, B_COUNT_
 };
 
 // B_OUT: the counters and histograms one call reads back, laid out as the host copy of them (one
@@ -130,6 +130,7 @@ struct CfCtx {
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     CfRun run;
     int last_grid = 0, last_warps = 0;
+    bool one_clean = false;        // the one-launch build's key counts are zero
     int one_blocks = -1;           // blocks of the one-launch build (0: not taken, -1: not asked yet)
     int launches = 0;              // kernels launched by the current call
     uint64_t gen = 0;              // bumped whenever device or pinned scratch is reallocated

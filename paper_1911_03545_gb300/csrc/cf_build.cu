@@ -993,10 +993,16 @@ __global__ void __launch_bounds__(256, GP ? 3 : 4)
 }
 
 // ---------------------------------------------------------------------------------------------
-// The whole build in one cooperative launch: one block per SM and a barrier over the grid between the
-// steps (zero the counters, assign, scan, scatter, cell boxes, work list).  Eight separate launches and
-// memsets cost 3 to 5 us each, most of it launch latency, ramp and tail.  The points of all sets are one
-// index range.  Only plain (coherent) loads read what the kernel wrote.
+// The whole build in one cooperative launch: one block per SM and three barriers over the grid between the
+// steps.  Eight separate launches and memsets cost 3 to 5 us each, most of it launch latency, ramp and
+// tail, and a barrier about 3 us, so the steps are few:
+//   assign: the points' keys and ranks; the call's counters to zero;
+//   scatter: every block scans all key counts for itself in shared memory (at most CFB_ONE_KEYS), so no
+//     barrier orders a scan;
+//   the cells' boxes, and the key counts back to zero for the next launch (boxes by atomic minima and maxima
+//     of the points in the scatter step would save a barrier, but cost more: 16 us more at 260k points);
+//   the work list.
+// The points of all sets are one index range.  Only plain (coherent) loads read what the kernel wrote.
 // ---------------------------------------------------------------------------------------------
 
 // Barrier over the grid (all blocks are resident: cooperative launch).  bar[0] counts arrivals and is back at 0
@@ -1033,15 +1039,13 @@ __device__ __forceinline__ bool cf_grid_barrier(uint32_t *bar, uint32_t *late)
 
 __global__ void __launch_bounds__(CFB_ONE_THREADS, 1) cf_one_build_kernel(const CfOneBuild A)
 {
+    extern __shared__ __align__(16) uint32_t s_start[];       // first place of each key
+    __shared__ uint32_t s_warp[CFB_ONE_THREADS / 32];
     const uint32_t rank = blockIdx.x, nct = gridDim.x;
     const uint32_t tid = rank * blockDim.x + threadIdx.x, nth = nct * blockDim.x;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t ns = (uint32_t)(A.sub * A.sub * A.sub);
-    __shared__ uint32_t s_warp[CFB_ONE_THREADS / 32];
-    // ---- counters ----
-    for (uint32_t i = tid; i < A.nfine; i += nth) A.count[i] = 0u;
-    for (uint32_t i = tid; i < A.zero_words; i += nth) A.zero[i] = 0u;
-    if (!cf_grid_barrier(A.bar, A.late)) return;
+    const uint32_t cshift = 31u - __clz(ns), ncell = A.nfine >> cshift;
     // the set of point p: the last one that starts at or before it
     auto set_of = [&](uint32_t p) {
         int lo = 0, hi = A.nsets - 1;
@@ -1059,84 +1063,61 @@ __global__ void __launch_bounds__(CFB_ONE_THREADS, 1) cf_one_build_kernel(const 
         A.key[p] = k;
         A.slot[p] = atomicAdd(A.count + k, 1u);
     }
+    for (uint32_t i = tid; i < A.zero_words; i += nth) A.zero[i] = 0u;
     if (!cf_grid_barrier(A.bar, A.late)) return;
-    // ---- scan: each block a contiguous share of the keys; the blocks' totals through global memory ----
-    const uint32_t per = ((A.nfine + nct - 1) / nct + 3u) & ~3u;
-    const uint32_t k0 = min(rank * per, A.nfine), k1 = min(k0 + per, A.nfine);
-    auto block_sum = [&](uint32_t v) {          // the sum over the block, in every thread
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(CF_FULL, v, o);
-        __syncthreads();
-        if (lane == 0) s_warp[warp] = v;
-        __syncthreads();
-        uint32_t t = lane < blockDim.x / 32 ? s_warp[lane] : 0u;
-        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(CF_FULL, t, o);
-        return t;
-    };
-    {
-        uint32_t v = 0;
-        for (uint32_t i = k0 + threadIdx.x; i < k1; i += blockDim.x) v += A.count[i];
-        v = block_sum(v);
-        if (threadIdx.x == 0) A.part[rank] = v;
+    // ---- scan: each thread a run of keys, of an odd number of 16-byte words (no bank conflicts) ----
+    const uint32_t nw = (A.nfine + 3u) >> 2;            // words of four keys; the last keys past nfine count zero
+    uint4 *const sw = reinterpret_cast<uint4 *>(s_start);
+    for (uint32_t i = threadIdx.x; i < nw; i += blockDim.x) sw[i] = reinterpret_cast<const uint4 *>(A.count)[i];
+    __syncthreads();
+    const uint32_t per = ((nw + blockDim.x - 1) / blockDim.x) | 1u;
+    const uint32_t k0 = min(threadIdx.x * per, nw), k1 = min(k0 + per, nw);
+    uint32_t sum = 0;
+    for (uint32_t i = k0; i < k1; i++) {
+        const uint4 v = sw[i];
+        sum += v.x + v.y + v.z + v.w;
     }
-    if (!cf_grid_barrier(A.bar, A.late)) return;
-    uint32_t carry = 0;
-    for (uint32_t r = threadIdx.x; r < rank; r += blockDim.x) carry += A.part[r];
-    carry = block_sum(carry);
-    const uint32_t cmask = ns - 1u;
-    const int cshift = 31 - __clz(ns);
-    for (uint32_t b0 = k0; b0 < k1; b0 += 4u * blockDim.x) {
-        // four consecutive keys per thread
-        const uint32_t i = b0 + 4u * threadIdx.x;
-        uint32_t v[4], sum = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            v[q] = i + q < k1 ? A.count[i + q] : 0u;
-            sum += v[q];
-        }
-        uint32_t x = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(CF_FULL, x, o);
-            if ((int)lane >= o) x += t;
-        }
-        __syncthreads();
-        if (lane == 31) s_warp[warp] = x;
-        __syncthreads();
-        uint32_t w = lane < blockDim.x / 32 ? s_warp[lane] : 0u, wi = w;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(CF_FULL, wi, o);
-            if ((int)lane >= o) wi += t;
-        }
-        uint32_t pre = carry + __shfl_sync(CF_FULL, wi - w, warp) + x - sum;
-        carry += __shfl_sync(CF_FULL, wi, 31);
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (i + q >= k1) break;
-            A.fstart[i + q] = pre;
-            if (((i + q) & cmask) == 0u) A.cell_start[(i + q) >> cshift] = pre;
-            pre += v[q];
-        }
+    uint32_t x = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(CF_FULL, x, o);
+        if ((int)lane >= o) x += t;
     }
-    if (tid == 0) {
-        A.fstart[A.nfine] = A.npts;
-        A.cell_start[A.nfine >> cshift] = A.npts;
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    uint32_t w = lane < blockDim.x / 32 ? s_warp[lane] : 0u;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(CF_FULL, w, o);
+        if ((int)lane >= o) w += t;
     }
-    if (!cf_grid_barrier(A.bar, A.late)) return;
+    uint32_t pre = x - sum;
+    w = __shfl_sync(CF_FULL, w, warp ? warp - 1 : 0);
+    if (warp) pre += w;
+    for (uint32_t i = k0; i < k1; i++) {
+        const uint4 v = sw[i];
+        const uint4 r = make_uint4(pre, pre + v.x, pre + v.x + v.y, pre + v.x + v.y + v.z);
+        sw[i] = r;
+        pre = r.w + v.w;
+    }
+    __syncthreads();
+    for (uint32_t c = tid; c < ncell; c += nth) A.cell_start[c] = s_start[c << cshift];
+    if (tid == 0) A.cell_start[ncell] = A.npts;
     // ---- scatter ----
     for (uint32_t p = tid; p < A.npts; p += nth) {
         const CfSetDesc &S = A.sets[set_of(p)];
         const uint32_t k = A.key[p];
-        cf_scatter_point(A.plan, S, (int64_t)p - S.pbeg, k, ns, (int64_t)A.fstart[k] + A.slot[p], A.pt, A.pabs, A.plo,
+        cf_scatter_point(A.plan, S, (int64_t)p - S.pbeg, k, ns, (int64_t)s_start[k] + A.slot[p], A.pt, A.pabs, A.plo,
                          A.pabslo, A.orig);
     }
     if (!cf_grid_barrier(A.bar, A.late)) return;
     // ---- cell boxes ----
+    for (uint32_t i = tid; i < A.nfine; i += nth) A.count[i] = 0u;
     if (A.cbox) {
-        for (uint32_t c = tid >> 5; c < (A.nfine >> cshift); c += nth >> 5) cf_cell_box(A.cell_start, c, A.pt, A.cbox, nullptr);
+        for (uint32_t c = warp * nct + rank; c < ncell; c += nth >> 5) cf_cell_box(A.cell_start, c, A.pt, A.cbox, nullptr);
         if (!cf_grid_barrier(A.bar, A.late)) return;
     }
     // ---- work list ----
-    cf_items_body<false>(A.plan, A.sets, A.jobs, A.stencil, A.cell_start, A.cbox, nullptr, nullptr, nullptr, 2, A.nitems,
-                         nullptr, A.items, A.items_cap, A.evaluated, A.total64, rank, nct);
+    cf_items_body<false>(A.plan, A.sets, A.jobs, A.stencil, A.cell_start, A.cbox, nullptr,
+                         nullptr, nullptr, 2, A.nitems, nullptr, A.items, A.items_cap, A.evaluated, A.total64, rank, nct);
 }
 
 // sum of w^2 per set (self pairs of a weighted auto-correlation whose first edge is 0)
@@ -1257,8 +1238,11 @@ int cfb_one_init(int num_sms)
 {
     int per_sm = 0, coop = 0, dev = 0;
     cudaGetDevice(&dev);
+    const int smem = 4 * CFB_ONE_KEYS;
     const bool ok = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cf_one_build_kernel, CFB_ONE_THREADS, 0) ==
+                    cudaFuncSetAttribute(cf_one_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+                        cudaSuccess &&
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cf_one_build_kernel, CFB_ONE_THREADS, smem) ==
                         cudaSuccess && per_sm >= 1;
     cudaGetLastError();
     return ok ? num_sms : 0;
@@ -1268,7 +1252,8 @@ cudaError_t cfb_one_build(const CfOneBuild &A, int blocks, cudaStream_t st)
 {
     CfOneBuild arg = A;
     void *args[1] = {&arg};
-    return cudaLaunchCooperativeKernel((const void *)cf_one_build_kernel, dim3(blocks), dim3(CFB_ONE_THREADS), args, 0, st);
+    return cudaLaunchCooperativeKernel((const void *)cf_one_build_kernel, dim3(blocks), dim3(CFB_ONE_THREADS), args,
+                                       4 * (((size_t)A.nfine + 3) & ~(size_t)3), st);
 }
 
 cudaError_t cfb_wsq(const CfSetDesc *sets, int nsets, int64_t nmax, double *out, cudaStream_t st)

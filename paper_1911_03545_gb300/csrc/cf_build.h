@@ -50,6 +50,7 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
 // The whole build, from zeroing the call's counters to the work list, in one cooperative launch of one block
 // per SM: see cf_one_build_kernel.  3-D grids without group pruning only.
 #define CFB_ONE_THREADS 512
+#define CFB_ONE_KEYS 49152         // sort keys at most (192 KB of shared memory, beside the 25 KB item stage)
 struct CfOneBuild {
     const CfDevPlan *plan;
     const CfSetDesc *sets;
@@ -61,8 +62,8 @@ struct CfOneBuild {
     uint32_t zero_words;
     uint32_t *bar;               // the grid barrier's two words (0 before the first launch)
     uint32_t *late;              // set when a barrier was given up
-    uint32_t *part;              // one word per block
-    uint32_t *count, *key, *slot, *fstart, *cell_start, *orig;
+    uint32_t *count;             // nfine key counts (a multiple of four of them is read): 0 before the launch, and after it
+    uint32_t *key, *slot, *cell_start, *orig;
     float4 *pt, *pabs, *plo, *pabslo;
     float *cbox;                 // NULL: no boxes, every stencil neighbour is visited
     CfItem *items;
