@@ -490,7 +490,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     // so that the work-list pass does not spend a warp iteration on each empty cell
     R.live_units = R.nunit >= 65536 && R.nunit > R.npts;
     R.one_build = !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
-    // points sort by (cell, Morton sub-cell): the finest order whose key array stays within about
+    // points sort by (cell, sub-cell): the finest order whose key array stays within about
     // twice the points (and 1M keys).  The one-launch build scans the keys in shared memory, so it takes fewer:
     // sub-cells of 1/8 or a whole cell in place of 1/64 there cost the pair kernel 1 % at 200k points and
     // nothing measurable below.

@@ -69,7 +69,7 @@ struct CfRun {
     int64_t npts = 0, nmax = 0, np = 1, ncell = 0, ncell_all = 0, nst = 0, nunit = 0;
     const float *cbox = nullptr;   // cell boxes for pruning (nullptr: every stencil neighbour)
     const float *gbox = nullptr;   // 32-point group boxes for pruning inside cell pairs (or nullptr)
-    int sub = 1;                   // Morton sub-cells per axis inside a cell (1, 2, 4)
+    int sub = 1;                   // sub-cells per axis inside a cell (1, 2, 4)
     int64_t nfine = 0;             // ncell_all * sub^3 counting-sort keys
     size_t nslot = 0, hsz = 0;
     bool self_pairs = false;
