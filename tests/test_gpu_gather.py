@@ -56,3 +56,10 @@ def test_gathered_blocks(ctx, kind, n):
             got = gpu_count(ctx, kind, edges, d1, None if auto else d2, autocorr=auto, **kw)
             exp = oracle_count(kind, edges, d1, None if auto else d2, autocorr=auto, mode="brute", **kw)
             assert_match(got, exp, sums, sums)
+
+
+@pytest.mark.parametrize("n", [2, 8, 9, 16, 17, 24, 36, 40, 48])
+@pytest.mark.parametrize("kind", ["r", "rppi", "wp", "theta", "mocks"])
+def test_groups_that_share_the_warp(ctx, kind, n):
+    """Last groups of up to 4, 8 and 16 points, which have several lanes per point."""
+    test_gathered_blocks(ctx, kind, n)
