@@ -1,0 +1,32 @@
+"""The work list of cell pairs of many items: every tile pair of a cell with itself (the triangle) and with
+another cell exactly once, at the edges of tiles and ranges and with the smallest of both."""
+import numpy as np
+import pytest
+
+import gen
+from tests.gpu_util import gpu_count
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [32, 33, 64, 65, 97, 1000, 4097, 30_001])
+def test_every_pair_of_a_cell_once(n):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        a, b = gen.uniform_box(n, 1.0, 1, np.float32), gen.uniform_box(n // 3 + 1, 1.0, 2, np.float32)
+        edges = [0.0, 1.0, 2.0]          # every pair of the unit box counts
+        for tile, jchunk in ((0, 0), (32, 32), (64, 128)):
+            cf.cf_set_option(ctx, cf.CF_OPT_TILE, tile)
+            cf.cf_set_option(ctx, cf.CF_OPT_JCHUNK, jchunk)
+            for refine in (1, 2):
+                kw = dict(periodic=False, refine=(refine,) * 3)
+                auto = gpu_count(ctx, "r", edges, a, autocorr=True, **kw)
+                assert int(np.asarray(auto["npairs"]).astype(np.uint64).sum()) == n * n       # the points themselves too
+                cross = gpu_count(ctx, "r", edges, a, b, autocorr=False, **kw)
+                assert int(np.asarray(cross["npairs"]).astype(np.uint64).sum()) == n * (n // 3 + 1)
+    finally:
+        cf.cf_destroy(ctx)
