@@ -558,7 +558,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     const bool mocks = p->kind == CF_DD_RPPI_MOCKS;
     CF_TRY(C->ensure(B_PT, 16 * (size_t)R.np));
     if (mocks) CF_TRY(C->ensure(B_PABS, 16 * (size_t)R.np));
-    CF_TRY(C->ensure(B_ORIG, 4 * (size_t)R.np));
+    if (D.weighted) CF_TRY(C->ensure(B_ORIG, 4 * (size_t)R.np));      // else in the points' fourth word
     CF_TRY(C->ensure(B_CBOX, 24 * (size_t)R.ncell_all));
     if (C->opt[CF_OPT_CELL_PRUNE] == 0 && C->opt[CF_OPT_BLOCK_PRUNE] == 1) CF_TRY(C->ensure(B_GBOX, 24 * (size_t)R.np));
     if (D.f64lo) CF_TRY(C->ensure(B_PLO, 16 * (size_t)R.np));
@@ -665,7 +665,7 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
         S.key = (uint32_t *)C->buf[B_CELLID].p;
         S.slot = (uint32_t *)C->buf[B_SLOT].p;
         S.cell_start = cstart;
-        S.orig = (uint32_t *)C->buf[B_ORIG].p;
+        S.orig = R.plan.d.weighted ? (uint32_t *)C->buf[B_ORIG].p : nullptr;
         S.pt = (float4 *)C->buf[B_PT].p;
         S.pabs = (float4 *)C->buf[B_PABS].p;
         S.plo = (float4 *)C->buf[B_PLO].p;
@@ -702,7 +702,8 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
           "scan cells");
     CF_CU(cfb_scatter(dplan, dsets, R.nsets, R.np, R.sub, fstart, (uint32_t *)C->buf[B_CELLID].p,
                       (uint32_t *)C->buf[B_SLOT].p, (float4 *)C->buf[B_PT].p, (float4 *)C->buf[B_PABS].p,
-                      (float4 *)C->buf[B_PLO].p, (float4 *)C->buf[B_PABSLO].p, (uint32_t *)C->buf[B_ORIG].p, st),
+                      (float4 *)C->buf[B_PLO].p, (float4 *)C->buf[B_PABSLO].p,
+                      R.plan.d.weighted ? (uint32_t *)C->buf[B_ORIG].p : nullptr, st),
           "scatter");
     const float *cbox = nullptr;
     float *gbox = nullptr;
@@ -853,7 +854,7 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     A.pabs = (const float4 *)C->buf[B_PABS].p;
     A.plo = (const float4 *)C->buf[B_PLO].p;
     A.pabslo = (const float4 *)C->buf[B_PABSLO].p;
-    A.orig = (const uint32_t *)C->buf[B_ORIG].p;
+    A.orig = R.plan.d.weighted ? (const uint32_t *)C->buf[B_ORIG].p : nullptr;
     A.hcnt = hcnt;
     A.hw = hw;
     A.hr = hr;
@@ -889,7 +890,7 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     if (per_warp && !A.ghist && !C->capturing) fixed_point_scales(R, D.weighted != 0, R.cfg.ravg != 0, A);
     int grid = 0, warps = 0;
     if (R.items_cap > 0 && C->opt[CF_OPT_AUDIT]) {
-        CF_CU(cfp_launch_audit(A.items, A.nitems_dev, A.items_cap, A.orig, A.queue, A.qcount, A.qcap, C->num_sms,
+        CF_CU(cfp_launch_audit(A.items, A.nitems_dev, A.items_cap, A.orig, A.pt, A.queue, A.qcount, A.qcap, C->num_sms,
                                st), "audit");
     } else if (R.items_cap > 0) {
         cudaError_t e = cfp_launch_pair(R.cfg, A, C->num_sms, st, &grid, &warps);

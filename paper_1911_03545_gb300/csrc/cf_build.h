@@ -89,7 +89,7 @@ struct CfPairArgs {
     const float4 *pt;            // (-X, -Y, -Z, w)
     const float4 *pabs;          // mocks: absolute positions
     const float4 *plo, *pabslo;  // low parts (float64 inputs with ravg)
-    const uint32_t *orig;
+    const uint32_t *orig;        // NULL without weights: the index is in pt's fourth word
     unsigned long long *hcnt;    // [njobs][nslot]
     double *hw;                  // [njobs][nslot]
     double *hr;                  // [njobs][nslot]
@@ -137,7 +137,8 @@ cudaError_t cfp_launch_pair(const CfPairCfg &c, const CfPairArgs &a, int num_sms
 // CF_OPT_AUDIT: queue every pair of every work item for the FP64 recheck (launched instead of the
 // pair kernel).
 cudaError_t cfp_launch_audit(const CfItem *items, const uint32_t *nitems_dev, uint32_t items_cap,
-                             const uint32_t *orig, uint4 *queue, unsigned long long *qcount, uint32_t qcap, int num_sms,
+                             const uint32_t *orig, const float4 *pt, uint4 *queue, unsigned long long *qcount, uint32_t qcap,
+                             int num_sms,
                              cudaStream_t st);
 cudaError_t cfp_launch_recheck(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobDesc *jobs,
                                const uint4 *queue, const unsigned long long *qcount, uint32_t qcap,

@@ -83,6 +83,11 @@ __device__ __forceinline__ float f_sqrt_approx(float x)
 }
 
 // ---- cell origin: precomputed on the host (cfp_origin in cf_plan.cpp) ----
+// index in its input arrays of sorted point p
+__device__ __forceinline__ uint32_t cf_orig(const uint32_t *orig, const float4 *pt, uint32_t p)
+{
+    return orig ? orig[p] : __float_as_uint(pt[p].w);
+}
 __device__ __forceinline__ double cf_origin(const CfDevPlan *plan, int a, int i) { return plan->origin[plan->ooff[a] + i]; }
 // origin of cell c on axis a: the 3-D grid's per-axis table (index ia), or the angular grid's per-cell one
 __device__ __forceinline__ double cf_cell_origin(const CfDevPlan *plan, int a, int c, int ia)

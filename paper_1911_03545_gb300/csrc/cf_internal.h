@@ -10,7 +10,7 @@
 //     pabs[p] = float4(x, y, z, 0), the absolute position rounded to float32
 //   and for float64 inputs with ravg the low parts: x - o = X + Xlo, x = float(x) + xlo
 //     plo[p] = float4(-Xlo, -Ylo, -Zlo, 0), pabslo[p] = float4(xlo, ylo, zlo, 0) (mocks)
-//     orig[p] = index of the point in its input arrays
+//     orig[p] = index of the point in its input arrays (without weights kept in pt[p].w)
 //   cell_start[set cell offset + c] .. [c+1] delimit a cell's points.
 //   A work item is one (i tile, j range, shift) triple of a cell pair (Sec. 4.3).
 #pragma once

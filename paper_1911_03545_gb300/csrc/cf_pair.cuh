@@ -194,7 +194,7 @@ __device__ __forceinline__ u64 wrap2(u64 d, float L, float invL)
 static __device__ __noinline__ void push_recheck(const CfPairArgs &a, uint32_t ip, uint32_t jp, uint32_t job)
 {
     const unsigned long long k = atomicAdd(a.qcount, 1ull);
-    if (k < a.qcap) a.queue[k] = make_uint4(a.orig[ip], a.orig[jp], job, 0u);
+    if (k < a.qcap) a.queue[k] = make_uint4(cf_orig(a.orig, a.pt, ip), cf_orig(a.orig, a.pt, jp), job, 0u);
 }
 
 // rp of a counted pair of the mocks kind, for ravg (Appendix A.2.1).  rp^2 = |s x l|^2 / |l|^2,

@@ -101,7 +101,7 @@ __global__ void cf_recheck_kernel(const CfDevPlan *__restrict__ P, const CfSetDe
 // one atomic.  Entries past the queue capacity are dropped: the host sees the count and repeats the
 // call with a larger queue.
 __global__ void cf_audit_kernel(const CfItem *__restrict__ items, const uint32_t *__restrict__ nitems_dev,
-                                uint32_t items_cap, const uint32_t *__restrict__ orig, uint4 *__restrict__ queue,
+                                uint32_t items_cap, const uint32_t *__restrict__ orig, const float4 *__restrict__ pt, uint4 *__restrict__ queue,
                                 unsigned long long *__restrict__ qcount, uint32_t qcap)
 {
     const uint32_t n = min(*nitems_dev, items_cap);
@@ -117,18 +117,19 @@ __global__ void cf_audit_kernel(const CfItem *__restrict__ items, const uint32_t
             if (j0 >= jc) continue;
             const uint32_t cnt = jc - j0;
             const unsigned long long base = atomicAdd(qcount, (unsigned long long)cnt);
-            const uint32_t oi = orig[it.ibeg + il];
+            const uint32_t oi = cf_orig(orig, pt, it.ibeg + il);
             for (uint32_t k = 0; k < cnt; k++)
-                if (base + k < qcap) queue[base + k] = make_uint4(oi, orig[it.jbeg + j0 + k], jo, 0u);
+                if (base + k < qcap) queue[base + k] = make_uint4(oi, cf_orig(orig, pt, it.jbeg + j0 + k), jo, 0u);
         }
     }
 }
 
 cudaError_t cfp_launch_audit(const CfItem *items, const uint32_t *nitems_dev, uint32_t items_cap,
-                             const uint32_t *orig, uint4 *queue, unsigned long long *qcount, uint32_t qcap, int num_sms,
+                             const uint32_t *orig, const float4 *pt, uint4 *queue, unsigned long long *qcount, uint32_t qcap,
+                             int num_sms,
                              cudaStream_t st)
 {
-    cf_audit_kernel<<<num_sms * 4, 256, 0, st>>>(items, nitems_dev, items_cap, orig, queue, qcount, qcap);
+    cf_audit_kernel<<<num_sms * 4, 256, 0, st>>>(items, nitems_dev, items_cap, orig, pt, queue, qcount, qcap);
     return cudaGetLastError();
 }
 
