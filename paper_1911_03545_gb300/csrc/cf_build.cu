@@ -3,6 +3,8 @@
 #include "cf_build.h"
 #include "cf_device.cuh"
 
+#include <math_constants.h>
+
 // ---------------------------------------------------------------------------------------------
 // Bounding box and validity of every point set: min / max per axis, count of non-finite values.
 // grid = (blocks, nsets); out[s*W + 0..5] = key(min x,y,z), key(max x,y,z); out[s*W+6] = bad;
@@ -613,33 +615,41 @@ __device__ __forceinline__ void cf_cell_box(const uint32_t *cell_start, int64_t 
         return;
     }
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (uint32_t p0 = b; p0 < e; p0 += 32u) {
-        float glo[3] = {INFINITY, INFINITY, INFINITY}, ghi[3] = {-INFINITY, -INFINITY, -INFINITY};
-        const uint32_t p = p0 + lane;
-        if (p < e) {
-            const float4 A = pt[p];
-            const float v[3] = {-A.x, -A.y, -A.z};
-            for (int a = 0; a < 3; a++) glo[a] = ghi[a] = v[a];
+    // four groups' loads in flight: one at a time, cells of many points waited for each in turn
+    for (uint32_t p0 = b; p0 < e; p0 += 128u) {
+        float4 A[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4u; u++) {
+            A[u] = make_float4(CUDART_NAN_F, CUDART_NAN_F, CUDART_NAN_F, 0.f);       // drops out below
+            if (p0 + 32u * u + lane < e) A[u] = pt[p0 + 32u * u + lane];
         }
-        if (gbox) {
-            for (int o = 16; o; o >>= 1)
+#pragma unroll
+        for (uint32_t u = 0; u < 4u; u++) {
+            const float v[3] = {-A[u].x, -A[u].y, -A[u].z};
+            const uint32_t q = p0 + 32u * u;
+            if (gbox && q < e) {
+                float glo[3], ghi[3];
                 for (int a = 0; a < 3; a++) {
-                    glo[a] = fminf(glo[a], __shfl_xor_sync(CF_FULL, glo[a], o));
-                    ghi[a] = fmaxf(ghi[a], __shfl_xor_sync(CF_FULL, ghi[a], o));
+                    glo[a] = cf_redux_min(v[a]);
+                    ghi[a] = cf_redux_max(v[a]);
                 }
-            if (lane < 6u) gbox[6 * (size_t)p0 + lane] = lane < 3u ? glo[lane] : ghi[lane - 3u];
-        }
-        for (int a = 0; a < 3; a++) {
-            lo[a] = fminf(lo[a], glo[a]);
-            hi[a] = fmaxf(hi[a], ghi[a]);
+                if (lane < 6u)
+                    gbox[6 * (size_t)q + lane] = lane < 3u ? (lane == 0u ? glo[0] : (lane == 1u ? glo[1] : glo[2]))
+                                                          : (lane == 3u ? ghi[0] : (lane == 4u ? ghi[1] : ghi[2]));
+            }
+            for (int a = 0; a < 3; a++) {
+                lo[a] = fminf(lo[a], v[a]);
+                hi[a] = fmaxf(hi[a], v[a]);
+            }
         }
     }
-    for (int o = 16; o; o >>= 1)
-        for (int a = 0; a < 3; a++) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(CF_FULL, lo[a], o));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(CF_FULL, hi[a], o));
-        }
-    if (lane < 6u) box[6 * c + lane] = lane < 3u ? lo[lane] : hi[lane - 3u];
+    for (int a = 0; a < 3; a++) {
+        lo[a] = cf_redux_min(lo[a]);
+        hi[a] = cf_redux_max(hi[a]);
+    }
+    if (lane < 6u)
+        box[6 * c + lane] = lane < 3u ? (lane == 0u ? lo[0] : (lane == 1u ? lo[1] : lo[2]))
+                                      : (lane == 3u ? hi[0] : (lane == 4u ? hi[1] : hi[2]));
 }
 
 __global__ void cf_cellbox_kernel(const uint32_t *__restrict__ cell_start, int64_t ncell_all,
