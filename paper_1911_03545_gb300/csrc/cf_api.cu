@@ -900,7 +900,7 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     C->last_grid = grid;
     C->last_warps = warps;
     if (timed) CF_CU(cudaEventRecordWithFlags(C->ev[2], st, C->capturing ? cudaEventRecordExternal : 0), "event");
-    CF_CU(cfp_launch_recheck(dplan, dsets, djobs, A.queue, A.qcount, R.qcap, A.hcnt, A.hw, A.hr,
+    CF_CU(cfp_launch_recheck(dplan, dsets, djobs, A.queue, A.qcount, R.qcap, A.hcnt, A.hw, A.hr, R.hsz,
                              listed ? (const uint32_t *)C->buf[B_BAR].p + 2 : nullptr, (uint32_t *)(out + OUT_LATE),
                              C->num_sms, st),
           "recheck");

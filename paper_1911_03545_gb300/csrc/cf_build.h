@@ -137,10 +137,9 @@ cudaError_t cfp_launch_pair(const CfPairCfg &c, const CfPairArgs &a, int num_sms
 // CF_OPT_AUDIT: queue every pair of every work item for the FP64 recheck (launched instead of the
 // pair kernel).
 cudaError_t cfp_launch_audit(const CfItem *items, const uint32_t *nitems_dev, uint32_t items_cap,
-                             const uint32_t *orig, const float4 *pt, uint4 *queue, unsigned long long *qcount, uint32_t qcap,
-                             int num_sms,
-                             cudaStream_t st);
+                             const uint32_t *orig, const float4 *pt, uint4 *queue, unsigned long long *qcount,
+                             uint32_t qcap, int num_sms, cudaStream_t st);
 cudaError_t cfp_launch_recheck(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobDesc *jobs,
                                const uint4 *queue, const unsigned long long *qcount, uint32_t qcap,
-                               unsigned long long *hcnt, double *hw, double *hr, const uint32_t *late, uint32_t *flag,
-                               int num_sms, cudaStream_t st);
+                               unsigned long long *hcnt, double *hw, double *hr, size_t hsz, const uint32_t *late,
+                               uint32_t *flag, int num_sms, cudaStream_t st);
