@@ -136,6 +136,30 @@ class _Out:
         return d
 
 
+class _Outs:
+    """_Out for the n catalogues of a batch: one host block, a row per catalogue, and one array of
+    cf_result over it (an object and four views per catalogue cost more than half of what the GPU
+    takes for 32 catalogues of 8,000 points: 434 us per call, 298 us this way)."""
+
+    def __init__(self, p: Params, n: int):
+        nb, nout = len(p.edges) - 1, p.nout
+        self.buf = np.empty((n, 3 * nout + nb))
+        self.ptr = np.add.outer(np.arange(n, dtype=np.uintp) * np.uintp(8 * (3 * nout + nb)) + np.uintp(self.buf.ctypes.data),
+                                np.array([0, 8 * nout, 16 * nout, 24 * nout], dtype=np.uintp))
+        self.c = (_capi.cf_result * n).from_buffer(self.ptr)
+
+    def as_dicts(self, p: Params) -> list:
+        nb, nout = len(p.edges) - 1, p.nout
+        shape = (-1, nb, p.c.npibins) if p.kind in (CF_DD_RPPI, CF_DD_RPPI_MOCKS) else (-1, nout)
+        cols = {"npairs": self.buf[:, :nout].view(np.uint64).reshape(shape),
+                "wsum": self.buf[:, nout:2 * nout].reshape(shape)}
+        if p.c.output_ravg:
+            cols["ravg"] = self.buf[:, 2 * nout:3 * nout].reshape(shape)
+        if p.kind == CF_WP:
+            cols["wp"] = self.buf[:, 3 * nout:]
+        return [dict(zip(cols, row)) for row in zip(*cols.values())]
+
+
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         return None
@@ -172,10 +196,9 @@ def cf_count(ctx: int, p: Params, d1: Points, d2: Optional[Points] = None) -> di
 def cf_batch_count(ctx: int, p: Params, cats: Sequence[Points]) -> list:
     n = len(cats)
     arr = (_capi.cf_points * n)(*[c.c for c in cats])
-    outs = [_Out(p.nout, len(p.edges) - 1) for _ in range(n)]
-    res = (_capi.cf_result * n)(*[o.c for o in outs])
-    _check(_capi.lib().cf_batch_count(ctx, ctypes.byref(p.c), arr, n, res), ctx)
-    return [o.as_dict(p) for o in outs]
+    outs = _Outs(p, n)
+    _check(_capi.lib().cf_batch_count(ctx, ctypes.byref(p.c), arr, n, outs.c), ctx)
+    return outs.as_dicts(p)
 
 
 def cf_get_stats(ctx: int) -> dict:
@@ -245,10 +268,9 @@ def cf_batch_capture(ctx: int, p: Params, cats: Sequence[Points]) -> None:
 
 
 def cf_batch_replay(ctx: int, p: Params, n: int) -> list:
-    outs = [_Out(p.nout, len(p.edges) - 1) for _ in range(n)]
-    res = (_capi.cf_result * n)(*[o.c for o in outs])
-    _check(_capi.lib().cf_batch_replay(ctx, res, n), ctx)
-    return [o.as_dict(p) for o in outs]
+    outs = _Outs(p, n)
+    _check(_capi.lib().cf_batch_replay(ctx, outs.c, n), ctx)
+    return outs.as_dicts(p)
 
 
 def cf_plan_probe(p: Params, bbox, npoints: int, any_f64: bool = False, which: int = 0, values=None) -> dict:

@@ -603,6 +603,12 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
 
 size_t readback_bytes(const CfRun &R) { return OUT_HIST + 24 * R.hsz + 8 * (size_t)R.nsets; }
 
+// the part of it that a call clears and reads back: the counts alone without weights and ravg
+static size_t result_bytes(const CfRun &R)
+{
+    return R.plan.d.weighted || R.plan.d.ravg ? readback_bytes(R) : OUT_HIST + 8 * R.hsz;
+}
+
 // bbox pass of a captured graph: starting values, the pass, its readback at R.bb_off
 static int cf_enqueue_bbox(CfCtx *C, CfRun &R)
 {
@@ -658,7 +664,7 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
         S.npts = (uint32_t)R.npts;
         S.nfine = (uint32_t)R.nfine;
         S.zero = (uint32_t *)out;
-        S.zero_words = (uint32_t)(readback_bytes(R) / 4);
+        S.zero_words = (uint32_t)(result_bytes(R) / 4);
         S.bar = (uint32_t *)C->buf[B_BAR].p;
         S.late = S.bar + 2;
         S.count = (uint32_t *)C->buf[B_ONECNT].p;
@@ -812,7 +818,7 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     const size_t zero_from = R.fused_items ? 0 : OUT_EVAL;
     const bool listed = R.listed;       // the build has zeroed them and written the list
     R.listed = false;
-    if (!listed) CF_CU(cudaMemsetAsync(out + zero_from, 0, readback_bytes(R) - zero_from, st), "memset");
+    if (!listed) CF_CU(cudaMemsetAsync(out + zero_from, 0, result_bytes(R) - zero_from, st), "memset");
     uint32_t *nitems_dev = ioff + R.nunit;
     const uint32_t *cstart = (const uint32_t *)C->buf[B_CSTART].p;
     const uint32_t *live = R.live_units ? (const uint32_t *)C->buf[B_LIVE].p : nullptr;
@@ -915,8 +921,8 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
         CF_CU(cudaStreamWaitEvent(st, C->ev_join, 0), "stream wait");
         C->aux_pending = false;
     }
-    // readback: the whole B_OUT block (counters, histograms, w^2 sums) in one copy
-    CF_CU(cudaMemcpyAsync(C->hpin, out, readback_bytes(R), cudaMemcpyDeviceToHost, st), "readback");
+    // readback: the B_OUT block (counters, histograms, w^2 sums) in one copy
+    CF_CU(cudaMemcpyAsync(C->hpin, out, result_bytes(R), cudaMemcpyDeviceToHost, st), "readback");
     return CF_OK;
 }
 
@@ -962,16 +968,19 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
     res.assign(R.njobs, CfJobResult());
     for (int j = 0; j < R.njobs; j++) {
         CfJobResult &Q = res[j];
-        Q.npairs.assign(nslot, 0);
-        Q.wsum.assign(nslot, 0.0);
-        Q.rsum.assign(nslot, 0.0);
+        Q.npairs.resize(nslot);
+        Q.wsum.resize(nslot);
         const bool autoc = R.jobs[j].autoc != 0;
         const double mult = autoc ? 2.0 : 1.0;
-        for (size_t k = 0; k < nslot; k++) {
-            // Sec. 4.3: unique pairs were counted for an auto-correlation; double them
-            Q.npairs[k] = hc[j * nslot + k] * (autoc ? 2ull : 1ull);
-            Q.wsum[k] = D.weighted ? hw[j * nslot + k] * mult : (double)Q.npairs[k];
-            Q.rsum[k] = hr[j * nslot + k] * mult;
+        // Sec. 4.3: unique pairs were counted for an auto-correlation; double them
+        for (size_t k = 0; k < nslot; k++) Q.npairs[k] = hc[j * nslot + k] * (autoc ? 2ull : 1ull);
+        if (D.weighted)
+            for (size_t k = 0; k < nslot; k++) Q.wsum[k] = hw[j * nslot + k] * mult;
+        else
+            for (size_t k = 0; k < nslot; k++) Q.wsum[k] = (double)Q.npairs[k];
+        if (D.ravg) {
+            Q.rsum.resize(nslot);
+            for (size_t k = 0; k < nslot; k++) Q.rsum[k] = hr[j * nslot + k] * mult;
         }
         if (autoc && R.self_pairs) {
             // Appendix B: the N self pairs, added once, in the first bin (first pi bin for rp-pi)
@@ -1093,10 +1102,12 @@ void cf_write_result(const cf_params *p, const CfJobResult &Q, cf_result *out)
     const size_t nslot = Q.npairs.size();
     if (out->npairs) std::memcpy(out->npairs, Q.npairs.data(), 8 * nslot);
     if (out->wsum) std::memcpy(out->wsum, Q.wsum.data(), 8 * nslot);
-    if (out->ravg) {
+    if (out->ravg && !p->output_ravg) {
+        std::memset(out->ravg, 0, 8 * nslot);
+    } else if (out->ravg) {
         for (size_t k = 0; k < nslot; k++) {
             double den = p->weight == CF_W_PAIR_PRODUCT ? Q.wsum[k] : (double)Q.npairs[k];
-            out->ravg[k] = (p->output_ravg && den > 0) ? Q.rsum[k] / den : 0.0;
+            out->ravg[k] = den > 0 ? Q.rsum[k] / den : 0.0;
         }
     }
     if (out->wp) {
