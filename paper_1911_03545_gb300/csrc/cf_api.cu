@@ -771,7 +771,6 @@ static float fixed_scale(double tmin, double tmax)
 static void fixed_point_scales(const CfRun &R, bool weighted, bool ravg, CfPairArgs &A)
 {
     A.fxw = A.fxr = 0.f;
-    A.ifxw = 0.0;
     double pmin = 1.0, pmax = 1.0;
     if (weighted) {
         if (R.wneg) return;
@@ -795,7 +794,6 @@ static void fixed_point_scales(const CfRun &R, bool weighted, bool ravg, CfPairA
     }
     // one form for every sum the call keeps: fixed point only where all of them allow it
     if ((weighted && A.fxw == 0.f) || (ravg && A.fxr == 0.f)) A.fxw = A.fxr = 0.f;
-    if (A.fxw != 0.f) A.ifxw = 1.0 / (double)A.fxw;
 }
 
 // work items -> pair kernel -> recheck -> readback (device only; records ev[1..3] when `timed`)

@@ -110,7 +110,6 @@ struct CfPairArgs {
     float fxw;                   // rp-pi / mocks per-warp weight sums in fixed point (two 32-bit words
                                  // per slot, see cf_pair.cuh) at this power-of-two scale (0: FP64)
     float fxr;                   // nonzero: the ravg sums too, those of rp bin k at scale fxr_bin[k]
-    double ifxw;                 // 1 / fxw
     float fxr_bin[CF_MAX_BINS];
 };
 
