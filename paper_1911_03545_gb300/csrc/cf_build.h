@@ -111,6 +111,7 @@ struct CfPairArgs {
                                  // per slot, see cf_pair.cuh) at this power-of-two scale (0: FP64)
     float fxr;                   // nonzero: the ravg sums too, those of rp bin k at scale fxr_bin[k]
     float fxr_bin[CF_MAX_BINS];
+    uint32_t nwarps;             // warps of the launch (set by the launcher)
 };
 
 // Static configuration of a pair-kernel launch (selects the template instance and the shared
