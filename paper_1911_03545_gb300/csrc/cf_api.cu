@@ -271,7 +271,7 @@ static const int64_t CF_ONE_MAX = 262144;
 
 // work-list capacity (48 bytes an item) up to which a call on a new plan takes an estimate instead of
 // counting the items first
-static const uint64_t CF_GUESS_MAX = 1u << 21;
+static const uint64_t CF_GUESS_MAX = 1u << 22;
 
 static uint64_t items_guess(const CfRun &R)
 {
@@ -281,7 +281,10 @@ static uint64_t items_guess(const CfRun &R)
         const double na = (double)R.sets[J.a].n, nb = (double)R.sets[J.b].n, nc = (double)D.g.ncell;
         const double cells = std::min(nc, na);      // i cells that may hold points
         const double pairs = D.ang ? 25.0 : (J.autoc ? 0.5 * (R.nst + 1) : (double)R.nst);
-        n += cells * std::min(pairs, nb) * (na / cells / D.tile + 1.0) * (nb / std::min(nc, std::max(1.0, nb)) / D.jchunk + 1.0);
+        const double ti = na / cells / D.tile, tj = nb / std::min(nc, std::max(1.0, nb)) / D.jchunk;
+        // (halved cells have many neighbours, of which more lie out of reach or are empty)
+        n += cells * std::min(pairs, nb) * (D.g.k[0] > 1 ? std::max(1.0, ti + 0.5) * std::max(1.0, tj + 0.5)
+                                                         : (ti + 1.0) * (tj + 1.0));
     }
     return n < 4e18 ? (uint64_t)n : (uint64_t)4e18;
 }
@@ -444,6 +447,11 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     bool open_grid = !angular && C->opt[CF_OPT_REFINE] == 0 && C->opt[CF_OPT_CELL_ORDER] == 0 && !C->opt[CF_OPT_AUDIT];
     for (int a = 0; a < 3; a++) open_grid = open_grid && p->refine[a] == 0;
     const double fill = open_grid ? CFI_MIN_FILL : 0.0;
+    // size of the set that a point of the call is in on average, for the cells' width (0: not halved, since the
+    // longer work list may not fit a cap on the scratch)
+    double sq = 0.0;
+    for (int s = 0; s < nsets; s++) sq += (double)pts[s]->n * (double)pts[s]->n;
+    const int64_t dense_n = C->mem_cap || R.npts == 0 ? 0 : (int64_t)(sq / (double)R.npts);
     // |v| of the point nearest the observer (its square was summed in float32 for float32 inputs:
     // a few roundings high or low)
     const double vmin = std::isfinite(vmin2) ? std::sqrt(vmin2) * (1.0 - 1e-6) : 0.0;
@@ -457,6 +465,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         put(p->edges, sizeof(double) * (size_t)(p->nbins + 1));
         put(bbox, sizeof(bbox));
         put(&R.npts, sizeof(R.npts));
+        put(&dense_n, sizeof(dense_n));
         const int ints[6] = {any_f64 ? 1 : 0, refine[0] * 16 + refine[1] * 4 + refine[2], tile, jchunk, angular ? 1 : 0,
                              open_grid ? 1 : 0};
         put(ints, sizeof(ints));
@@ -464,7 +473,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         if (key != C->plan_key) {
             C->plan_key.clear();
             rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0, vmin,
-                               fill * nsets);
+                               fill * nsets, dense_n);
             // wider cells have wider error bands: what fails with them may pass without
             if (rc && fill > 0.0)
                 rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0,

@@ -30,6 +30,9 @@
 #define CFI_FINE_FLAG 0x100u      // coarse entry >= this: index of a fine entry + flag
 #define CFI_MIN_FILL 40.0         // points per cell and set below which the cells are widened (widen_cells)
 #define CFI_WIDEN_MIN 32768       // points of a call below which they are not
+#define CFI_DENSE 500.0           // points of a set per cell from which cells are halved (dense_cells)
+#define CFI_DENSE_CYL 800.0       // the same for the cylinder of rp-pi and wp
+#define CFI_DENSE_MAX (1 << 24)   // points of a set above which they are not
 #define CFI_JMAX 512              // longest j range of a work item (9-bit j in a candidate)
 
 // Pair-kernel item (48 bytes, three 16-byte loads)
