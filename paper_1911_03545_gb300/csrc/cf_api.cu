@@ -292,6 +292,13 @@ static uint64_t items_guess(const CfRun &R)
 // work lists longer than this (3 GB) are made again with the largest items when their shape was left open
 static const uint32_t CF_FINE_ITEMS = 1u << 26;
 
+// the shape of the items was left open and is not the largest
+static bool may_coarsen(const CfCtx *C, const CfRun &R)
+{
+    return !R.coarse && R.plan.d.tile * R.plan.d.jchunk < 128 * CFI_JMAX && C->opt[CF_OPT_TILE] == 0 &&
+           C->opt[CF_OPT_JCHUNK] == 0;
+}
+
 int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &pts,
                const std::vector<CfJobDesc> &jobs, CfRun &R)
 {
@@ -1050,10 +1057,16 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
             cap = (uint32_t)guess;
         }
     }
-    if (R.fused_items) {
-        R.items_cap = cap;
-        CF_TRY(ensure_items(C, cap));
-    }
+    // a list that does not fit (a cap on the scratch) is made with the largest items before the call fails
+    auto grow = [&](uint32_t n) {      // 1: start again
+        const int rc = ensure_items(C, n);
+        if (rc != CF_ERR_OOM || !may_coarsen(C, R)) return rc;
+        C->coarse_key = C->plan_key;
+        C->items_hint = 0;
+        return 1;
+    };
+    if (R.fused_items && ensure_items(C, cap) != CF_OK) R.fused_items = false;      // no room for the headroom: count first
+    if (R.fused_items) R.items_cap = cap;
     CF_CU(cudaEventRecord(C->ev[0], st), "event");
     CF_TRY(cf_enqueue_build(C, R));
     if (!R.fused_items) {
@@ -1065,14 +1078,15 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     }
     // concentrated points make far more items than their mean density says: take the largest ones then
     auto too_fine = [&] {
-        return R.items_cap > CF_FINE_ITEMS && !R.coarse && R.plan.d.tile * R.plan.d.jchunk < 128 * CFI_JMAX &&
-               C->opt[CF_OPT_TILE] == 0 && C->opt[CF_OPT_JCHUNK] == 0;
+        return R.items_cap > CF_FINE_ITEMS && may_coarsen(C, R);
     };
     if (!R.fused_items && too_fine()) {
         C->coarse_key = C->plan_key;
         return cf_run(C, p, pts, jobs, res);
     }
-    CF_TRY(ensure_items(C, R.items_cap));
+    int grown = grow(R.items_cap);
+    if (grown > 0) return cf_run(C, p, pts, jobs, res);
+    CF_TRY(grown);
     for (int attempt = 0; attempt < 4; attempt++) {
         CF_TRY(cf_enqueue_count(C, R, true));
         CF_CU(cudaStreamSynchronize(st), "count sync");
@@ -1098,7 +1112,11 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
             C->items_hint = 0;
             return cf_run(C, p, pts, jobs, res);
         }
-        if (retry == 2) CF_TRY(ensure_items(C, R.items_cap));
+        if (retry == 2) {
+            grown = grow(R.items_cap);
+            if (grown > 0) return cf_run(C, p, pts, jobs, res);
+            CF_TRY(grown);
+        }
     }
     return C->fail(CF_ERR_INTERNAL, "recheck queue kept overflowing");
 }
@@ -1273,7 +1291,13 @@ cf_status cf_batch_capture(void *ctx, const cf_params *params, const cf_points *
     // the graph sizes its work list here (one pass writes it) and runs its own bbox pass in line
     R.fused_items = true;
     R.bbox_aux = false;
-    if ((rc = ensure_items(C, R.items_cap))) return (cf_status)rc;
+    rc = ensure_items(C, R.items_cap);
+    if (rc == CF_ERR_OOM && may_coarsen(C, R)) {
+        C->coarse_key = C->plan_key;
+        C->items_hint = 0;
+        return cf_batch_capture(ctx, params, cats, ncat);
+    }
+    if (rc) return (cf_status)rc;
     R.qcap = std::max(R.qcap, (uint32_t)std::min<int64_t>(CF_MAX_ENTRIES, C->stats.rechecked_pairs * 2 + 4096));
     if ((rc = C->ensure(B_QUEUE, 16 * (size_t)R.qcap))) return (cf_status)rc;
     // the graph also re-runs the bbox pass, read back past the results, so that a replay can

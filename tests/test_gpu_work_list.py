@@ -30,3 +30,34 @@ def test_every_pair_of_a_cell_once(n):
                 assert int(np.asarray(cross["npairs"]).astype(np.uint64).sum()) == n * (n // 3 + 1)
     finally:
         cf.cf_destroy(ctx)
+
+
+def test_a_list_that_does_not_fit_takes_larger_items():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    n = 60_000
+    cat = gen.uniform_box(n, 100.0, 1, np.float32)
+    edges, kw = gen.log_edges(0.1, 10.0, 8), dict(autocorr=True, periodic=True, box=100.0)
+    free, capped = (cf.cf_create(0, torch.cuda.current_stream()) for _ in range(2))
+    try:
+        exp = gpu_count(free, "r", edges, cat, **kw)
+        fine = cf.cf_get_stats(free)["work_items"]
+        used = 0
+        for cap in range(1 << 21, 1 << 25, 1 << 18):
+            cf.cf_set_option(capped, cf.CF_OPT_MEM_CAP, cap)
+            try:
+                got = gpu_count(capped, "r", edges, cat, **kw)
+            except cf.CfError as e:
+                assert "cap" in str(e)
+                continue
+            used = cf.cf_get_stats(capped)["work_items"]
+            break
+        assert 0 < used < fine
+        np.testing.assert_array_equal(got["npairs"], exp["npairs"])
+        again = gpu_count(capped, "r", edges, cat, **kw)
+        np.testing.assert_array_equal(again["npairs"], exp["npairs"])
+    finally:
+        cf.cf_destroy(free)
+        cf.cf_destroy(capped)
