@@ -20,8 +20,10 @@ enum CfBuf {
 // of units with points in their i cell (u32, when the work list visits only those), the same length in 64 bits,
 // evaluated pairs, the pair kernel's work cursor (u32), recheck-queue length, then from OUT_HIST
 // hcnt[hsz] (u64), hw[hsz], hr[hsz] (f64) and the sum of w^2 per point set (f64); at OUT_SCAN the
-// tickets of the build's two scans, at OUT_LATE a flag that the one-launch build gave up at a barrier.  The build zeroes the first OUT_HIST bytes, the count phase
-// everything from OUT_EVAL on (from 0 for the one-pass work list), each with one memset.
+// tickets of the build's two scans, at OUT_LATE a flag that the one-launch build gave up at a barrier.
+// The build zeroes the first OUT_HIST bytes, the count phase everything from OUT_EVAL on (from 0 for the
+// one-pass work list), each with one memset; the one-launch build zeroes all of it.  Without weights and ravg
+// what follows hcnt is neither zeroed nor read back.
 #define OUT_NITEMS 0
 #define OUT_NLIVE 4
 #define OUT_ITEMS64 8

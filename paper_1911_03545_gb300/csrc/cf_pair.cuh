@@ -20,15 +20,18 @@
 // the proven FP32 error band of an edge is not binned: the pair goes to a global queue and is
 // re-evaluated in FP64 by the recheck kernel, so counts equal the FP64 result.
 //
-// What bounds it: instruction issue (70 to 80 % of the slots).  Counting costs 17 (DD(theta), counts only)
-// to 30 (weights and ravg) instructions per gathered point and warp, gathering about 70 per 32 j points,
-// so the layout aims at few gathered points per pair in range: on the clustered catalogues 1.6 to
-// 2.0 times the in-range pairs are formed, where whole cell pairs form 4 to 8 times as many.  Gathering
-// also fills the blocks: a cell's ragged end costs at most three points of a range's last block.
+// What bounds it: instruction issue for the counts (rp-pi 86 % of the slots, r 84 %, mocks 78 %; theta 82 % of the
+// shared-memory wavefronts, one histogram word per pair), for the sums the shared-memory wavefronts (72 to 77 %:
+// a 16-byte Kahan update per pair and lane, five atomics per pair of rp-pi) at the 16 warps per SM that their
+// histograms leave.  Counting costs 17 (DD(theta), counts only) to 30 (weights and ravg) instructions per gathered
+// point and warp, gathering about 70 per 32 j points, so the layout aims at few gathered points per pair in
+// range: on the clustered catalogues 1.6 to 2.0 times the in-range pairs are formed, where whole cell pairs form 4
+// to 8 times as many.  Gathering also fills the blocks: a cell's ragged end costs at most three points of a
+// range's last block, and a tile's last group shares the warp (below).
 // Measured against whole cell pairs with a branch per pair in range (pair kernel, one GB300): DD(r) of
-// 1M clustered points with weights and ravg 1.546 -> 1.102 ms, counts to twice the separation
-// 5.25 -> 2.53 ms, DD(rp, pi) of 2M points 1.505 -> 1.016 ms, its DR against 4M randoms 5.17 -> 3.03 ms,
-// DD(theta) of 1M points 1.176 -> 0.687 ms, DR of the survey cone 5.48 -> 2.48 ms.
+// 1M clustered points with weights and ravg 1.546 -> 0.981 ms, counts to twice the separation
+// 5.25 -> 2.06 ms, DD(rp, pi) of 2M points 1.505 -> 0.879 ms, its DR against 4M randoms 5.17 -> 2.70 ms,
+// DD(theta) of 1M points 1.176 -> 0.623 ms, DR of the survey cone 5.48 -> 1.81 ms.
 //
 // Histograms live in shared memory per warp (Sec. 4.8: private histograms, merged once): for
 // r / theta / wp one private copy per lane (no bank conflicts, no contention; weighted sums
