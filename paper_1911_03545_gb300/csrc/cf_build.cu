@@ -697,8 +697,9 @@ __global__ void cf_live_units_kernel(const CfDevPlan *__restrict__ plan, const C
 // mode 0 writes the item count of each (job, cell) and adds the number of items, counted in 64 bits,
 // to *evaluated (the 32-bit scan of the counts would wrap silently past 2^32 items); mode 1 writes
 // the items at the scanned offsets and adds the pairs they hold to *evaluated.  Mode 2 needs no
-// count pass: per 32 stencil entries the warps of a block reserve their items' places together, with one
-// atomic on counts[0] (the list's length when the kernel ends); the angular grid's warps, whose stencils
+// count pass: for a stencil of up to 32 entries the warps of a block reserve their items' places together, with one
+// atomic on counts[0] (the list's length when the kernel ends); for larger ones a block first collects its items in
+// shared memory (a reservation per 32 entries made 28,672 cells of 125 entries take 40 us more); the angular grid's warps, whose stencils
 // differ, each reserve for themselves.  The number of items is added in 64 bits to *total64.  The list's
 // order then follows the blocks' arrival instead of (job, cell).
 // Bound by the latency of the loads, the reservation and the barriers around it, not by the 48 bytes per
@@ -730,15 +731,19 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
     const uint32_t lane = threadIdx.x & 31u;
     unsigned long long ev = 0, nres = 0;
     constexpr int MAXW = CFB_ONE_THREADS / 32;
-    __shared__ uint32_t s_cnt[MAXW], s_base[MAXW];
+    __shared__ uint32_t s_cnt[MAXW], s_base[MAXW], s_n;
+    __shared__ __align__(16) CfItem s_items[CFB_ITEM_STAGE];
     // every warp of a block runs the same number of iterations (block-wide barriers in mode 2)
     const uint32_t wpb = blockDim.x >> 5, warp = threadIdx.x >> 5;
     // mode 2 on the 3-D grid: the warps of a block reserve their places in the list together
     const bool joint = mode == 2 && !plan->ang;
+    // with more than 32 stencil entries they collect the items in shared memory first
+    const bool stage = joint && nst > 32;
     // with a list of the units whose i cell holds points, only those (the same count in every thread)
     const uint32_t nloop = live ? min(*nlive, (uint32_t)nunit) : (uint32_t)nunit;
-    // neighbouring units go to one block, unless that leaves blocks without any
-    const bool spread = nloop < nblk * wpb;
+    // neighbouring units go to one block, unless that leaves SMs without any (the one-launch build; listed units
+    // are fewer than the grid has warps for, and blocks of idle warps would only take room)
+    const bool spread = !live && nloop < nblk * wpb;
     for (uint32_t ub = spread ? 0u : bid * wpb; ub < nloop; ub += nblk * wpb) {
         const uint32_t un = spread ? warp * nblk + bid : ub + warp;
         {
@@ -752,6 +757,7 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
             const uint32_t ia = cell_start[A.cbeg + c], na = have ? cell_start[A.cbeg + c + 1] - ia : 0u;
             uint32_t total = 0;
             // (a block of empty cells has nothing to reserve)
+            if (stage && threadIdx.x == 0) s_n = 0u;
             if (joint ? __syncthreads_or(na != 0u) != 0 : na != 0u) {
                 const int cxy = c / g.n[2], cx = cxy / g.n[1];
                 const int ci[3] = {cx, cxy - cx * g.n[1], c - cxy * g.n[2]};
@@ -938,7 +944,28 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                     }
                     const uint32_t ctot = __shfl_sync(CF_FULL, incl, 31);
                     uint32_t cbase = base + total;
-                    if (joint) {
+                    bool staged = false;
+                    if (stage) {
+                        uint32_t r = 0, in = 0;
+                        if (lane == 0 && ctot) {
+                            // a place in the stage when the items fit (the CAS only fails when another warp of the
+                            // block reserved; bounded), else in the list
+                            uint32_t old = *(volatile uint32_t *)&s_n;
+                            for (int t = 0; t < 64 && old + ctot <= CFB_ITEM_STAGE; t++) {
+                                const uint32_t seen = atomicCAS(&s_n, old, old + ctot);
+                                if (seen == old) {
+                                    r = old;
+                                    in = 1;
+                                    break;
+                                }
+                                old = seen;
+                            }
+                            if (!in) r = atomicAdd(counts, ctot);
+                        }
+                        cbase = __shfl_sync(CF_FULL, r, 0);
+                        staged = __shfl_sync(CF_FULL, in, 0) != 0u;
+                        nres += ctot;
+                    } else if (joint) {
                         // one reservation per block: 40,000 warps that each added to the list's length would
                         // wait for one another
                         if (lane == 0) s_cnt[warp] = ctot;
@@ -985,8 +1012,8 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                         }
                         auto put = [&](uint32_t o, uint32_t i0, uint32_t ic, uint32_t jbeg, uint32_t jc, bool dflag,
                                        const float (&vh)[3], const float (&vl)[3]) {
-                            if (o < items_cap) {
-                                uint4 *p = reinterpret_cast<uint4 *>(items + o);
+                            if (staged || o < items_cap) {
+                                uint4 *p = reinterpret_cast<uint4 *>(staged ? s_items + o : items + o);
                                 p[0] = make_uint4(ia + i0, jbeg, ic | (jc << 16), (uint32_t)job | (dflag ? CFI_ITEM_DIAG : 0u));
                                 p[1] = make_uint4(__float_as_uint(vh[0]), __float_as_uint(vh[1]), __float_as_uint(vh[2]), 0u);
                                 p[2] = make_uint4(__float_as_uint(vl[0]), __float_as_uint(vl[1]), __float_as_uint(vl[2]), 0u);
@@ -1048,6 +1075,18 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                         }
                     }
                     total += __shfl_sync(CF_FULL, incl, 31);
+                }
+                if (stage) {
+                    // one reservation, then 16-byte stores
+                    __syncthreads();
+                    const uint32_t n = s_n;
+                    if (threadIdx.x == 0 && n) s_base[0] = atomicAdd(counts, n);
+                    __syncthreads();
+                    const uint32_t b0 = s_base[0];
+                    for (uint32_t k = threadIdx.x; k < 3u * n; k += blockDim.x)
+                        if (b0 + k / 3u < items_cap)
+                            reinterpret_cast<uint4 *>(items + b0)[k] = reinterpret_cast<const uint4 *>(s_items)[k];
+                    __syncthreads();
                 }
             }
             if (mode == 0 && lane == 0 && have) counts[u] = total;
