@@ -254,7 +254,9 @@ static int cf_check_bbox(CfCtx *C, CfRun &R, const unsigned long long *bb, doubl
 // wp of 100k 222 -> 183 us, DD(r) of 200k with sums 568 -> 528 us with 64 x 128; DD(r) of 1M with sums
 // 1.213 -> 1.177 ms, DD(rp, pi) of 2M 1.191 -> 1.168 ms with 64 x 256 (64 x 128: 1.207 and 1.171).  Dense cells
 // make long lists of items whatever their shape: at 1000 points per cell 64 x 256 took 2.735 ms against 2.587 with
-// 128 x 512, at 56 x 558 (survey cone, data x randoms) 64 x 512 2.70 ms, 64 x 256 2.72 and 128 x 512 2.82.
+// 128 x 512, at 56 x 558 (survey cone, data x randoms) 64 x 512 2.70 ms, 64 x 256 2.72 and 128 x 512 2.82 (both in
+// whole cells; dense_cells halves such cells since, which leaves the large shape to pinned refinements, capped
+// scratch and the densities between the two marks).
 static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
 {
     double da = 0.0, db = 0.0;      // mean points per cell, i and j side

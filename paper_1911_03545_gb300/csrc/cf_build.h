@@ -50,7 +50,7 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
 // per SM: see cf_one_build_kernel.  3-D grids without group pruning only.
 #define CFB_ITEM_STAGE 256      // work items a block collects in shared memory (stencils of more than 32 entries)
 #define CFB_ONE_THREADS 512
-#define CFB_ONE_KEYS 49152         // sort keys at most (192 KB of shared memory, beside the 25 KB item stage)
+#define CFB_ONE_KEYS 49152         // sort keys at most (192 KB of shared memory, beside the 12 KB item stage)
 struct CfOneBuild {
     const CfDevPlan *plan;
     const CfSetDesc *sets;
