@@ -294,6 +294,8 @@ static uint64_t items_guess(const CfRun &R)
 // work lists longer than this (3 GB) are made again with the largest items when their shape was left open
 static const uint32_t CF_FINE_ITEMS = 1u << 26;
 
+static const char TOO_MANY_ITEMS[] = "the work list exceeds 2^32 - 2^20 items (fewer points per call, or a coarser grid)";
+
 // the shape of the items was left open and is not the largest
 static bool may_coarsen(const CfCtx *C, const CfRun &R)
 {
@@ -956,8 +958,13 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
     }
     // work items and queue entries are indexed in 32 bits, with headroom for the grid-stride
     // loops and the work cursor's overshoot
-    if (*(const unsigned long long *)(h + OUT_ITEMS64) > CF_MAX_ENTRIES)
-        return C->fail(CF_ERR_ARG, "the work list exceeds 2^32 - 2^20 items (fewer points per call, or a coarser grid)");
+    if (*(const unsigned long long *)(h + OUT_ITEMS64) > CF_MAX_ENTRIES) {
+        // (the largest items may make a list that fits: cf_run starts again with them)
+        if (!may_coarsen(C, R)) return C->fail(CF_ERR_ARG, TOO_MANY_ITEMS);
+        R.items_cap = (uint32_t)CF_MAX_ENTRIES;
+        *retry = 2;
+        return CF_OK;
+    }
     // the audit queues every evaluated pair
     if (C->opt[CF_OPT_AUDIT] && *(const unsigned long long *)(h + OUT_EVAL) >= 0xF0000000ull)
         return C->fail(CF_ERR_ARG, "CF_OPT_AUDIT needs fewer than 2^32 - 2^28 evaluated pairs");
@@ -1072,11 +1079,14 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     CF_CU(cudaEventRecord(C->ev[0], st), "event");
     CF_TRY(cf_enqueue_build(C, R));
     if (!R.fused_items) {
-        // size the work list from the device count (one small readback)
-        CF_CU(cudaMemcpyAsync(C->hpin, (uint32_t *)C->buf[B_IOFF].p + R.nunit, 4, cudaMemcpyDeviceToHost, st),
-              "items total");
+        // size the work list from the device count (one small readback): its length, and the same in 64 bits
+        CF_CU(cudaMemcpyAsync(C->hpin, C->buf[B_OUT].p, OUT_EVAL, cudaMemcpyDeviceToHost, st), "items total");
         CF_CU(cudaStreamSynchronize(st), "items sync");
-        R.items_cap = *(const uint32_t *)C->hpin;
+        R.items_cap = *(const uint32_t *)((const char *)C->hpin + OUT_NITEMS);
+        if (*(const unsigned long long *)((const char *)C->hpin + OUT_ITEMS64) > CF_MAX_ENTRIES) {
+            if (!may_coarsen(C, R)) return C->fail(CF_ERR_ARG, TOO_MANY_ITEMS);
+            R.items_cap = (uint32_t)CF_MAX_ENTRIES;
+        }
     }
     // concentrated points make far more items than their mean density says: take the largest ones then
     auto too_fine = [&] {

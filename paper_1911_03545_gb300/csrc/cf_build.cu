@@ -861,6 +861,7 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                 for (int s0 = 0; s0 < ncand; s0 += 32) {
                     const int s = na ? s0 + (int)lane : ncand;
                     uint32_t cnt = 0, jb = 0, nb = 0, ntj = 0, tsj = 0;
+                    uint64_t cnt64 = 0;
                     bool diag = false;
                     int ct = 0, tj[3] = {0, 0, 0};
                     double delta[3] = {0.0, 0.0, 0.0};      // image of the j point: x_j + delta
@@ -925,17 +926,29 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                                         ntj = nb <= jchunk ? 1u : (nb + jchunk - 1) / jchunk;
                                         tsj = ntj == 1u ? nb : (nb + ntj - 1) / ntj;
                                     }
-                                    cnt = diag ? nti * (nti + 1) / 2 : nti * ntj;
+                                    cnt64 = cfi_item_count(nti, ntj, diag);
                                     if (GP && gp) {
-                                        cnt = 0;
+                                        cnt64 = 0;
                                         group_items(diag, jb, nb, sh32, mc, 1,
-                                                    [&](uint32_t, uint32_t, uint32_t, uint32_t, bool) { cnt++; });
+                                                    [&](uint32_t, uint32_t, uint32_t, uint32_t, bool) { cnt64++; });
                                     }
-                                    if (mode == 0) ev += cnt;
+                                    if (mode == 0) ev += cnt64;
                                 }
                             }
                         }
                     }
+                    if (__any_sync(CF_FULL, (cnt64 >> 27) != 0u)) {
+                        // (32 lanes below 2^27 stay below 2^32.)  More items than any list takes are only counted:
+                        // the host finds the total past its limit and does not use the list.
+                        uint64_t all = cnt64;
+#pragma unroll
+                        for (int o = 16; o; o >>= 1) all += __shfl_xor_sync(CF_FULL, all, o);
+                        if (all > CFI_MAX_ENTRIES) {
+                            cnt64 = 0;
+                            if (mode == 2) nres += all;
+                        }
+                    }
+                    cnt = (uint32_t)cnt64;
                     uint32_t incl = cnt;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
@@ -951,7 +964,7 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                             // a place in the stage when the items fit (the CAS only fails when another warp of the
                             // block reserved; bounded), else in the list
                             uint32_t old = *(volatile uint32_t *)&s_n;
-                            for (int t = 0; t < 64 && old + ctot <= CFB_ITEM_STAGE; t++) {
+                            for (int t = 0; t < 64 && ctot <= CFB_ITEM_STAGE - old; t++) {
                                 const uint32_t seen = atomicCAS(&s_n, old, old + ctot);
                                 if (seen == old) {
                                     r = old;
@@ -1056,18 +1069,13 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                                     vl[a] = __shfl_sync(CF_FULL, sl[a], own);
                                 }
                                 if (k0 + lane >= ctot) continue;
-                                uint32_t t = k - first, a0, b;
+                                const uint32_t t = k - first;
+                                uint32_t a0, b;
                                 if (on) {
                                     a0 = on == 1u ? t : t / on;
                                     b = t - a0 * on;
                                 } else {
-                                    // tile pairs a0 <= b, row by row: counted from the end they are a triangle
-                                    t = nti * (nti + 1u) / 2u - 1u - t;
-                                    uint32_t q = (uint32_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-                                    while (q * (q + 1u) / 2u > t) q--;
-                                    while ((q + 1u) * (q + 2u) / 2u <= t) q++;
-                                    a0 = nti - 1u - q;
-                                    b = nti - 1u - (t - q * (q + 1u) / 2u);
+                                    cfi_tile_pair(nti, t, a0, b);
                                 }
                                 const uint32_t i0 = a0 * tile, j0 = b * ots;
                                 put(cbase + k, i0, min(tile, na - i0), ojb + j0, min(ots, onb - j0), !on && a0 == b, vh, vl);

@@ -14,6 +14,7 @@
 //   cell_start[set cell offset + c] .. [c+1] delimit a cell's points.
 //   A work item is one (i tile, j range, shift) triple of a cell pair (Sec. 4.3).
 #pragma once
+#include <math.h>
 #include <stdint.h>
 
 #include "cf.h"
@@ -48,6 +49,34 @@ struct CfItem {
 };
 #define CFI_ITEM_DIAG (1u << 30)
 #define CFI_ITEM_JOBMASK 0xFFFFFu
+// most work items and recheck-queue entries of one call: both are indexed in 32 bits, and the
+// grid-stride loops and the work cursor run a few thousand past the end
+#define CFI_MAX_ENTRIES 0xFFF00000ull   // 2^32 - 2^20
+
+#ifdef __CUDACC__
+#define CFI_HD __host__ __device__ __forceinline__
+#else
+#define CFI_HD inline
+#endif
+
+// Work items of a cell pair: every tile of the i cell with every range of the j cell, or of a cell with itself the
+// tile pairs a <= b.  64 bits: a cell of 4.2 million points has 65,625 tiles of 64, whose square does not fit 32.
+CFI_HD uint64_t cfi_item_count(uint32_t nti, uint32_t ntj, bool diag)
+{
+    return diag ? (uint64_t)nti * (nti + 1ull) / 2u : (uint64_t)nti * ntj;
+}
+
+// The k-th tile pair of a cell with itself, row by row (a = 0: b = 0, 1, ..; then a = 1: b = 1, ..).  Counted from
+// the end the rows are a triangle.  k < cfi_item_count(nti, nti, true), which must fit 32 bits.
+CFI_HD void cfi_tile_pair(uint32_t nti, uint32_t k, uint32_t &a, uint32_t &b)
+{
+    const uint32_t t = (uint32_t)(cfi_item_count(nti, nti, true) - 1u - k);
+    uint32_t q = (uint32_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while ((uint64_t)q * (q + 1u) / 2u > t) q--;
+    while ((uint64_t)(q + 1u) * (q + 2u) / 2u <= t) q++;
+    a = nti - 1u - q;
+    b = nti - 1u - (uint32_t)(t - (uint64_t)q * (q + 1u) / 2u);
+}
 
 // A point set (input view + where its sorted points and cells live)
 struct CfSetDesc {
