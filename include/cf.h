@@ -150,8 +150,10 @@ const char *cf_last_error(const void *ctx);
  * kernel evaluates to the FP64 recheck instead of binning it in FP32, so the call returns the FP64
  * result of every evaluated pair: equal counts with and without it show that the FP32 path
  * misclassified nothing (the band audit; slow, and CF_ERR_ARG above 2^32 - 2^28 evaluated pairs,
- * as the queue's entries are indexed in 32 bits); CF_OPT_ITER_LIMIT is reserved and has no
- * effect (no kernel of this library waits on a flag: every device loop is bounded by its data);
+ * as the queue's entries are indexed in 32 bits); CF_OPT_ITER_LIMIT bounds how
+ * often a block of the one-launch build looks at a barrier of its grid (0, and at most, 2^22 times: two to three
+ * seconds); when it runs out the call is built again by kernels that wait for nothing, as are all later calls
+ * of the context (no other kernel of this library waits on a flag: every device loop is bounded by its data);
  * CF_OPT_WARPS and CF_OPT_REFINE are the autotuner's knobs. */
 typedef enum {
     CF_OPT_MEM_CAP = 1,

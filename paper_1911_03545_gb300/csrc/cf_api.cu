@@ -527,7 +527,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     R.one_build = R.one_build && R.nfine <= CFB_ONE_KEYS;
     if (R.one_build && C->one_blocks < 0) {
         CF_TRY(C->ensure(B_BAR, 64));
-        CF_CU(cudaMemsetAsync(C->buf[B_BAR].p, 0, 64, st), "memset barrier");
+        C->one_clean = false;
         C->one_blocks = cfb_one_init(C->num_sms);
     }
     R.one_build = R.one_build && C->one_blocks > 0;
@@ -686,7 +686,6 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
         S.zero = (uint32_t *)out;
         S.zero_words = (uint32_t)(result_bytes(R) / 4);
         S.bar = (uint32_t *)C->buf[B_BAR].p;
-        S.late = S.bar + 2;
         S.count = (uint32_t *)C->buf[B_ONECNT].p;
         S.key = (uint32_t *)C->buf[B_CELLID].p;
         S.slot = (uint32_t *)C->buf[B_SLOT].p;
@@ -703,8 +702,14 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
         S.evaluated = (unsigned long long *)(out + OUT_EVAL);
         S.total64 = (unsigned long long *)(out + OUT_ITEMS64);
         // a new buffer, or one that a launch may have left half done
-        if (!C->one_clean) CF_CU(cudaMemsetAsync(S.count, 0, C->buf[B_ONECNT].cap, st), "memset counts");
-        if (!C->capturing) C->one_clean = true;
+        if (!C->one_clean) {
+            CF_CU(cudaMemsetAsync(S.count, 0, C->buf[B_ONECNT].cap, st), "memset counts");
+            CF_CU(cudaMemsetAsync(S.bar, 0, 64, st), "memset barrier");
+            if (C->one_polls)
+                CF_CU(cudaMemcpyAsync(S.bar + 3, &C->one_polls, 4, cudaMemcpyHostToDevice, st), "poll limit");
+        }
+        // (set again once the read-back says that it finished)
+        if (!C->capturing) C->one_clean = false;
         CF_CU(cfb_one_build(S, C->one_blocks, st), "build");
         R.cbox = S.cbox;
         R.gbox = nullptr;
@@ -944,6 +949,16 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
     return CF_OK;
 }
 
+// After the stream is synchronised, before anything else of a call whose build was one launch: whether it gave up
+// at a barrier.  The context then builds with the general kernels, which wait for nothing.
+static bool one_build_gave_up(CfCtx *C)
+{
+    C->one_clean = *(const uint32_t *)((const char *)C->hpin + OUT_LATE) == 0u;
+    if (C->one_clean) return false;
+    C->one_blocks = 0;
+    return true;
+}
+
 // after the stream is synchronised: overflow checks (*retry = 1 queue, 2 items) and finalize
 int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
 {
@@ -951,11 +966,6 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
     const unsigned long long qn = *(const unsigned long long *)(h + OUT_QCOUNT);
     const uint32_t nitems = *(const uint32_t *)(h + OUT_NITEMS);
     *retry = 0;
-    if (*(const uint32_t *)(h + OUT_LATE)) {
-        C->one_blocks = -1;         // start the barrier and the key counts afresh
-        C->one_clean = false;
-        return C->fail(CF_ERR_TIMEOUT, "the build gave up waiting at a barrier");
-    }
     // work items and queue entries are indexed in 32 bits, with headroom for the grid-stride
     // loops and the work cursor's overshoot
     if (*(const unsigned long long *)(h + OUT_ITEMS64) > CF_MAX_ENTRIES) {
@@ -1102,6 +1112,7 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     for (int attempt = 0; attempt < 4; attempt++) {
         CF_TRY(cf_enqueue_count(C, R, true));
         CF_CU(cudaStreamSynchronize(st), "count sync");
+        if (attempt == 0 && R.one_build && R.fused_items && one_build_gave_up(C)) return cf_run(C, p, pts, jobs, res);
         if (R.bbox_deferred && attempt == 0) {
             // the inputs' check that a periodic call did not wait for (its plan needs only L)
             double bb[6], nd, v2;
@@ -1222,6 +1233,17 @@ cf_status cf_set_option(void *ctx, int option, int64_t value)
     if (value < 0) return (cf_status)C->fail(CF_ERR_ARG, "option values must be >= 0");
     C->opt[option] = value;
     if (option == CF_OPT_MEM_CAP) C->mem_cap = (size_t)value;
+    if (option == CF_OPT_ITER_LIMIT) {
+        // in device memory, where a captured graph reads it too
+        C->one_polls = (uint32_t)std::min<int64_t>(value, CFB_POLLS);
+        if (C->buf[B_BAR].p) {
+            DeviceGuard g(C->device);
+            cudaError_t e = cudaMemcpyAsync((uint32_t *)C->buf[B_BAR].p + 3, &C->one_polls, 4, cudaMemcpyHostToDevice,
+                                            C->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(C->stream);
+            return (cf_status)C->cuda(e, "poll limit");
+        }
+    }
     return CF_OK;
 }
 
@@ -1369,11 +1391,12 @@ cf_status cf_batch_replay(void *ctx, cf_result *outs, int ncat)
     CfRun &R = C->run;
     std::vector<CfJobResult> res;
     int retry = 0;
-    if (!bbox_within(R, (const unsigned long long *)((const char *)C->hpin + R.bb_off))) retry = 3;
+    if (R.one_build && one_build_gave_up(C)) retry = 3;
+    else if (!bbox_within(R, (const unsigned long long *)((const char *)C->hpin + R.bb_off))) retry = 3;
     else if ((rc = cf_finish(C, R, res, &retry))) return (cf_status)rc;
     if (retry) {
-        // the new data left the captured plan's box (or are not finite), or the work list or the
-        // recheck queue outgrew the captured capacity: count without the graph (same inputs,
+        // the new data left the captured plan's box (or are not finite), the work list or the
+        // recheck queue outgrew the captured capacity, or the build gave up at a barrier: count without the graph (same inputs,
         // checked and planned afresh) and drop the graph so that the next capture sizes it again
         std::vector<const cf_points *> pts;
         for (auto &q : R.pts) pts.push_back(&q);

@@ -130,8 +130,9 @@ struct CfCtx {
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     CfRun run;
     int last_grid = 0, last_warps = 0;
-    bool one_clean = false;        // the one-launch build's key counts are zero
+    bool one_clean = false;        // the last one-launch build was seen to finish: barrier words and key counts are clear
     int one_blocks = -1;           // blocks of the one-launch build (0: not taken, -1: not asked yet)
+    uint32_t one_polls = 0;        // CF_OPT_ITER_LIMIT
     int launches = 0;              // kernels launched by the current call
     uint64_t gen = 0;              // bumped whenever device or pinned scratch is reallocated
     cudaGraph_t graph = nullptr;

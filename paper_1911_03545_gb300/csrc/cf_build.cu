@@ -1136,16 +1136,20 @@ __global__ void __launch_bounds__(256, GP ? 3 : 4)
 // ---------------------------------------------------------------------------------------------
 
 // Barrier over the grid (all blocks are resident: cooperative launch).  bar[0] counts arrivals and is back at 0
-// after each barrier, bar[1] counts barriers; both start at 0 once and keep across launches.  A wait is
-// bounded: past the limit the block reports it and goes on to its end (ok = false), and the host
-// fails the call.
-__device__ __forceinline__ bool cf_grid_barrier(uint32_t *bar, uint32_t *late)
+// after each barrier, bar[1] counts barriers; both start at 0 and keep across launches that finish.  A wait is
+// bounded by bar[3] polls (0: CFB_POLLS): past the limit the block reports it in bar[2] and returns (ok = false).  The
+// blocks that gave up never arrive at the next barrier, so the others give up there: what lies between two
+// barriers only runs when every block has finished what is before them.  The host then clears the words and the
+// key counts and builds without this kernel.
+__device__ __forceinline__ bool cf_grid_barrier(uint32_t *bar)
 {
     __shared__ bool s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         s_ok = true;
         const uint32_t gen = *(volatile uint32_t *)(bar + 1);
+        uint32_t limit = *(volatile uint32_t *)(bar + 3);
+        if (!limit) limit = CFB_POLLS;
         __threadfence();
         if (atomicAdd(bar, 1u) == gridDim.x - 1) {
             *(volatile uint32_t *)bar = 0u;
@@ -1154,8 +1158,8 @@ __device__ __forceinline__ bool cf_grid_barrier(uint32_t *bar, uint32_t *late)
         } else {
             uint32_t n = 0;
             while (*(volatile uint32_t *)(bar + 1) == gen) {
-                if (++n > (1u << 22)) {
-                    atomicExch(late, 1u);
+                if (++n > limit) {
+                    atomicExch(bar + 2, 1u);
                     s_ok = false;
                     break;
                 }
@@ -1194,7 +1198,7 @@ __global__ void __launch_bounds__(CFB_ONE_THREADS, 1) cf_one_build_kernel(const 
         A.slot[p] = atomicAdd(A.count + k, 1u);
     }
     for (uint32_t i = tid; i < A.zero_words; i += nth) A.zero[i] = 0u;
-    if (!cf_grid_barrier(A.bar, A.late)) return;
+    if (!cf_grid_barrier(A.bar)) return;
     // ---- scan: each thread a run of keys, of an odd number of 16-byte words (no bank conflicts) ----
     const uint32_t nw = (A.nfine + 3u) >> 2;            // words of four keys; the last keys past nfine count zero
     uint4 *const sw = reinterpret_cast<uint4 *>(s_start);
@@ -1238,12 +1242,12 @@ __global__ void __launch_bounds__(CFB_ONE_THREADS, 1) cf_one_build_kernel(const 
         cf_scatter_point(A.plan, S, (int64_t)p - S.pbeg, k, ns, (int64_t)s_start[k] + A.slot[p], A.pt, A.pabs, A.plo,
                          A.pabslo, A.orig);
     }
-    if (!cf_grid_barrier(A.bar, A.late)) return;
+    if (!cf_grid_barrier(A.bar)) return;
     // ---- cell boxes ----
     for (uint32_t i = tid; i < A.nfine; i += nth) A.count[i] = 0u;
     if (A.cbox) {
         for (uint32_t c = warp * nct + rank; c < ncell; c += nth >> 5) cf_cell_box(A.cell_start, c, A.pt, A.cbox, nullptr);
-        if (!cf_grid_barrier(A.bar, A.late)) return;
+        if (!cf_grid_barrier(A.bar)) return;
     }
     // ---- work list ----
     cf_items_body<false>(A.plan, A.sets, A.jobs, A.stencil, A.cell_start, A.cbox, nullptr,

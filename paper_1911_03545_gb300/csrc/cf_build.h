@@ -50,6 +50,7 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
 // per SM: see cf_one_build_kernel.  3-D grids without group pruning only.
 #define CFB_ITEM_STAGE 256      // work items a block collects in shared memory (stencils of more than 32 entries)
 #define CFB_ONE_THREADS 512
+#define CFB_POLLS (1u << 22)       // of a block at a barrier: two to three seconds
 #define CFB_ONE_KEYS 49152         // sort keys at most (192 KB of shared memory, beside the 12 KB item stage)
 struct CfOneBuild {
     const CfDevPlan *plan;
@@ -60,8 +61,7 @@ struct CfOneBuild {
     uint32_t npts, nfine;
     uint32_t *zero;              // counters and histograms of the call
     uint32_t zero_words;
-    uint32_t *bar;               // the grid barrier's two words (0 before the first launch)
-    uint32_t *late;              // set when a barrier was given up
+    uint32_t *bar;               // the grid barrier's words: arrivals, barriers, given up, poll limit
     uint32_t *count;             // nfine key counts (a multiple of four of them is read): 0 before the launch, and after it
     uint32_t *key, *slot, *cell_start, *orig;
     float4 *pt, *pabs, *plo, *pabslo;
