@@ -476,6 +476,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         put(p->edges, sizeof(double) * (size_t)(p->nbins + 1));
         put(bbox, sizeof(bbox));
         put(&R.npts, sizeof(R.npts));
+        put(&nsets, sizeof(nsets));
         put(&dense_n, sizeof(dense_n));
         const int ints[6] = {any_f64 ? 1 : 0, refine[0] * 16 + refine[1] * 4 + refine[2], tile, jchunk, angular ? 1 : 0,
                              open_grid ? 1 : 0};

@@ -1,0 +1,47 @@
+"""What a context counted before, or was limited to before, decides neither the grid nor the work list of a call."""
+import numpy as np
+import pytest
+
+import gen
+from tests.gpu_util import assert_match, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def make():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    made = []
+
+    def new(**opts):
+        made.append(cf.cf_create(0, torch.cuda.current_stream()))
+        for k, v in opts.items():
+            cf.cf_set_option(made[-1], getattr(cf, k), v)
+        return made[-1]
+    yield new
+    for c in made:
+        cf.cf_destroy(c)
+
+
+@pytest.mark.parametrize("cap", [0, 1 << 30])
+def test_the_number_of_sets_is_part_of_the_plan(make, cap):
+    """64,000 points of one catalogue or of 32 in the same box: the cells' width goes by their number."""
+    import paper_1911_03545_gb300 as cf
+    p = cf.params(kind="r", edges=gen.log_edges(0.1, 5.0, 7), autocorr=True, periodic=True, box=200.0)
+    whole = gen.uniform_box(64_000, 200.0, 1, np.float32)
+    one = [cf.points(*to_dev(whole, "cuda:0", False))]
+    many = [cf.points(*to_dev(gen.uniform_box(2_000, 200.0, 5 + i, np.float32), "cuda:0", False)) for i in range(32)]
+    cells = {}
+    for name, first, second in (("one", many, one), ("many", one, many)):
+        fresh, used = make(CF_OPT_MEM_CAP=cap), make(CF_OPT_MEM_CAP=cap)
+        exp = cf.cf_batch_count(fresh, p, second)
+        cells[name] = cf.cf_get_stats(fresh)["cells"]
+        cf.cf_batch_count(used, p, first)
+        got = cf.cf_batch_count(used, p, second)
+        assert cf.cf_get_stats(used)["cells"] == cells[name]
+        for g, e in zip(got, exp):
+            assert_match(g, e)
+    assert cells["many"] < cells["one"]
