@@ -303,6 +303,16 @@ static bool may_coarsen(const CfCtx *C, const CfRun &R)
            C->opt[CF_OPT_JCHUNK] == 0;
 }
 
+static uint64_t with_headroom(uint32_t items) { return std::min<uint64_t>(CF_MAX_ENTRIES, (uint64_t)items + items / 4 + 1024); }
+
+// the current plan gets the largest items from here on; n: length of the list that did not fit (0: none that could)
+static void take_largest(CfCtx *C, uint32_t n)
+{
+    C->coarse_key = C->plan_key;
+    C->coarse_bytes = C->mem_cap && n ? sizeof(CfItem) * with_headroom(n) : 0;
+    C->items_hint = 0;
+}
+
 int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &pts,
                const std::vector<CfJobDesc> &jobs, CfRun &R)
 {
@@ -593,6 +603,12 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
                                       : C->qcap_default;
     CF_TRY(C->ensure(B_QUEUE, 16 * (size_t)R.qcap));
     CF_TRY(C->ensure_host(readback_bytes(R)));
+    if (R.coarse && C->coarse_bytes && C->mem_used - C->buf[B_ITEMS].cap + C->coarse_bytes <= C->mem_cap) {
+        // a cap raised since then has the room
+        C->coarse_key.clear();
+        R.coarse = false;
+        item_shape(R, tile, jchunk, D);
+    }
 
     {
         // one upload through pinned staging (no wait for the transfer); the angular grid's origins
@@ -1081,8 +1097,7 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     auto grow = [&](uint32_t n) {      // 1: start again
         const int rc = ensure_items(C, n);
         if (rc != CF_ERR_OOM || !may_coarsen(C, R)) return rc;
-        C->coarse_key = C->plan_key;
-        C->items_hint = 0;
+        take_largest(C, n);
         return 1;
     };
     if (R.fused_items && ensure_items(C, cap) != CF_OK) R.fused_items = false;      // no room for the headroom: count first
@@ -1104,7 +1119,7 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
         return R.items_cap > CF_FINE_ITEMS && may_coarsen(C, R);
     };
     if (!R.fused_items && too_fine()) {
-        C->coarse_key = C->plan_key;
+        take_largest(C, 0);
         return cf_run(C, p, pts, jobs, res);
     }
     int grown = grow(R.items_cap);
@@ -1123,7 +1138,7 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
         CF_TRY(cf_finish(C, R, res, &retry));
         if (!retry) {
             const uint32_t n = (uint32_t)C->stats.work_items;
-            C->items_hint = (uint32_t)std::min<uint64_t>(CF_MAX_ENTRIES, (uint64_t)n + n / 4 + 1024);
+            C->items_hint = (uint32_t)with_headroom(n);
             C->items_key = ikey;
             record_times(C, attempt == 0);
             C->stats.ms_total =
@@ -1132,8 +1147,7 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
         }
         if (retry == 1) CF_TRY(C->ensure(B_QUEUE, 16 * (size_t)R.qcap));
         if (retry == 2 && too_fine()) {
-            C->coarse_key = C->plan_key;
-            C->items_hint = 0;
+            take_largest(C, 0);
             return cf_run(C, p, pts, jobs, res);
         }
         if (retry == 2) {
@@ -1328,8 +1342,7 @@ cf_status cf_batch_capture(void *ctx, const cf_params *params, const cf_points *
     R.bbox_aux = false;
     rc = ensure_items(C, R.items_cap);
     if (rc == CF_ERR_OOM && may_coarsen(C, R)) {
-        C->coarse_key = C->plan_key;
-        C->items_hint = 0;
+        take_largest(C, R.items_cap);
         return cf_batch_capture(ctx, params, cats, ncat);
     }
     if (rc) return (cf_status)rc;

@@ -113,6 +113,8 @@ struct CfCtx {
     int smem_optin = 0;            // largest dynamic shared memory of one CTA (opt-in)
     std::string plan_key;          // inputs of the plan held in run.plan (empty: none)
     std::string coarse_key;        // plan whose work list is made of the largest items (see CF_FINE_ITEMS)
+    size_t coarse_bytes = 0;       // room, with headroom, that its list of smaller items would have needed under the cap
+                                   // (0: not for the cap's sake)
     std::string err;
     size_t mem_cap = 0, mem_used = 0;
     Buf buf[B_COUNT_];

@@ -45,3 +45,27 @@ def test_the_number_of_sets_is_part_of_the_plan(make, cap):
         for g, e in zip(got, exp):
             assert_match(g, e)
     assert cells["many"] < cells["one"]
+
+
+def test_a_larger_cap_gives_the_small_items_back(make):
+    """A list that did not fit is made with the largest items; once the cap is raised the shape is open again."""
+    import paper_1911_03545_gb300 as cf
+    p = cf.params(kind="r", edges=gen.log_edges(0.1, 10.0, 8), autocorr=True, periodic=True, box=100.0)
+    pts = cf.points(*to_dev(gen.uniform_box(60_000, 100.0, 1, np.float32), "cuda:0", False))
+    exp = cf.cf_count(make(CF_OPT_MEM_CAP=1 << 30), p, pts)
+    wide = make(CF_OPT_MEM_CAP=1 << 30)
+    cf.cf_count(wide, p, pts)
+    fine = cf.cf_get_stats(wide)["work_items"]
+    ctx = make()
+    for cap in range(1 << 21, 1 << 25, 1 << 18):
+        cf.cf_set_option(ctx, cf.CF_OPT_MEM_CAP, cap)
+        try:
+            assert_match(cf.cf_count(ctx, p, pts), exp)
+        except cf.CfError as e:
+            assert "cap" in str(e)
+            continue
+        break
+    assert cf.cf_get_stats(ctx)["work_items"] < fine
+    cf.cf_set_option(ctx, cf.CF_OPT_MEM_CAP, 1 << 30)
+    assert_match(cf.cf_count(ctx, p, pts), exp)
+    assert cf.cf_get_stats(ctx)["work_items"] == fine
