@@ -468,11 +468,17 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     bool open_grid = !angular && C->opt[CF_OPT_REFINE] == 0 && C->opt[CF_OPT_CELL_ORDER] == 0 && !C->opt[CF_OPT_AUDIT];
     for (int a = 0; a < 3; a++) open_grid = open_grid && p->refine[a] == 0;
     const double fill = open_grid ? CFI_MIN_FILL : 0.0;
-    // size of the set that a point of the call is in on average, for the cells' width (0: not halved, since the
-    // longer work list may not fit a cap on the scratch)
+    // size of the set that a point of the call is in on average
     double sq = 0.0;
     for (int s = 0; s < nsets; s++) sq += (double)pts[s]->n * (double)pts[s]->n;
-    const int64_t dense_n = C->mem_cap || R.npts == 0 ? 0 : (int64_t)(sq / (double)R.npts);
+    const int64_t typ_n = R.npts ? (int64_t)(sq / (double)R.npts) : 0;
+    // sizes of the sets of a pair, the larger and the smaller, each the least over the jobs, for the cells' width
+    // (0: not halved, since the longer work list may not fit a cap on the scratch)
+    int64_t dense_n[2] = {C->mem_cap ? 0 : R.npts, C->mem_cap ? 0 : R.npts};
+    for (const CfJobDesc &J : jobs) {
+        dense_n[0] = std::min(dense_n[0], std::max(pts[J.a]->n, pts[J.b]->n));
+        dense_n[1] = std::min(dense_n[1], std::min(pts[J.a]->n, pts[J.b]->n));
+    }
     // |v| of the point nearest the observer (its square was summed in float32 for float32 inputs:
     // a few roundings high or low)
     const double vmin = std::isfinite(vmin2) ? std::sqrt(vmin2) * (1.0 - 1e-6) : 0.0;
@@ -487,7 +493,8 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         put(bbox, sizeof(bbox));
         put(&R.npts, sizeof(R.npts));
         put(&nsets, sizeof(nsets));
-        put(&dense_n, sizeof(dense_n));
+        put(&typ_n, sizeof(typ_n));
+        put(dense_n, sizeof(dense_n));
         const int ints[6] = {any_f64 ? 1 : 0, refine[0] * 16 + refine[1] * 4 + refine[2], tile, jchunk, angular ? 1 : 0,
                              open_grid ? 1 : 0};
         put(ints, sizeof(ints));
@@ -495,7 +502,7 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
         if (key != C->plan_key) {
             C->plan_key.clear();
             rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0, vmin,
-                               fill * nsets, dense_n);
+                               fill * nsets, typ_n, dense_n[0], dense_n[1]);
             // wider cells have wider error bands: what fails with them may pass without
             if (rc && fill > 0.0)
                 rc = cfp_make_plan(p, bbox, R.npts, any_f64 ? 1 : 0, refine, 128, CFI_JMAX, &H, err, angular ? 1 : 0,

@@ -30,9 +30,14 @@
 #define CFI_CLS_AMB 0xFFu         // class: within the FP32 error band of an edge
 #define CFI_FINE_FLAG 0x100u      // coarse entry >= this: index of a fine entry + flag
 #define CFI_MIN_FILL 40.0         // points per cell and set below which the cells are widened (widen_cells)
+#define CFI_BIG_FILL 2.0          // times that: points per cell of the typical point's own set that stop the widening
 #define CFI_WIDEN_MIN 32768       // points of a call below which they are not
-#define CFI_DENSE 500.0           // points of a set per cell from which cells are halved (dense_cells)
-#define CFI_DENSE_CYL 800.0       // the same for the cylinder of rp-pi and wp
+#define CFI_DENSE 800.0           // points per cell of a pair's larger set from which cells are halved (dense_cells)
+#define CFI_DENSE_MOCKS 500.0     // the same for mocks,
+#define CFI_DENSE_FEW 500.0       // and for r where that set has at most
+#define CFI_DENSE_FEW_N (1 << 17) // so many points
+#define CFI_DENSE_I_CYL 90.0      // points per cell of the smaller set below which they are not: rp-pi and wp,
+#define CFI_DENSE_I_MOCKS 16.0    // mocks (r: those of the larger set)
 #define CFI_DENSE_MAX (1 << 24)   // points of a set above which they are not
 #define CFI_JMAX 512              // longest j range of a work item (9-bit j in a candidate)
 

@@ -287,14 +287,19 @@ void trig_range(double a0, double a1, int c, double &mn, double &mx)
 // points with 3-degree and finer cells 335 / 229 / 228 / 218 / 215 us and 418 / 319 / 295 / 276 / 308, at 100
 // 197 and 273.  Small catalogues gain nothing (DD(r) of 20k points 124 to 128 us throughout: launches and
 // latency) and keep their grid.
-void widen_cells(bool periodic, int kind, const double extent[3], double fill, int64_t npoints, int n[3])
+// A large set among many small ones has most of the pairs: the cells are not widened past twice that mark of
+// it.  Batches of one set and many small ones, whole cells / that / twice as far, by the large set's points per whole
+// cell: 300k and 30 x 3k points over (rp, pi) at 69 0.59 / 0.61 / 0.65 ms, 500k and 300 x 1k at 93 2.81 / 2.82 / 3.02, 200k and
+// 20 x 5k by r at 135 0.42 / 0.44 / 0.44, 50k and 100 x 2k at 3 0.51 / 0.44 / 0.47; without the limit 2M and 4000 x 200 by r 55 / 198.
+void widen_cells(bool periodic, int kind, const double extent[3], double fill, int64_t npoints, int64_t typ_n, int n[3])
 {
     const bool sphere = kind == CF_DD_THETA;
     if (sphere) fill *= 3.0;
+    const double big = CFI_BIG_FILL * CFI_MIN_FILL * (sphere ? 3.0 : 1.0);
     for (int it = 0; it < 1 << 20; it++) {
         double c = (double)n[0] * n[1] * n[2];
         if (sphere) c = std::min(c, 1.5 * std::pow(c, 2.0 / 3.0));
-        if ((double)npoints >= fill * c) break;
+        if ((double)npoints >= fill * c || (double)typ_n >= big * c) break;
         int a = -1;
         for (int b = 0; b < 3; b++)
             if (n[b] > (periodic ? 3 : 1) && (a < 0 || extent[b] / n[b] < extent[a] / n[a])) a = b;
@@ -304,26 +309,41 @@ void widen_cells(bool periodic, int kind, const double extent[3], double fill, i
 }
 
 // Dense cells: half as wide (refinement 2), since their groups of 32 points are then gathered against fewer
-// points out of reach, and the longer list and the build of more cells cost less than that.  By the points
-// per cell of the larger set, whole call at refinement 1 -> 2: DD(r) at 82 0.51 -> 0.75 ms, 244 0.94 -> 1.00, 364 1.26 ->
-// 1.25, 579 1.70 -> 1.57, 1000 2.48 -> 2.23, 100k points at 1,560 0.53 -> 0.41; with both sums at 244 1.98 -> 1.90 and 579
-// 3.67 -> 3.28; mocks at 140 0.80 -> 0.92, 279 1.33 -> 1.34, 558 2.37 -> 2.19.  The cylinder of rp and pi gains later:
-// DD(rp, pi) at 391 2.60 -> 2.74, 940 1.86 -> 1.76, 990 5.43 -> 5.25.  Not measured above 2M points: left alone above 16M,
-// where the longer list would also take a GB.
-bool dense_cells(bool periodic, int kind, int64_t set_n, const int n[3])
+// points out of reach, and the longer list and the build of more cells cost less than that.  That takes groups on
+// both sides: the smaller set's points per cell count too.  Whole call at refinement 1 / 2, by the points per cell of
+// the set(s), clusters and uniform points alike unless noted.  DD(r) of 4M to 8M points at 600 8.71 / 9.84 ms, 800 14.7 /
+// 15.6, of 0.5M to 2M at 520 1.10 / 1.20, 800 2.03 / 2.08, 1000 (to 40) 2.48 / 2.23, 1400 5.36 / 5.17, 2000 11.2 / 10.6, of
+// 0.1M at 600 0.35 / 0.29, 800 0.47 / 0.39, 1000 0.58 / 0.52.  DR(r) at 20 x 2000 0.91 / 2.21, 250 x 1000 2.14 / 2.35, 500 x 2000
+// 7.04 / 7.19, 1000 x 1000 6.30 / 6.36, 1000 x 2000 12.3 / 12.1.  DD(rp, pi) at 800 1.93 / 1.90, 1000 2.80 / 2.67; DR(rp, pi) at
+// 60 x 600 0.40 / 0.41, 90 x 900 0.74 / 0.69, 200 x 2000 2.72 / 2.52 (wp of uniform points 3.15 / 3.25).  Mocks at 84 0.24 /
+// 0.27, 167 0.39 / 0.43, 558 10.4 / 9.7, 6 x 558 0.55 / 0.50 (uniform 0.96 / 1.20), 19 x 558 0.99 / 0.93 (2.06 / 2.14), 56 x 558
+// 2.38 / 2.14 (4.37 / 4.47).  Sets of one batch go by the smallest: a million points with 20 x 100,000 in the same cells
+// 4.37 / 5.58, with 20 x 10,000 3.45 / 3.66.  Not measured above 8M points: left alone above 16M, where the longer list
+// would also take a GB.
+bool dense_cells(bool periodic, int kind, int64_t big_n, int64_t small_n, const int n[3])
 {
-    if (kind == CF_DD_THETA || set_n > CFI_DENSE_MAX) return false;
+    if (kind == CF_DD_THETA || big_n > CFI_DENSE_MAX) return false;
     for (int a = 0; a < 3; a++)
         if (periodic && n[a] < 3) return false;      // its minimum image is explicit, and would stay so
-    const double need = kind == CF_DD_RPPI || kind == CF_WP ? CFI_DENSE_CYL : CFI_DENSE;
-    return (double)set_n >= need * n[0] * n[1] * n[2];
+    double big = CFI_DENSE, small = 0.0;
+    if (kind == CF_DD_RPPI_MOCKS) {
+        big = CFI_DENSE_MOCKS;
+        small = CFI_DENSE_I_MOCKS;
+    } else if (kind == CF_DD_RPPI || kind == CF_WP) {
+        small = CFI_DENSE_I_CYL;
+    } else {
+        if (big_n <= CFI_DENSE_FEW_N) big = CFI_DENSE_FEW;
+        small = big;
+    }
+    const double cells = (double)n[0] * n[1] * n[2];
+    return (double)big_n >= big * cells && (double)small_n >= small * cells;
 }
 
 }  // namespace
 
 int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int f64,
                   const int refine[3], int tile, int jchunk, CfHostPlan *out, std::string &err, int angular,
-                  double vmin, double min_fill, int64_t set_n)
+                  double vmin, double min_fill, int64_t typ_n, int64_t big_n, int64_t small_n)
 {
     CfHostPlan &H = *out;
     std::memset(&H.d, 0, sizeof(H.d));
@@ -387,8 +407,8 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
         G.n[a] = std::max(G.k[a], (int)(G.n[a] * 0.8));
     }
     if (min_fill > 0.0 && npoints >= CFI_WIDEN_MIN) {
-        widen_cells(p->periodic != 0, p->kind, extent, min_fill, npoints, G.n);
-        if (G.k[0] == 1 && G.k[1] == 1 && G.k[2] == 1 && dense_cells(p->periodic != 0, p->kind, set_n, G.n))
+        widen_cells(p->periodic != 0, p->kind, extent, min_fill, npoints, typ_n, G.n);
+        if (G.k[0] == 1 && G.k[1] == 1 && G.k[2] == 1 && dense_cells(p->periodic != 0, p->kind, big_n, small_n, G.n))
             for (int a = 0; a < 3; a++) {
                 G.n[a] *= 2;
                 G.k[a] = 2;
@@ -792,7 +812,8 @@ extern "C" cf_status cf_plan_probe(const cf_params *params, const double bbox[6]
     int refine[3];
     for (int a = 0; a < 3; a++) refine[a] = params->refine[a] > 0 ? params->refine[a] : 1;
     const double fill = params->refine[0] || params->refine[1] || params->refine[2] ? 0.0 : CFI_MIN_FILL;
-    int rc = cfp_make_plan(params, bbox, npoints, any_f64, refine, 128, 512, H, err, angular, -1.0, fill, npoints);
+    int rc = cfp_make_plan(params, bbox, npoints, any_f64, refine, 128, 512, H, err, angular, -1.0, fill, npoints,
+                           npoints, npoints);
     if (rc && fill > 0.0) rc = cfp_make_plan(params, bbox, npoints, any_f64, refine, 128, 512, H, err, angular);
     if (rc) {
         delete H;

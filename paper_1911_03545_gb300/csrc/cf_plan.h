@@ -34,10 +34,13 @@ void cfp_edges(const cf_params *p, double *e2, double *pe);
 // angular = 1 (DD(theta) only): DEC bands x RA cells instead of the 3-D grid over unit vectors.
 // vmin (mocks only): a lower bound on |v| over the points (negative: derived from bbox).
 // min_fill: cells are widened until they hold this many points on average (0: as wide as the separation).
-// set_n: points of a set by which they may be halved (0: they are not).
+// typ_n: size of the set that a point of the call is in on average (holds the widening back).
+// big_n, small_n: points of the larger and of the smaller set of a pair that is counted, each the least over the
+// pairs, by which the cells may be halved (0: they are not).
 int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int f64,
                   const int refine[3], int tile, int jchunk, CfHostPlan *out, std::string &err,
-                  int angular = 0, double vmin = -1.0, double min_fill = 0.0, int64_t set_n = 0);
+                  int angular = 0, double vmin = -1.0, double min_fill = 0.0, int64_t typ_n = 0,
+                  int64_t big_n = 0, int64_t small_n = 0);
 
 // Origin of cell i on an axis starting at lo with cell width w.  For float32 coordinates x in
 // the cell, x - origin is exact in float32: the origin is a multiple of the float32 spacing at

@@ -76,3 +76,43 @@ def test_halved_cells_keep_results(kind, auto, periodic, n):
         assert_match(got, exp, True, True)
     finally:
         cf.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("kind,sizes,auto,halved", [
+    ("r", (2_000, 100_000), False, False), ("r", (100_000, 2_000), False, False), ("r", (60_000, 100_000), False, False),
+    ("r", (70_000, 100_000), False, True), ("r", (100_000, 3_000, 40_000), True, False),
+    ("r", (60_000,) + (100,) * 20, True, False), ("r", (100_000, 60_000), True, False), ("r", (100_000, 70_000), True, True),       # 480 and 560 per cell
+    ("rppi", (2_000, 100_000), False, False), ("rppi", (20_000, 100_000), False, True),
+    ("mocks", (500, 100_000), False, False), ("mocks", (5_000, 100_000), False, True)])
+def test_unequal_sets_are_not_halved(kind, sizes, auto, halved):
+    """Cells are halved where both sets of every pair fill them: a few points against dense ones, or small catalogues
+    beside a large one, keep whole cells, which the small ones do not widen either."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    from tests.gpu_util import to_dev
+    box, edges = 60.0, gen.log_edges(0.1, 12.0, 7)
+    kw = dict(kind=kind, edges=edges, autocorr=auto, periodic=kind != "mocks", box=box)
+    if kind != "r":
+        kw.update(pimax=12.0 if kind == "rppi" else 6.0, npibins=5)
+    cats = [gen.uniform_box(n, box, 3 + i, np.float32) for i, n in enumerate(sizes)]
+    if kind == "mocks":
+        for c in cats:
+            for a in (c.x, c.y, c.z):
+                a += np.float32(300.0)
+    pts = [cf.points(*to_dev(c, "cuda:0", False)) for c in cats]
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        outs, cells = [], []
+        for refine in ((0, 0, 0), (1, 1, 1)):
+            p = cf.params(refine=refine, **kw)
+            outs.append(cf.cf_batch_count(ctx, p, pts) if auto else [cf.cf_count(ctx, p, *pts)])
+            want = 2 if halved and refine[0] == 0 else 1
+            assert cf.cf_get_stats(ctx)["refine"] == [want] * 3
+            cells.append(cf.cf_get_stats(ctx)["cells"])
+        assert cells[0] == (8 if halved else 1) * cells[1]
+        for got, exp in zip(*outs):
+            assert_match(got, exp)
+    finally:
+        cf.cf_destroy(ctx)
