@@ -861,7 +861,7 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                 for (int s0 = 0; s0 < ncand; s0 += 32) {
                     const int s = na ? s0 + (int)lane : ncand;
                     uint32_t cnt = 0, jb = 0, nb = 0, ntj = 0, tsj = 0;
-                    uint64_t cnt64 = 0;
+                    uint64_t cnt64 = 0;                     // with group pruning
                     bool diag = false;
                     int ct = 0, tj[3] = {0, 0, 0};
                     double delta[3] = {0.0, 0.0, 0.0};      // image of the j point: x_j + delta
@@ -926,36 +926,41 @@ __device__ __forceinline__ void cf_items_body(const CfDevPlan *__restrict__ plan
                                         ntj = nb <= jchunk ? 1u : (nb + jchunk - 1) / jchunk;
                                         tsj = ntj == 1u ? nb : (nb + ntj - 1) / ntj;
                                     }
-                                    cnt64 = cfi_item_count(nti, ntj, diag);
+                                    cnt = max(nti, ntj) >= CFI_FEW_TILES ? CFI_MANY_ITEMS
+                                                                         : (diag ? cfi_triangle(nti) : nti * ntj);
                                     if (GP && gp) {
-                                        cnt64 = 0;
                                         group_items(diag, jb, nb, sh32, mc, 1,
                                                     [&](uint32_t, uint32_t, uint32_t, uint32_t, bool) { cnt64++; });
+                                        cnt = cnt64 < CFI_MANY_ITEMS ? (uint32_t)cnt64 : CFI_MANY_ITEMS;
                                     }
-                                    if (mode == 0) ev += cnt64;
                                 }
                             }
                         }
                     }
-                    if (__any_sync(CF_FULL, (cnt64 >> 27) != 0u)) {
-                        // (32 lanes below 2^27 stay below 2^32.)  More items than any list takes are only counted:
-                        // the host finds the total past its limit and does not use the list.
-                        uint64_t all = cnt64;
+                    uint32_t incl, ctot;
+                    auto scan = [&] {
+                        incl = cnt;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const uint32_t v = __shfl_up_sync(CF_FULL, incl, o);
+                            if ((int)lane >= o) incl += v;
+                        }
+                        ctot = __shfl_sync(CF_FULL, incl, 31);
+                    };
+                    scan();
+                    if (ctot >= CFI_MANY_ITEMS) {
+                        // in 64 bits.  More than any list takes are only counted: the host finds the total past its
+                        // limit and does not use the list.
+                        const uint64_t own = GP && gp ? cnt64 : (ntj ? cfi_item_count(nti, ntj, diag) : 0u);
+                        uint64_t all = own;
 #pragma unroll
                         for (int o = 16; o; o >>= 1) all += __shfl_xor_sync(CF_FULL, all, o);
-                        if (all > CFI_MAX_ENTRIES) {
-                            cnt64 = 0;
-                            if (mode == 2) nres += all;
-                        }
+                        cnt = all > CFI_MAX_ENTRIES ? 0u : (uint32_t)own;
+                        if (mode == 0) ev += own - cnt;
+                        if (mode == 2 && all > CFI_MAX_ENTRIES) nres += all;
+                        scan();
                     }
-                    cnt = (uint32_t)cnt64;
-                    uint32_t incl = cnt;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t v = __shfl_up_sync(CF_FULL, incl, o);
-                        if ((int)lane >= o) incl += v;
-                    }
-                    const uint32_t ctot = __shfl_sync(CF_FULL, incl, 31);
+                    if (mode == 0) ev += cnt;
                     uint32_t cbase = base + total;
                     bool staged = false;
                     if (stage) {

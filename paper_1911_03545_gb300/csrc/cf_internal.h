@@ -70,17 +70,23 @@ CFI_HD uint64_t cfi_item_count(uint32_t nti, uint32_t ntj, bool diag)
 {
     return diag ? (uint64_t)nti * (nti + 1ull) / 2u : (uint64_t)nti * ntj;
 }
+// below this many tiles and ranges a count stays below CFI_MANY_ITEMS, and 32 of those fit 32 bits
+#define CFI_FEW_TILES 8192u
+#define CFI_MANY_ITEMS (1u << 26)
+
+// q (q + 1) / 2 without a product larger than it
+CFI_HD uint32_t cfi_triangle(uint32_t q) { return ((q + 1u) >> 1) * (q | 1u); }
 
 // The k-th tile pair of a cell with itself, row by row (a = 0: b = 0, 1, ..; then a = 1: b = 1, ..).  Counted from
 // the end the rows are a triangle.  k < cfi_item_count(nti, nti, true), which must fit 32 bits.
 CFI_HD void cfi_tile_pair(uint32_t nti, uint32_t k, uint32_t &a, uint32_t &b)
 {
-    const uint32_t t = (uint32_t)(cfi_item_count(nti, nti, true) - 1u - k);
+    const uint32_t t = cfi_triangle(nti) - 1u - k;
     uint32_t q = (uint32_t)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-    while ((uint64_t)q * (q + 1u) / 2u > t) q--;
-    while ((uint64_t)(q + 1u) * (q + 2u) / 2u <= t) q++;
+    while (cfi_triangle(q) > t) q--;
+    while (cfi_triangle(q + 1u) <= t) q++;
     a = nti - 1u - q;
-    b = nti - 1u - (uint32_t)(t - (uint64_t)q * (q + 1u) / 2u);
+    b = nti - 1u - (t - cfi_triangle(q));
 }
 
 // A point set (input view + where its sorted points and cells live)
