@@ -63,3 +63,48 @@ def test_gathered_blocks(ctx, kind, n):
 def test_groups_that_share_the_warp(ctx, kind, n):
     """Last groups of up to 4, 8 and 16 points, which have several lanes per point."""
     test_gathered_blocks(ctx, kind, n)
+
+
+@pytest.mark.parametrize("kind,box,rmax,pimax", [
+    ("r", (20.0, 20.0, 20.0), 9.99, 0.0),           # one or two cells on every axis, almost to half the side
+    ("r", (90.0, 20.0, 33.0), 9.0, 0.0),            # cells on x and z, explicit on y
+    ("rppi", (40.0, 40.0, 25.0), 4.0, 12.5),        # explicit along the line of sight, to half the side
+    ("wp", (16.0, 50.0, 30.0), 7.0, 8.0)])
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("sums", [False, True])
+def test_gathering_across_an_explicit_minimum_image(kind, box, rmax, pimax, dtype, sums):
+    """Groups near and across the faces of a box whose axes have fewer than three cells: clumps on the corners, points
+    on the faces themselves and on a lattice of half the side.  An explicit minimum image rounds the unwrapped difference,
+    and the side, at the side's magnitude, so a pair's separation is off by up to 2 sqrt(3) 2^-24 L besides."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    rng = np.random.default_rng(11)
+    L = np.array(box)
+    pts = [rng.uniform(0.0, 1.0, (900, 3)) * L, (rng.normal(0.0, 0.4, (700, 3)) % L),
+           (L / 2 + rng.normal(0.0, 0.4, (700, 3))), rng.integers(0, 3, (200, 3)) * (L / 2)]
+    x = np.concatenate(pts).astype(dtype)
+    x = np.minimum(np.maximum(x, 0), L.astype(dtype))
+    cats = []
+    for part in (x, x[::3] * dtype(0.5)):
+        c = gen.uniform_box(len(part), 1.0, 1, dtype)
+        c.x, c.y, c.z = (np.ascontiguousarray(part[:, a]) for a in range(3))
+        c.w = gen.uniform_weights(len(part), 0.5, 1.5, 2).astype(dtype)
+        cats.append(c)
+    edges = gen.log_edges(0.05, rmax, 9)
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        for auto in (True, False):
+            kw = dict(autocorr=auto, periodic=True, box=box, weighted=sums, ravg=sums)
+            if pimax:
+                kw.update(pimax=pimax, npibins=5)
+            d2 = None if auto else cats[1]
+            got = gpu_count(ctx, kind, edges, cats[0], d2, **kw)
+            exp = oracle_count(kind, edges, cats[0], d2, **kw)
+            assert_match(got, exp, sums)
+            if sums:
+                tol = 1e-6 * np.asarray(exp["ravg"]) + 2.0 * 3.0 ** 0.5 * 2.0 ** -24 * max(box)
+                assert np.all(np.abs(got["ravg"] - exp["ravg"]) <= tol)
+    finally:
+        cf.cf_destroy(ctx)
