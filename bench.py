@@ -561,7 +561,7 @@ def run_gpu(args, wl, world, rank, local):
     from paper_1911_03545_gb300 import tune
     npts = wl.d1.n + (0 if wl.autocorr else wl.d2.n)
     if args.config:
-        tuned = dict(tune.DEFAULT, **_parse_config(args.config))
+        tuned = tune.pinned(tune.DEFAULT, **_parse_config(args.config))
         tune.apply(ctx, tuned)
     elif args.no_tune:
         tuned = dict(tune.DEFAULT)
@@ -968,7 +968,7 @@ def main(argv=None):
     ap.add_argument("--no-tune", action="store_true")
     ap.add_argument("--no-tune-cache", action="store_true")
     ap.add_argument("--config", default="", help="pin the launch configuration instead of tuning, "
-                    "e.g. variant=2,warps=8 (knobs of paper_1911_03545_gb300.tune)")
+                    "e.g. refine=2,warps=8 (knobs of paper_1911_03545_gb300.tune)")
     ap.add_argument("--ncat", type=int, default=256)
     ap.add_argument("--batch-min", type=float, default=5e4, help="smallest catalogue of the batch workload")
     ap.add_argument("--batch-max", type=float, default=8e5, help="largest catalogue of the batch workload")

@@ -1,7 +1,7 @@
 """Autotuner for the pair-counting launch configuration.
 
 Knobs (all results are identical across them; only speed changes):
-  variant accepted for stored configurations; the pair kernel has one form
+  variant accepted in configurations, not searched; the pair kernel has one form
   refine  sub-cells per Rmax cell (Sec. 4.2): 1, 2, 3
   warps   warps per CTA of the persistent pair kernel (CTA shape; occupancy follows from the
           shared-memory histograms): 0 (as many as fit), 12, 8, 6, 4
@@ -13,6 +13,9 @@ Knobs (all results are identical across them; only speed changes):
           largest edge of the i tile; 0 whole cells.  Searched only with tune(..., block=True): it
           lowers the evaluated-pair count, so evaluated-pair rates with and without it differ
   thetagrid DD(theta) only: 0 the 3-D grid over unit vectors, 1 declination bands x RA cells
+  open    the knobs among refine, tile and jchunk that are left to the library, which goes by the number and the
+          density of the points (wider or halved cells, item shapes); the configuration's values of those are not
+          applied.  The search starts with all three open, so the library's own choice is always a candidate
 
 The tuner times `cf_count` on the caller's own catalogue (coordinate descent from the default,
 repeated while a pass still improves, at most twice). Each candidate runs alternately with the
@@ -31,13 +34,14 @@ import time
 from . import (CF_DD_RPPI_MOCKS, CF_DD_THETA, CF_OPT_BLOCK_PRUNE, CF_OPT_CELL_PRUNE, CF_OPT_JCHUNK, CF_OPT_REFINE,
                CF_OPT_THETA_GRID, CF_OPT_TILE, CF_OPT_VARIANT, CF_OPT_WARPS, cf_count, cf_get_stats, cf_set_option)
 
-KNOBS = {"variant": [1, 2], "refine": [1, 2, 3], "warps": [0, 12, 8, 6, 4], "tile": [128, 64],
+KNOBS = {"variant": [1], "refine": [1, 2, 3], "warps": [0, 12, 8, 6, 4], "tile": [128, 64],
          "jchunk": [512, 256, 128], "noprune": [0, 1], "thetagrid": [0, 1]}
 OPT = {"variant": CF_OPT_VARIANT, "refine": CF_OPT_REFINE, "warps": CF_OPT_WARPS, "tile": CF_OPT_TILE,
        "jchunk": CF_OPT_JCHUNK, "noprune": CF_OPT_CELL_PRUNE, "block": CF_OPT_BLOCK_PRUNE,
        "thetagrid": CF_OPT_THETA_GRID}
+OPEN = ("jchunk", "refine", "tile")
 DEFAULT = {"variant": 1, "refine": 1, "warps": 0, "tile": 128, "jchunk": 512, "noprune": 0, "block": 0,
-           "thetagrid": 0}
+           "thetagrid": 0, "open": list(OPEN)}
 MARGIN = 0.01
 
 
@@ -70,13 +74,25 @@ def occupancy_class(p, npoints: int) -> int:
 
 
 def _key(device_name: str, p, npoints: int) -> str:
-    return "|".join([device_name, str(p.kind), f"w{p.c.weight}", f"r{p.c.output_ravg}", f"p{p.c.periodic}",
+    return "|".join([device_name, "open", str(p.kind), f"w{p.c.weight}", f"r{p.c.output_ravg}", f"p{p.c.periodic}",
                      f"n{len(p.edges) - 1}", f"occ{occupancy_class(p, npoints)}"])
 
 
 def apply(ctx, cfg: dict) -> None:
+    left = cfg.get("open", ())
     for k, v in cfg.items():
-        cf_set_option(ctx, OPT[k], int(v))
+        if k != "open":
+            cf_set_option(ctx, OPT[k], 0 if k in left else int(v))
+
+
+def pinned(cfg: dict, **knobs) -> dict:
+    """cfg with these knobs' values (None: left open), none of them open any more."""
+    out = dict(cfg, open=[k for k in cfg.get("open", ()) if k not in knobs])
+    for k, v in knobs.items():
+        if v is None:
+            out["open"] = sorted(out["open"] + [k])
+        out[k] = DEFAULT[k] if v is None else v
+    return out
 
 
 def reset(ctx) -> None:
@@ -127,7 +143,7 @@ def tune(ctx, p, d1, d2=None, *, device_name: str = "gpu", npoints: int = 0, rep
         cfg = cache[key]["cfg"]
         apply(ctx, cfg)
         return cfg
-    cfg = dict(DEFAULT)
+    cfg = pinned(DEFAULT)
     apply(ctx, cfg)
     _time(ctx, p, d1, d2, 1, timer)               # warm up
     best_t = _time(ctx, p, d1, d2, reps, timer)
@@ -136,11 +152,10 @@ def tune(ctx, p, d1, d2=None, *, device_name: str = "gpu", npoints: int = 0, rep
     for _ in range(passes):
         moved = False
         for knob, values in knobs_for(p, block).items():
-            for v in values:
-                if v == cfg[knob]:
+            for v in values + ([None] if knob in OPEN else []):
+                if v == (None if knob in cfg["open"] else cfg[knob]):
                     continue
-                cand = dict(cfg)
-                cand[knob] = v
+                cand = pinned(cfg, **{knob: v})
                 # the candidate against the current best, measured alternately; a move must win
                 # by a margin (a marginal win of a few repetitions is often noise)
                 tc, tb = _duel(ctx, p, d1, d2, cand, cfg, reps, timer)

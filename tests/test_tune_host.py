@@ -67,3 +67,37 @@ def test_tuner_searches_group_pruning_on_request(monkeypatch):
     tune, timer = _fake(monkeypatch, times, noise=0.002, seed=5)
     assert tune.tune(None, _P(), None, use_cache=False, timer=timer)["block"] == 0
     assert tune.tune(None, _P(), None, use_cache=False, timer=timer, block=True)["block"] == 1
+
+
+def test_tuner_keeps_what_the_library_chooses(monkeypatch):
+    # the library's own cells and item shapes 20 % faster than any pinned ones; 8 warps 5 % faster
+    def times(c):
+        return (0.8 if set(c["open"]) == {"refine", "tile", "jchunk"} else 1.0) * (0.95 if c["warps"] == 8 else 1.0)
+    tune, timer = _fake(monkeypatch, times, noise=0.002, seed=7)
+    cfg = tune.tune(None, _P(), None, use_cache=False, timer=timer)
+    assert sorted(cfg["open"]) == ["jchunk", "refine", "tile"] and cfg["warps"] == 8
+
+
+def test_tuner_pins_one_knob_and_opens_it_again(monkeypatch):
+    # refinement 2 is best while the warps are 0, the open one once they are 4
+    def times(c):
+        if c["warps"] == 4:
+            return 0.7 if "refine" in c["open"] else 0.8
+        return 0.9 if c["refine"] == 2 and "refine" not in c["open"] else 1.0
+    tune, timer = _fake(monkeypatch, times, noise=0.002, seed=8)
+    cfg = tune.tune(None, _P(), None, use_cache=False, timer=timer)
+    assert cfg["warps"] == 4 and "refine" in cfg["open"]
+
+
+def test_open_knobs_reach_the_library_as_zero(monkeypatch):
+    from paper_1911_03545_gb300 import tune
+    got = {}
+    monkeypatch.setattr(tune, "cf_set_option", lambda ctx, opt, v: got.update({opt: v}))
+    tune.apply(None, tune.DEFAULT)
+    assert set(got) == set(tune.OPT.values())
+    assert [got[tune.OPT[k]] for k in ("refine", "tile", "jchunk")] == [0, 0, 0]
+    tune.apply(None, tune.pinned(tune.DEFAULT, tile=64, warps=8))
+    assert (got[tune.OPT["tile"]], got[tune.OPT["warps"]], got[tune.OPT["refine"]]) == (64, 8, 0)
+    tune.apply(None, {"refine": 2, "tile": 128})          # a plain dict of knobs
+    assert (got[tune.OPT["refine"]], got[tune.OPT["tile"]]) == (2, 128)
+    assert tune.KNOBS["variant"] == [1]                   # nothing to search: the pair kernel has one form
