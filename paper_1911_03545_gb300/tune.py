@@ -63,9 +63,14 @@ def cache_path() -> str:
 
 
 def occupancy_class(p, npoints: int) -> int:
-    """log2 of the mean points per cell of the unrefined grid (Sec. 4.1)."""
+    """log2 of the mean points per cell of the unrefined grid (Sec. 4.1): refinement 1 pinned, since the plan of
+    an open refinement widens or halves cells by their density."""
     from . import cf_plan_probe
+    import copy
     import numpy as np
+    p = copy.copy(p)
+    p.c = type(p.c).from_buffer_copy(p.c)
+    p.c.refine[:] = [1, 1, 1]
     box = list(p.c.box) if p.c.periodic else [1.0, 1.0, 1.0]
     bb = [0.0, 0.0, 0.0] + box
     info = cf_plan_probe(p, bb, max(1, npoints))

@@ -101,3 +101,15 @@ def test_open_knobs_reach_the_library_as_zero(monkeypatch):
     tune.apply(None, {"refine": 2, "tile": 128})          # a plain dict of knobs
     assert (got[tune.OPT["refine"]], got[tune.OPT["tile"]]) == (2, 128)
     assert tune.KNOBS["variant"] == [1]                   # nothing to search: the pair kernel has one form
+
+
+@pytest.mark.parametrize("box,few,many", [(1000.0, 40_000, 320_000), (200.0, 62_000, 500_000)])
+def test_occupancy_class_is_of_whole_cells(box, few, many):
+    """Eight times the points are up to three classes further, also where the plan widens or halves the cells."""
+    from paper_1911_03545_gb300 import build, params, tune
+    build.build()
+    p = params(kind="r", edges=[0.1, 20.0], autocorr=True, periodic=True, box=box)
+    whole = int(box / 20.0) ** 3
+    a, b = tune.occupancy_class(p, few), tune.occupancy_class(p, many)
+    assert (a, b) == tuple(max(0, round(np.log2(n / whole))) for n in (few, many))
+    assert list(p.c.refine) == [0, 0, 0]                  # the caller's parameters stay as they are
