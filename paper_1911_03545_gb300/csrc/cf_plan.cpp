@@ -738,6 +738,11 @@ int cfp_make_plan(const cf_params *p, const double bbox[6], int64_t npoints, int
         D.pi_n = n;
         D.pi_inv = (float)(n / p->pimax);
         D.pi_tol = ceil32(1.01 * off / w + 16 * u * n + 4 * u);
+        if (n / p->pimax > 3e38) {
+            // the quotient does not fit float32: every value goes through the table (a pi of 1 and more is out of range)
+            D.pi_inv = 3e38f;
+            D.pi_tol = 1.0f;
+        }
     }
     // ---- lookup tables ----
     {

@@ -108,3 +108,18 @@ def test_gathering_across_an_explicit_minimum_image(kind, box, rmax, pimax, dtyp
                 assert np.all(np.abs(got["ravg"] - exp["ravg"]) <= tol)
     finally:
         cf.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("kind,npi", [("rppi", 3), ("wp", 1), ("rppi", 1)])
+@pytest.mark.parametrize("pimax,step", [(2.5e-39, 1e-39), (4e20, 1.7e20)])
+def test_pi_limits_at_the_ends_of_float32(ctx, kind, npi, pimax, step):
+    """Limits along the line of sight whose inverse, or whose square, does not fit float32."""
+    rng = np.random.default_rng(4)
+    n = 700
+    c = gen.uniform_box(n, 10.0, 3, np.float32)
+    c.z = (rng.integers(0, 6, n) * step).astype(np.float32)
+    edges, kw = gen.log_edges(0.1, 5.0, 5), dict(autocorr=True, periodic=False, pimax=pimax, npibins=npi)
+    got = gpu_count(ctx, kind, edges, c, None, **kw)
+    exp = oracle_count(kind, edges, c, None, mode="brute", **kw)
+    assert 0 < int(np.asarray(got["npairs"]).sum()) < n * n
+    assert_match(got, exp)
