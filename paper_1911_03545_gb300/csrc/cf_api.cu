@@ -66,7 +66,7 @@ int CfCtx::ensure(int b, size_t bytes)
     if (bytes == 0) bytes = 16;
     Buf &B = buf[b];
     if (B.cap >= bytes) return CF_OK;
-    size_t want = bytes + bytes / 4 + 256;
+    size_t want = tight ? bytes : bytes + bytes / 4 + 256;
     size_t used_other = mem_used - B.cap;
     if (mem_cap && used_other + want > mem_cap) {
         want = bytes;
@@ -74,13 +74,7 @@ int CfCtx::ensure(int b, size_t bytes)
             return fail(CF_ERR_OOM, "device scratch would exceed the context's memory cap (" +
                                         std::to_string(used_other + want) + " > " + std::to_string(mem_cap) + " bytes)");
     }
-    if (B.p) {
-        cudaStreamSynchronize(stream);
-        cudaFree(B.p);
-        mem_used -= B.cap;
-        B.p = nullptr;
-        B.cap = 0;
-    }
+    release(b);
     gen++;
     cudaError_t e = cudaMalloc(&B.p, want);
     if (e != cudaSuccess) {
@@ -91,6 +85,18 @@ int CfCtx::ensure(int b, size_t bytes)
     B.cap = want;
     mem_used += want;
     return CF_OK;
+}
+
+void CfCtx::release(int b)
+{
+    Buf &B = buf[b];
+    if (!B.p) return;
+    gen++;
+    cudaStreamSynchronize(stream);
+    cudaFree(B.p);
+    mem_used -= B.cap;
+    B.p = nullptr;
+    B.cap = 0;
 }
 
 int CfCtx::ensure_host(size_t bytes)
@@ -993,7 +999,7 @@ int cf_finish(CfCtx *C, CfRun &R, std::vector<CfJobResult> &res, int *retry)
     // work items and queue entries are indexed in 32 bits, with headroom for the grid-stride
     // loops and the work cursor's overshoot
     if (*(const unsigned long long *)(h + OUT_ITEMS64) > CF_MAX_ENTRIES) {
-        // (the largest items may make a list that fits: cf_run starts again with them)
+        // (the largest items may make a list that fits: the call starts again with them)
         if (!may_coarsen(C, R)) return C->fail(CF_ERR_ARG, TOO_MANY_ITEMS);
         R.items_cap = (uint32_t)CF_MAX_ENTRIES;
         *retry = 2;
@@ -1072,8 +1078,8 @@ static void record_times(CfCtx *C, bool with_build)
     cudaGetLastError();
 }
 
-int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &pts, const std::vector<CfJobDesc> &jobs,
-           std::vector<CfJobResult> &res)
+static int run_once(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &pts,
+                    const std::vector<CfJobDesc> &jobs, std::vector<CfJobResult> &res)
 {
     auto t0 = std::chrono::steady_clock::now();
     CfRun &R = C->run;
@@ -1127,15 +1133,15 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     };
     if (!R.fused_items && too_fine()) {
         take_largest(C, 0);
-        return cf_run(C, p, pts, jobs, res);
+        return run_once(C, p, pts, jobs, res);
     }
     int grown = grow(R.items_cap);
-    if (grown > 0) return cf_run(C, p, pts, jobs, res);
+    if (grown > 0) return run_once(C, p, pts, jobs, res);
     CF_TRY(grown);
     for (int attempt = 0; attempt < 4; attempt++) {
         CF_TRY(cf_enqueue_count(C, R, true));
         CF_CU(cudaStreamSynchronize(st), "count sync");
-        if (attempt == 0 && R.one_build && R.fused_items && one_build_gave_up(C)) return cf_run(C, p, pts, jobs, res);
+        if (attempt == 0 && R.one_build && R.fused_items && one_build_gave_up(C)) return run_once(C, p, pts, jobs, res);
         if (R.bbox_deferred && attempt == 0) {
             // the inputs' check that a periodic call did not wait for (its plan needs only L)
             double bb[6], nd, v2;
@@ -1152,18 +1158,45 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
                 (float)std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
             return CF_OK;
         }
-        if (retry == 1) CF_TRY(C->ensure(B_QUEUE, 16 * (size_t)R.qcap));
+        if (retry == 1) {
+            int rc = C->ensure(B_QUEUE, 16 * (size_t)R.qcap);
+            const bool again = rc == CF_ERR_OOM && may_coarsen(C, R);
+            if (again) {
+                // the shorter list of the largest items leaves more room
+                take_largest(C, R.items_cap);
+                C->release(B_ITEMS);
+                rc = run_once(C, p, pts, jobs, res);
+            }
+            if (rc == CF_ERR_OOM) C->qcap_default = 1u << 20;       // a smaller call need not have that queue
+            if (rc || again) return rc;
+        }
         if (retry == 2 && too_fine()) {
             take_largest(C, 0);
-            return cf_run(C, p, pts, jobs, res);
+            return run_once(C, p, pts, jobs, res);
         }
         if (retry == 2) {
             grown = grow(R.items_cap);
-            if (grown > 0) return cf_run(C, p, pts, jobs, res);
+            if (grown > 0) return run_once(C, p, pts, jobs, res);
             CF_TRY(grown);
         }
     }
     return C->fail(CF_ERR_INTERNAL, "recheck queue kept overflowing");
+}
+
+int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &pts, const std::vector<CfJobDesc> &jobs,
+           std::vector<CfJobResult> &res)
+{
+    int rc = run_once(C, p, pts, jobs, res);
+    if (rc != CF_ERR_OOM) return rc;
+    // the headroom of some buffers, or what earlier calls left, may have taken the room of others: once more from
+    // nothing, without headroom, so that a call fits a cap whatever came before it
+    for (int b = 0; b < B_COUNT_; b++)
+        if (b != B_BAR) C->release(b);
+    C->one_clean = false;
+    C->tight = true;
+    rc = run_once(C, p, pts, jobs, res);
+    C->tight = false;
+    return rc;
 }
 
 void cf_write_result(const cf_params *p, const CfJobResult &Q, cf_result *out)

@@ -141,6 +141,7 @@ struct CfCtx {
     cudaGraphExec_t graph_exec = nullptr;
     uint64_t graph_gen = 0;
     int graph_ncat = 0;
+    bool tight = false;            // buffers are made without headroom (a call that did not fit with it)
     bool capturing = false;
     cudaStream_t cap_stream = nullptr;   // stream used to record the batch graph
     cudaStream_t aux = nullptr;          // side stream of the deferred bbox pass (runs beside the build)
@@ -150,6 +151,7 @@ struct CfCtx {
     int fail(int status, const std::string &msg);
     int cuda(cudaError_t e, const char *what);
     int ensure(int b, size_t bytes);
+    void release(int b);
     int ensure_host(size_t bytes);
     int ensure_upload(size_t bytes);
     int ensure_aux();

@@ -69,3 +69,61 @@ def test_a_larger_cap_gives_the_small_items_back(make):
     cf.cf_set_option(ctx, cf.CF_OPT_MEM_CAP, 1 << 30)
     assert_match(cf.cf_count(ctx, p, pts), exp)
     assert cf.cf_get_stats(ctx)["work_items"] == fine
+
+
+def _fits(cf, make, cap, *calls):
+    """Whether the calls (params, points) all pass in turn, twice each, in a new context with that cap."""
+    ctx = make(CF_OPT_MEM_CAP=int(cap))
+    try:
+        for p, pts in calls:
+            for _ in range(2):
+                cf.cf_count(ctx, p, pts)
+    except cf.CfError as e:
+        assert "cap" in str(e)
+        return False
+    return True
+
+
+@pytest.mark.parametrize("n,box", [(10_000, 100.0), (60_000, 100.0)])
+def test_a_larger_cap_never_refuses_what_a_smaller_one_takes(make, n, box):
+    import paper_1911_03545_gb300 as cf
+    p = cf.params(kind="r", edges=gen.log_edges(0.1, 10.0, 10), autocorr=True, periodic=True, box=box)
+    pts = cf.points(*to_dev(gen.uniform_box(n, box, 1, np.float32), "cuda:0", False))
+    took = [_fits(cf, make, cap, (p, pts)) for cap in range(16_000_000, 28_000_000, 250_000)]
+    assert True in took and False in took
+    assert took == sorted(took)
+
+
+def test_a_call_that_fits_alone_fits_after_another(make):
+    """Dense points make a long list; the cap then has to hold more points with a short one."""
+    import paper_1911_03545_gb300 as cf
+    dense = (cf.params(kind="r", edges=gen.log_edges(0.1, 12.0, 8), autocorr=True, periodic=True, box=60.0, refine=(2, 2, 2)),
+             cf.points(*to_dev(gen.uniform_box(150_000, 60.0, 1, np.float32), "cuda:0", False)))
+    wide = (cf.params(kind="r", edges=gen.log_edges(0.1, 2.0, 8), autocorr=True, periodic=True, box=200.0),
+            cf.points(*to_dev(gen.uniform_box(400_000, 200.0, 2, np.float32), "cuda:0", False)))
+    lo, hi = 1 << 20, 1 << 28
+    while hi - lo > 1 << 17:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if _fits(cf, make, mid, wide) else (mid, hi)
+    ctx = make(CF_OPT_MEM_CAP=hi)
+    try:
+        cf.cf_count(ctx, *dense)
+    except cf.CfError as e:
+        assert "cap" in str(e)
+    assert_match(cf.cf_count(ctx, *wide), cf.cf_count(make(), *wide))
+
+
+def test_a_queue_that_does_not_fit_is_forgotten(make):
+    """A lattice whose separations all lie on edges needs a queue past the cap; the next call does not."""
+    import paper_1911_03545_gb300 as cf
+    k = np.arange(40, dtype=np.float32)
+    x, y, z = (np.ascontiguousarray(a.ravel()) for a in np.meshgrid(k, k, k, indexing="ij"))
+    grid = gen.Catalogue(x, y, z, None)
+    p = cf.params(kind="r", edges=[1.0, 2.0, 3.0, 4.0], autocorr=True, periodic=True, box=40.0)
+    small = (cf.params(kind="r", edges=gen.log_edges(0.1, 10.0, 10), autocorr=True, periodic=True, box=100.0),
+             cf.points(*to_dev(gen.uniform_box(10_000, 100.0, 1, np.float32), "cuda:0", False)))
+    ctx = make(CF_OPT_MEM_CAP=28_000_000)
+    for _ in range(2):
+        with pytest.raises(cf.CfError, match="cap"):
+            cf.cf_count(ctx, p, cf.points(*to_dev(grid, "cuda:0", False)))
+        assert_match(cf.cf_count(ctx, *small), cf.cf_count(make(), *small))
