@@ -223,6 +223,8 @@ cf_status cf_get_stats(const void *ctx, cf_stats *out);
  * chord; which = 1: |dz|, or pi^2 for mocks): classes[i] = bin index, 0xFE outside every bin, 0xFF within a band.
  * which = 2 / 3 classify with an FP32 cut at the table's tail in place of the lookup's upper clamp;
  * 0xFD there would mean an index past the table.
+ * Adding 8 to `which` (0 or 1) gives what the pair kernel decides before it asks that table: a bin, 0xFE, or 0xFC where it
+ * leaves the value to the table (0xFD there would mean that its square root's last bits change the decision).
  * Adding 4 to `which` plans DD(theta) on the angular grid (CF_OPT_THETA_GRID = 1): grid[] then
  * reports the bands, the most RA cells of a band, and 1. 
  * Grid and refinement: Sec. 4.1-4.2; bins in squared space: Sec. 4.7. */

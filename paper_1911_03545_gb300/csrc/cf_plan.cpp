@@ -801,6 +801,32 @@ uint32_t cfp_lut_class(const CfHostPlan &H, int which, uint32_t vb)
     return c;
 }
 
+// What the pair kernel decides of a value without the full tables (bin4 in cf_pair.cuh): its byte table over the
+// separation, or the multiplication by 1 / width for pi.  Its square root is off by up to 2^-22: every cell
+// between both ends counts.  0xFC: nothing decided; 0xFD: different cells decide differently.
+static uint32_t kernel_class(const CfHostPlan &H, int which, float v)
+{
+    const CfDevPlan &D = H.d;
+    const bool root = !(which & 1) || D.kind == CF_DD_RPPI_MOCKS;
+    const double s = root ? std::sqrt((double)v) : (double)v, w = root ? 1.0 / 4194304.0 : 0.0;
+    uint32_t out = 0xFCu;
+    auto decide = [&](uint32_t c) { out = out == 0xFCu || out == c ? c : 0xFDu; };
+    if (which & 1) {
+        for (int e = -1; e <= 1; e++) {
+            const float t = (float)(s * (1.0 + e * w)) * D.pi_inv;
+            const float n = std::floor(t), f = (t - n) - 0.5f;
+            if (t < 8388608.0f && !(std::fabs(f) > 0.5f - D.pi_tol)) decide(n < (float)D.pi_n ? (uint32_t)n : CFI_CLS_OUT);
+        }
+        return out;
+    }
+    // denormals count as 0
+    const double last = D.nlut8 - 1.0, low = v < 1.17549435e-38f ? 0.0 : s * (1.0 - w), high = s * (1.0 + w);
+    const int i0 = (int)std::min(last, std::nearbyint(low * D.lut8_scale)), i1 = (int)std::min(last, std::nearbyint(high * D.lut8_scale));
+    for (int i = i0; i <= i1; i++)
+        if (H.lut8[i] <= D.nb) decide(H.lut8[i] < D.nb ? H.lut8[i] : CFI_CLS_OUT);
+    return out;
+}
+
 extern "C" cf_status cf_plan_probe(const cf_params *params, const double bbox[6], int64_t npoints, int any_f64,
                                    cf_plan_info *info, double *bands_r, double *bands_p, int which,
                                    const float *values, int64_t nv, uint32_t *classes)
@@ -809,8 +835,9 @@ extern "C" cf_status cf_plan_probe(const cf_params *params, const double bbox[6]
     std::string err;
     if (cfp_check_params(params, err) != CF_OK) return CF_ERR_ARG;
     const bool rppi_like = params->kind == CF_DD_RPPI || params->kind == CF_WP || params->kind == CF_DD_RPPI_MOCKS;
-    if (which < 0 || which > 7) return CF_ERR_ARG;
+    if (which < 0 || which > 15) return CF_ERR_ARG;
     const int angular = (which & 4) ? 1 : 0;
+    const bool kernel = (which & 8) != 0;
     which &= 3;
     if ((which & 1) && !rppi_like && nv > 0) return CF_ERR_ARG;
     CfHostPlan *H = new CfHostPlan();
@@ -846,7 +873,7 @@ extern "C" cf_status cf_plan_probe(const cf_params *params, const double bbox[6]
     for (int64_t i = 0; i < nv; i++) {
         uint32_t b;
         std::memcpy(&b, values + i, 4);
-        classes[i] = cfp_lut_class(*H, which, b);
+        classes[i] = kernel ? kernel_class(*H, which, values[i]) : cfp_lut_class(*H, which, b);
     }
     delete H;
     return CF_OK;

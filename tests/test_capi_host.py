@@ -351,3 +351,51 @@ def test_tables_at_the_largest_sizes(cf, kind):
     for which in ((1, 3) if kind == "rppi" else (1,)):
         out = cf.cf_plan_probe(p, bb, 1600, which=which, values=vals)
         _check_classes(vals, out["classes"], P, out["bands_p"], 252)
+
+
+KERNEL_RULES = {
+    "clustered_r": dict(kind="r", edges=gen.log_edges(0.1, 20.0, 20), box=420.0),
+    "sums": dict(kind="r", edges=gen.log_edges(0.1, 20.0, 20), box=420.0, weighted=True, ravg=True),
+    "wide_range": dict(kind="r", edges=gen.log_edges(1e-4, 20.0, 12), box=60.0),
+    "zero_first": dict(kind="r", edges=[0.0, 0.5, 1.0, 2.0, 4.0, 8.0], box=420.0),
+    "many_bins": dict(kind="r", edges=np.linspace(0.5, 30.0, 253), box=300.0),
+    "dense_edges": dict(kind="r", edges=np.concatenate([gen.log_edges(1.0, 1.2, 30), [5.0]]), box=420.0),
+    "theta": dict(kind="theta", edges=gen.log_edges(0.001, 1.0, 20)),
+    "rppi": dict(kind="rppi", edges=gen.log_edges(0.1, 25.0, 14), box=1000.0, pimax=40.0, npibins=40),
+    "rppi_uneven": dict(kind="rppi", edges=gen.log_edges(0.1, 25.0, 14), box=100.0, pimax=37.3, npibins=252),
+    "rppi_tiny_pi": dict(kind="rppi", edges=gen.log_edges(0.1, 25.0, 14), pimax=2.5e-39, npibins=3),
+    "wp": dict(kind="wp", edges=gen.log_edges(0.1, 25.0, 14), box=1000.0, pimax=40.0, npibins=40),
+    "mocks": dict(kind="mocks", edges=gen.log_edges(0.5, 42.0, 14), pimax=42.0, npibins=42),
+}
+
+
+@pytest.mark.parametrize("f64", [False, True])
+@pytest.mark.parametrize("name", sorted(KERNEL_RULES))
+def test_kernel_rules_agree_with_the_full_tables(cf, name, f64):
+    """What the pair kernel decides by its byte table and by multiplication is what the full tables say, never inside
+    an error band and whichever way its square root rounds; it leaves them few values."""
+    kw = dict(KERNEL_RULES[name])
+    L = kw.get("box", 0.0)
+    p = cf.params(autocorr=True, periodic=L > 0, **kw)
+    bb = {"theta": [0.0, 0.0, -0.17, 1.0, 1.0, 0.5], "mocks": [300.0] * 3 + [800.0] * 3}.get(kw["kind"], [0.0] * 3 + [L or 500.0] * 3)
+    import oracle
+    E = oracle.squared_edges(kw["kind"], np.asarray(kw["edges"], dtype=np.float64))
+    rng = np.random.default_rng(2)
+    vals = np.concatenate([_values_near(E[E > 0]), (rng.uniform(0.0, 1.2, 300_000) * E[-1] ** 0.5).astype(np.float32) ** 2,
+                           np.float32([0.0, 1e-45, 1e-39, 1.2e-38, 1e-30, 3e38, np.inf])])
+    rules = [(0, vals)]
+    if "pimax" in kw:
+        n = 1 if kw["kind"] == "wp" else kw["npibins"]
+        pe = np.arange(n + 1) * (kw["pimax"] / n)
+        pi = np.concatenate([rng.uniform(0.0, 1.5, 200_000) * kw["pimax"],
+                             np.concatenate([e * (1.0 + np.arange(-40, 41) * 2.0 ** -23) for e in pe])])
+        pi = np.concatenate([pi, [0.0, 1e-45, 1.0, 1e30]]).astype(np.float32)
+        rules.append((1, pi if kw["kind"] != "mocks" else pi[pi < 1e18] ** 2))
+    for which, v in rules:
+        full = cf.cf_plan_probe(p, bb, 10 ** 6, f64, which=which, values=v)["classes"]
+        got = cf.cf_plan_probe(p, bb, 10 ** 6, f64, which=which + 8, values=v)["classes"]
+        decided = got != 0xFC
+        np.testing.assert_array_equal(got[decided], full[decided])
+        assert not np.any(full[decided] == 0xFF)
+        if which == 0 and name == "clustered_r":
+            assert np.mean(decided[-200_000:]) > 0.99
