@@ -533,6 +533,9 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     // a grid with more cells than points (most of them empty): list the units with points first,
     // so that the work-list pass does not spend a warp iteration on each empty cell
     R.live_units = R.nunit >= 65536 && R.nunit > R.npts;
+    R.nvisit = 0;
+    for (const CfJobDesc &J : jobs) R.nvisit += pts[J.a]->n;      // each point makes at most one unit of a job live
+    R.nvisit = R.live_units ? std::min(R.nunit, R.nvisit) : R.nunit;
     R.one_build = !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
     // points sort by (cell, sub-cell): the finest order whose key array stays within about
     // twice the points (and 1M keys).  The one-launch build scans the keys in shared memory, so it takes fewer:
@@ -794,7 +797,7 @@ int cf_enqueue_build(CfCtx *C, CfRun &R)
               "live units");
         C->launches += 1;
     }
-    CF_CU(cfb_items(dplan, dsets, djobs, R.d_stencil, cstart, cbox, gbox, live, nlive, R.nunit, 0, icnt, nullptr,
+    CF_CU(cfb_items(dplan, dsets, djobs, R.d_stencil, cstart, cbox, gbox, live, nlive, R.nvisit, 0, icnt, nullptr,
                     nullptr, 0, items64, nullptr, st),
           "items count");
     CF_CU(cfb_scan(icnt, ioff, R.nunit, (uint32_t *)C->buf[B_SCAN].p, (uint32_t *)(out + OUT_SCAN + 4), st,
@@ -886,12 +889,12 @@ int cf_enqueue_count(CfCtx *C, CfRun &R, bool timed)
                   "live units");
             C->launches += 1;
         }
-        CF_CU(cfb_items(dplan, dsets, djobs, R.d_stencil, cstart, R.cbox, R.gbox, live, nlive, R.nunit, 2,
+        CF_CU(cfb_items(dplan, dsets, djobs, R.d_stencil, cstart, R.cbox, R.gbox, live, nlive, R.nvisit, 2,
                         nitems_dev, nullptr, (CfItem *)C->buf[B_ITEMS].p, R.items_cap, evaluated,
                         (unsigned long long *)(out + OUT_ITEMS64), st),
               "items");
     } else {
-        CF_CU(cfb_items(dplan, dsets, djobs, R.d_stencil, cstart, R.cbox, R.gbox, live, nlive, R.nunit, 1,
+        CF_CU(cfb_items(dplan, dsets, djobs, R.d_stencil, cstart, R.cbox, R.gbox, live, nlive, R.nvisit, 1,
                         (uint32_t *)C->buf[B_ICNT].p, ioff, (CfItem *)C->buf[B_ITEMS].p, R.items_cap, evaluated,
                         nullptr, st),
               "items emit");

@@ -82,6 +82,7 @@ struct CfRun {
     bool listed = false;           // the build has written the work list and zeroed the call's counters
     bool one_build = false;        // the build is one launch (cfb_one_build)
     bool live_units = false;       // the work list visits only the units whose i cell holds points
+    int64_t nvisit = 0;            // units it visits at most
     bool bbox_aux = false;         // the bbox pass runs on the side stream: join before the readback
     // the call's plan, tables and descriptors inside the B_PLANBLK device block
     const CfDevPlan *d_plan = nullptr;

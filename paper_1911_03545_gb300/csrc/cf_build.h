@@ -36,7 +36,7 @@ cudaError_t cfb_live_units(const CfDevPlan *plan, const CfSetDesc *sets, const C
                            cudaStream_t st);
 // cbox: the boxes above, or nullptr to visit every stencil neighbour; gbox: the group boxes, or
 // nullptr for j ranges over whole cells; live / nlive: the units to visit (cfb_live_units), or
-// nullptr for all of them (with a list, mode 0 writes the counts of the listed units only: the
+// nullptr for all of them; nunits: units visited at most, for the size of the grid (with a list, mode 0 writes the counts of the listed units only: the
 // caller zeroes the rest).  mode 0: per-unit item counts
 // into counts[], their number in 64 bits added to *evaluated; mode 1: items at offsets[]; mode 2:
 // count and emit in one pass, items reserved on the counter counts[0] (zeroed by the caller), their
