@@ -116,3 +116,30 @@ def test_unequal_sets_are_not_halved(kind, sizes, auto, halved):
             assert_match(got, exp)
     finally:
         cf.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,cells", [(3, 97), (40_000, 90), (5_003, 41), (20_000, 60)])
+def test_boxes_of_mostly_empty_cells(n, cells):
+    """Grids of more cells than the boxes' pass has warps for one each (a warp then takes up to 32), and one of just
+    more: counts of the call that uses no boxes."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    box = 10.0 * cells
+    cat = gen.uniform_box(n, box, 5, np.float32)
+    for a in (cat.x, cat.y, cat.z):
+        a[n // 2:] = a[: n - n // 2] + np.float32(0.3)       # pairs, one of them in the next cell here and there
+        np.minimum(a, np.float32(box), out=a)
+    edges = gen.log_edges(0.1, 10.0, 7)
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        outs = []
+        for prune in (0, 1):
+            cf.cf_set_option(ctx, cf.CF_OPT_CELL_PRUNE, prune)
+            outs.append(gpu_count(ctx, "r", edges, cat, autocorr=True, periodic=True, box=box, refine=(1, 1, 1)))
+            assert cf.cf_get_stats(ctx)["cells"] > 65_536
+        assert int(np.asarray(outs[0]["npairs"]).sum()) > n // 2
+        assert_match(outs[0], outs[1])
+    finally:
+        cf.cf_destroy(ctx)
