@@ -39,7 +39,7 @@
 #define CFI_DENSE_I_CYL 90.0      // points per cell of the smaller set below which they are not: rp-pi and wp,
 #define CFI_DENSE_I_MOCKS 16.0    // mocks (r: those of the larger set)
 #define CFI_DENSE_MAX (1 << 24)   // points of a set above which they are not
-#define CFI_JMAX 512              // longest j range of a work item (9-bit j in a candidate)
+#define CFI_JMAX 512              // longest j range of a work item
 
 // Pair-kernel item (48 bytes, three 16-byte loads)
 struct CfItem {

@@ -20,13 +20,14 @@
 // the proven FP32 error band of an edge is not binned: the pair goes to a global queue and is
 // re-evaluated in FP64 by the recheck kernel, so counts equal the FP64 result.
 //
-// What bounds it: instruction issue for the counts (rp-pi 86 % of the slots, r 84 %, mocks 78 %; theta 82 % of the
-// shared-memory wavefronts, one histogram word per pair), for the sums the shared-memory wavefronts (72 to 77 %:
-// a 16-byte Kahan update per pair and lane, five atomics per pair of rp-pi) at the 16 warps per SM that their
+// What bounds it: instruction issue for the counts (rp-pi 86 to 88 % of the slots, wp 85 %, theta 83 % beside 81 % of the
+// shared-memory wavefronts, mocks 78 %), for the sums the shared-memory wavefronts (73 % for r, 88 % for 2M points of
+// rp-pi: a 16-byte Kahan update per pair and lane, five atomics per pair of rp-pi) at the 16 warps per SM that their
 // histograms leave.  Counting costs 17 (DD(theta), counts only) to 30 (weights and ravg) instructions per gathered
 // point and warp, gathering about 70 per 32 j points, so the layout aims at few gathered points per pair in
-// range: on the clustered catalogues 1.6 to 2.0 times the in-range pairs are formed, where whole cell pairs form 4
-// to 8 times as many.  Gathering also fills the blocks: a cell's ragged end costs at most three points of a
+// range: counted in the kernel, clustered catalogues form 1.34 (1M points, separations to 40) to 1.84 (angles) pairs per
+// pair in range, mocks 2.40 (their reach is a sphere, a counted pair lies in a cylinder), where whole cell pairs form 4
+// to 8.  Gathering also fills the blocks: a cell's ragged end costs at most three points of a
 // range's last block, and a tile's last group shares the warp (below).
 // Measured against whole cell pairs with a branch per pair in range (pair kernel, one GB300): DD(r) of
 // 1M clustered points with weights and ravg 1.546 -> 0.981 ms, counts to twice the separation
@@ -267,7 +268,8 @@ struct Warp {
     uint32_t *h_cnt;        // lane-private [nslot][32] (this and the sums: at the lane's column) or
                             // per-warp [nslot]
     float2 *h_w;            // lane-private Kahan pairs of the sum kept (interleaved when both are)
-    uint32_t *d_cnt;        // the CTA's spare row: count and sums nobody reads
+    uint32_t *d_cnt;        // the CTA's spare row: count and sums nobody reads (all of its warps write there without
+                            // atomics: what they lose of one another does not matter)
     float2 *d_w;
     double *h_wd, *h_rd;    // per-warp sums (rp-pi, mocks): FP64, or with FX two 32-bit words per slot
                             // (nslot low words, then nslot high words)
