@@ -1192,7 +1192,9 @@ int cf_run(CfCtx *C, const cf_params *p, const std::vector<const cf_points *> &p
     int rc = run_once(C, p, pts, jobs, res);
     if (rc != CF_ERR_OOM) return rc;
     // the headroom of some buffers, or what earlier calls left, may have taken the room of others: once more from
-    // nothing, without headroom, so that a call fits a cap whatever came before it
+    // nothing, without headroom, so that a call fits a cap whatever came before it.  The failed attempt may have left
+    // its bbox pass on the side stream, which reads two of the buffers.
+    if (C->aux && cudaStreamSynchronize(C->aux) != cudaSuccess) cudaGetLastError();
     for (int b = 0; b < B_COUNT_; b++)
         if (b != B_BAR) C->release(b);
     C->one_clean = false;
