@@ -276,6 +276,8 @@ static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
 
 // points of a call up to which one launch builds it
 static const int64_t CF_ONE_MAX = 262144;
+// and units times 32 stencil entries up to which, where a unit has more of them than 32
+static const int64_t CF_ONE_TURNS = 65536;
 
 // work-list capacity (48 bytes an item) up to which a call on a new plan takes an estimate instead of
 // counting the items first
@@ -537,6 +539,11 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     for (const CfJobDesc &J : jobs) R.nvisit += pts[J.a]->n;      // each point makes at most one unit of a job live
     R.nvisit = R.live_units ? std::min(R.nunit, R.nvisit) : R.nunit;
     R.one_build = !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
+    // stencils of more than 32 entries on many units are the work list's time, which the general build's more and
+    // smaller blocks balance better: refinement 2 on 13,824 / 21,952 / 46,656 cells of 3,000 points 0.98 / 0.94 / 0.84 of its
+    // speed, refinement 3 on 9,261 and 19,683 0.97 and 0.94 (on 8,000 and 3,375 cells 1.10 and 1.06)
+    const int64_t turns = (R.nst + 31) / 32;
+    if (turns > 1 && R.nunit * turns > CF_ONE_TURNS) R.one_build = false;
     // points sort by (cell, sub-cell): the finest order whose key array stays within about
     // twice the points (and 1M keys).  The one-launch build scans the keys in shared memory, so it takes fewer:
     // sub-cells of 1/8 or a whole cell in place of 1/64 there cost the pair kernel 1 % at 200k points and

@@ -1150,7 +1150,8 @@ __global__ void __launch_bounds__(256, GP ? 3 : 4)
 //     barrier orders a scan;
 //   the cells' boxes, and the key counts back to zero for the next launch (boxes by atomic minima and maxima
 //     of the points in the scatter step would save a barrier, but cost more: 16 us more at 260k points);
-//   the work list.
+//   the work list, latency-bound like the kernel of its own: 32 warps per SM as there.  With 16 it took longer than the
+//     general build from about 24,000 units on (3,000 points on 46,656 cells 98 us against 70, now 74; 32 catalogues 50 -> 43).
 // The points of all sets are one index range.  Only plain (coherent) loads read what the kernel wrote.
 // ---------------------------------------------------------------------------------------------
 
@@ -1195,8 +1196,10 @@ __global__ void __launch_bounds__(CFB_ONE_THREADS, 1) cf_one_build_kernel(const 
     extern __shared__ __align__(16) uint32_t s_start[];       // first place of each key
     __shared__ uint32_t s_warp[CFB_ONE_THREADS / 32];
     const uint32_t rank = blockIdx.x, nct = gridDim.x;
-    const uint32_t tid = rank * blockDim.x + threadIdx.x, nth = nct * blockDim.x;
+    // neighbouring warps of the index range go to different blocks: 20k points are a fifth of the threads, and
+    // a block of them after another would leave most SMs' FP64 pipes idle
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t tid = (warp * nct + rank) * 32u + lane, nth = nct * blockDim.x;
     const uint32_t ns = (uint32_t)(A.sub * A.sub * A.sub);
     const uint32_t cshift = 31u - __clz(ns), ncell = A.nfine >> cshift;
     // the set of point p: the last one that starts at or before it

@@ -49,7 +49,7 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
 // The whole build, from zeroing the call's counters to the work list, in one cooperative launch of one block
 // per SM: see cf_one_build_kernel.  3-D grids without group pruning only.
 #define CFB_ITEM_STAGE 256      // work items a block collects in shared memory (stencils of more than 32 entries)
-#define CFB_ONE_THREADS 512
+#define CFB_ONE_THREADS 1024
 #define CFB_POLLS (1u << 22)       // of a block at a barrier: two to three seconds
 #define CFB_ONE_KEYS 49152         // sort keys at most (192 KB of shared memory, beside the 12 KB item stage)
 struct CfOneBuild {

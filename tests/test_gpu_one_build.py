@@ -40,3 +40,23 @@ def test_one_launch_build_keeps_counts():
     finally:
         cf.cf_destroy(one)
         cf.cf_destroy(gen_ctx)
+
+
+@pytest.mark.parametrize("refine,whole,small", [(2, 12, True), (2, 14, False), (3, 6, True), (3, 10, False)])
+def test_refined_grids_of_many_cells_take_the_general_build(refine, whole, small):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    cat = gen.uniform_box(9_001, 10.0 * whole, 4, np.float32)
+    edges = gen.log_edges(0.1, 10.0, 8)
+    kw = dict(autocorr=True, periodic=True, box=10.0 * whole)
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        for _ in range(2):
+            got = gpu_count(ctx, "r", edges, cat, None, refine=(refine,) * 3, **kw)
+            assert cf.cf_get_stats(ctx)["cells"] == (refine * whole) ** 3
+            assert (cf.cf_get_stats(ctx)["kernel_launches"] <= 4) == small
+        assert_match(got, gpu_count(ctx, "r", edges, cat, None, refine=(1, 1, 1), **kw))
+    finally:
+        cf.cf_destroy(ctx)
