@@ -262,7 +262,10 @@ static int cf_check_bbox(CfCtx *C, CfRun &R, const unsigned long long *bb, doubl
 // make long lists of items whatever their shape: at 1000 points per cell 64 x 256 took 2.735 ms against 2.587 with
 // 128 x 512, at 56 x 558 (survey cone, data x randoms) 64 x 512 2.70 ms, 64 x 256 2.72 and 128 x 512 2.82 (both in
 // whole cells; dense_cells halves such cells since, which leaves the large shape to pinned refinements, capped
-// scratch and the densities between the two marks).
+// scratch and the densities between the two marks).  A few j points per cell against many i points make an item
+// per i tile however few they are: with 128 in place of 64 points 1M x 50k (296 x 15 per cell, uniform j) take 0.80 to 0.93
+// of the time, 108 x 5 0.73 to 0.92, 296 x 30 0.94 to 0.97, with clustered j points 0.99 to 1.05; 300k x 15k 0.87 to 0.95 and 1.02
+// to 1.05, which stay at 64.
 static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
 {
     double da = 0.0, db = 0.0;      // mean points per cell, i and j side
@@ -270,7 +273,8 @@ static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
         da = std::max(da, (double)R.sets[J.a].n / D.g.ncell);
         db = std::max(db, (double)R.sets[J.b].n / D.g.ncell);
     }
-    D.tile = tile ? tile : (da >= 400.0 || R.coarse ? 128 : 64);
+    const bool lopsided = db < 16.0 && da > 4.0 * db && R.npts > 400000;
+    D.tile = tile ? tile : (da >= 400.0 || lopsided || R.coarse ? 128 : 64);
     D.jchunk = jchunk ? jchunk : (db >= 400.0 || R.coarse ? CFI_JMAX : (R.npts <= 400000 ? 128 : 256));
 }
 

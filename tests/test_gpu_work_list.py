@@ -61,3 +61,26 @@ def test_a_list_that_does_not_fit_takes_larger_items():
     finally:
         cf.cf_destroy(free)
         cf.cf_destroy(capped)
+
+
+@pytest.mark.parametrize("n,m,large", [(420_000, 5_000, True), (5_000, 420_000, False), (300_000, 5_000, False)])
+def test_few_j_points_per_cell_take_large_tiles(n, m, large):
+    """Counts of the pinned tile, and the number of items that the open one makes."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    cats = [gen.uniform_box(k, 200.0, s, np.float32) for s, k in ((1, n), (2, m))]
+    edges = gen.log_edges(0.1, 12.0, 7)
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        outs, items = [], []
+        for tile in (0, 64, 128):
+            cf.cf_set_option(ctx, cf.CF_OPT_TILE, tile)
+            outs.append(gpu_count(ctx, "r", edges, *cats, autocorr=False, periodic=True, box=200.0))
+            items.append(cf.cf_get_stats(ctx)["work_items"])
+        assert items[0] == items[2 if large else 1]
+        for o in outs[1:]:
+            np.testing.assert_array_equal(o["npairs"], outs[0]["npairs"])
+    finally:
+        cf.cf_destroy(ctx)
