@@ -542,7 +542,14 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     R.nvisit = 0;
     for (const CfJobDesc &J : jobs) R.nvisit += pts[J.a]->n;      // each point makes at most one unit of a job live
     R.nvisit = R.live_units ? std::min(R.nunit, R.nvisit) : R.nunit;
-    R.one_build = !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
+    // A one-pass list is in the order of the blocks' arrival.  Past the units that all blocks take at once its jobs
+    // interleave, and every item of another job flushes a warp's histogram: eight catalogues of 36k to 290k points on
+    // 114,048 cells each, one pass / in order, DD(rp, pi) counts with 560 slots 8.5 / 9.3 ms, 1000 10.3 / 8.9, 2000 18.7 / 8.9,
+    // 4000 53 / 13, with both sums 560 29 / 9.9, DD(r) counts 7.3 / 7.1 (20 bins), 11.8 / 9.2 (100) and 18.9 / 11.4 (252), with both
+    // sums 34 / 7.7 (20 bins) and 927 / 70 (252).
+    R.ordered = njobs > 1 && R.nvisit > 8 * CFB_ITEM_BLOCKS &&
+                (D.weighted || D.ravg || D.nslot > (D.npi > 1 ? 768 : 32));
+    R.one_build = !R.ordered && !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
     // stencils of more than 32 entries on many units are the work list's time, which the general build's more and
     // smaller blocks balance better: refinement 2 on 13,824 / 21,952 / 46,656 cells of 3,000 points 0.98 / 0.94 / 0.84 of its
     // speed, refinement 3 on 9,261 and 19,683 0.97 and 0.94 (on 8,000 and 3,375 cells 1.10 and 1.06)
@@ -1109,9 +1116,9 @@ static int run_once(CfCtx *C, const cf_params *p, const std::vector<const cf_poi
     // write the list in one pass, and let cf_finish run the count again in the rare case that the
     // list outgrew it
     R.listed = false;
-    R.fused_items = C->items_hint && C->items_key == ikey;
+    R.fused_items = !R.ordered && C->items_hint && C->items_key == ikey;
     uint32_t cap = C->items_hint;
-    if (!R.fused_items && !C->opt[CF_OPT_AUDIT] && !C->mem_cap) {
+    if (!R.fused_items && !R.ordered && !C->opt[CF_OPT_AUDIT] && !C->mem_cap) {
         // a new plan: the size that evenly spread points would need, while that is modest; a longer list
         // only costs a second attempt, whose pair kernel the first one leaves out
         const uint64_t guess = items_guess(R);
@@ -1393,8 +1400,9 @@ cf_status cf_batch_capture(void *ctx, const cf_params *params, const cf_points *
     if (rc) return (cf_status)rc;
     CfRun &R = C->run;
     R.items_cap = R.items_cap + R.items_cap / 4 + 1024;
-    // the graph sizes its work list here (one pass writes it) and runs its own bbox pass in line
-    R.fused_items = true;
+    // the graph sizes its work list here (one pass writes it, unless it has to be in order) and runs its own bbox pass
+    // in line
+    R.fused_items = !R.ordered;
     R.bbox_aux = false;
     rc = ensure_items(C, R.items_cap);
     if (rc == CF_ERR_OOM && may_coarsen(C, R)) {

@@ -79,6 +79,7 @@ struct CfRun {
     bool angular = false;          // DD(theta) on the angular grid (needs unit vectors)
     bool bbox_deferred = false;    // periodic call planned from L: its bbox is checked after the final sync
     bool fused_items = false;      // the work list is counted and written in one pass (size known)
+    bool ordered = false;          // the work list has to come job by job: counted first, then written in order
     bool listed = false;           // the build has written the work list and zeroed the call's counters
     bool one_build = false;        // the build is one launch (cfb_one_build)
     bool live_units = false;       // the work list visits only the units whose i cell holds points

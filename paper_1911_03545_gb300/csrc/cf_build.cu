@@ -1385,7 +1385,7 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
                       cudaStream_t st)
 {
     // (a list of few units gets few blocks: 8192 blocks with their item stage cost 4,000 points on 970,299 cells 7 us of 128)
-    const int nb = blocks_for(nunits * 32, 256, 8192);
+    const int nb = blocks_for(nunits * 32, 256, CFB_ITEM_BLOCKS);
     if (gbox)
         cf_items_kernel<true><<<nb, 256, 0, st>>>(plan, sets, jobs, stencil, cell_start, cbox, gbox, live, nlive,
                                                   mode, counts, offsets, items, items_cap, evaluated, total64);

@@ -48,6 +48,7 @@ cudaError_t cfb_items(const CfDevPlan *plan, const CfSetDesc *sets, const CfJobD
                       cudaStream_t st);
 // The whole build, from zeroing the call's counters to the work list, in one cooperative launch of one block
 // per SM: see cf_one_build_kernel.  3-D grids without group pruning only.
+#define CFB_ITEM_BLOCKS 8192    // of the work-list kernel, at most; 8 units at a time each
 #define CFB_ITEM_STAGE 256      // work items a block collects in shared memory (stencils of more than 32 entries)
 #define CFB_ONE_THREADS 1024
 #define CFB_POLLS (1u << 22)       // of a block at a barrier: two to three seconds
