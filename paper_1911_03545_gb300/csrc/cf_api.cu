@@ -265,7 +265,11 @@ static int cf_check_bbox(CfCtx *C, CfRun &R, const unsigned long long *bb, doubl
 // scratch and the densities between the two marks).  A few j points per cell against many i points make an item
 // per i tile however few they are: with 128 in place of 64 points 1M x 50k (296 x 15 per cell, uniform j) take 0.80 to 0.93
 // of the time, 108 x 5 0.73 to 0.92, 296 x 30 0.94 to 0.97, with clustered j points 0.99 to 1.05; 300k x 15k 0.87 to 0.95 and 1.02
-// to 1.05, which stay at 64.
+// to 1.05, which stay at 64.  Dense cells of a small call make too few items of 128 x 512 for the 4,864 warps: whole call with
+// those / with 64 x 128, 660 x 7,700 points of one cell 96 / 671 items 240 / 140 us (over (rp, pi) with weights of both signs 2,038 /
+// 423), 30k of 64 cells 4,230 / 28,817 items 233 / 176, 100k of 125 cells 25,898 / 156,685 items 478 / 423, 200k of 343 cells
+// 49,761 / 232,401 items 568 / 565; but not where a cell makes thousands of them, which one warp writes: 8k of one cell 2,016 /
+// 7,875 items 186 / 230, 30k 27,730 / 110,215 items 818 / 1,659.
 static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
 {
     double da = 0.0, db = 0.0;      // mean points per cell, i and j side
@@ -273,9 +277,19 @@ static void item_shape(const CfRun &R, int tile, int jchunk, CfDevPlan &D)
         da = std::max(da, (double)R.sets[J.a].n / D.g.ncell);
         db = std::max(db, (double)R.sets[J.b].n / D.g.ncell);
     }
+    // items of 128 x 512 per i cell, and of all
+    double unit = 0.0, all = 0.0;
+    const double nst = std::min<double>(D.ang ? 25.0 : D.g.nstencil, D.g.ncell);       // (the others lie outside)
+    for (const CfJobDesc &J : R.jobs) {
+        const double ti = std::ceil((double)R.sets[J.a].n / D.g.ncell / 128.0), tj = std::ceil((double)R.sets[J.b].n / D.g.ncell / 512.0);
+        const double u = J.autoc ? 0.5 * ti * (ti + 1.0) + 0.5 * (nst - 1.0) * ti * tj : nst * ti * tj;
+        unit = std::max(unit, u);
+        all += u * D.g.ncell;
+    }
+    const bool few = all < 32768.0 && unit < 512.0 && !R.coarse;
     const bool lopsided = db < 16.0 && da > 4.0 * db && R.npts > 400000;
-    D.tile = tile ? tile : (da >= 400.0 || lopsided || R.coarse ? 128 : 64);
-    D.jchunk = jchunk ? jchunk : (db >= 400.0 || R.coarse ? CFI_JMAX : (R.npts <= 400000 ? 128 : 256));
+    D.tile = tile ? tile : ((da >= 400.0 && !few) || lopsided || R.coarse ? 128 : 64);
+    D.jchunk = jchunk ? jchunk : ((db >= 400.0 && !few) || R.coarse ? CFI_JMAX : (R.npts <= 400000 ? 128 : 256));
 }
 
 // points of a call up to which one launch builds it

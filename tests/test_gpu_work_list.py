@@ -84,3 +84,28 @@ def test_few_j_points_per_cell_take_large_tiles(n, m, large):
             np.testing.assert_array_equal(o["npairs"], outs[0]["npairs"])
     finally:
         cf.cf_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,m,box,small", [(660, 7_700, 8.0, True), (2_000, 0, 8.0, True), (8_000, 0, 8.0, False),
+                                           (30_000, 0, 41.0, True)])
+def test_small_dense_calls_take_small_items(n, m, box, small):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1911_03545_gb300 as cf
+    cats = [gen.uniform_box(k, box, s, np.float32) for s, k in ((1, n), (2, max(m, 1)))]
+    edges = gen.log_edges(0.1, 10.0, 7)
+    ctx = cf.cf_create(0, torch.cuda.current_stream())
+    try:
+        outs, items = [], []
+        for tile, jchunk in ((0, 0), (64, 128), (128, 512)):
+            cf.cf_set_option(ctx, cf.CF_OPT_TILE, tile)
+            cf.cf_set_option(ctx, cf.CF_OPT_JCHUNK, jchunk)
+            outs.append(gpu_count(ctx, "r", edges, cats[0], cats[1] if m else None, autocorr=not m, periodic=False,
+                                  refine=(1, 1, 1)))
+            items.append(cf.cf_get_stats(ctx)["work_items"])
+        assert items[1] != items[2] and items[0] == items[1 if small else 2]
+        for o in outs[1:]:
+            np.testing.assert_array_equal(o["npairs"], outs[0]["npairs"])
+    finally:
+        cf.cf_destroy(ctx)
