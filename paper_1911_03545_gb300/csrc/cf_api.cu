@@ -560,9 +560,13 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     // interleave, and every item of another job flushes a warp's histogram: eight catalogues of 36k to 290k points on
     // 114,048 cells each, one pass / in order, DD(rp, pi) counts with 560 slots 8.5 / 9.3 ms, 1000 10.3 / 8.9, 2000 18.7 / 8.9,
     // 4000 53 / 13, with both sums 560 29 / 9.9, DD(r) counts 7.3 / 7.1 (20 bins), 11.8 / 9.2 (100) and 18.9 / 11.4 (252), with both
-    // sums 34 / 7.7 (20 bins) and 927 / 70 (252).
-    R.ordered = njobs > 1 && R.nvisit > 8 * CFB_ITEM_BLOCKS &&
-                (D.weighted || D.ravg || D.nslot > (D.npi > 1 ? 768 : 32));
+    // sums 34 / 7.7 (20 bins) and 927 / 70 (252).  The blocks of the one-launch build take the units of all jobs at once; with sums
+    // and large histograms order is worth its launches there too: 8 x 20k points, one launch / in order, DD(r) with both sums and
+    // 20 bins 0.51 / 0.42 ms, 40 0.92 / 0.53, 252 17.3 / 2.1, 100 x 1,500 points 0.67 / 0.77, 1.10 / 1.21 and 17.0 / 6.1, DD(rp, pi) with 560
+    // slots 0.45 / 0.52, 800 0.56 / 0.59, 2400 2.05 / 0.96.
+    const int64_t hist = (int64_t)D.nslot * (D.npi > 1 ? 1 : 32);       // words of a warp's counts
+    const bool heavy = (D.weighted || D.ravg) && hist > 1200;
+    R.ordered = njobs > 1 && (heavy || (R.nvisit > 8 * CFB_ITEM_BLOCKS && (D.weighted || D.ravg || hist > 768)));
     R.one_build = !R.ordered && !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
     // stencils of more than 32 entries on many units are the work list's time, which the general build's more and
     // smaller blocks balance better: refinement 2 on 13,824 / 21,952 / 46,656 cells of 3,000 points 0.98 / 0.94 / 0.84 of its

@@ -273,22 +273,23 @@ def test_mocks_batched_and_served(cf):
             np.testing.assert_allclose(r["ravg"], e["ravg"], rtol=TOL)
 
 
-@pytest.mark.parametrize("weighted,nbins,npi", [(True, 6, 4), (False, 20, 50), (False, 6, 4)])
-def test_batches_of_many_units_repeat_and_replay(cf, weighted, nbins, npi):
-    """More units than the work-list kernel takes at once: the list comes job by job (or not, with few slots) in the
-    first call, in the next ones and in a graph, with the results of each catalogue alone."""
+@pytest.mark.parametrize("weighted,nbins,npi,box", [(True, 6, 4, 62.0), (False, 20, 50, 62.0), (False, 6, 4, 62.0),
+                                                    (True, 40, 40, 20.0)])
+def test_batches_of_many_units_repeat_and_replay(cf, weighted, nbins, npi, box):
+    """More units than the work-list kernel takes at once, or histograms that are long to flush: the list comes job by
+    job (or not, with few slots) in the first call, in the next ones and in a graph, with the results of each catalogue alone."""
     import torch
     sizes = [9_000, 30, 4_001]
-    cats = [gen.uniform_box(n, 62.0, 40 + i, np.float32) for i, n in enumerate(sizes)]
+    cats = [gen.uniform_box(n, box, 40 + i, np.float32) for i, n in enumerate(sizes)]
     for i, c in enumerate(cats):
         c.w = gen.uniform_weights(c.n, 0.5, 1.5, 60 + i)
-    p = cf.params(kind="rppi", edges=gen.log_edges(0.1, 2.0, nbins), autocorr=True, periodic=True, box=62.0, pimax=2.0,
+    p = cf.params(kind="rppi", edges=gen.log_edges(0.1, 2.0, nbins), autocorr=True, periodic=True, box=box, pimax=2.0,
                   npibins=npi, weighted=weighted, ravg=weighted, refine=(1, 1, 1))
     pts = [cf.points(*to_dev(c, "cuda:0", weighted)) for c in cats]
     ctx = cf.cf_create(0, torch.cuda.current_stream())
     try:
         alone = [cf.cf_count(ctx, p, q) for q in pts]
-        assert 3 * cf.cf_get_stats(ctx)["cells"] > 65_536
+        assert (3 * cf.cf_get_stats(ctx)["cells"] > 65_536) == (box > 60.0)
         runs = [cf.cf_batch_count(ctx, p, pts) for _ in range(3)]
         cf.cf_batch_capture(ctx, p, pts)
         runs += [cf.cf_batch_replay(ctx, p, 3) for _ in range(2)]
@@ -296,7 +297,7 @@ def test_batches_of_many_units_repeat_and_replay(cf, weighted, nbins, npi):
         keep = [[t.clone() for t in q.keep if t is not None] for q in pts]
         for q in pts:
             for t in q.keep[:3]:
-                t.copy_(62.0 - t)
+                t.copy_(box - t)
         moved = cf.cf_batch_replay(ctx, p, 3)
         for got, exp in zip(moved, alone):
             assert abs(int(got["npairs"].sum()) - int(exp["npairs"].sum())) <= 0.01 * int(exp["npairs"].sum()) + 4
