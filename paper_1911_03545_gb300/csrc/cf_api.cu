@@ -307,6 +307,7 @@ static uint64_t items_guess(const CfRun &R)
     double n = 4096.0;
     for (const CfJobDesc &J : R.jobs) {
         const double na = (double)R.sets[J.a].n, nb = (double)R.sets[J.b].n, nc = (double)D.g.ncell;
+        if (na == 0.0 || nb == 0.0) continue;
         const double cells = std::min(nc, na);      // i cells that may hold points
         const double pairs = D.ang ? 25.0 : (J.autoc ? 0.5 * (R.nst + 1) : (double)R.nst);
         const double ti = na / cells / D.tile, tj = nb / std::min(nc, std::max(1.0, nb)) / D.jchunk;
@@ -565,7 +566,8 @@ int cf_prepare(CfCtx *C, const cf_params *p, const std::vector<const cf_points *
     // 20 bins 0.51 / 0.42 ms, 40 0.92 / 0.53, 252 17.3 / 2.1, 100 x 1,500 points 0.67 / 0.77, 1.10 / 1.21 and 17.0 / 6.1, DD(rp, pi) with 560
     // slots 0.45 / 0.52, 800 0.56 / 0.59, 2400 2.05 / 0.96.
     const int64_t hist = (int64_t)D.nslot * (D.npi > 1 ? 1 : 32);       // words of a warp's counts
-    const bool heavy = (D.weighted || D.ravg) && hist > 1200;
+    // (not for a list of an item or two per warp: a count pass costs about 30 us)
+    const bool heavy = njobs > 1 && (D.weighted || D.ravg) && hist > 1200 && items_guess(R) > 16384;
     R.ordered = njobs > 1 && (heavy || (R.nvisit > 8 * CFB_ITEM_BLOCKS && (D.weighted || D.ravg || hist > 768)));
     R.one_build = !R.ordered && !D.ang && !R.live_units && R.npts <= CF_ONE_MAX && C->opt[CF_OPT_BLOCK_PRUNE] == 0;
     // stencils of more than 32 entries on many units are the work list's time, which the general build's more and
